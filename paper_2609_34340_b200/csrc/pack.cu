@@ -1,20 +1,12 @@
 // vp_pack: stage one rank's routed token rows in activation x destination order
 // (Section 5, "Device-resident buffer layout").
 //
-// Four kernels on the caller's stream:
-//   count + plan : per 256-copy chunk, how many copies go to each destination rank; one more
-//           block builds, meanwhile, the rank's segment table: for every destination, the
-//           activations that send to it, with the stream position they start at and their
-//           first staged row (from the plan's send offsets)
-//   scan  : exclusive scan of the chunk counts over chunks, one warp per destination
-//   map   : stable position of every copy inside its destination's stream ->
-//           staged row (binary search in the segment table); writes src_map
-//   copy  : token-major: every source row is read ONCE and written to each of
-//           its staged rows.  Rows travel global -> shared -> global as bulk
-//           asynchronous copies (TMA): one warp per CTA drives a ring of
-//           shared-memory stages, an mbarrier per stage signals the load, and
-//           the up to topk stores of a token form one bulk group whose read
-//           completion frees the stage.
+// Up to kSmallItems routed copies: one kernel (pack_small_kernel).  More: three kernels on the caller's stream:
+//   count : per chunk of copies a histogram of destination ranks; one more CTA builds, meanwhile, the rank's run table
+//           (for every destination the activations that send to it, with the stream position they start at and their
+//           first staged row) from the plan's send offsets
+//   map   : stable position of every copy inside its destination's stream -> staged row; writes src_map and the status
+//   copy  : token-major: every source row is read ONCE and written to each of its staged rows (row_copy.cuh)
 #include <cuda_runtime.h>
 
 #include "row_copy.cuh"
@@ -22,19 +14,24 @@
 
 namespace {
 
-constexpr int kItems = 8;                  // 32-copy rounds per warp chunk
-constexpr int kChunk = 32 * kItems;        // copies per warp chunk
-constexpr int kWarpsPerBlock = 8;
+struct PackArgs {
+    const int32_t* n_steps;
+    const int16_t* lane_dst;
+    const int64_t *lane_bytes, *send_off;
+    int N, rank, k_max, T, topk, epr;
+    const int32_t* idx;
+    int64_t row_bytes, capacity;
+    int32_t *src_map, *status;
+};
 
 struct PackWs {
-    int32_t* flags;      // [0] abort, [1] n_segments
+    int32_t* flags;      // [0] abort, [1] status bits of the run table
     int32_t* hist;       // [n_chunks][N] copies of each chunk per destination
-    int32_t* base;       // [n_chunks][N] copies to that destination in earlier chunks
-    int32_t* len;        // [N] routed copies per destination
-    int32_t* planned;    // [N] rows the plan sends to each destination
-    int32_t* seg_ptr;    // [N+1]
-    int32_t* seg_start;  // [k_max] stream position of a segment's first row
-    int32_t* seg_row;    // [k_max] staged row of a segment's first row
+    int32_t* bad;        // [n_chunks] status bits of each chunk
+    int32_t* total;      // [N] rows the plan sends to each destination
+    int32_t* ptr;        // [N+1] \ run table (see Runs)
+    int32_t* start;      // [k_max] |
+    int32_t* row;        // [k_max] /
     int32_t* dst_row;    // [T*topk] staged row of each copy, -1 = not staged
     size_t bytes;
 };
@@ -42,199 +39,195 @@ struct PackWs {
 PackWs carve(void* base, int N, int T, int topk, int k_max) {
     PackWs w;
     size_t o = 0;
-    auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (char*)base + at; };
-    long long E = (long long)T * topk;
-    int n_chunks = (int)((E + kChunk - 1) / kChunk);
-    w.flags = (int32_t*)take(256);
-    w.hist = (int32_t*)take((size_t)n_chunks * N * 4);
-    w.base = (int32_t*)take((size_t)n_chunks * N * 4);
-    w.len = (int32_t*)take((size_t)N * 4);
-    w.planned = (int32_t*)take((size_t)N * 4);
-    w.seg_ptr = (int32_t*)take((size_t)(N + 1) * 4);
-    w.seg_start = (int32_t*)take((size_t)k_max * 4);
-    w.seg_row = (int32_t*)take((size_t)k_max * 4);
-    w.dst_row = (int32_t*)take((size_t)E * 4);
+    auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (int32_t*)((char*)base + at); };
+    const long long E = (long long)T * topk, chunk = chunk_items(E, N);
+    const size_t n_chunks = (size_t)((E + chunk - 1) / chunk);
+    w.flags = take(256);
+    w.hist = take(n_chunks * N * 4);
+    w.bad = take(n_chunks * 4);
+    w.total = take((size_t)N * 4);
+    w.ptr = take((size_t)(N + 1) * 4);
+    w.start = take((size_t)k_max * 4);
+    w.row = take((size_t)k_max * 4);
+    w.dst_row = take((size_t)E * 4);
     w.bytes = o;
     return w;
 }
 
-__device__ __forceinline__ int dest_of(int x, int experts_per_rank, int N, int rank) {
-    // destination rank of a routed copy, or -1 if it is not staged (dropped, local, out of range)
+// Destination rank of a routed copy, or -1 if it is not staged (dropped, local, out of range: that one sets `bad`).
+__device__ __forceinline__ int dest_of(int x, const PackArgs& a, int& bad) {
     if (x < 0) return -1;
-    int j = x / experts_per_rank;
-    return (j >= N || j == rank) ? -1 : j;
+    const int j = (int)((unsigned)x / (unsigned)a.epr);
+    if (j >= a.N) { bad = VP_ST_PACK_MISMATCH; return -1; }
+    return j == a.rank ? -1 : j;
 }
 
-__device__ __forceinline__ void count_block(const int32_t* __restrict__ idx, long long E, int N, int rank, int experts_per_rank,
-                                            int32_t* __restrict__ hist, int32_t* __restrict__ status) {
-    __shared__ int wh[kWarpsPerBlock][VP_MAX_N];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long chunk = (long long)blockIdx.x * kWarpsPerBlock + warp;
-    const long long e0 = chunk * kChunk;
-    if (e0 >= E) return;
-    for (int j = lane; j < N; j += 32) wh[warp][j] = 0;
-    __syncwarp();
-    bool bad = false;
-    for (int it = 0; it < kItems; it++) {
-        long long e = e0 + it * 32 + lane;
-        if (e < E) {
-            int x = idx[e];
-            int j = dest_of(x, experts_per_rank, N, rank);
-            if (x >= 0 && x / experts_per_rank >= N) bad = true;
-            if (j >= 0) atomicAdd(&wh[warp][j], 1);
-        }
-    }
-    __syncwarp();
-    for (int j = lane; j < N; j += 32) hist[chunk * N + j] = wh[warp][j];
-    if (bad) atomicOr(status, VP_ST_PACK_MISMATCH);
+__device__ __forceinline__ int steps_in_use(const PackArgs& a) { return min(max(*a.n_steps, 0), a.k_max); }
+
+// Status bits of the run table, the same in every thread.
+__device__ __forceinline__ int pack_runs(const PackArgs& a, int K, Runs out, int* cnt, int* scratch) {
+    int bad = 0;
+    build_runs(K, a.N, [&](int k, int& j, int& rows, int& row0) {
+        const size_t at = (size_t)k * a.N + a.rank;
+        const int64_t bytes = a.lane_bytes[at];
+        j = a.lane_dst[at];
+        if (j >= a.N) j = -1;
+        rows = (int)(bytes / a.row_bytes);
+        row0 = (int)(a.send_off[at] / a.row_bytes);
+        if (j >= 0 && bytes % a.row_bytes) bad = VP_ST_PACK_MISMATCH;
+    }, out, cnt, scratch);
+    if (threadIdx.x == 0 && out.total[a.rank] != 0) bad = VP_ST_PACK_MISMATCH;
+    return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
 }
 
-// One block of VP_MAX_N threads.  Thread j owns destination j; the rank's column of the plan is staged
-// through shared memory a tile of steps at a time so that its global loads run in parallel.
-__device__ __forceinline__ void segments_block(const int32_t* __restrict__ n_steps_p, const int16_t* __restrict__ lane_dst,
-                                               const int64_t* __restrict__ lane_bytes, const int64_t* __restrict__ send_off, int N,
-                                               int rank, int k_max, int64_t row_bytes, int64_t capacity_bytes, PackWs w,
-                                               int32_t* __restrict__ status) {
-    __shared__ int s_cnt[VP_MAX_N + 1];
-    __shared__ int16_t t_dst[VP_MAX_N];
-    __shared__ int32_t t_rows[VP_MAX_N], t_base[VP_MAX_N];
-    const int j = threadIdx.x, NT = blockDim.x;
-    int K = *n_steps_p;
-    if (K > k_max) K = k_max;
-    if (K < 0) K = 0;
-    // pass 1: how many activations send to each destination
-    int cnt = 0;
-    for (int k0 = 0; k0 < K; k0 += NT) {
-        const int k = k0 + j;
-        t_dst[j] = k < K ? lane_dst[(size_t)k * N + rank] : (int16_t)-1;
-        __syncthreads();
-        if (j < N) {
-            const int n = min(NT, K - k0);
-            for (int i = 0; i < n; i++) cnt += (t_dst[i] == j);
-        }
-        __syncthreads();
-    }
-    if (j < N) s_cnt[j] = cnt;
+// ---- one launch -------------------------------------------------------------------------------------------------
+
+struct PackSmall { int cnt, hist, total, ptr, start, row, src, dst, scratch, ints; };   // offsets in ints
+__host__ __device__ inline PackSmall pack_small_layout(int N, int k_max) {
+    PackSmall L;
+    int o = 0;
+    L.cnt = o;     o += N;
+    L.hist = o;    o += N;
+    L.total = o;   o += N;
+    L.ptr = o;     o += N + 1;
+    L.start = o;   o += k_max;
+    L.row = o;     o += k_max;
+    L.src = o;     o += kSmallOwn;
+    L.dst = o;     o += kSmallOwn;
+    L.scratch = o; o += runs_scratch_ints(N);
+    L.ints = o;
+    return L;
+}
+
+// Decode steps and prefill chunks of a few thousand tokens.  Bound by latency (launch, two trips to L2 for plan and routing,
+// one for the rows), then by HBM writes.  CTA c owns the tokens [c T / grid, (c + 1) T / grid) -- or one of `pieces` column
+// ranges of one token while there are fewer tokens than SMs -- and finds their places by itself: the run table from the
+// plan, and how many copies to each destination come before its own.  The last CTA thereby sees every copy and writes the
+// status.  Replaces two memsets and four kernels: 128 tokens x top-8 of 14,336 B 30 -> 18 us a call.
+template <typename V>
+__global__ void __launch_bounds__(kIdxThreads, 2)
+pack_small_kernel(PackArgs a, const char* __restrict__ rows, char* __restrict__ staged, int pieces) {
+    extern __shared__ int sm[];
+    const PackSmall L = pack_small_layout(a.N, a.k_max);
+    int* const hist = sm + L.hist;
+    const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
+    const int t0 = (int)((long long)a.T * c / n_cta), t1 = (int)((long long)a.T * (c + 1) / n_cta);
+    for (int j = tid; j < a.N; j += kIdxThreads) hist[j] = 0;
+    grid_wait();
+    const int K = steps_in_use(a);
+    const bool over = a.send_off[(size_t)K * a.N + a.rank] > a.capacity;
     __syncthreads();
-    if (j == 0) {
-        int run = 0;
-        for (int d = 0; d < N; d++) { int v = s_cnt[d]; s_cnt[d] = run; run += v; }
-        s_cnt[N] = run;
-        w.seg_ptr[N] = run;
-        if (send_off[(size_t)K * N + rank] > capacity_bytes) { atomicOr(status, VP_ST_PACK_CAPACITY); w.flags[0] = 1; }
-    }
-    __syncthreads();
-    // pass 2: the segments of each destination: stream position and staged row where each one starts
-    int p = j < N ? s_cnt[j] : 0;
-    long long cum = 0;
-    bool bad = false;
-    if (j < N) w.seg_ptr[j] = p;
-    for (int k0 = 0; k0 < K; k0 += NT) {
-        const int k = k0 + j;
-        if (k < K) {
-            const int64_t bytes = lane_bytes[(size_t)k * N + rank];
-            t_dst[j] = lane_dst[(size_t)k * N + rank];
-            t_rows[j] = (int32_t)(bytes / row_bytes);
-            t_base[j] = (int32_t)(send_off[(size_t)k * N + rank] / row_bytes);
-            if (t_dst[j] >= 0 && bytes % row_bytes) bad = true;
-        } else {
-            t_dst[j] = -1;
-        }
-        __syncthreads();
-        if (j < N) {
-            const int n = min(NT, K - k0);
-            for (int i = 0; i < n; i++) {
-                if (t_dst[i] != j) continue;
-                w.seg_start[p] = (int32_t)cum;
-                w.seg_row[p] = t_base[i];
-                cum += t_rows[i];
-                p++;
-            }
-        }
-        __syncthreads();
-    }
-    if (j < N) {
-        w.planned[j] = (int32_t)cum;
-        if (j == rank && cum != 0) bad = true;
-    }
-    if (bad) atomicOr(status, VP_ST_PACK_MISMATCH);
-}
-
-// The count blocks and, as the last block of the grid, the segment table: the two need nothing from each other.
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-pack_count_plan_kernel(const int32_t* __restrict__ idx, long long E, int N, int rank, int experts_per_rank,
-                       const int32_t* __restrict__ n_steps_p, const int16_t* __restrict__ lane_dst,
-                       const int64_t* __restrict__ lane_bytes, const int64_t* __restrict__ send_off, int k_max,
-                       int64_t row_bytes, int64_t capacity_bytes, PackWs w, int32_t* __restrict__ status) {
-    static_assert(kWarpsPerBlock * 32 == VP_MAX_N, "the segment block has one thread per destination");
-    if (blockIdx.x == gridDim.x - 1) segments_block(n_steps_p, lane_dst, lane_bytes, send_off, N, rank, k_max, row_bytes, capacity_bytes, w, status);
-    else count_block(idx, E, N, rank, experts_per_rank, w.hist, status);
-}
-
-// Exclusive scan of the chunk counts, per destination: one warp per destination, 32 chunks per step; then the
-// routed copies of a destination must be as many as the plan sends there.
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-pack_scan_kernel(int N, int rank, int n_chunks, PackWs w, int32_t* __restrict__ status) {
-    const int lane = threadIdx.x & 31, d = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (d >= N) return;
-    int run = 0;
-    const int32_t* __restrict__ in = w.hist;
-    int32_t* __restrict__ out = w.base;
+    int bad = 0;
 #pragma unroll 4
-    for (int b0 = 0; b0 < n_chunks; b0 += 32) {
-        const int c = b0 + lane;
-        const int v = c < n_chunks ? in[(size_t)c * N + d] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (c < n_chunks) out[(size_t)c * N + d] = run + incl - v;
-        run += __shfl_sync(0xffffffffu, incl, 31);
+    for (int e = tid; e < t0 * a.topk; e += kIdxThreads) {
+        const int j = dest_of(a.idx[e], a, bad);
+        if (j >= 0) atomicAdd(&hist[j], 1);
     }
-    if (lane == 0) {
-        w.len[d] = run;
-        if (d != rank && run != w.planned[d]) atomicOr(status, VP_ST_PACK_MISMATCH);
+    const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
+    const int st = pack_runs(a, K, runs, sm + L.cnt, sm + L.scratch);   // (ends with a barrier: the histogram is complete, too)
+    int *const src = sm + L.src, *const dst = sm + L.dst;
+    if (tid < 32)
+        warp_positions(t0 * a.topk, t1 * a.topk, hist, [&](long long e) { return dest_of(a.idx[e], a, bad); },
+                       [&](long long e, int j, int p) {
+                           const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
+                           dst[e - t0 * a.topk] = row;
+                           if (row >= 0 && a.src_map && piece == 0) a.src_map[row] = (int)e;
+                       });
+    else
+        for (int i = tid - 32; i < t1 - t0; i += kIdxThreads - 32) src[i] = t0 + i;
+    __syncthreads();
+    if (c == n_cta - 1 && piece == 0) {              // every copy has been counted here
+        if (tid < a.N && tid != a.rank && hist[tid] != runs.total[tid]) bad = VP_ST_PACK_MISMATCH;
+        const int any = __syncthreads_or(bad);
+        if (tid == 0) *a.status = st | (any ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
     }
+    if (over) return;
+    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
+    move_rows<V>(rows, staged, a.row_bytes, t1 - t0, a.topk, src, dst, (int)((long long)vecs * piece / pieces),
+                 (int)((long long)vecs * (piece + 1) / pieces));
 }
 
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-pack_map_kernel(const int32_t* __restrict__ idx, long long E, int N, int rank, int experts_per_rank, PackWs w,
-                int32_t* __restrict__ src_map) {
-    __shared__ int base[kWarpsPerBlock][VP_MAX_N];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long chunk = (long long)blockIdx.x * kWarpsPerBlock + warp;
-    const long long e0 = chunk * kChunk;
-    if (e0 >= E) return;
-    const bool aborted = w.flags[0] != 0;
-    for (int j = lane; j < N; j += 32) base[warp][j] = w.base[chunk * N + j];
-    __syncwarp();
-    for (int it = 0; it < kItems; it++) {
-        long long e = e0 + it * 32 + lane;
-        int j = -1;
-        if (e < E) j = dest_of(idx[e], experts_per_rank, N, rank);
-        const unsigned peers = __match_any_sync(0xffffffffu, j >= 0 ? j : -1 - lane);
-        int row = -1;
-        if (j >= 0) {
-            const int p = base[warp][j] + __popc(peers & ((1u << lane) - 1));   // position in stream_j
-            if (!aborted && p < w.planned[j]) {
-                int lo = w.seg_ptr[j], hi = w.seg_ptr[j + 1] - 1;              // last segment starting at or before p
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (w.seg_start[mid] <= p) lo = mid; else hi = mid - 1;
-                }
-                row = w.seg_row[lo] + (p - w.seg_start[lo]);
-            }
+// ---- chunked form -----------------------------------------------------------------------------------------------
+
+// CTA b < n_chunks counts chunk b; the last CTA builds the run table: the two need nothing from each other.
+__global__ void __launch_bounds__(kIdxThreads) pack_count_kernel(PackArgs a, PackWs w, int chunk, int n_chunks) {
+    extern __shared__ int sm[];
+    const int tid = threadIdx.x, N = a.N;
+    grid_wait();
+    if ((int)blockIdx.x == n_chunks) {
+        const int K = steps_in_use(a);
+        const int st = pack_runs(a, K, Runs{w.start, w.row, w.ptr, w.total}, sm, sm + N);
+        if (tid == 0) {
+            const bool over = a.send_off[(size_t)K * N + a.rank] > a.capacity;
+            w.flags[0] = over;
+            w.flags[1] = st | (over ? VP_ST_PACK_CAPACITY : 0);
         }
-        __syncwarp();
-        if (j >= 0 && (peers & ((1u << lane) - 1)) == 0) base[warp][j] += __popc(peers);
-        __syncwarp();
-        if (e < E) {
-            w.dst_row[e] = row;
-            if (row >= 0 && src_map) src_map[row] = (int32_t)e;
-        }
+        return;
     }
+    const long long E = (long long)a.T * a.topk, e0 = (long long)blockIdx.x * chunk, e1 = min(e0 + chunk, E);
+    for (int j = tid; j < N; j += kIdxThreads) sm[j] = 0;
+    __syncthreads();
+    int bad = 0;
+#pragma unroll 4
+    for (long long e = e0 + tid; e < e1; e += kIdxThreads) {
+        const int j = dest_of(a.idx[e], a, bad);
+        if (j >= 0) atomicAdd(&sm[j], 1);
+    }
+    bad = __syncthreads_or(bad);
+    for (int j = tid; j < N; j += kIdxThreads) w.hist[(size_t)blockIdx.x * N + j] = sm[j];
+    if (tid == 0) w.bad[blockIdx.x] = bad ? VP_ST_PACK_MISMATCH : 0;
+}
+
+// CTA b maps chunk b, every warp a contiguous slice of it; the last CTA, whose base and own counts are all counts, checks
+// them against the plan and writes the status.
+__global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackWs w, int chunk) {
+    extern __shared__ int sm[];                      // [N] base, then [kIdxWarps][N] next position of every warp's slice
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N = a.N;
+    int* const base = sm;
+    int* const next = sm + N + warp * N;
+    for (int j = tid; j < N * (kIdxWarps + 1); j += kIdxThreads) sm[j] = 0;
+    __syncthreads();
+    grid_wait();
+#pragma unroll 4
+    for (int i = tid; i < (int)blockIdx.x * N; i += kIdxThreads) {
+        const int v = w.hist[i];
+        if (v) atomicAdd(&base[i % N], v);
+    }
+    const long long E = (long long)a.T * a.topk, e0 = (long long)blockIdx.x * chunk, e1 = min(e0 + chunk, E);
+    const long long s0 = min(e0 + (long long)warp * (chunk / kIdxWarps), e1), s1 = min(s0 + chunk / kIdxWarps, e1);
+    int ignore = 0;
+    for (long long e = s0 + lane; e < s1; e += 32) {
+        const int j = dest_of(a.idx[e], a, ignore);
+        if (j >= 0) atomicAdd(&next[j], 1);
+    }
+    __syncthreads();
+    for (int j = tid; j < N; j += kIdxThreads) {     // exclusive prefix over the warps
+        int run = base[j];
+        for (int v = 0; v < kIdxWarps; v++) {
+            int* const at = sm + N + v * N + j;
+            const int x = *at;
+            *at = run;
+            run += x;
+        }
+        base[j] = run;                               // copies up to the end of this chunk
+    }
+    __syncthreads();
+    if (blockIdx.x == gridDim.x - 1) {
+        int bad = w.flags[1];
+        for (int j = tid; j < N; j += kIdxThreads)
+            if (j != a.rank && base[j] != w.total[j]) bad |= VP_ST_PACK_MISMATCH;
+        for (int b = tid; b < (int)gridDim.x; b += kIdxThreads) bad |= w.bad[b];
+        const int mismatch = __syncthreads_or(bad & VP_ST_PACK_MISMATCH);
+        if (tid == 0) *a.status = (bad & VP_ST_PACK_CAPACITY) | (mismatch ? VP_ST_PACK_MISMATCH : 0);
+    }
+    const bool over = w.flags[0] != 0;
+    const Runs runs{w.start, w.row, w.ptr, w.total};
+    warp_positions(s0, s1, next, [&](long long e) { return dest_of(a.idx[e], a, ignore); },
+                   [&](long long e, int j, int p) {
+                       const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
+                       w.dst_row[e] = row;
+                       if (row >= 0 && a.src_map) a.src_map[row] = (int)e;
+                   });
 }
 
 }  // namespace
@@ -259,23 +252,35 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < vp_pack_workspace_bytes(N, T, topk, k_max))
         return VP_E_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    PackWs w = carve(workspace, N, T, topk, k_max);
     const long long E = (long long)T * topk;
-    const int n_chunks = (int)((E + kChunk - 1) / kChunk);
-    const int blocks = (n_chunks + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    if (cudaMemsetAsync(w.flags, 0, 256, stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess) return VP_E_CUDA;
+    const PackArgs a{n_steps_b, lane_dst_b, lane_bytes_b, send_off_b, N, rank, k_max, T, topk, experts_per_rank,
+                     expert_idx, row_bytes, staged_capacity_bytes, src_map, status};
+    const int sms = sm_count_of_device();
+    if (!sms) return VP_E_CUDA;
+    if (E <= kSmallItems && k_max <= kSmallSteps) {
+        const SmallSplit s = small_split(T, sms);
+        const int n_cta = s.grid / s.pieces;
+        if ((long long)((T + n_cta - 1) / n_cta) * topk <= kSmallOwn) {
+            const size_t smem = (size_t)pack_small_layout(N, k_max).ints * 4;
+            const char* from = (const char*)rows;
+            const int width = copy_width(rows, staged, row_bytes);
+            vp_prof_mark(2, 0, stream);
+            const cudaError_t e = width == 16 ? launch_wide(pack_small_kernel<uint4>, s.grid, smem, stream, a, from, (char*)staged, s.pieces)
+                                : width == 4 ? launch_wide(pack_small_kernel<uint32_t>, s.grid, smem, stream, a, from, (char*)staged, s.pieces)
+                                             : launch_wide(pack_small_kernel<uint8_t>, s.grid, smem, stream, a, from, (char*)staged, s.pieces);
+            vp_prof_mark(2, 1, stream);
+            return e == cudaSuccess ? VP_OK : VP_E_CUDA;
+        }
+    }
+    const PackWs w = carve(workspace, N, T, topk, k_max);
+    const int chunk = chunk_items(E, N), n_chunks = (int)((E + chunk - 1) / chunk);
     vp_prof_mark(1, 0, stream);
-    pack_count_plan_kernel<<<blocks + 1, kWarpsPerBlock * 32, 0, stream>>>(expert_idx, E, N, rank, experts_per_rank, n_steps_b,
-                                                                         lane_dst_b, lane_bytes_b, send_off_b, k_max, row_bytes,
-                                                                         staged_capacity_bytes, w, status);
-    pack_scan_kernel<<<(N + kWarpsPerBlock - 1) / kWarpsPerBlock, kWarpsPerBlock * 32, 0, stream>>>(N, rank, n_chunks, w, status);
-    pack_map_kernel<<<blocks, kWarpsPerBlock * 32, 0, stream>>>(expert_idx, E, N, rank, experts_per_rank, w, src_map);
-    g_vp_launches += 3;
+    cudaError_t e = launch_after(pack_count_kernel, n_chunks + 1, kIdxThreads, (size_t)(N + runs_scratch_ints(N)) * 4, stream, a, w, chunk, n_chunks);
+    if (e == cudaSuccess) e = launch_after(pack_map_kernel, n_chunks, kIdxThreads, (size_t)N * (kIdxWarps + 1) * 4, stream, a, w, chunk);
     vp_prof_mark(1, 1, stream);
+    if (e != cudaSuccess) return VP_E_CUDA;
     vp_prof_mark(2, 0, stream);
-
-    const int rc = launch_row_copy(rows, staged, w.dst_row, w.flags, T, topk, row_bytes, status, stream);
+    const int rc = launch_row_copy(rows, staged, w.dst_row, w.flags, T, topk, false, false, row_bytes, status, stream);
     vp_prof_mark(2, 1, stream);
     return rc;
 }
@@ -322,8 +327,7 @@ extern "C" int vp_pack_static(const int32_t* n_steps_b, const int16_t* lane_dst_
     void* scratch = nullptr;
     const int rc = static_scratch_address(&scratch);
     if (rc != VP_OK) return rc;
-    // vp_pack zeroes the flags it needs and overwrites every other scratch word it reads, so whatever the
-    // previous call left in the block does not matter
+    // vp_pack writes every scratch word before it reads it, so whatever the previous call left in the block does not matter
     return vp_pack(n_steps_b, lane_dst_b, lane_bytes_b, send_off_b, N, rank, k_max, expert_idx, T, topk,
                    experts_per_rank, rows, row_bytes, staged, staged_capacity_bytes, src_map, status, scratch,
                    (size_t)VP_PACK_STATIC_SCRATCH_BYTES, cuda_stream);

@@ -1,120 +1,132 @@
-// Row copy shared by the pack and the unpack: every source row is read once and written to each of its
-// destination rows (given by a row map, -1 = none).  Rows of at least 2 KB that are 16-byte aligned travel
-// global -> shared -> global as bulk asynchronous copies (TMA): one warp per CTA drives a ring of
-// shared-memory stages, an mbarrier per stage signals the load, the stores of a source row form one bulk
-// group whose read completion frees the stage, and the mbarrier wait is bounded.  Other rows take a
-// plain vector-load kernel.  Included by the translation units that launch it.
+// Row copy shared by the pack and the unpack directions: every source row is read once and written to each of its
+// destination rows.  The map is either map[row * fanout + slot] = destination row, or (gather, fan-out 1) map[i] = source
+// row of destination row i; -1 = none.  Rows of at least 2 KB that are 16-byte aligned travel global -> shared -> global as
+// bulk asynchronous copies (TMA): one warp per CTA drives a ring of shared-memory stages, an mbarrier per stage signals the
+// load, the stores of a source row form one bulk group whose read completion frees the stage, and the mbarrier wait is
+// bounded.  Other rows take a plain vector-load kernel.  Included by the translation units that launch it.
 #pragma once
 #include <cuda_runtime.h>
 
 #include "bulk_copy.cuh"
+#include "route_index.cuh"
 #include "vp_internal.h"
 
 namespace {
 
 constexpr int kPiece = 16384;              // bytes per bulk transfer (rows longer than this are split)
+constexpr int kStages = 6;
 constexpr int kMinBulkRow = 2048;          // shorter rows use the plain-load kernel
 constexpr unsigned kSpinLimit = 1u << 22;  // bounded mbarrier wait
 
-// One warp per CTA.  A "unit" is one piece (<= kPiece bytes) of one source row.  Units are dealt to CTAs round
-// robin.  Unit u is loaded into stage u % S, kLook units ahead of its stores.  The destination rows of a unit
-// (lane = slot, up to 32 slots per round) are fetched one unit ahead of the load that needs them and kept in
-// registers until the unit's stores, so no global-memory latency sits between two bulk copies.
-template <int S>
-__global__ void __launch_bounds__(32)
-pack_copy_bulk_kernel(const char* __restrict__ rows, char* __restrict__ staged, const int32_t* __restrict__ dst_row,
-                      const int32_t* __restrict__ flags, int T, int topk, long long row_bytes, int pieces,
-                      int32_t* __restrict__ status) {
-    constexpr int kLook = S / 2;
-    static_assert(kLook == 3, "the destination-row registers below form a ring of three");
+struct RowCopy {
+    const char* rows;
+    char* out;
+    const int32_t* map;
+    const int32_t* flags;      // device: [0] != 0 turns the copy into a no-op; [2] = rows in use when `bounded`
+    int n, fanout, gather, bounded;
+    long long row_bytes;
+    int pieces, stage_bytes, run;      // bulk form: pieces per row, ring stage, consecutive rows a CTA takes at a time
+    int32_t* status;
+};
+
+// One warp per CTA.  A "unit" is one piece (<= kPiece bytes) of one source row.  CTAs take runs of `run` consecutive rows,
+// dealt round robin.  Unit m is loaded into stage m % S, S / 2 units ahead of its stores.
+//
+// The map entries of a whole run are fetched by one coalesced load while the run before is in flight.  (With one fetch per
+// unit each unit waited for a trip to L2: 0.85 us a unit and CTA whatever its size, so rows of 4 to 8 KB reached half of
+// the bandwidth with two CTAs per SM.)  Stores carry no L2 policy: marking them evict-first cost 10 % at fan-out 1
+// (32,768 rows of 14,336 B: 157 -> 142 us) and at 4 KB rows (214 -> 195 us), and changed nothing elsewhere.
+__global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
+    constexpr int S = kStages, kLook = S / 2;
     extern __shared__ __align__(128) unsigned char ring[];
     __shared__ __align__(8) unsigned long long bars[S];
+    __shared__ int32_t sdst[S][32];                  // destination row of this lane's slot, per unit in flight
     const int lane = threadIdx.x;
-    if (flags[0]) return;
-    const unsigned long long stream_policy = l2_evict_first_policy();
     if (lane == 0) {
         for (int s = 0; s < S; s++) mbar_init(smem_u32(&bars[s]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    const long long units = (long long)T * pieces;
-    const long long count = units > blockIdx.x ? (units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    const int rounds = (topk + 31) / 32;            // destinations are handled 32 slots at a time
-    const bool one_round = rounds == 1;
+    grid_wait();
+    if (c.flags[0]) return;
+    const int n = c.bounded ? min(c.n, c.flags[2]) : c.n;
+    const int F = c.fanout, pieces = c.pieces, run = c.run, per_run = run * pieces;
+    const bool wide = F > 32;                        // destinations of a row are then handled 32 slots at a time
+    const int n_runs = (n + run - 1) / run;
+    const int my_runs = n_runs > (int)blockIdx.x ? (n_runs - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     unsigned phase = 0;                              // parity per stage (bit s)
     unsigned loaded = 0;                             // stage holds a load that was issued (bit s)
     bool failed = false;
-    // destination row of this lane's slot: for the unit whose load is issued next (fetched), and for the three
-    // units in flight (r2 newest .. r0 oldest); used when all slots fit one round
-    int fetched = -1, r0 = -1, r1 = -1, r2 = -1;
-    if (one_round && count > 0 && lane < topk) fetched = dst_row[(long long)(blockIdx.x / pieces) * topk + lane];
-    for (long long it = 0; it < count + kLook && !failed; it++) {
-        int rows_m = r0;                             // unit it - kLook
-        r0 = r1; r1 = r2; r2 = -1;
-        if (it < count) {                            // ---- issue the load of unit `it`
-            const long long u = blockIdx.x + it * gridDim.x;
-            const long long t = u / pieces;
-            const int s = (int)(it % S);
-            bool any = false;
-            if (one_round) {
-                r2 = fetched;
-                any = fetched >= 0;
-                fetched = -1;
-                if (it + 1 < count && lane < topk) fetched = dst_row[((u + gridDim.x) / pieces) * topk + lane];
+    auto fetch = [&](int q) {                        // map entries of the q-th run: lane = row in run x fan-out + slot
+        const long long e = ((long long)blockIdx.x + (long long)q * gridDim.x) * run * F + lane;
+        return !wide && q < my_runs && lane < run * F && e < (long long)n * F ? c.map[e] : -1;
+    };
+    int cur = -1, nxt = fetch(0);
+    // position of the next load (run, row in run, piece) and of the next store; s_*: ring stages
+    int lq = 0, li = 0, lp = 0, ls = 0, sq = 0, si = 0, sp = 0, ss = 0;
+    const long long units = (long long)my_runs * per_run;
+    for (long long it = 0; it < units + kLook && !failed; it++) {
+        if (it < units) {                            // ---- issue the load of unit `it`
+            if (li == 0 && lp == 0) { cur = nxt; nxt = fetch(lq + 1); }
+            const long long r = ((long long)blockIdx.x + (long long)lq * gridDim.x) * run + li;
+            int d = wide ? -1 : __shfl_sync(0xffffffffu, cur, min(li * F + lane, 31));
+            if (lane >= F) d = -1;
+            bool any;
+            long long src = r;
+            if (wide) {
+                any = false;
+                for (int f = lane; f < F && r < n; f += 32) any |= c.map[r * F + f] >= 0;
+                any = __any_sync(0xffffffffu, any);
             } else {
-                for (int r = 0; r < rounds; r++) {
-                    const int slot = r * 32 + lane;
-                    any |= slot < topk && dst_row[t * topk + slot] >= 0;
+                any = __any_sync(0xffffffffu, d >= 0);
+                if (c.gather) {
+                    src = __shfl_sync(0xffffffffu, d, 0);
+                    d = any && lane == 0 ? (int)r : -1;
                 }
             }
-            any = __any_sync(0xffffffffu, any);
             bulk_wait_read<S - kLook - 1>();         // every lane: its stores that last read this stage are done
             __syncwarp();
-            if (lane == 0) {
-                if (any) {
-                    const int p = (int)(u % pieces);
-                    const unsigned bytes = (unsigned)min((long long)kPiece, row_bytes - (long long)p * kPiece);
-                    const unsigned bar = smem_u32(&bars[s]);
-                    mbar_expect_tx(bar, bytes);
-                    bulk_load_stream(smem_u32(ring + (size_t)s * kPiece), rows + t * row_bytes + (long long)p * kPiece, bytes, bar, stream_policy);
-                }
+            sdst[ls][lane] = d;
+            if (any && lane == 0) {
+                const unsigned bytes = (unsigned)min((long long)kPiece, c.row_bytes - (long long)lp * kPiece);
+                const unsigned bar = smem_u32(&bars[ls]);
+                mbar_expect_tx(bar, bytes);
+                bulk_load(smem_u32(ring + (size_t)ls * c.stage_bytes), c.rows + src * c.row_bytes + (long long)lp * kPiece, bytes, bar);
             }
-            loaded = any ? (loaded | (1u << s)) : (loaded & ~(1u << s));
+            loaded = any ? (loaded | (1u << ls)) : (loaded & ~(1u << ls));
+            ls = ls + 1 == S ? 0 : ls + 1;
+            if (++lp == pieces) { lp = 0; if (++li == run) { li = 0; lq++; } }
         }
-        const long long m = it - kLook;
-        if (m >= 0) {                                // ---- unit m: wait for its load, issue its stores
-            const long long u = blockIdx.x + m * gridDim.x;
-            const long long t = u / pieces;
-            const int p = (int)(u % pieces);
-            const int s = (int)(m % S);
-            if (loaded & (1u << s)) {
-                const unsigned bar = smem_u32(&bars[s]);
+        if (it >= kLook) {                           // ---- unit it - kLook: wait for its load, issue its stores
+            if (loaded & (1u << ss)) {
+                const unsigned bar = smem_u32(&bars[ss]);
                 unsigned spins = 0;
-                while (!mbar_try_wait(bar, (phase >> s) & 1u)) {
+                while (!mbar_try_wait(bar, (phase >> ss) & 1u)) {
                     if (++spins > kSpinLimit) { failed = true; break; }
                 }
                 failed = __any_sync(0xffffffffu, failed);
-                phase ^= 1u << s;
-                if (!failed) loaded &= ~(1u << s);   // this stage's load has landed
+                phase ^= 1u << ss;
                 if (!failed) {
-                    const unsigned bytes = (unsigned)min((long long)kPiece, row_bytes - (long long)p * kPiece);
+                    loaded &= ~(1u << ss);           // this stage's load has landed
+                    const unsigned bytes = (unsigned)min((long long)kPiece, c.row_bytes - (long long)sp * kPiece);
+                    const unsigned from = smem_u32(ring + (size_t)ss * c.stage_bytes);
+                    char* const to = c.out + (long long)sp * kPiece;
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    if (one_round) {
-                        if (rows_m >= 0)
-                            bulk_store_stream(staged + (long long)rows_m * row_bytes + (long long)p * kPiece,
-                                              smem_u32(ring + (size_t)s * kPiece), bytes, stream_policy);
+                    if (!wide) {
+                        const int d = sdst[ss][lane];
+                        if (d >= 0) bulk_store(to + (long long)d * c.row_bytes, from, bytes);
                     } else {
-                        for (int r = 0; r < rounds; r++) {
-                            const int slot = r * 32 + lane;
-                            const int row = slot < topk ? dst_row[t * topk + slot] : -1;
-                            if (row >= 0)
-                                bulk_store_stream(staged + (long long)row * row_bytes + (long long)p * kPiece,
-                                                  smem_u32(ring + (size_t)s * kPiece), bytes, stream_policy);
+                        const long long r = ((long long)blockIdx.x + (long long)sq * gridDim.x) * run + si;
+                        for (int f = lane; f < F; f += 32) {
+                            const int d = c.map[r * F + f];
+                            if (d >= 0) bulk_store(to + (long long)d * c.row_bytes, from, bytes);
                         }
                     }
                 }
             }
             bulk_commit();                           // one group per unit from every lane, empty or not
+            ss = ss + 1 == S ? 0 : ss + 1;
+            if (++sp == pieces) { sp = 0; if (++si == run) { si = 0; sq++; } }
         }
     }
     bulk_wait_all();                                 // stores must finish before shared memory is released
@@ -129,81 +141,112 @@ pack_copy_bulk_kernel(const char* __restrict__ rows, char* __restrict__ staged, 
                    ++spins < (1u << 18)) {
             }
         }
-        if (lane == 0) atomicOr(status, VP_ST_INTERNAL_TIMEOUT);
+        if (lane == 0) atomicOr(c.status, VP_ST_INTERNAL_TIMEOUT);
     }
 }
 
-// Plain-load path (short or unaligned rows): one warp per token, V-byte vectors.
+// Plain-load path (short or unaligned rows): a warp takes 32 U vectors of one row at a time, all loads in flight before the
+// first store (one load per lane at a time left a few KB in flight per SM: 4,100-byte rows ran at a third of the bandwidth).
 template <typename V>
-__global__ void __launch_bounds__(256)
-pack_copy_plain_kernel(const char* __restrict__ rows, char* __restrict__ staged, const int32_t* __restrict__ dst_row,
-                       const int32_t* __restrict__ flags, int T, int topk, long long row_bytes) {
-    if (flags[0]) return;
+__global__ void __launch_bounds__(256) row_copy_plain_kernel(RowCopy c) {
+    constexpr int U = PieceOf<V>::U;
+    grid_wait();
+    if (c.flags[0]) return;
+    const int n = c.bounded ? min(c.n, c.flags[2]) : c.n, F = c.fanout;
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long vecs = row_bytes / (long long)sizeof(V);
-    for (long long t = warp; t < T; t += n_warps) {
-        const V* src = (const V*)(rows + t * row_bytes);
-        for (int s0 = 0; s0 < topk; s0 += 8) {
-            int row[8];
+    const int vecs = (int)(c.row_bytes / (long long)sizeof(V)), pieces = (vecs + 32 * U - 1) / (32 * U);
+    for (long long it = warp; it < (long long)n * pieces; it += n_warps) {
+        const long long r = it / pieces;
+        const int v0 = (int)(it - r * pieces) * 32 * U + lane;
+        long long src = r;
+        if (c.gather) {
+            src = c.map[r];
+            if (src < 0) continue;
+        } else {
             bool any = false;
+            for (int f = lane; f < F; f += 32) any |= c.map[r * F + f] >= 0;
+            if (!__any_sync(0xffffffffu, any)) continue;
+        }
+        const V* from = (const V*)(c.rows + src * c.row_bytes);
+        V x[U];
 #pragma unroll
-            for (int s = 0; s < 8; s++) {
-                row[s] = (s0 + s < topk) ? dst_row[t * topk + s0 + s] : -1;
-                any |= row[s] >= 0;
-            }
-            if (!any) continue;
-            for (long long v = lane; v < vecs; v += 32) {
-                const V x = src[v];
+        for (int u = 0; u < U; u++)
+            if (v0 + 32 * u < vecs) x[u] = __ldg(from + v0 + 32 * u);
+        for (int f = 0; f < F; f++) {
+            const long long d = c.gather ? r : (long long)c.map[r * F + f];
+            if (d < 0) continue;
+            V* to = (V*)(c.out + d * c.row_bytes);
 #pragma unroll
-                for (int s = 0; s < 8; s++)
-                    if (row[s] >= 0) ((V*)(staged + (long long)row[s] * row_bytes))[v] = x;
-            }
+            for (int u = 0; u < U; u++)
+                if (v0 + 32 * u < vecs) to[v0 + 32 * u] = x[u];
         }
     }
 }
 
-
-// Enqueue the copy of `n_src` source rows, each to its up to `fanout` destination rows dst_row[src * fanout + slot].
-// `flags[0] != 0` (device) turns the copy into a no-op.  Returns VP_OK or VP_E_CUDA.
-inline int launch_row_copy(const void* rows, void* out, const int32_t* dst_row, const int32_t* flags, int n_src, int fanout,
-                           long long row_bytes, int32_t* status, cudaStream_t stream) {
-    // per device, once: the SM count and the bulk kernel's shared-memory limit (kept out of the per-call path)
+// SMs of the current device, asked once per device.
+inline int sm_count_of_device() {
     static int s_sms[64] = {0};
-    static bool s_attr_set[64] = {false};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return VP_E_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     const bool cached = dev >= 0 && dev < 64;
-    int sms = cached ? s_sms[dev] : 0;
+    int sms = cached ? __atomic_load_n(&s_sms[dev], __ATOMIC_RELAXED) : 0;
     if (!sms) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return VP_E_CUDA;
-        if (cached) s_sms[dev] = sms;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        if (cached) __atomic_store_n(&s_sms[dev], sms, __ATOMIC_RELAXED);
     }
-    const bool aligned16 = row_bytes % 16 == 0 && ((uintptr_t)rows & 15) == 0 && ((uintptr_t)out & 15) == 0;
-    if (aligned16 && row_bytes >= kMinBulkRow) {
-        constexpr int S = 6;
-        const int pieces = (int)((row_bytes + kPiece - 1) / kPiece);
-        const size_t smem = (size_t)S * kPiece;
-        if (!cached || !s_attr_set[dev]) {
-            if (cudaFuncSetAttribute(pack_copy_bulk_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return sms;
+}
+
+// Widest vector (bytes) that source, destination and row size allow.
+inline int copy_width(const void* rows, const void* out, long long row_bytes) {
+    const uintptr_t mix = (uintptr_t)rows | (uintptr_t)out | (uintptr_t)row_bytes;
+    return mix % 16 == 0 ? 16 : (mix % 4 == 0 ? 4 : 1);
+}
+
+// Enqueues the copy behind the kernel that wrote map and flags.  With `bounded`, only the first flags[2] rows (device) are
+// in use.  Returns VP_OK or VP_E_CUDA.
+inline int launch_row_copy(const void* rows, void* out, const int32_t* map, const int32_t* flags, int n, int fanout, bool gather,
+                           bool bounded, long long row_bytes, int32_t* status, cudaStream_t stream) {
+    static bool s_attr_set[64] = {false};       // per device, once: the bulk kernel's shared-memory limit
+    int dev = 0;
+    const int sms = sm_count_of_device();
+    if (!sms || cudaGetDevice(&dev) != cudaSuccess) return VP_E_CUDA;
+    RowCopy c;
+    c.rows = (const char*)rows; c.out = (char*)out; c.map = map; c.flags = flags;
+    c.n = n; c.fanout = fanout; c.gather = gather; c.bounded = bounded; c.row_bytes = row_bytes; c.status = status;
+    c.pieces = 1; c.stage_bytes = 0; c.run = 1;
+    const int width = copy_width(rows, out, row_bytes);
+    cudaError_t e;
+    if (width == 16 && row_bytes >= kMinBulkRow) {
+        if (dev < 0 || dev >= 64 || !s_attr_set[dev]) {
+            if (cudaFuncSetAttribute(row_copy_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * kPiece) != cudaSuccess)
                 return VP_E_CUDA;
-            if (cached) s_attr_set[dev] = true;
+            if (dev >= 0 && dev < 64) s_attr_set[dev] = true;
         }
-        pack_copy_bulk_kernel<S><<<sms * 2, 32, smem, stream>>>((const char*)rows, (char*)out, dst_row, flags, n_src, fanout,
-                                                                row_bytes, pieces, status);
+        c.pieces = (int)((row_bytes + kPiece - 1) / kPiece);
+        c.stage_bytes = row_bytes < kPiece ? (int)((row_bytes + 127) & ~127ll) : kPiece;
+        // About 170 KB of ring per SM: two CTAs at 14 KB rows, four at 7 KB, eight at most.  With a fan-out the stores are
+        // most of the traffic and more than two CTAs per SM only scatter them (4 KB rows, fan-out 8: 195 us with two, 215
+        // with four and more).
+        int per_sm = 176 * 1024 / (kStages * c.stage_bytes);
+        per_sm = per_sm < 2 ? 2 : (per_sm > 8 ? 8 : per_sm);
+        if (fanout >= 4) per_sm = 2;
+        const int grid = sms * per_sm;
+        int run = fanout <= 32 ? 32 / fanout : 1;
+        if (run > 8) run = 8;
+        while (run > 1 && (long long)n < (long long)grid * run * 8) run >>= 1;   // eight runs per CTA at least: an even last wave
+        c.run = run;
+        e = launch_after(row_copy_bulk_kernel, grid, 32, (size_t)kStages * c.stage_bytes, stream, c);
+    } else if (width == 16) {
+        e = launch_after(row_copy_plain_kernel<uint4>, sms * 8, 256, 0, stream, c);
+    } else if (width == 4) {
+        e = launch_after(row_copy_plain_kernel<uint32_t>, sms * 8, 256, 0, stream, c);
     } else {
-        const int grid = sms * 8;
-        const uintptr_t mix = (uintptr_t)rows | (uintptr_t)out | (uintptr_t)row_bytes;
-        if (mix % 16 == 0)
-            pack_copy_plain_kernel<uint4><<<grid, 256, 0, stream>>>((const char*)rows, (char*)out, dst_row, flags, n_src, fanout, row_bytes);
-        else if (mix % 4 == 0)
-            pack_copy_plain_kernel<uint32_t><<<grid, 256, 0, stream>>>((const char*)rows, (char*)out, dst_row, flags, n_src, fanout, row_bytes);
-        else
-            pack_copy_plain_kernel<uint8_t><<<grid, 256, 0, stream>>>((const char*)rows, (char*)out, dst_row, flags, n_src, fanout, row_bytes);
+        e = launch_after(row_copy_plain_kernel<uint8_t>, sms * 8, 256, 0, stream, c);
     }
-    g_vp_launches++;
-    return cudaGetLastError() == cudaSuccess ? VP_OK : VP_E_CUDA;
+    return e == cudaSuccess ? VP_OK : VP_E_CUDA;
 }
 
 }  // namespace

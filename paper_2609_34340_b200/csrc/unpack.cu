@@ -5,11 +5,13 @@
 // (at recv_off[k][rank]).  The output is expert-major: all rows of local expert 0, then 1, ...; inside an
 // expert by source rank; inside a source in arrival order.  That is a stable sort of the received rows by
 // the key (expert, source), done as a counting sort:
-//   plan  : the rank's receive segments (first row, source rank) from the plan
-//   count : key of every row (binary search of its segment), per 256-row chunk a histogram of keys
-//   scan  : per key an exclusive scan over the chunks; then an exclusive scan over the keys
+//   steps : receive row and sender of every step (only for plans too large for every count CTA to read)
+//   count : key of every row (binary search of its step), per chunk of rows a histogram of keys
 //   map   : stable position of every row among the rows of its key -> output row
 //   copy  : the row copy shared with the pack (each received row read once, written once)
+// vp_unpack_tokens, the return direction, sorts the routed copies by expert id the same way; a copy's position among the
+// copies to its expert's rank is its position in that sender's stream, whose runs give the receive row.
+// Up to kSmallItems rows (copies) each call is one kernel (see route_index.cuh).
 #include <cuda_runtime.h>
 
 #include "row_copy.cuh"
@@ -17,224 +19,449 @@
 
 namespace {
 
-constexpr int kItems = 8;                  // 32-row rounds per warp chunk
-constexpr int kChunk = 32 * kItems;
-constexpr int kWarps = 8;
-constexpr int kMaxKeys = 1024;             // experts_per_rank x N
+struct UnpackArgs {
+    const int32_t* n_steps;
+    const int16_t* lane_dst;
+    const int64_t *lane_bytes, *recv_off;    // (lane_bytes: return direction only)
+    int N, rank, k_max, epr, keys, items;    // items: capacity in rows, or routed copies
+    const int32_t* item_expert;              // local expert of each received row, or global expert of each routed copy
+    int64_t row_bytes, capacity_rows;
+    int32_t *expert_off, *out_src, *out_map, *status;
+};
 
 struct UnpackWs {
-    int32_t* flags;      // [0] abort, [1] number of segments, [2] rows received
-    int32_t* seg_row0;   // [k_max] first receive row of a segment
-    int32_t* seg_end;    // [k_max] one past its last receive row
-    int32_t* seg_src;    // [k_max] its source rank
+    int32_t* flags;      // [0] abort, [1] status bits, [2] rows received
+    int32_t* bad;        // [n_chunks] status bits of each chunk
+    int32_t* step_row;   // [k_max + 1] first receive row of a step
+    int32_t* step_peer;  // [k_max] its sender, -1 = none
     int32_t* hist;       // [n_chunks][keys]
-    int32_t* base;       // [n_chunks][keys] rows of that key in earlier chunks
-    int32_t* key_total;  // [keys]
-    int32_t* key_base;   // [keys + 1] first output row of a key
-    int32_t* row_key;    // [capacity] key of a received row, -1 = none
-    int32_t* out_row;    // [capacity] output row of a received row, -1 = none
+    int32_t* item_key;   // [items] key of a received row or routed copy, -1 = none
+    int32_t* map;        // [items] output row of a received row, or receive row of a routed copy; -1 = none
+    int32_t *total, *ptr, *start, *row;      // (return direction) run table of the senders, see Runs
     size_t bytes;
 };
 
-UnpackWs carve(void* base, int keys, long long capacity_rows, int k_max) {
+UnpackWs carve(void* base, int N, int keys, long long items, int k_max) {
     UnpackWs w;
     size_t o = 0;
-    auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (char*)base + at; };
-    const long long n_chunks = (capacity_rows + kChunk - 1) / kChunk;
-    w.flags = (int32_t*)take(256);
-    w.seg_row0 = (int32_t*)take((size_t)k_max * 4);
-    w.seg_end = (int32_t*)take((size_t)k_max * 4);
-    w.seg_src = (int32_t*)take((size_t)k_max * 4);
-    w.hist = (int32_t*)take((size_t)n_chunks * keys * 4);
-    w.base = (int32_t*)take((size_t)n_chunks * keys * 4);
-    w.key_total = (int32_t*)take((size_t)keys * 4);
-    w.key_base = (int32_t*)take((size_t)(keys + 1) * 4);
-    w.row_key = (int32_t*)take((size_t)capacity_rows * 4);
-    w.out_row = (int32_t*)take((size_t)capacity_rows * 4);
+    auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (int32_t*)((char*)base + at); };
+    const long long chunk = chunk_items(items, keys);
+    const size_t n_chunks = (size_t)((items + chunk - 1) / chunk);
+    w.flags = take(256);
+    w.bad = take(n_chunks * 4);
+    w.step_row = take((size_t)(k_max + 1) * 4);
+    w.step_peer = take((size_t)k_max * 4);
+    w.hist = take(n_chunks * keys * 4);
+    w.item_key = take((size_t)items * 4);
+    w.map = take((size_t)items * 4);
+    w.total = take((size_t)N * 4);
+    w.ptr = take((size_t)(N + 1) * 4);
+    w.start = take((size_t)k_max * 4);
+    w.row = take((size_t)k_max * 4);
     w.bytes = o;
     return w;
 }
 
-__global__ void __launch_bounds__(256)
-unpack_plan_kernel(const int32_t* __restrict__ n_steps_p, const int16_t* __restrict__ lane_dst,
-                   const int64_t* __restrict__ recv_off, int N, int rank, int k_max, int64_t row_bytes,
-                   long long capacity_rows, UnpackWs w, int32_t* __restrict__ status) {
-    __shared__ int t_row0[256], t_src[256], t_rows[256];
-    __shared__ int s_n;
-    const int tid = threadIdx.x;
-    int K = *n_steps_p;
-    K = K < 0 ? 0 : (K > k_max ? k_max : K);
-    if (tid == 0) {
-        s_n = 0;
-        const int64_t total = recv_off[(size_t)K * N + rank];
-        int st = 0;
-        if (total % row_bytes) st |= VP_ST_PACK_MISMATCH;
-        if (total / row_bytes > capacity_rows) { st |= VP_ST_PACK_CAPACITY; w.flags[0] = 1; }
-        w.flags[2] = (int32_t)(total / row_bytes > capacity_rows ? 0 : total / row_bytes);
-        if (st) atomicOr(status, st);
-    }
-    __syncthreads();
-    bool bad = false;
-    for (int k0 = 0; k0 < K; k0 += 256) {
-        const int k = k0 + tid;
-        t_rows[tid] = 0;
-        if (k < K) {
-            const int64_t lo = recv_off[(size_t)k * N + rank], hi = recv_off[(size_t)(k + 1) * N + rank];
-            if (hi > lo && (lo % row_bytes || hi % row_bytes)) bad = true;   // such a segment is left out
-            else if (hi > lo) {
-                int src = -1;
-                for (int i = 0; i < N; i++)
-                    if (lane_dst[(size_t)k * N + i] == rank) src = i;
-                if (src < 0) bad = true;
-                t_row0[tid] = (int)(lo / row_bytes);
-                t_rows[tid] = (int)(hi / row_bytes - lo / row_bytes);
-                t_src[tid] = src;
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {                                    // steps are in receive order: append in order
-            int n = s_n;
-            for (int i = 0; i < 256 && k0 + i < K; i++)
-                if (t_rows[i] > 0) { w.seg_row0[n] = t_row0[i]; w.seg_end[n] = t_row0[i] + t_rows[i]; w.seg_src[n] = t_src[i]; n++; }
-            s_n = n;
-        }
-        __syncthreads();
-    }
-    if (tid == 0) w.flags[1] = s_n;
-    if (bad) atomicOr(status, VP_ST_PACK_MISMATCH);
+__device__ __forceinline__ int steps_in_use(const UnpackArgs& a) { return min(max(*a.n_steps, 0), a.k_max); }
+
+// Rows this rank receives in K steps (0 when they exceed the buffer), with status bits.
+__device__ __forceinline__ int rows_received(const UnpackArgs& a, int K, int& st) {
+    const int64_t total = a.recv_off[(size_t)K * a.N + a.rank];
+    const bool over = total / a.row_bytes > a.capacity_rows;
+    st = (total % a.row_bytes ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
+    return over ? 0 : (int)(total / a.row_bytes);
 }
 
-// by_routing = 0: item r is a received row, key = (local expert, source rank of its segment)
-// by_routing = 1: item c is a routed copy, key = its global expert id (copies to `rank` itself or dropped: none)
-__global__ void __launch_bounds__(kWarps * 32)
-unpack_count_kernel(const int32_t* __restrict__ recv_expert, long long capacity_rows, int N, int experts_per_rank,
-                    int keys, UnpackWs w, int32_t* __restrict__ status, int by_routing, int rank) {
-    __shared__ int wh[kWarps][kMaxKeys];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long chunk = (long long)blockIdx.x * kWarps + warp;
-    const long long r0 = chunk * kChunk;
-    if (r0 >= capacity_rows) return;
-    const int R = w.flags[0] ? 0 : w.flags[2], n_seg = w.flags[1];
-    for (int j = lane; j < keys; j += 32) wh[warp][j] = 0;
-    __syncwarp();
-    bool bad = false;
-    for (int it = 0; it < kItems; it++) {
-        const long long r = r0 + it * 32 + lane;
-        if (r >= capacity_rows) continue;
-        int key = -1;
-        if (by_routing) {
-            const int e = recv_expert[r];
-            if (!w.flags[0] && e >= 0 && e < keys && e / experts_per_rank != rank) { key = e; atomicAdd(&wh[warp][key], 1); }
-        } else if (r < R) {
-            int lo = 0, hi = n_seg - 1;                    // last segment starting at or before r
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (w.seg_row0[mid] <= r) lo = mid; else hi = mid - 1;
-            }
-            const int e = recv_expert[r];
-            const int src = n_seg > 0 && w.seg_row0[lo] <= r && r < w.seg_end[lo] ? w.seg_src[lo] : -1;
-            if (e < 0 || e >= experts_per_rank || src < 0) bad = true;
-            else { key = e * N + src; atomicAdd(&wh[warp][key], 1); }
-        }
-        w.row_key[r] = key;
-    }
-    __syncwarp();
-    for (int j = lane; j < keys; j += 32) w.hist[chunk * keys + j] = wh[warp][j];
-    if (bad) atomicOr(status, VP_ST_PACK_MISMATCH);
+// Step k of the dispatch plan from its sender: first receive row; a step whose bytes are not whole rows, or that has bytes
+// and no sender, is left out (peer -1) and reported.
+__device__ __forceinline__ int check_step(const UnpackArgs& a, int k, int& peer, int& bad) {
+    const int64_t lo = a.recv_off[(size_t)k * a.N + a.rank], hi = a.recv_off[(size_t)(k + 1) * a.N + a.rank];
+    if (hi > lo && (peer < 0 || lo % a.row_bytes || hi % a.row_bytes)) { peer = -1; bad = VP_ST_PACK_MISMATCH; }
+    return (int)(lo / a.row_bytes);
 }
 
-// one warp per key: exclusive scan of its counts over the chunks
-__global__ void __launch_bounds__(kWarps * 32)
-unpack_scan_kernel(int keys, int n_chunks, UnpackWs w) {
-    const int lane = threadIdx.x & 31, key = blockIdx.x * kWarps + (threadIdx.x >> 5);
-    if (key >= keys) return;
-    const int32_t* __restrict__ in = w.hist;
-    int32_t* __restrict__ out = w.base;
+// Key of a received row r < R: (local expert, sender of its step), -1 if either is missing.
+__device__ __forceinline__ int row_key_of(const UnpackArgs& a, int r, int K, const int* step_row, const int* step_peer) {
+    int lo = 0, hi = K - 1;                                        // last step starting at or before r
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (step_row[mid] <= r) lo = mid; else hi = mid - 1;
+    }
+    const int e = a.item_expert[r], src = K > 0 ? step_peer[lo] : -1;
+    return e < 0 || e >= a.epr || src < 0 ? -1 : e * a.N + src;
+}
+
+// Key of a routed copy: its expert id, -1 if it does not travel.
+__device__ __forceinline__ int copy_key_of(const UnpackArgs& a, long long c) {
+    const int e = a.item_expert[c];
+    return e >= 0 && e < a.keys && (int)((unsigned)e / (unsigned)a.epr) != a.rank ? e : -1;
+}
+
+// Run table of the return plan: bucket = sender, runs = its segments in the receive buffer.  peer(k) is the sender of step k.
+template <typename Peer>
+__device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, Peer peer, Runs out, int* cnt, int* scratch) {
+    int bad = 0;
+    build_runs(K, a.N, [&](int k, int& j, int& rows, int& row0) {
+        j = peer(k);
+        rows = row0 = 0;
+        if (j < 0) return;
+        const int64_t bytes = a.lane_bytes[(size_t)k * a.N + j], at = a.recv_off[(size_t)k * a.N + a.rank];
+        if (bytes % a.row_bytes || at % a.row_bytes) { bad = VP_ST_PACK_MISMATCH; j = -1; return; }   // left out
+        rows = (int)(bytes / a.row_bytes);
+        row0 = (int)(at / a.row_bytes);
+        if (rows <= 0) j = -1;
+    }, out, cnt, scratch);
+    return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
+}
+
+// total[key] -> exclusive prefix over the keys in first[0 .. keys]; all threads.
+__device__ __forceinline__ void scan_keys(const int* total, int* first, int keys, int* wsum) {
     int run = 0;
+    for (int k0 = 0; k0 < keys; k0 += kIdxThreads) {
+        const int k = k0 + threadIdx.x;
+        int all;
+        const int at = cta_exclusive_scan(k < keys ? total[k] : 0, wsum, all);
+        if (k < keys) first[k] = run + at;
+        run += all;
+    }
+    if (threadIdx.x == 0) first[keys] = run;
+    __syncthreads();
+}
+
+// ---- one launch -------------------------------------------------------------------------------------------------
+
+struct UnpackSmall { int peer, step_row, all, next, first, wsum, cnt, total, ptr, start, row, src, dst, scratch, ints; };
+__host__ __device__ inline UnpackSmall unpack_small_layout(int N, int keys, int k_max, bool tokens) {
+    UnpackSmall L;
+    int o = 0;
+    L.peer = o;     o += k_max;
+    L.step_row = o; o += tokens ? 0 : k_max + 1;
+    L.all = o;      o += keys;
+    L.next = o;     o += keys;
+    L.first = o;    o += keys + 1;
+    L.wsum = o;     o += kIdxWarps + 1;
+    L.cnt = o;      o += tokens ? N : 0;
+    L.total = o;    o += tokens ? N : 0;
+    L.ptr = o;      o += tokens ? N + 1 : 0;
+    L.start = o;    o += tokens ? k_max : 0;
+    L.row = o;      o += tokens ? k_max : 0;
+    L.src = o;      o += kSmallOwn;
+    L.dst = o;      o += kSmallOwn;
+    L.scratch = o;  o += tokens ? runs_scratch_ints(N) : 0;
+    L.ints = o;
+    return L;
+}
+
+// Receive side of small calls.  Every CTA reads the plan and the keys of all received rows, counts them (all of them, and
+// those before its own), and moves its own contiguous range of rows.  Bound by latency, then by HBM.  Replaces two memsets
+// and six kernels.
+template <typename V>
+__global__ void __launch_bounds__(kIdxThreads, 2)
+unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, int pieces) {
+    extern __shared__ int sm[];
+    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, false);
+    int *const peer = sm + L.peer, *const step_row = sm + L.step_row, *const all = sm + L.all, *const next = sm + L.next;
+    const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
+    for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
+    grid_wait();
+    const int K = steps_in_use(a);
+    int st, bad = 0;
+    const int R = rows_received(a, K, st);
+    find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+    for (int k = tid; k < K; k += kIdxThreads) {
+        int p = peer[k];
+        step_row[k] = check_step(a, k, p, bad);
+        peer[k] = p;
+    }
+    __syncthreads();
+    const int r0 = (int)((long long)R * c / n_cta), r1 = (int)((long long)R * (c + 1) / n_cta);
+    for (int r = tid; r < R; r += kIdxThreads) {
+        const int key = row_key_of(a, r, K, step_row, peer);
+        if (key < 0) { bad = VP_ST_PACK_MISMATCH; continue; }
+        atomicAdd(&all[key], 1);
+        if (r < r0) atomicAdd(&next[key], 1);
+    }
+    bad = __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
+    int* const first = sm + L.first;
+    scan_keys(all, first, a.keys, sm + L.wsum);
+    if (blockIdx.x == 0) {
+        for (int e = tid; e <= a.epr; e += kIdxThreads) a.expert_off[e] = first[e * a.N];
+        if (tid == 0) *a.status = st | bad | (!(st & VP_ST_PACK_CAPACITY) && first[a.keys] != R ? VP_ST_PACK_MISMATCH : 0);
+    }
+    int *const src = sm + L.src, *const dst = sm + L.dst;
+    if (tid < 32)
+        warp_positions(r0, r1, next, [&](long long r) { return row_key_of(a, (int)r, K, step_row, peer); },
+                       [&](long long r, int key, int p) {
+                           const int o = p >= 0 ? first[key] + p : -1;
+                           src[r - r0] = o >= 0 ? (int)r : -1;
+                           dst[r - r0] = o;
+                           if (o >= 0 && piece == 0) {
+                               if (a.out_src) a.out_src[o] = key % a.N;
+                               if (a.out_map) a.out_map[o] = (int)r;
+                           }
+                       });
+    __syncthreads();
+    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
+    move_rows<V>(recv, out, a.row_bytes, r1 - r0, 1, src, dst, (int)((long long)vecs * piece / pieces),
+                 (int)((long long)vecs * (piece + 1) / pieces));
+}
+
+// Return direction of small calls, the same way: own range = output rows (routed copies).
+template <typename V>
+__global__ void __launch_bounds__(kIdxThreads, 2)
+tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, int pieces) {
+    extern __shared__ int sm[];
+    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, true);
+    int *const peer = sm + L.peer, *const all = sm + L.all, *const next = sm + L.next, *const first = sm + L.first;
+    const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
+    for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
+    grid_wait();
+    const int K = steps_in_use(a);
+    const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row_bytes;      // nothing is unpacked then
+    find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+    const int c0 = (int)((long long)a.items * c / n_cta), c1 = (int)((long long)a.items * (c + 1) / n_cta);
 #pragma unroll 4
-    for (int b0 = 0; b0 < n_chunks; b0 += 32) {
-        const int c = b0 + lane;
-        const int v = c < n_chunks ? in[(size_t)c * keys + key] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (c < n_chunks) out[(size_t)c * keys + key] = run + incl - v;
-        run += __shfl_sync(0xffffffffu, incl, 31);
+    for (int i = tid; i < a.items; i += kIdxThreads) {
+        const int key = copy_key_of(a, i);
+        if (key < 0) continue;
+        atomicAdd(&all[key], 1);
+        if (i < c0) atomicAdd(&next[key], 1);
     }
-    if (lane == 0) w.key_total[key] = run;
+    const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
+    const int st = return_runs(a, K, [&](int k) { return peer[k]; }, runs, sm + L.cnt, sm + L.scratch);
+    scan_keys(all, first, a.keys, sm + L.wsum);
+    if (blockIdx.x == 0) {                           // every sender's stream is used up exactly
+        int bad = st;
+        if (tid < a.N && tid != a.rank && first[(tid + 1) * a.epr] - first[tid * a.epr] != runs.total[tid]) bad = VP_ST_PACK_MISMATCH;
+        bad = __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
+        if (tid == 0) *a.status = over ? VP_ST_PACK_CAPACITY : bad;
+    }
+    int *const src = sm + L.src, *const dst = sm + L.dst;
+    if (tid < 32)
+        warp_positions(c0, c1, next, [&](long long i) { return copy_key_of(a, i); },
+                       [&](long long i, int key, int p) {
+                           int row = -1;
+                           if (p >= 0 && !over) {
+                               const int j = key / a.epr;
+                               row = run_lookup(runs, j, first[key] + p - first[j * a.epr]);   // position in sender j's stream
+                           }
+                           src[i - c0] = row;
+                           dst[i - c0] = (int)i;
+                           if (a.out_map && piece == 0) a.out_map[i] = row;
+                       });
+    __syncthreads();
+    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
+    move_rows<V>(recv, out, a.row_bytes, c1 - c0, 1, src, dst, (int)((long long)vecs * piece / pieces),
+                 (int)((long long)vecs * (piece + 1) / pieces));
 }
 
-// one block: exclusive scan over the keys (expert-major, then source), expert offsets, consistency check
-__global__ void __launch_bounds__(kMaxKeys)
-unpack_keys_kernel(int keys, int N, int experts_per_rank, UnpackWs w, int32_t* __restrict__ expert_off,
-                   int32_t* __restrict__ status) {
-    __shared__ int s[kMaxKeys];
-    __shared__ int warp_sum[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int v = tid < keys ? w.key_total[tid] : 0;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int ws = warp_sum[lane], wi = ws;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
-        }
-        warp_sum[lane] = wi - ws;
-    }
-    __syncthreads();
-    const int excl = warp_sum[warp] + incl - v;
-    s[tid] = excl;
-    if (tid < keys) w.key_base[tid] = excl;
-    __syncthreads();
-    if (expert_off && tid < experts_per_rank) expert_off[tid] = s[tid * N];
-    if (tid == kMaxKeys - 1) {
-        const int total = excl + v;
-        w.key_base[keys] = total;
-        if (expert_off) {
-            expert_off[experts_per_rank] = total;
-            if (!w.flags[0] && total != w.flags[2]) atomicOr(status, VP_ST_PACK_MISMATCH);
-        }
-    }
+// ---- chunked form -----------------------------------------------------------------------------------------------
+
+// A count CTA reads the plan's lane_dst itself up to this many cells (64 KB, five 16-byte loads per thread for the 300 of
+// 512 activations a 64-rank plan uses); larger plans have their steps resolved by steps_kernel first.
+constexpr int kInlineCells = 32768;
+constexpr int kStepTile = 32;                        // steps per CTA of steps_kernel
+
+__global__ void __launch_bounds__(kIdxThreads) unpack_steps_kernel(UnpackArgs a, UnpackWs w) {
+    __shared__ int peer[kStepTile];
+    grid_wait();
+    const int K = steps_in_use(a);
+    const int k0 = blockIdx.x * kStepTile, k1 = min(k0 + kStepTile, K);
+    if (k0 >= k1) return;
+    find_senders(a.lane_dst, a.N, a.rank, k0, k1, peer);
+    if (k0 + (int)threadIdx.x < k1) w.step_peer[k0 + threadIdx.x] = peer[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(kWarps * 32)
-unpack_map_kernel(long long capacity_rows, int N, int keys, UnpackWs w, int32_t* __restrict__ out_src,
-                  int32_t* __restrict__ out_map) {
-    __shared__ int next[kWarps][kMaxKeys];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long chunk = (long long)blockIdx.x * kWarps + warp;
-    const long long r0 = chunk * kChunk;
-    if (r0 >= capacity_rows) return;
-    for (int j = lane; j < keys; j += 32) next[warp][j] = w.key_base[j] + w.base[chunk * keys + j];
-    __syncwarp();
-    for (int it = 0; it < kItems; it++) {
-        const long long r = r0 + it * 32 + lane;
-        const int key = r < capacity_rows ? w.row_key[r] : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, key >= 0 ? key : -1 - lane);
-        int o = -1;
-        if (key >= 0) o = next[warp][key] + __popc(peers & ((1u << lane) - 1));
-        __syncwarp();
-        if (key >= 0 && (peers & ((1u << lane) - 1)) == 0) next[warp][key] += __popc(peers);
-        __syncwarp();
-        if (r < capacity_rows) {
-            w.out_row[r] = o;
-            if (o >= 0) {
-                if (out_src) out_src[o] = key % N;
-                if (out_map) out_map[o] = (int32_t)r;
+// Chunks in use: those that hold one of the R rows received (return direction: all of them).
+__device__ __forceinline__ int chunks_of(int items, int chunk) { return (items + chunk - 1) / chunk; }
+
+// steps: 0 the plan is read here, 1 its senders come from unpack_steps_kernel, 2 the same, and the tables stay in the
+// workspace because they exceed shared memory (every CTA then writes the same values there).
+__global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a, UnpackWs w, int chunk, int steps) {
+    extern __shared__ int sm[];                      // [keys] histogram, [k_max] sender, [k_max] first row of every step
+    int* const hist = sm;
+    int* const peer = steps == 2 ? w.step_peer : sm + a.keys;
+    int* const step_row = steps == 2 ? w.step_row : sm + a.keys + a.k_max;
+    const int tid = threadIdx.x;
+    for (int j = tid; j < a.keys; j += kIdxThreads) hist[j] = 0;
+    grid_wait();
+    const int K = steps_in_use(a);
+    int st, bad = 0;
+    const int R = rows_received(a, K, st);
+    if (blockIdx.x == 0 && tid == 0) { w.flags[0] = (st & VP_ST_PACK_CAPACITY) != 0; w.flags[1] = st; w.flags[2] = R; }
+    if ((int)blockIdx.x > 0 && (int)blockIdx.x >= chunks_of(R, chunk)) return;     // (CTA 0 always reports on the plan)
+    if (steps == 0) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+    for (int k = tid; k < K; k += kIdxThreads) {
+        int p = steps == 0 ? peer[k] : w.step_peer[k];
+        step_row[k] = check_step(a, k, p, bad);
+        peer[k] = p;
+    }
+    __syncthreads();
+    const int r0 = blockIdx.x * chunk, r1 = min(r0 + chunk, R);
+    for (int r = r0 + tid; r < r1; r += kIdxThreads) {
+        const int key = row_key_of(a, r, K, step_row, peer);
+        w.item_key[r] = key;
+        if (key >= 0) atomicAdd(&hist[key], 1);
+        else bad = VP_ST_PACK_MISMATCH;
+    }
+    bad = __syncthreads_or(bad);
+    for (int j = tid; j < a.keys; j += kIdxThreads) w.hist[(size_t)blockIdx.x * a.keys + j] = hist[j];
+    if (tid == 0) w.bad[blockIdx.x] = bad ? VP_ST_PACK_MISMATCH : 0;
+}
+
+__global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a, UnpackWs w, int chunk, int n_chunks, int inline_steps) {
+    extern __shared__ int sm[];
+    const int tid = threadIdx.x;
+    grid_wait();
+    if ((int)blockIdx.x == n_chunks) {               // the senders' run table
+        int *const cnt = sm, *const scratch = sm + a.N, *const peer = scratch + runs_scratch_ints(a.N);
+        const int K = steps_in_use(a);
+        if (inline_steps) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+        const int st = return_runs(a, K, [&](int k) { return inline_steps ? peer[k] : w.step_peer[k]; },
+                                   Runs{w.start, w.row, w.ptr, w.total}, cnt, scratch);
+        if (tid == 0) {
+            const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row_bytes;
+            w.flags[0] = over;
+            w.flags[1] = over ? VP_ST_PACK_CAPACITY : st;
+        }
+        return;
+    }
+    for (int j = tid; j < a.keys; j += kIdxThreads) sm[j] = 0;
+    __syncthreads();
+    const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)a.items);
+#pragma unroll 4
+    for (long long i = i0 + tid; i < i1; i += kIdxThreads) {
+        const int key = copy_key_of(a, i);
+        if (key >= 0) atomicAdd(&sm[key], 1);
+    }
+    __syncthreads();
+    for (int j = tid; j < a.keys; j += kIdxThreads) w.hist[(size_t)blockIdx.x * a.keys + j] = sm[j];
+}
+
+// Map of one chunk: all counts, the counts before this chunk, their prefix over the keys, then stable positions, every warp
+// a contiguous slice.  Shared memory: [keys] all, [keys] before, [keys + 1] first, wsum, [kIdxWarps][keys] slices.
+__host__ __device__ inline int map_smem_ints(int keys) { return 3 * keys + 1 + kIdxWarps + 1 + kIdxWarps * keys; }
+
+template <bool TOKENS>
+__global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, UnpackWs w, int chunk) {
+    extern __shared__ int sm[];
+    const int keys = a.keys, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int *const all = sm, *const before = all + keys, *const first = before + keys, *const wsum = first + keys + 1;
+    int *const slices = wsum + kIdxWarps + 1, *const next = slices + warp * keys;
+    for (int j = tid; j < 2 * keys; j += kIdxThreads) all[j] = 0;
+    for (int j = tid; j < kIdxWarps * keys; j += kIdxThreads) slices[j] = 0;
+    __syncthreads();
+    grid_wait();
+    const bool over = w.flags[0] != 0;
+    const int items = TOKENS ? a.items : w.flags[2];
+    const int n_chunks = chunks_of(items, chunk);
+    if (!TOKENS && (int)blockIdx.x > 0 && (int)blockIdx.x >= n_chunks) return;
+#pragma unroll 4
+    for (int i = tid; i < n_chunks * keys; i += kIdxThreads) {
+        const int v = w.hist[i];
+        if (v) {
+            const int b = i / keys, key = i - b * keys;
+            atomicAdd(&all[key], v);
+            if (b < (int)blockIdx.x) atomicAdd(&before[key], v);
+        }
+    }
+    const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)items);
+    const long long s0 = min(i0 + (long long)warp * (chunk / kIdxWarps), i1), s1 = min(s0 + chunk / kIdxWarps, i1);
+    auto key_of = [&](long long i) { return TOKENS ? copy_key_of(a, i) : w.item_key[i]; };
+    for (long long i = s0 + lane; i < s1; i += 32) {
+        const int key = key_of(i);
+        if (key >= 0) atomicAdd(&next[key], 1);
+    }
+    __syncthreads();
+    scan_keys(all, first, keys, wsum);
+    if (blockIdx.x == 0) {
+        int bad = 0;
+        if (TOKENS) {                                // every sender's stream is used up exactly
+            for (int j = tid; j < a.N; j += kIdxThreads)
+                if (j != a.rank && first[(j + 1) * a.epr] - first[j * a.epr] != w.total[j]) bad = VP_ST_PACK_MISMATCH;
+        } else {
+            for (int e = tid; e <= a.epr; e += kIdxThreads) a.expert_off[e] = first[e * a.N];
+            for (int b = tid; b < (n_chunks > 1 ? n_chunks : 1); b += kIdxThreads) bad |= w.bad[b];
+            if (!over && first[keys] != items) bad = VP_ST_PACK_MISMATCH;
+        }
+        bad = __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
+        if (tid == 0) *a.status = w.flags[1] | (TOKENS && over ? 0 : bad);
+    }
+    for (int j = tid; j < keys; j += kIdxThreads) {  // start of every warp's slice: key, chunks before, warps before
+        int run = first[j] + before[j];
+        for (int v = 0; v < kIdxWarps; v++) {
+            const int x = slices[v * keys + j];
+            slices[v * keys + j] = run;
+            run += x;
+        }
+    }
+    __syncthreads();
+    const Runs runs{w.start, w.row, w.ptr, w.total};
+    warp_positions(s0, s1, next, key_of, [&](long long i, int key, int p) {
+        if (TOKENS) {
+            int row = -1;
+            if (p >= 0 && !over) {
+                const int j = key / a.epr;
+                row = run_lookup(runs, j, p - first[j * a.epr]);
+            }
+            w.map[i] = row;
+            if (a.out_map) a.out_map[i] = row;
+        } else {
+            w.map[i] = p;
+            if (p >= 0) {
+                if (a.out_src) a.out_src[p] = key % a.N;
+                if (a.out_map) a.out_map[p] = (int)i;
             }
         }
+    });
+}
+
+// Both calls once their arguments are checked.
+template <bool TOKENS>
+int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* workspace, cudaStream_t stream) {
+    const int sms = sm_count_of_device();
+    if (!sms) return VP_E_CUDA;
+    const long long items = a.items;
+    // (shared memory of unpack_count_kernel: histogram and both step tables)
+    const bool steps_fit = ((long long)a.keys + 2ll * a.k_max) * 4 <= (long long)kSmemLimit;
+    const bool inline_steps = (long long)a.k_max * a.N <= kInlineCells && steps_fit;
+    cudaError_t e = cudaSuccess;
+    if (items <= kSmallItems && a.k_max <= kSmallSteps && inline_steps) {
+        const SmallSplit s = small_split(a.items, sms);
+        const int n_cta = s.grid / s.pieces;
+        const size_t smem = (size_t)unpack_small_layout(a.N, a.keys, a.k_max, TOKENS).ints * 4;
+        if ((items + n_cta - 1) / n_cta <= kSmallOwn) {
+            const char* from = (const char*)recv;
+            vp_prof_mark(3, 0, stream);
+            const auto go = [&](auto fn) { return launch_wide(fn, s.grid, smem, stream, a, from, (char*)out, s.pieces); };
+            const int width = copy_width(recv, out, a.row_bytes);
+            if constexpr (TOKENS)
+                e = width == 16 ? go(tokens_small_kernel<uint4>) : width == 4 ? go(tokens_small_kernel<uint32_t>) : go(tokens_small_kernel<uint8_t>);
+            else
+                e = width == 16 ? go(unpack_small_kernel<uint4>) : width == 4 ? go(unpack_small_kernel<uint32_t>) : go(unpack_small_kernel<uint8_t>);
+            vp_prof_mark(3, 1, stream);
+            return e == cudaSuccess ? VP_OK : VP_E_CUDA;
+        }
     }
+    const UnpackWs w = carve(workspace, a.N, a.keys, items, a.k_max);
+    const int chunk = chunk_items(items, a.keys), n_chunks = (int)((items + chunk - 1) / chunk);
+    if (!inline_steps) e = launch_after(unpack_steps_kernel, (a.k_max + kStepTile - 1) / kStepTile, kIdxThreads, 0, stream, a, w);
+    if (e == cudaSuccess) {
+        if constexpr (TOKENS) {
+            const size_t ints_runs = (size_t)a.N + runs_scratch_ints(a.N) + (inline_steps ? a.k_max : 0);
+            const size_t ints = ints_runs > (size_t)a.keys ? ints_runs : (size_t)a.keys;
+            e = launch_wide(tokens_count_kernel, n_chunks + 1, ints * 4, stream, a, w, chunk, n_chunks, (int)inline_steps);
+        } else {
+            const size_t ints = (size_t)a.keys + (steps_fit ? 2 * (size_t)a.k_max : 0);
+            e = launch_wide(unpack_count_kernel, n_chunks, ints * 4, stream, a, w, chunk, inline_steps ? 0 : (steps_fit ? 1 : 2));
+        }
+    }
+    if (e == cudaSuccess) e = launch_wide(unpack_map_kernel<TOKENS>, n_chunks, (size_t)map_smem_ints(a.keys) * 4, stream, a, w, chunk);
+    if (e != cudaSuccess) return VP_E_CUDA;
+    vp_prof_mark(3, 0, stream);
+    const int rc = launch_row_copy(recv, out, w.map, w.flags, a.items, 1, TOKENS, !TOKENS, a.row_bytes, a.status, stream);
+    vp_prof_mark(3, 1, stream);
+    return rc;
 }
 
 }  // namespace
@@ -242,7 +469,7 @@ unpack_map_kernel(long long capacity_rows, int N, int keys, UnpackWs w, int32_t*
 extern "C" size_t vp_unpack_workspace_bytes(int N, int64_t capacity_rows, int experts_per_rank, int k_max) {
     if (N <= 0 || N > VP_MAX_N || capacity_rows <= 0 || experts_per_rank <= 0 || k_max <= 0) return 0;
     if ((long long)N * experts_per_rank > kMaxKeys || capacity_rows >= ((int64_t)1 << 31)) return 0;
-    return carve(nullptr, N * experts_per_rank, capacity_rows, k_max).bytes;
+    return carve(nullptr, N, N * experts_per_rank, capacity_rows, k_max).bytes;
 }
 
 extern "C" int vp_unpack(const int32_t* n_steps_b, const int16_t* lane_dst_b, const int64_t* recv_off_b, int N, int rank,
@@ -253,171 +480,20 @@ extern "C" int vp_unpack(const int32_t* n_steps_b, const int16_t* lane_dst_b, co
     if (N <= 0 || N > VP_MAX_N || rank < 0 || rank >= N || k_max <= 0 || row_bytes <= 0 || capacity_rows <= 0 ||
         experts_per_rank <= 0)
         return VP_E_BAD_ARG;
-    const int keys = N * experts_per_rank;
     if ((long long)N * experts_per_rank > kMaxKeys || capacity_rows >= ((int64_t)1 << 31)) return VP_E_UNSUPPORTED;
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < vp_unpack_workspace_bytes(N, capacity_rows, experts_per_rank, k_max))
         return VP_E_WORKSPACE;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    UnpackWs w = carve(workspace, keys, capacity_rows, k_max);
-    const int n_chunks = (int)((capacity_rows + kChunk - 1) / kChunk);
-    const int blocks = (n_chunks + kWarps - 1) / kWarps;
-    if (cudaMemsetAsync(w.flags, 0, 256, stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess) return VP_E_CUDA;
-    unpack_plan_kernel<<<1, 256, 0, stream>>>(n_steps_b, lane_dst_b, recv_off_b, N, rank, k_max, row_bytes, capacity_rows, w, status);
-    unpack_count_kernel<<<blocks, kWarps * 32, 0, stream>>>(recv_expert, capacity_rows, N, experts_per_rank, keys, w, status, 0, rank);
-    unpack_scan_kernel<<<(keys + kWarps - 1) / kWarps, kWarps * 32, 0, stream>>>(keys, n_chunks, w);
-    unpack_keys_kernel<<<1, kMaxKeys, 0, stream>>>(keys, N, experts_per_rank, w, expert_off, status);
-    unpack_map_kernel<<<blocks, kWarps * 32, 0, stream>>>(capacity_rows, N, keys, w, out_src, out_map);
-    g_vp_launches += 5;
-    if (cudaGetLastError() != cudaSuccess) return VP_E_CUDA;
-    vp_prof_mark(3, 0, stream);
-    const int rc = launch_row_copy(recv, out, w.out_row, w.flags, (int)capacity_rows, 1, row_bytes, status, stream);
-    vp_prof_mark(3, 1, stream);
-    return rc;
+    const UnpackArgs a{n_steps_b, lane_dst_b, nullptr, recv_off_b, N, rank, k_max, experts_per_rank, N * experts_per_rank,
+                       (int)capacity_rows, recv_expert, row_bytes, capacity_rows, expert_off, out_src, out_map, status};
+    return unpack_launch<false>(a, recv, out, workspace, (cudaStream_t)cuda_stream);
 }
 
 // ---- return direction: receive buffer -> token layout ---------------------------------------------------
 
-namespace {
-
-struct TokWs {
-    UnpackWs u;            // flags, histograms, scans, key of every copy (row_key), inverse map (out_row)
-    int32_t* step_sender;  // [k_max] sender of the step's segment for this rank, -1 = none
-    int32_t* step_row0;    // [k_max] first receive row of the segment
-    int32_t* step_rows;    // [k_max] its rows
-    int32_t* sender_ptr;   // [N + 1] segments of sender j are sseg_*[sender_ptr[j] .. sender_ptr[j+1])
-    int32_t* sender_total; // [N] rows sender j delivers
-    int32_t* sseg_stream0; // [k_max] position of the segment's first row in the sender's stream
-    int32_t* sseg_row0;    // [k_max]
-    int32_t* sseg_rows;    // [k_max]
-    size_t bytes;
-};
-
-TokWs carve_tokens(void* base, int N, int keys, long long copies, long long capacity_rows, int k_max) {
-    TokWs w;
-    size_t o = 0;
-    auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (char*)base + at; };
-    const long long n_chunks = (copies + kChunk - 1) / kChunk;
-    w.u.flags = (int32_t*)take(256);
-    w.u.seg_row0 = w.u.seg_end = w.u.seg_src = nullptr;
-    w.u.hist = (int32_t*)take((size_t)n_chunks * keys * 4);
-    w.u.base = (int32_t*)take((size_t)n_chunks * keys * 4);
-    w.u.key_total = (int32_t*)take((size_t)keys * 4);
-    w.u.key_base = (int32_t*)take((size_t)(keys + 1) * 4);
-    w.u.row_key = (int32_t*)take((size_t)copies * 4);
-    w.u.out_row = (int32_t*)take((size_t)capacity_rows * 4);
-    w.step_sender = (int32_t*)take((size_t)k_max * 4);
-    w.step_row0 = (int32_t*)take((size_t)k_max * 4);
-    w.step_rows = (int32_t*)take((size_t)k_max * 4);
-    w.sender_ptr = (int32_t*)take((size_t)(N + 1) * 4);
-    w.sender_total = (int32_t*)take((size_t)N * 4);
-    w.sseg_stream0 = (int32_t*)take((size_t)k_max * 4);
-    w.sseg_row0 = (int32_t*)take((size_t)k_max * 4);
-    w.sseg_rows = (int32_t*)take((size_t)k_max * 4);
-    w.bytes = o;
-    return w;
-}
-
-// One block of VP_MAX_N threads: the segment every step delivers to `rank`, then per sender its segments in step order.
-__global__ void __launch_bounds__(VP_MAX_N)
-tokens_plan_kernel(const int32_t* __restrict__ n_steps_p, const int16_t* __restrict__ lane_dst,
-                   const int64_t* __restrict__ lane_bytes, const int64_t* __restrict__ recv_off, int N, int rank, int k_max,
-                   int64_t row_bytes, long long capacity_rows, TokWs w, int32_t* __restrict__ status) {
-    __shared__ int s_cnt[VP_MAX_N + 1];
-    const int tid = threadIdx.x;
-    int K = *n_steps_p;
-    K = K < 0 ? 0 : (K > k_max ? k_max : K);
-    const bool over = recv_off[(size_t)K * N + rank] > capacity_rows * row_bytes;      // nothing is unpacked then
-    if (tid == 0 && over) { atomicOr(status, VP_ST_PACK_CAPACITY); w.u.flags[0] = 1; }
-    bool bad = false;
-    for (int k = tid; k < K; k += blockDim.x) {
-        int sender = -1;
-        for (int j = 0; j < N; j++)
-            if (lane_dst[(size_t)k * N + j] == rank) sender = j;
-        int rows = 0, row0 = 0;
-        if (sender >= 0) {
-            const int64_t bytes = lane_bytes[(size_t)k * N + sender], at = recv_off[(size_t)k * N + rank];
-            if (bytes % row_bytes || at % row_bytes) { bad = true; sender = -1; }       // such a segment is left out
-            else { rows = (int)(bytes / row_bytes); row0 = (int)(at / row_bytes); }
-        }
-        w.step_sender[k] = rows > 0 ? sender : -1;
-        w.step_row0[k] = row0;
-        w.step_rows[k] = rows;
-    }
-    if (bad && !over) atomicOr(status, VP_ST_PACK_MISMATCH);
-    __syncthreads();
-    int cnt = 0;
-    if (tid < N)
-        for (int k = 0; k < K; k++) cnt += w.step_sender[k] == tid;
-    s_cnt[tid] = tid < N ? cnt : 0;
-    __syncthreads();
-    if (tid == 0) {
-        int run = 0;
-        for (int j = 0; j < N; j++) { const int c = s_cnt[j]; s_cnt[j] = run; run += c; }
-        s_cnt[N] = run;
-    }
-    __syncthreads();
-    if (tid <= N) w.sender_ptr[tid] = s_cnt[tid];
-    if (tid < N) {
-        int at = s_cnt[tid], stream = 0;
-        for (int k = 0; k < K; k++)
-            if (w.step_sender[k] == tid) {
-                w.sseg_stream0[at] = stream; w.sseg_row0[at] = w.step_row0[k]; w.sseg_rows[at] = w.step_rows[k];
-                stream += w.step_rows[k]; at++;
-            }
-        w.sender_total[tid] = stream;
-    }
-}
-
-__global__ void __launch_bounds__(kWarps * 32)
-tokens_map_kernel(long long copies, int N, int experts_per_rank, int keys, int rank, TokWs w, int32_t* __restrict__ out_map,
-                  int32_t* __restrict__ status) {
-    __shared__ int next[kWarps][kMaxKeys];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (blockIdx.x == 0 && threadIdx.x < N && threadIdx.x != rank && !w.u.flags[0]) {      // every sender's stream is used up exactly
-        const int j = threadIdx.x;
-        if (w.u.key_base[(j + 1) * experts_per_rank] - w.u.key_base[j * experts_per_rank] != w.sender_total[j])
-            atomicOr(status, VP_ST_PACK_MISMATCH);
-    }
-    const long long chunk = (long long)blockIdx.x * kWarps + warp;
-    const long long c0 = chunk * kChunk;
-    if (c0 >= copies) return;
-    for (int j = lane; j < keys; j += 32) next[warp][j] = w.u.key_base[j] + w.u.base[chunk * keys + j];
-    __syncwarp();
-    for (int it = 0; it < kItems; it++) {
-        const long long c = c0 + it * 32 + lane;
-        const int key = c < copies ? w.u.row_key[c] : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, key >= 0 ? key : -1 - lane);
-        int gpos = -1;
-        if (key >= 0) gpos = next[warp][key] + __popc(peers & ((1u << lane) - 1));
-        __syncwarp();
-        if (key >= 0 && (peers & ((1u << lane) - 1)) == 0) next[warp][key] += __popc(peers);
-        __syncwarp();
-        if (c >= copies) continue;
-        int rrow = -1;
-        if (key >= 0) {
-            const int j = key / experts_per_rank;
-            const int pos = gpos - w.u.key_base[j * experts_per_rank];           // position in sender j's stream
-            int lo = w.sender_ptr[j], hi = w.sender_ptr[j + 1] - 1;
-            if (hi >= lo && pos < w.sender_total[j]) {
-                while (lo < hi) {                                                // last segment starting at or before pos
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (w.sseg_stream0[mid] <= pos) lo = mid; else hi = mid - 1;
-                }
-                rrow = w.sseg_row0[lo] + pos - w.sseg_stream0[lo];
-                w.u.out_row[rrow] = (int32_t)c;
-            }
-        }
-        if (out_map) out_map[c] = rrow;
-    }
-}
-
-}  // namespace
-
 extern "C" size_t vp_unpack_tokens_workspace_bytes(int N, int T, int topk, int experts_per_rank, int64_t capacity_rows, int k_max) {
     if (N <= 0 || N > VP_MAX_N || T <= 0 || topk <= 0 || capacity_rows <= 0 || experts_per_rank <= 0 || k_max <= 0) return 0;
     if ((long long)N * experts_per_rank > kMaxKeys || capacity_rows >= ((int64_t)1 << 31) || (long long)T * topk >= ((long long)1 << 31)) return 0;
-    return carve_tokens(nullptr, N, N * experts_per_rank, (long long)T * topk, capacity_rows, k_max).bytes;
+    return carve(nullptr, N, N * experts_per_rank, (long long)T * topk, k_max).bytes;
 }
 
 extern "C" int vp_unpack_tokens(const int32_t* n_steps_b, const int16_t* lane_dst_b, const int64_t* lane_bytes_b,
@@ -431,25 +507,7 @@ extern "C" int vp_unpack_tokens(const int32_t* n_steps_b, const int16_t* lane_ds
     const size_t need = vp_unpack_tokens_workspace_bytes(N, T, topk, experts_per_rank, capacity_rows, k_max);
     if (!need) return VP_E_UNSUPPORTED;
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < need) return VP_E_WORKSPACE;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    const int keys = N * experts_per_rank;
-    const long long copies = (long long)T * topk;
-    TokWs w = carve_tokens(workspace, N, keys, copies, capacity_rows, k_max);
-    const int n_chunks = (int)((copies + kChunk - 1) / kChunk);
-    const int blocks = (n_chunks + kWarps - 1) / kWarps;
-    if (cudaMemsetAsync(w.u.flags, 0, 256, stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaMemsetAsync(w.u.out_row, 0xFF, (size_t)capacity_rows * 4, stream) != cudaSuccess) return VP_E_CUDA;
-    tokens_plan_kernel<<<1, VP_MAX_N, 0, stream>>>(n_steps_b, lane_dst_b, lane_bytes_b, recv_off_b, N, rank, k_max, row_bytes,
-                                                   capacity_rows, w, status);
-    unpack_count_kernel<<<blocks, kWarps * 32, 0, stream>>>(expert_idx, copies, N, experts_per_rank, keys, w.u, status, 1, rank);
-    unpack_scan_kernel<<<(keys + kWarps - 1) / kWarps, kWarps * 32, 0, stream>>>(keys, n_chunks, w.u);
-    unpack_keys_kernel<<<1, kMaxKeys, 0, stream>>>(keys, N, experts_per_rank, w.u, nullptr, status);
-    tokens_map_kernel<<<blocks, kWarps * 32, 0, stream>>>(copies, N, experts_per_rank, keys, rank, w, out_map, status);
-    g_vp_launches += 5;
-    if (cudaGetLastError() != cudaSuccess) return VP_E_CUDA;
-    vp_prof_mark(3, 0, stream);
-    const int rc = launch_row_copy(recv, out, w.u.out_row, w.u.flags, (int)capacity_rows, 1, row_bytes, status, stream);
-    vp_prof_mark(3, 1, stream);
-    return rc;
+    const UnpackArgs a{n_steps_b, lane_dst_b, lane_bytes_b, recv_off_b, N, rank, k_max, experts_per_rank, N * experts_per_rank,
+                       T * topk, expert_idx, row_bytes, capacity_rows, nullptr, nullptr, out_map, status};
+    return unpack_launch<true>(a, recv, out, workspace, (cudaStream_t)cuda_stream);
 }

@@ -1,0 +1,78 @@
+"""GPU parity of the pack and both unpack directions where their index work changes form: one self-contained launch up to
+16,384 items and 1,024 plan rows, chunked histograms beyond; the plan's senders read in place or resolved by a kernel of
+their own; fewer rows than SMs (a row split over CTAs) and more; every copy width."""
+import numpy as np
+import pytest
+import torch
+
+import tests.test_gpu_pack as tp
+import tests.test_gpu_unpack as tu
+from tests.test_gpu_pack import vp  # noqa: F401  (fixture)
+from workloads import SchedParams as WParams
+from workloads.configs import catalog_for
+from workloads.demand import demand_from_routing, moe_routing
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(nodes, tokens, topk, row_bytes, k_max=0, seed=0):
+    """One call on ``nodes`` nodes; row_bytes a multiple of two: int16 rows, otherwise bytes."""
+    cat = catalog_for(nodes, "complete" if nodes <= 2 else "template")
+    N = cat.topology.N
+    E = 4 * N if N <= 128 else N
+    rank = (seed * 5 + 3) % N
+    idx = moe_routing(N * tokens, E, topk, 0.8, seed=seed, device="cuda")
+    D = demand_from_routing(idx, torch.arange(N, device="cuda").repeat_interleave(tokens), N, E, row_bytes).cpu()
+    gen = torch.Generator().manual_seed(seed)
+    if row_bytes % 2:
+        rows = torch.randint(0, 256, (tokens, row_bytes), dtype=torch.uint8, generator=gen)
+    else:
+        rows = torch.randint(-32768, 32768, (tokens, row_bytes // 2), dtype=torch.int16, generator=gen)
+    w = WParams(granule_bytes=row_bytes, k_max=k_max).resolved(N)
+    return dict(catalog=cat, demand=D.unsqueeze(0), params=w, rank=rank, rows=rows, row_bytes=row_bytes, topk=topk,
+                expert_idx=idx.view(N, tokens, topk)[rank].cpu().contiguous(), experts_per_rank=E // N)
+
+
+# (nodes, tokens, topk, row bytes, k_max): one CTA per token; a token over several CTAs; exactly the limit of the one-launch
+# form and one token more; long plans (k_max above 1,024, above what a count CTA reads itself); 64, 128 and 256 ranks; rows that
+# are multiples of 16, 4 and 1 bytes on both sides of 2 KB, and rows of more than one 16 KB piece
+CASES = [(2, 1, 1, 4096, 0), (2, 5, 8, 14336, 0), (1, 149, 3, 4100, 0), (2, 700, 6, 333, 0), (2, 2048, 8, 96, 0), (2, 2049, 8, 96, 0),
+         (2, 2400, 8, 2064, 0), (2, 2100, 8, 4100, 0), (2, 300, 8, 2048, 1025), (2, 300, 8, 2048, 40000), (8, 40, 6, 7392, 0),
+         (8, 2300, 8, 1536, 0), (16, 30, 4, 4096, 2048), (32, 12, 8, 512, 4096), (2, 2100, 8, 16400, 0)]
+
+
+@pytest.mark.parametrize("nodes,tokens,topk,row_bytes,k_max", CASES)
+def test_pack_forms(vp, oracle_lib, nodes, tokens, topk, row_bytes, k_max):  # noqa: F811
+    res = tp._run_case(vp, oracle_lib, _case(nodes, tokens, topk, row_bytes, k_max, seed=tokens))
+    assert res[2] == 0
+    tp._assert_pack(res)
+
+
+@pytest.mark.parametrize("nodes,tokens,topk,row_bytes,k_max", CASES)
+def test_unpack_forms(vp, oracle_lib, nodes, tokens, topk, row_bytes, k_max):  # noqa: F811
+    case = _case(nodes, tokens, topk, row_bytes, k_max, seed=tokens + 1)
+    oc, plan, one = tu._plans(vp, oracle_lib, case["catalog"], case["demand"], case["params"])
+    R, recv, expert = tu._receive_case(case, case["rank"], case["experts_per_rank"], seed=1,
+                                       dtype=torch.uint8 if row_bytes % 2 else torch.int16, extra_rows=5)
+    got, want, cap = tu._run(vp, oc, plan, one, case["rank"], recv, expert, case["experts_per_rank"])
+    assert got[4] == 0 and int(got[1][-1]) == R
+    tu._assert_unpack(got, want, cap)
+
+
+@pytest.mark.parametrize("nodes,tokens,topk,row_bytes,k_max", [c for c in CASES if c[3] % 2 == 0])
+def test_unpack_tokens_forms(vp, oracle_lib, nodes, tokens, topk, row_bytes, k_max):  # noqa: F811
+    case = _case(nodes, tokens, topk, row_bytes, k_max, seed=tokens + 2)
+    oc, plan, one, R, recv = tu._return_case(vp, oracle_lib, case, case["rank"], seed=2, extra_rows=3)
+    st, w_map = tu._run_tokens(vp, oc, plan, one, case["rank"], case["expert_idx"], case["experts_per_rank"], recv)
+    assert st == 0 and int((w_map >= 0).sum()) == R
+
+
+@pytest.mark.parametrize("tokens", [300, 2300])
+def test_pack_mismatch_and_capacity_in_both_forms(vp, oracle_lib, tokens):  # noqa: F811
+    case = _case(2, tokens, 8, 1024, seed=7)
+    R = int(case["demand"][0, case["rank"]].sum().item() // 1024)
+    res = tp._run_case(vp, oracle_lib, case, capacity_rows=R - 1)
+    assert res[2] == vp.ST_PACK_CAPACITY == res[5] and not res[0][:R - 1].any()
+    case["expert_idx"][0, 0] = 1 << 20                         # an expert on no rank
+    res = tp._run_case(vp, oracle_lib, case)
+    assert res[2] == vp.ST_PACK_MISMATCH and res[5] & vp.ST_PACK_MISMATCH
