@@ -18,9 +18,11 @@ struct PackArgs {
     const int32_t* n_steps;
     const int16_t* lane_dst;
     const int64_t *lane_bytes, *send_off;
-    int N, rank, k_max, T, topk, epr;
+    int N, rank, k_max, T, topk;
+    SmallDiv epr;
     const int32_t* idx;
-    int64_t row_bytes, capacity;
+    RowDiv row;
+    int64_t capacity;
     int32_t *src_map, *status;
 };
 
@@ -57,25 +59,27 @@ PackWs carve(void* base, int N, int T, int topk, int k_max) {
 // Destination rank of a routed copy, or -1 if it is not staged (dropped, local, out of range: that one sets `bad`).
 __device__ __forceinline__ int dest_of(int x, const PackArgs& a, int& bad) {
     if (x < 0) return -1;
-    const int j = (int)((unsigned)x / (unsigned)a.epr);
+    const int j = a.epr.div(x);
     if (j >= a.N) { bad = VP_ST_PACK_MISMATCH; return -1; }
     return j == a.rank ? -1 : j;
 }
 
 __device__ __forceinline__ int steps_in_use(const PackArgs& a) { return min(max(*a.n_steps, 0), a.k_max); }
 
+__device__ __forceinline__ Step pack_step(const PackArgs& a, int k, int& bad) {
+    const size_t at = (size_t)k * a.N + a.rank;
+    int64_t odd, ignore;
+    const int j = a.lane_dst[at];
+    const int64_t rows = a.row.div(a.lane_bytes[at], odd), row0 = a.row.div(a.send_off[at], ignore);
+    if (j < 0 || j >= a.N) return Step{-1, 0, 0};
+    if (odd) bad = VP_ST_PACK_MISMATCH;
+    return Step{j, (int)rows, (int)row0};
+}
+
 // Status bits of the run table, the same in every thread.
-__device__ __forceinline__ int pack_runs(const PackArgs& a, int K, Runs out, int* cnt, int* scratch) {
-    int bad = 0;
-    build_runs(K, a.N, [&](int k, int& j, int& rows, int& row0) {
-        const size_t at = (size_t)k * a.N + a.rank;
-        const int64_t bytes = a.lane_bytes[at];
-        j = a.lane_dst[at];
-        if (j >= a.N) j = -1;
-        rows = (int)(bytes / a.row_bytes);
-        row0 = (int)(a.send_off[at] / a.row_bytes);
-        if (j >= 0 && bytes % a.row_bytes) bad = VP_ST_PACK_MISMATCH;
-    }, out, cnt, scratch);
+__device__ __forceinline__ int pack_runs(const PackArgs& a, int K, Step first, int bad, Runs out, int* cnt, int* scratch) {
+    if ((int)threadIdx.x >= K) bad = 0;
+    build_runs(K, a.N, first, [&](int k) { return pack_step(a, k, bad); }, out, cnt, scratch);
     if (threadIdx.x == 0 && out.total[a.rank] != 0) bad = VP_ST_PACK_MISMATCH;
     return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
 }
@@ -114,17 +118,17 @@ pack_small_kernel(PackArgs a, const char* __restrict__ rows, char* __restrict__ 
     const int t0 = (int)((long long)a.T * c / n_cta), t1 = (int)((long long)a.T * (c + 1) / n_cta);
     for (int j = tid; j < a.N; j += kIdxThreads) hist[j] = 0;
     grid_wait();
+    int bad = 0, bad_step = 0;
+    const Step first = tid < a.k_max ? pack_step(a, tid, bad_step) : Step{-1, 0, 0};
     const int K = steps_in_use(a);
     const bool over = a.send_off[(size_t)K * a.N + a.rank] > a.capacity;
     __syncthreads();
-    int bad = 0;
-#pragma unroll 4
-    for (int e = tid; e < t0 * a.topk; e += kIdxThreads) {
-        const int j = dest_of(a.idx[e], a, bad);
+    for_each_item(a.idx, 0, t0 * a.topk, [&](int, int x) {
+        const int j = dest_of(x, a, bad);
         if (j >= 0) atomicAdd(&hist[j], 1);
-    }
+    });
     const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
-    const int st = pack_runs(a, K, runs, sm + L.cnt, sm + L.scratch);   // (ends with a barrier: the histogram is complete, too)
+    const int st = pack_runs(a, K, first, bad_step, runs, sm + L.cnt, sm + L.scratch);   // (ends with a barrier: the histogram is complete, too)
     int *const src = sm + L.src, *const dst = sm + L.dst;
     if (tid < 32)
         warp_positions(t0 * a.topk, t1 * a.topk, hist, [&](long long e) { return dest_of(a.idx[e], a, bad); },
@@ -142,8 +146,8 @@ pack_small_kernel(PackArgs a, const char* __restrict__ rows, char* __restrict__ 
         if (tid == 0) *a.status = st | (any ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
     }
     if (over) return;
-    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
-    move_rows<V>(rows, staged, a.row_bytes, t1 - t0, a.topk, src, dst, (int)((long long)vecs * piece / pieces),
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
+    move_rows<V>(rows, staged, a.row.d, t1 - t0, a.topk, src, dst, (int)((long long)vecs * piece / pieces),
                  (int)((long long)vecs * (piece + 1) / pieces));
 }
 
@@ -155,8 +159,10 @@ __global__ void __launch_bounds__(kIdxThreads) pack_count_kernel(PackArgs a, Pac
     const int tid = threadIdx.x, N = a.N;
     grid_wait();
     if ((int)blockIdx.x == n_chunks) {
+        int bad = 0;
+        const Step first = tid < a.k_max ? pack_step(a, tid, bad) : Step{-1, 0, 0};
         const int K = steps_in_use(a);
-        const int st = pack_runs(a, K, Runs{w.start, w.row, w.ptr, w.total}, sm, sm + N);
+        const int st = pack_runs(a, K, first, bad, Runs{w.start, w.row, w.ptr, w.total}, sm, sm + N);
         if (tid == 0) {
             const bool over = a.send_off[(size_t)K * N + a.rank] > a.capacity;
             w.flags[0] = over;
@@ -179,20 +185,18 @@ __global__ void __launch_bounds__(kIdxThreads) pack_count_kernel(PackArgs a, Pac
 }
 
 // CTA b maps chunk b, every warp a contiguous slice of it; the last CTA, whose base and own counts are all counts, checks
-// them against the plan and writes the status.
+// them against the plan and writes the status.  The routing is read before the wait for the count kernel: that kernel has
+// started, so whatever wrote the routing has finished.
+constexpr int kMapRuns = 2048;                       // runs whose table is copied to shared memory
+__host__ __device__ inline int pack_map_ints(int N, int k_max) { return N * (kIdxWarps + 1) + 2 * N + 1 + 2 * (k_max < kMapRuns ? k_max : kMapRuns); }
+
 __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackWs w, int chunk) {
-    extern __shared__ int sm[];                      // [N] base, then [kIdxWarps][N] next position of every warp's slice
+    extern __shared__ int sm[];                      // [N] base, [kIdxWarps][N] next position of every warp's slice, run table
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N = a.N;
     int* const base = sm;
     int* const next = sm + N + warp * N;
     for (int j = tid; j < N * (kIdxWarps + 1); j += kIdxThreads) sm[j] = 0;
     __syncthreads();
-    grid_wait();
-#pragma unroll 4
-    for (int i = tid; i < (int)blockIdx.x * N; i += kIdxThreads) {
-        const int v = w.hist[i];
-        if (v) atomicAdd(&base[i % N], v);
-    }
     const long long E = (long long)a.T * a.topk, e0 = (long long)blockIdx.x * chunk, e1 = min(e0 + chunk, E);
     const long long s0 = min(e0 + (long long)warp * (chunk / kIdxWarps), e1), s1 = min(s0 + chunk / kIdxWarps, e1);
     int ignore = 0;
@@ -200,6 +204,14 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
         const int j = dest_of(a.idx[e], a, ignore);
         if (j >= 0) atomicAdd(&next[j], 1);
     }
+    grid_wait();
+#pragma unroll 8
+    for (int i = tid; i < (int)blockIdx.x * N; i += kIdxThreads) {
+        const int v = w.hist[i];
+        if (v) atomicAdd(&base[i % N], v);
+    }
+    const bool over = w.flags[0] != 0;
+    const Runs runs = runs_to_shared(Runs{w.start, w.row, w.ptr, w.total}, N, kMapRuns, sm + N * (kIdxWarps + 1));
     __syncthreads();
     for (int j = tid; j < N; j += kIdxThreads) {     // exclusive prefix over the warps
         int run = base[j];
@@ -215,13 +227,11 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
     if (blockIdx.x == gridDim.x - 1) {
         int bad = w.flags[1];
         for (int j = tid; j < N; j += kIdxThreads)
-            if (j != a.rank && base[j] != w.total[j]) bad |= VP_ST_PACK_MISMATCH;
+            if (j != a.rank && base[j] != runs.total[j]) bad |= VP_ST_PACK_MISMATCH;
         for (int b = tid; b < (int)gridDim.x; b += kIdxThreads) bad |= w.bad[b];
         const int mismatch = __syncthreads_or(bad & VP_ST_PACK_MISMATCH);
         if (tid == 0) *a.status = (bad & VP_ST_PACK_CAPACITY) | (mismatch ? VP_ST_PACK_MISMATCH : 0);
     }
-    const bool over = w.flags[0] != 0;
-    const Runs runs{w.start, w.row, w.ptr, w.total};
     warp_positions(s0, s1, next, [&](long long e) { return dest_of(a.idx[e], a, ignore); },
                    [&](long long e, int j, int p) {
                        const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
@@ -253,8 +263,8 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
         return VP_E_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const long long E = (long long)T * topk;
-    const PackArgs a{n_steps_b, lane_dst_b, lane_bytes_b, send_off_b, N, rank, k_max, T, topk, experts_per_rank,
-                     expert_idx, row_bytes, staged_capacity_bytes, src_map, status};
+    const PackArgs a{n_steps_b, lane_dst_b, lane_bytes_b, send_off_b, N, rank, k_max, T, topk, small_div(experts_per_rank),
+                     expert_idx, row_div(row_bytes), staged_capacity_bytes, src_map, status};
     const int sms = sm_count_of_device();
     if (!sms) return VP_E_CUDA;
     if (E <= kSmallItems && k_max <= kSmallSteps) {
@@ -276,7 +286,7 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
     const int chunk = chunk_items(E, N), n_chunks = (int)((E + chunk - 1) / chunk);
     vp_prof_mark(1, 0, stream);
     cudaError_t e = launch_after(pack_count_kernel, n_chunks + 1, kIdxThreads, (size_t)(N + runs_scratch_ints(N)) * 4, stream, a, w, chunk, n_chunks);
-    if (e == cudaSuccess) e = launch_after(pack_map_kernel, n_chunks, kIdxThreads, (size_t)N * (kIdxWarps + 1) * 4, stream, a, w, chunk);
+    if (e == cudaSuccess) e = launch_after(pack_map_kernel, n_chunks, kIdxThreads, (size_t)pack_map_ints(N, k_max) * 4, stream, a, w, chunk);
     vp_prof_mark(1, 1, stream);
     if (e != cudaSuccess) return VP_E_CUDA;
     vp_prof_mark(2, 0, stream);

@@ -22,12 +22,37 @@ namespace {
 constexpr int kIdxThreads = 512;                    // threads of every index CTA
 constexpr int kIdxWarps = kIdxThreads / 32;
 constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
-// Items up to which one self-contained launch is used.  Its last CTA counts every item itself: 32 loads and shared-memory
-// atomics per thread at this limit, about what the two extra launches of the chunked form cost.
-constexpr int kSmallItems = 16384;
+// Items up to which one self-contained launch is used.  Its last CTA counts every item itself, and the rows move by plain loads
+// and stores (10 % behind the bulk copy).  At 8,192 items the two forms cost the same: index work of 10 and 11 us.
+constexpr int kSmallItems = 8192;
 constexpr int kSmallSteps = 1024;                   // plan arrays longer than this do not fit its run table
 constexpr int kSmallOwn = 1024;                     // rows or copies one CTA may own there
-constexpr int kMinChunk = 2048;                     // items per histogram of the chunked form, at least
+constexpr int kMinChunk = kIdxThreads;              // items per histogram of the chunked form, at least: one per thread
+
+// Division by the row size and by the experts per rank without a divide sequence: plan offsets are below 2^52, so the
+// product with the rounded reciprocal is off by one at most; expert ids are below 2^31 (multiply-high and shift, exact).
+struct RowDiv {
+    int64_t d;
+    double inv;
+    __device__ __forceinline__ int64_t div(int64_t x, int64_t& rem) const {
+        int64_t q = __double2ll_rz((double)x * inv), r = x - q * d;
+        if (r < 0) { q--; r += d; }
+        else if (r >= d) { q++; r -= d; }
+        rem = r;
+        return q;
+    }
+};
+inline RowDiv row_div(int64_t d) { return RowDiv{d, 1.0 / (double)d}; }
+struct SmallDiv {
+    uint32_t m;
+    int shift;
+    __device__ __forceinline__ int div(int x) const { return (int)((__umulhi(m, (uint32_t)x) + (uint32_t)x) >> shift); }
+};
+inline SmallDiv small_div(int d) {
+    int l = 0;
+    while (((int64_t)1 << l) < d) l++;
+    return SmallDiv{(uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << l) - (uint64_t)d)) / (uint64_t)d + 1), l};
+}
 
 // Launch that may start while the kernel ahead of it in the stream drains (its griddepcontrol.wait holds it back).
 template <typename... P, typename... A>
@@ -97,10 +122,13 @@ __device__ __forceinline__ int cta_exclusive_scan(int v, int* wsum, int& sum) {
 // Scratch of build_runs: counts and rows per (warp, bucket).
 __host__ __device__ inline int runs_scratch_ints(int N) { return 2 * kIdxWarps * N + kIdxWarps + 1; }
 
-// Builds the run table from the steps k < K; step(k, j, rows, row0) names the bucket (-1: none), the rows and the first row
-// of step k.  out.* may be shared or global memory (each element is written once, by one thread); cnt is [N] ints of shared memory.
-template <typename Step>
-__device__ __forceinline__ void build_runs(int K, int N, Step step, Runs out, int* cnt, int* scratch) {
+// One step of the plan as the rank sees it: bucket (-1: none), rows, first row.
+struct Step { int j, rows, row0; };
+
+// Builds the run table from the steps step(k), k < K.  `first` is step(threadIdx.x), which the caller fetches before it knows K
+// (the plan arrays have k_max rows, and a trip to L2 is saved); what lies beyond K is ignored here.  out.* may be shared or global memory (each element is written once, by one thread); cnt is [N] ints of shared memory.
+template <typename StepFn>
+__device__ __forceinline__ void build_runs(int K, int N, Step first, StepFn step, Runs out, int* cnt, int* scratch) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int* wcnt = scratch;
     int* wrow = scratch + kIdxWarps * N;
@@ -108,29 +136,24 @@ __device__ __forceinline__ void build_runs(int K, int N, Step step, Runs out, in
     for (int j = tid; j < N; j += kIdxThreads) cnt[j] = 0;
     for (int e = tid; e < 2 * kIdxWarps * N; e += kIdxThreads) scratch[e] = 0;
     __syncthreads();
-    // the first tile's steps stay in registers: plans of at most kIdxThreads activations are read once
-    int j0 = -1, rows0 = 0, base0 = 0;
-    if (tid < K) step(tid, j0, rows0, base0);
-    if (j0 >= 0) atomicAdd(&cnt[j0], 1);
+    if (tid >= K) first.j = -1;
+    if (first.j >= 0) atomicAdd(&cnt[first.j], 1);
     for (int k = tid + kIdxThreads; k < K; k += kIdxThreads) {
-        int j, r, b;
-        step(k, j, r, b);
+        const int j = step(k).j;
         if (j >= 0) atomicAdd(&cnt[j], 1);
     }
     __syncthreads();
     int all;
     const int mine = tid < N ? cnt[tid] : 0;                       // (N <= 256 <= kIdxThreads)
-    const int first = cta_exclusive_scan(mine, wsum, all);
-    if (tid < N) { out.ptr[tid] = first; cnt[tid] = first; }       // from here on: next free run of every bucket
+    const int ptr = cta_exclusive_scan(mine, wsum, all);
+    if (tid < N) { out.ptr[tid] = ptr; cnt[tid] = ptr; }       // from here on: next free run of every bucket
     if (tid == 0) out.ptr[N] = all;
     __syncthreads();
     int run_rows = 0;                                              // rows of bucket tid in the tiles before
     for (int k0 = 0; k0 < K; k0 += kIdxThreads) {
-        int j = j0, rows = rows0, base = base0;
-        if (k0) {
-            j = -1; rows = 0; base = 0;
-            if (k0 + tid < K) step(k0 + tid, j, rows, base);
-        }
+        Step s = first;
+        if (k0) s = k0 + tid < K ? step(k0 + tid) : Step{-1, 0, 0};
+        const int j = s.j, rows = s.rows;
         // inside the warp: runs and rows of the same bucket in lower lanes
         const unsigned peers = __match_any_sync(0xffffffffu, j >= 0 ? j : -1 - lane);
         const unsigned lower = peers & ((1u << lane) - 1);
@@ -156,7 +179,7 @@ __device__ __forceinline__ void build_runs(int K, int N, Step step, Runs out, in
         if (j >= 0) {
             const int at = wcnt[warp * N + j] + __popc(lower);
             out.start[at] = wrow[warp * N + j] + pre;
-            out.row[at] = base;
+            out.row[at] = s.row0;
         }
         if (k0 + kIdxThreads < K) {
             __syncthreads();
@@ -166,6 +189,18 @@ __device__ __forceinline__ void build_runs(int K, int N, Step step, Runs out, in
     }
     if (tid < N) out.total[tid] = run_rows;
     __syncthreads();
+}
+
+// The run table of n buckets copied to shared memory (2 n_runs + 2 n + 1 words at `to`) if its runs fit `most`; all threads, no
+// barrier.  A look-up is half a dozen dependent reads: 30 cycles each there, ten times that in L2.
+__device__ __forceinline__ Runs runs_to_shared(const Runs& t, int n, int most, int* to) {
+    const int n_runs = t.ptr[n];
+    if (n_runs > most) return t;
+    const Runs s{to + 2 * n + 1, to + 2 * n + 1 + n_runs, to, to + n + 1};
+    for (int i = threadIdx.x; i < n_runs; i += kIdxThreads) { s.start[i] = t.start[i]; s.row[i] = t.row[i]; }
+    for (int i = threadIdx.x; i <= n; i += kIdxThreads) s.ptr[i] = t.ptr[i];
+    for (int i = threadIdx.x; i < n; i += kIdxThreads) s.total[i] = t.total[i];
+    return s;
 }
 
 // Row of position p in bucket j's stream, -1 beyond the plan.
@@ -205,6 +240,25 @@ __device__ __forceinline__ void find_senders(const int16_t* __restrict__ lane_ds
     __syncthreads();
 }
 
+// Calls f(x[i]) for lo <= i < hi over the CTA, sixteen loads of four values in flight per thread where x is 16-byte aligned.
+template <typename F>
+__device__ __forceinline__ void for_each_item(const int32_t* __restrict__ x, int lo, int hi, F f) {
+    const bool vec = ((uintptr_t)x & 15) == 0;
+    const int v0 = vec ? (lo + 3) & ~3 : hi, v1 = vec ? hi & ~3 : hi;
+    if (hi - lo >= 4 * kIdxThreads && v0 < v1) {     // (fewer: one value per thread spreads the work better)
+#pragma unroll 4
+        for (int v = v0 / 4 + threadIdx.x; v < v1 / 4; v += kIdxThreads) {
+            const int4 q = __ldg((const int4*)x + v);
+            f(4 * v, q.x); f(4 * v + 1, q.y); f(4 * v + 2, q.z); f(4 * v + 3, q.w);
+        }
+        if ((int)threadIdx.x < v0 - lo) f(lo + threadIdx.x, x[lo + threadIdx.x]);
+        if ((int)threadIdx.x < hi - v1) f(v1 + threadIdx.x, x[v1 + threadIdx.x]);
+    } else {
+#pragma unroll 4
+        for (int i = lo + threadIdx.x; i < hi; i += kIdxThreads) f(i, x[i]);
+    }
+}
+
 // Stable positions of the items lo <= i < hi, taken 32 at a time by ONE warp: key(i) names an item's key (-1: none),
 // next[] holds the position of the next item of every key and is carried on; put(i, key, position) is called for every
 // item, with position -1 where there is no key.
@@ -225,9 +279,9 @@ __device__ __forceinline__ void warp_positions(long long lo, long long hi, int* 
 }
 
 // Items per chunk and chunks of the chunked form: a map CTA adds up the histograms of all chunks, so their number times the
-// keys is kept within 64 K words (16 chunks at least, however many keys there are).
+// keys is kept within 16 K words (16 chunks at least, however many keys there are).
 inline int chunk_items(long long items, int keys) {
-    long long most = 65536 / keys;
+    long long most = 16384 / keys;
     if (most > 512) most = 512;
     if (most < 16) most = 16;
     long long c = (items + most - 1) / most;

@@ -24,8 +24,10 @@ struct UnpackArgs {
     const int16_t* lane_dst;
     const int64_t *lane_bytes, *recv_off;    // (lane_bytes: return direction only)
     int N, rank, k_max, epr, keys, items;    // items: capacity in rows, or routed copies
+    SmallDiv by_epr;
     const int32_t* item_expert;              // local expert of each received row, or global expert of each routed copy
-    int64_t row_bytes, capacity_rows;
+    RowDiv row;
+    int64_t capacity_rows;
     int32_t *expert_off, *out_src, *out_map, *status;
 };
 
@@ -66,51 +68,65 @@ __device__ __forceinline__ int steps_in_use(const UnpackArgs& a) { return min(ma
 
 // Rows this rank receives in K steps (0 when they exceed the buffer), with status bits.
 __device__ __forceinline__ int rows_received(const UnpackArgs& a, int K, int& st) {
-    const int64_t total = a.recv_off[(size_t)K * a.N + a.rank];
-    const bool over = total / a.row_bytes > a.capacity_rows;
-    st = (total % a.row_bytes ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
-    return over ? 0 : (int)(total / a.row_bytes);
+    int64_t odd;
+    const int64_t rows = a.row.div(a.recv_off[(size_t)K * a.N + a.rank], odd);
+    const bool over = rows > a.capacity_rows;
+    st = (odd ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
+    return over ? 0 : (int)rows;
 }
 
-// Step k of the dispatch plan from its sender: first receive row; a step whose bytes are not whole rows, or that has bytes
-// and no sender, is left out (peer -1) and reported.
-__device__ __forceinline__ int check_step(const UnpackArgs& a, int k, int& peer, int& bad) {
+// Step k of the dispatch plan, apart from its sender: first receive row, or -1 - row if its bytes are not whole rows;
+// `any` if it delivers something.
+__device__ __forceinline__ int step_rows(const UnpackArgs& a, int k, bool& any) {
     const int64_t lo = a.recv_off[(size_t)k * a.N + a.rank], hi = a.recv_off[(size_t)(k + 1) * a.N + a.rank];
-    if (hi > lo && (peer < 0 || lo % a.row_bytes || hi % a.row_bytes)) { peer = -1; bad = VP_ST_PACK_MISMATCH; }
-    return (int)(lo / a.row_bytes);
+    int64_t odd_lo, odd_hi;
+    const int row = (int)a.row.div(lo, odd_lo);
+    a.row.div(hi, odd_hi);
+    any = hi > lo;
+    return any && (odd_lo || odd_hi) ? -1 - row : row;
+}
+// With its sender: a step whose bytes are not whole rows, or that has bytes and no sender, is left out (peer -1) and reported.
+__device__ __forceinline__ int check_step(int row, bool any, int& peer, int& bad) {
+    if (any && (peer < 0 || row < 0)) { peer = -1; bad = VP_ST_PACK_MISMATCH; }
+    return row < 0 ? -1 - row : row;
 }
 
 // Key of a received row r < R: (local expert, sender of its step), -1 if either is missing.
-__device__ __forceinline__ int row_key_of(const UnpackArgs& a, int r, int K, const int* step_row, const int* step_peer) {
+__device__ __forceinline__ int row_key_of(const UnpackArgs& a, int r, int e, int K, const int* step_row, const int* step_peer) {
     int lo = 0, hi = K - 1;                                        // last step starting at or before r
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (step_row[mid] <= r) lo = mid; else hi = mid - 1;
     }
-    const int e = a.item_expert[r], src = K > 0 ? step_peer[lo] : -1;
+    const int src = K > 0 ? step_peer[lo] : -1;
     return e < 0 || e >= a.epr || src < 0 ? -1 : e * a.N + src;
 }
 
 // Key of a routed copy: its expert id, -1 if it does not travel.
-__device__ __forceinline__ int copy_key_of(const UnpackArgs& a, long long c) {
-    const int e = a.item_expert[c];
-    return e >= 0 && e < a.keys && (int)((unsigned)e / (unsigned)a.epr) != a.rank ? e : -1;
+__device__ __forceinline__ int copy_key_of(const UnpackArgs& a, int e) {
+    return e >= 0 && e < a.keys && a.by_epr.div(e) != a.rank ? e : -1;
 }
 
-// Run table of the return plan: bucket = sender, runs = its segments in the receive buffer.  peer(k) is the sender of step k.
+// Run table of the return plan: bucket = sender, runs = its segments in the receive buffer.  peer(k) is the sender of step k;
+// row0 is the first row of step threadIdx.x as return_row gives it.
+__device__ __forceinline__ int return_row(const UnpackArgs& a, int k) {
+    int64_t odd;
+    const int row = (int)a.row.div(a.recv_off[(size_t)k * a.N + a.rank], odd);
+    return odd ? -1 : row;
+}
 template <typename Peer>
-__device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, Peer peer, Runs out, int* cnt, int* scratch) {
+__device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, int row0, Peer peer, Runs out, int* cnt, int* scratch) {
     int bad = 0;
-    build_runs(K, a.N, [&](int k, int& j, int& rows, int& row0) {
-        j = peer(k);
-        rows = row0 = 0;
-        if (j < 0) return;
-        const int64_t bytes = a.lane_bytes[(size_t)k * a.N + j], at = a.recv_off[(size_t)k * a.N + a.rank];
-        if (bytes % a.row_bytes || at % a.row_bytes) { bad = VP_ST_PACK_MISMATCH; j = -1; return; }   // left out
-        rows = (int)(bytes / a.row_bytes);
-        row0 = (int)(at / a.row_bytes);
-        if (rows <= 0) j = -1;
-    }, out, cnt, scratch);
+    const auto step = [&](int k, int at) {
+        const int j = peer(k);
+        if (j < 0) return Step{-1, 0, 0};
+        int64_t odd;
+        const int64_t rows = a.row.div(a.lane_bytes[(size_t)k * a.N + j], odd);
+        if (odd || at < 0) { bad = VP_ST_PACK_MISMATCH; return Step{-1, 0, 0}; }   // left out
+        return Step{rows > 0 ? j : -1, (int)rows, at};
+    };
+    const Step first = (int)threadIdx.x < K ? step(threadIdx.x, row0) : Step{-1, 0, 0};
+    build_runs(K, a.N, first, [&](int k) { return step(k, return_row(a, k)); }, out, cnt, scratch);
     return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
 }
 
@@ -164,19 +180,24 @@ unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
     const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
     for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
     grid_wait();
+    bool any0 = false;
+    const int row0 = tid < a.k_max ? step_rows(a, tid, any0) : 0;      // (before K is known: a trip to L2 saved)
     const int K = steps_in_use(a);
     int st, bad = 0;
     const int R = rows_received(a, K, st);
     find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
     for (int k = tid; k < K; k += kIdxThreads) {
+        bool any = any0;
+        const int row = k == tid ? row0 : step_rows(a, k, any);
         int p = peer[k];
-        step_row[k] = check_step(a, k, p, bad);
+        step_row[k] = check_step(row, any, p, bad);
         peer[k] = p;
     }
     __syncthreads();
     const int r0 = (int)((long long)R * c / n_cta), r1 = (int)((long long)R * (c + 1) / n_cta);
+#pragma unroll 4
     for (int r = tid; r < R; r += kIdxThreads) {
-        const int key = row_key_of(a, r, K, step_row, peer);
+        const int key = row_key_of(a, r, a.item_expert[r], K, step_row, peer);
         if (key < 0) { bad = VP_ST_PACK_MISMATCH; continue; }
         atomicAdd(&all[key], 1);
         if (r < r0) atomicAdd(&next[key], 1);
@@ -190,7 +211,7 @@ unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
     }
     int *const src = sm + L.src, *const dst = sm + L.dst;
     if (tid < 32)
-        warp_positions(r0, r1, next, [&](long long r) { return row_key_of(a, (int)r, K, step_row, peer); },
+        warp_positions(r0, r1, next, [&](long long r) { return row_key_of(a, (int)r, a.item_expert[r], K, step_row, peer); },
                        [&](long long r, int key, int p) {
                            const int o = p >= 0 ? first[key] + p : -1;
                            src[r - r0] = o >= 0 ? (int)r : -1;
@@ -201,8 +222,8 @@ unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
                            }
                        });
     __syncthreads();
-    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
-    move_rows<V>(recv, out, a.row_bytes, r1 - r0, 1, src, dst, (int)((long long)vecs * piece / pieces),
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
+    move_rows<V>(recv, out, a.row.d, r1 - r0, 1, src, dst, (int)((long long)vecs * piece / pieces),
                  (int)((long long)vecs * (piece + 1) / pieces));
 }
 
@@ -216,19 +237,19 @@ tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
     const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
     for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
     grid_wait();
+    const int row0 = tid < a.k_max ? return_row(a, tid) : 0;           // (before K is known: a trip to L2 saved)
     const int K = steps_in_use(a);
-    const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row_bytes;      // nothing is unpacked then
+    const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row.d;      // nothing is unpacked then
     find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
     const int c0 = (int)((long long)a.items * c / n_cta), c1 = (int)((long long)a.items * (c + 1) / n_cta);
-#pragma unroll 4
-    for (int i = tid; i < a.items; i += kIdxThreads) {
-        const int key = copy_key_of(a, i);
-        if (key < 0) continue;
+    for_each_item(a.item_expert, 0, a.items, [&](int i, int e) {
+        const int key = copy_key_of(a, e);
+        if (key < 0) return;
         atomicAdd(&all[key], 1);
         if (i < c0) atomicAdd(&next[key], 1);
-    }
+    });
     const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
-    const int st = return_runs(a, K, [&](int k) { return peer[k]; }, runs, sm + L.cnt, sm + L.scratch);
+    const int st = return_runs(a, K, row0, [&](int k) { return peer[k]; }, runs, sm + L.cnt, sm + L.scratch);
     scan_keys(all, first, a.keys, sm + L.wsum);
     if (blockIdx.x == 0) {                           // every sender's stream is used up exactly
         int bad = st;
@@ -238,11 +259,11 @@ tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
     }
     int *const src = sm + L.src, *const dst = sm + L.dst;
     if (tid < 32)
-        warp_positions(c0, c1, next, [&](long long i) { return copy_key_of(a, i); },
+        warp_positions(c0, c1, next, [&](long long i) { return copy_key_of(a, a.item_expert[i]); },
                        [&](long long i, int key, int p) {
                            int row = -1;
                            if (p >= 0 && !over) {
-                               const int j = key / a.epr;
+                               const int j = a.by_epr.div(key);
                                row = run_lookup(runs, j, first[key] + p - first[j * a.epr]);   // position in sender j's stream
                            }
                            src[i - c0] = row;
@@ -250,8 +271,8 @@ tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
                            if (a.out_map && piece == 0) a.out_map[i] = row;
                        });
     __syncthreads();
-    const int vecs = (int)(a.row_bytes / (int64_t)sizeof(V));
-    move_rows<V>(recv, out, a.row_bytes, c1 - c0, 1, src, dst, (int)((long long)vecs * piece / pieces),
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
+    move_rows<V>(recv, out, a.row.d, c1 - c0, 1, src, dst, (int)((long long)vecs * piece / pieces),
                  (int)((long long)vecs * (piece + 1) / pieces));
 }
 
@@ -285,6 +306,8 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     const int tid = threadIdx.x;
     for (int j = tid; j < a.keys; j += kIdxThreads) hist[j] = 0;
     grid_wait();
+    bool any0 = false;
+    const int row0 = tid < a.k_max ? step_rows(a, tid, any0) : 0;
     const int K = steps_in_use(a);
     int st, bad = 0;
     const int R = rows_received(a, K, st);
@@ -292,14 +315,16 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     if ((int)blockIdx.x > 0 && (int)blockIdx.x >= chunks_of(R, chunk)) return;     // (CTA 0 always reports on the plan)
     if (steps == 0) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
     for (int k = tid; k < K; k += kIdxThreads) {
+        bool any = any0;
+        const int row = k == tid ? row0 : step_rows(a, k, any);
         int p = steps == 0 ? peer[k] : w.step_peer[k];
-        step_row[k] = check_step(a, k, p, bad);
+        step_row[k] = check_step(row, any, p, bad);
         peer[k] = p;
     }
     __syncthreads();
     const int r0 = blockIdx.x * chunk, r1 = min(r0 + chunk, R);
     for (int r = r0 + tid; r < r1; r += kIdxThreads) {
-        const int key = row_key_of(a, r, K, step_row, peer);
+        const int key = row_key_of(a, r, a.item_expert[r], K, step_row, peer);
         w.item_key[r] = key;
         if (key >= 0) atomicAdd(&hist[key], 1);
         else bad = VP_ST_PACK_MISMATCH;
@@ -315,12 +340,13 @@ __global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a,
     grid_wait();
     if ((int)blockIdx.x == n_chunks) {               // the senders' run table
         int *const cnt = sm, *const scratch = sm + a.N, *const peer = scratch + runs_scratch_ints(a.N);
+        const int row0 = tid < a.k_max ? return_row(a, tid) : 0;
         const int K = steps_in_use(a);
         if (inline_steps) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
-        const int st = return_runs(a, K, [&](int k) { return inline_steps ? peer[k] : w.step_peer[k]; },
+        const int st = return_runs(a, K, row0, [&](int k) { return inline_steps ? peer[k] : w.step_peer[k]; },
                                    Runs{w.start, w.row, w.ptr, w.total}, cnt, scratch);
         if (tid == 0) {
-            const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row_bytes;
+            const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row.d;
             w.flags[0] = over;
             w.flags[1] = over ? VP_ST_PACK_CAPACITY : st;
         }
@@ -331,7 +357,7 @@ __global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a,
     const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)a.items);
 #pragma unroll 4
     for (long long i = i0 + tid; i < i1; i += kIdxThreads) {
-        const int key = copy_key_of(a, i);
+        const int key = copy_key_of(a, a.item_expert[i]);
         if (key >= 0) atomicAdd(&sm[key], 1);
     }
     __syncthreads();
@@ -339,8 +365,14 @@ __global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a,
 }
 
 // Map of one chunk: all counts, the counts before this chunk, their prefix over the keys, then stable positions, every warp
-// a contiguous slice.  Shared memory: [keys] all, [keys] before, [keys + 1] first, wsum, [kIdxWarps][keys] slices.
-__host__ __device__ inline int map_smem_ints(int keys) { return 3 * keys + 1 + kIdxWarps + 1 + kIdxWarps * keys; }
+// a contiguous slice.  Shared memory: [keys] all, [keys] before, [keys + 1] first, wsum, [kIdxWarps][keys] slices, run table.
+// The return direction counts its slices before the wait for the count kernel: that kernel has started, so whatever wrote the
+// routing has finished.
+constexpr int kMapRuns = 2048;                       // runs whose table is copied to shared memory
+__host__ __device__ inline int map_ints(int keys) { return 3 * keys + 1 + kIdxWarps + 1 + kIdxWarps * keys; }
+inline int map_smem_ints(int N, int keys, int k_max, bool tokens) {
+    return map_ints(keys) + (tokens ? 2 * N + 1 + 2 * (k_max < kMapRuns ? k_max : kMapRuns) : 0);
+}
 
 template <bool TOKENS>
 __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, UnpackWs w, int chunk) {
@@ -351,34 +383,46 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, U
     for (int j = tid; j < 2 * keys; j += kIdxThreads) all[j] = 0;
     for (int j = tid; j < kIdxWarps * keys; j += kIdxThreads) slices[j] = 0;
     __syncthreads();
+    auto key_of = [&](long long i) { return TOKENS ? copy_key_of(a, a.item_expert[i]) : w.item_key[i]; };
+    long long s0, s1;
+    auto count_slice = [&](int items) {
+        const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)items);
+        s0 = min(i0 + (long long)warp * (chunk / kIdxWarps), i1);
+        s1 = min(s0 + chunk / kIdxWarps, i1);
+        for (long long i = s0 + lane; i < s1; i += 32) {
+            const int key = key_of(i);
+            if (key >= 0) atomicAdd(&next[key], 1);
+        }
+    };
+    if (TOKENS) count_slice(a.items);
     grid_wait();
     const bool over = w.flags[0] != 0;
     const int items = TOKENS ? a.items : w.flags[2];
     const int n_chunks = chunks_of(items, chunk);
     if (!TOKENS && (int)blockIdx.x > 0 && (int)blockIdx.x >= n_chunks) return;
-#pragma unroll 4
-    for (int i = tid; i < n_chunks * keys; i += kIdxThreads) {
-        const int v = w.hist[i];
-        if (v) {
-            const int b = i / keys, key = i - b * keys;
-            atomicAdd(&all[key], v);
-            if (b < (int)blockIdx.x) atomicAdd(&before[key], v);
+    if (!TOKENS) count_slice(items);
+    // thread t adds up column t mod keys of every (kIdxThreads / keys)-th chunk (keys <= kIdxThreads), or columns t, t + kIdxThreads
+    const int lanes = keys <= kIdxThreads ? kIdxThreads / keys : 1, mine = tid / min(keys, kIdxThreads);
+    for (int key = tid - mine * keys; mine < lanes && key < keys; key += kIdxThreads) {
+        int sum = 0, early = 0;
+#pragma unroll 8
+        for (int b = mine; b < n_chunks; b += lanes) {
+            const int v = w.hist[(size_t)b * keys + key];
+            sum += v;
+            early += b < (int)blockIdx.x ? v : 0;
         }
+        if (sum) atomicAdd(&all[key], sum);
+        if (early) atomicAdd(&before[key], early);
     }
-    const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)items);
-    const long long s0 = min(i0 + (long long)warp * (chunk / kIdxWarps), i1), s1 = min(s0 + chunk / kIdxWarps, i1);
-    auto key_of = [&](long long i) { return TOKENS ? copy_key_of(a, i) : w.item_key[i]; };
-    for (long long i = s0 + lane; i < s1; i += 32) {
-        const int key = key_of(i);
-        if (key >= 0) atomicAdd(&next[key], 1);
-    }
+    Runs runs{w.start, w.row, w.ptr, w.total};
+    if (TOKENS) runs = runs_to_shared(runs, a.N, kMapRuns, sm + map_ints(keys));
     __syncthreads();
     scan_keys(all, first, keys, wsum);
     if (blockIdx.x == 0) {
         int bad = 0;
         if (TOKENS) {                                // every sender's stream is used up exactly
             for (int j = tid; j < a.N; j += kIdxThreads)
-                if (j != a.rank && first[(j + 1) * a.epr] - first[j * a.epr] != w.total[j]) bad = VP_ST_PACK_MISMATCH;
+                if (j != a.rank && first[(j + 1) * a.epr] - first[j * a.epr] != runs.total[j]) bad = VP_ST_PACK_MISMATCH;
         } else {
             for (int e = tid; e <= a.epr; e += kIdxThreads) a.expert_off[e] = first[e * a.N];
             for (int b = tid; b < (n_chunks > 1 ? n_chunks : 1); b += kIdxThreads) bad |= w.bad[b];
@@ -396,12 +440,11 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, U
         }
     }
     __syncthreads();
-    const Runs runs{w.start, w.row, w.ptr, w.total};
     warp_positions(s0, s1, next, key_of, [&](long long i, int key, int p) {
         if (TOKENS) {
             int row = -1;
             if (p >= 0 && !over) {
-                const int j = key / a.epr;
+                const int j = a.by_epr.div(key);
                 row = run_lookup(runs, j, p - first[j * a.epr]);
             }
             w.map[i] = row;
@@ -434,7 +477,7 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
             const char* from = (const char*)recv;
             vp_prof_mark(3, 0, stream);
             const auto go = [&](auto fn) { return launch_wide(fn, s.grid, smem, stream, a, from, (char*)out, s.pieces); };
-            const int width = copy_width(recv, out, a.row_bytes);
+            const int width = copy_width(recv, out, a.row.d);
             if constexpr (TOKENS)
                 e = width == 16 ? go(tokens_small_kernel<uint4>) : width == 4 ? go(tokens_small_kernel<uint32_t>) : go(tokens_small_kernel<uint8_t>);
             else
@@ -456,10 +499,10 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
             e = launch_wide(unpack_count_kernel, n_chunks, ints * 4, stream, a, w, chunk, inline_steps ? 0 : (steps_fit ? 1 : 2));
         }
     }
-    if (e == cudaSuccess) e = launch_wide(unpack_map_kernel<TOKENS>, n_chunks, (size_t)map_smem_ints(a.keys) * 4, stream, a, w, chunk);
+    if (e == cudaSuccess) e = launch_wide(unpack_map_kernel<TOKENS>, n_chunks, (size_t)map_smem_ints(a.N, a.keys, a.k_max, TOKENS) * 4, stream, a, w, chunk);
     if (e != cudaSuccess) return VP_E_CUDA;
     vp_prof_mark(3, 0, stream);
-    const int rc = launch_row_copy(recv, out, w.map, w.flags, a.items, 1, TOKENS, !TOKENS, a.row_bytes, a.status, stream);
+    const int rc = launch_row_copy(recv, out, w.map, w.flags, a.items, 1, TOKENS, !TOKENS, a.row.d, a.status, stream);
     vp_prof_mark(3, 1, stream);
     return rc;
 }
@@ -484,7 +527,7 @@ extern "C" int vp_unpack(const int32_t* n_steps_b, const int16_t* lane_dst_b, co
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < vp_unpack_workspace_bytes(N, capacity_rows, experts_per_rank, k_max))
         return VP_E_WORKSPACE;
     const UnpackArgs a{n_steps_b, lane_dst_b, nullptr, recv_off_b, N, rank, k_max, experts_per_rank, N * experts_per_rank,
-                       (int)capacity_rows, recv_expert, row_bytes, capacity_rows, expert_off, out_src, out_map, status};
+                       (int)capacity_rows, small_div(experts_per_rank), recv_expert, row_div(row_bytes), capacity_rows, expert_off, out_src, out_map, status};
     return unpack_launch<false>(a, recv, out, workspace, (cudaStream_t)cuda_stream);
 }
 
@@ -508,6 +551,6 @@ extern "C" int vp_unpack_tokens(const int32_t* n_steps_b, const int16_t* lane_ds
     if (!need) return VP_E_UNSUPPORTED;
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < need) return VP_E_WORKSPACE;
     const UnpackArgs a{n_steps_b, lane_dst_b, lane_bytes_b, recv_off_b, N, rank, k_max, experts_per_rank, N * experts_per_rank,
-                       T * topk, expert_idx, row_bytes, capacity_rows, nullptr, nullptr, out_map, status};
+                       T * topk, small_div(experts_per_rank), expert_idx, row_div(row_bytes), capacity_rows, nullptr, nullptr, out_map, status};
     return unpack_launch<true>(a, recv, out, workspace, (cudaStream_t)cuda_stream);
 }
