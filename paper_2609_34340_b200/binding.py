@@ -1,6 +1,7 @@
-"""ctypes binding of ``libvariopath.so``; names follow the C ABI (``vp_*`` without the prefix).
+"""Binding of ``libvariopath.so``; names follow the C ABI (``vp_*`` without the prefix).
 
-PyTorch is used for device memory and streams only.
+PyTorch is used for device memory and streams only.  The calls of a serving or training step go through a small extension
+module (``csrc/calls.cpp``: about 1 us of host time instead of 10 to 15), everything else through ctypes.
 """
 from __future__ import annotations
 
@@ -121,6 +122,21 @@ def _load():
     return lib
 
 
+_calls = None
+
+
+def _load_calls():
+    """The extension module with the frequent calls (after the library, so that a missing library is reported first)."""
+    global _calls
+    _load()
+    try:
+        from . import _calls as module
+    except ImportError as e:
+        raise RuntimeError(f"{_PKG}/_calls.so cannot be loaded ({e}): build it with `python -m paper_2609_34340_b200.build`") from e
+    _calls = module
+    return module
+
+
 def _strerror(code: int) -> str:
     return _load().vp_strerror(int(code)).decode()
 
@@ -163,10 +179,9 @@ def exchange_put(plan: "Plan", b: int, rank: int, staged: torch.Tensor, recv_buf
                  arrived: Optional[torch.Tensor], status: torch.Tensor, stream=None) -> None:
     """``vp_exchange_put`` for matrix ``b`` of a device plan: ``recv_bufs`` / ``arrived`` are int64 device tensors ``[N]`` holding
     device addresses (``tensor.data_ptr()`` of every rank's receive buffer / counter), ``recv_capacity`` int64 ``[N]`` bytes."""
-    N = plan.lane_dst.shape[2]
-    _check(_load().vp_exchange_put(_ptr(plan.n_steps[b:]), _ptr(plan.lane_dst[b]), _ptr(plan.send_off[b]), _ptr(plan.recv_off[b]),
-                                   int(N), int(rank), int(plan.k_max), _ptr(staged), _ptr(recv_bufs), _ptr(recv_capacity),
-                                   _ptr(arrived), _ptr(status), _stream(stream)), "vp_exchange_put")
+    rc = (_calls or _load_calls()).exchange_put(plan, b, rank, staged, recv_bufs, recv_capacity, arrived, status, stream)
+    if rc:
+        _check(rc, "vp_exchange_put")
 
 
 def exchange_wait(plan: "Plan", b: int, rank: int, counter: torch.Tensor, base: int, max_polls: int, status: torch.Tensor,
@@ -317,27 +332,21 @@ class Plan:
         return out
 
 
-def _sched_call(fn, catalog, p, demand, tau_ns_in, B, plan, scratch, stream):
-    return fn(catalog._h, C.byref(p), _ptr(demand), _ptr(tau_ns_in), int(B), _ptr(plan.n_steps),
-              _ptr(plan.chan_id), _ptr(plan.lane_dst), _ptr(plan.lane_inst), _ptr(plan.lane_bytes),
-              _ptr(plan.send_off), _ptr(plan.recv_off), _ptr(plan.tau_ns), _ptr(plan.status),
-              _ptr(scratch), scratch.numel(), _stream(stream))
-
-
 def schedule_batch(catalog: Catalog, params: SchedParams, demand: torch.Tensor,
                    tau_ns_in: Optional[torch.Tensor] = None, plan: Optional[Plan] = None,
                    workspace: Optional[torch.Tensor] = None, stream=None) -> Plan:
     """``vp_schedule_batch`` on device tensors: ``demand`` is ``[B,N,N]`` int64 on the catalog's device."""
-    assert demand.is_cuda and demand.dtype == torch.int64 and demand.is_contiguous()
-    B, N = demand.shape[0], catalog.N
-    assert demand.shape == (B, N, N)
-    p = params._c(N)
-    if plan is None:
-        plan = Plan.empty(B, N, p.k_max, demand.device)
-    if workspace is None:
-        workspace = torch.empty(schedule_workspace_bytes(catalog, B, params), dtype=torch.uint8, device=demand.device)
-    _check(_sched_call(_load().vp_schedule_batch, catalog, p, demand, tau_ns_in, B, plan, workspace, stream),
-           "vp_schedule_batch")
+    if plan is None or workspace is None:
+        assert demand.is_cuda and demand.dtype == torch.int64 and demand.is_contiguous()
+        B, N = demand.shape[0], catalog.N
+        assert demand.shape == (B, N, N)
+        if plan is None:
+            plan = Plan.empty(B, N, params._c(N).k_max, demand.device)
+        if workspace is None:
+            workspace = torch.empty(schedule_workspace_bytes(catalog, B, params), dtype=torch.uint8, device=demand.device)
+    rc = (_calls or _load_calls()).schedule_batch(catalog, params, demand, tau_ns_in, plan, workspace, stream)
+    if rc:
+        _check(rc, "vp_schedule_batch")
     return plan
 
 
@@ -346,7 +355,6 @@ def schedule_batch_host(catalog: Catalog, params: SchedParams, demand: torch.Ten
                         scratch: Optional[torch.Tensor] = None, stream=None, used_only: bool = False) -> Plan:
     """``vp_schedule_batch_host``: host tensors in and out (pinned memory recommended).  ``used_only`` selects
     ``vp_schedule_batch_host_used``: only the rows below each matrix's ``n_steps`` come back."""
-    assert not demand.is_cuda and demand.dtype == torch.int64 and demand.is_contiguous()
     B, N = demand.shape[0], catalog.N
     p = params._c(N)
     if plan is None:
@@ -354,8 +362,9 @@ def schedule_batch_host(catalog: Catalog, params: SchedParams, demand: torch.Ten
     if scratch is None:
         need = int(_load().vp_schedule_host_scratch_bytes(catalog._h, B, C.byref(p)))
         scratch = torch.empty(need, dtype=torch.uint8, device=f"cuda:{catalog.device}")
-    fn = _load().vp_schedule_batch_host_used if used_only else _load().vp_schedule_batch_host
-    _check(_sched_call(fn, catalog, p, demand, tau_ns_in, B, plan, scratch, stream), "vp_schedule_batch_host")
+    calls = _calls or _load_calls()
+    fn = calls.schedule_batch_host_used if used_only else calls.schedule_batch_host
+    _check(fn(catalog, params, demand, tau_ns_in, plan, scratch, stream), "vp_schedule_batch_host")
     return plan
 
 
@@ -391,15 +400,13 @@ def demand_from_routing(expert_idx: torch.Tensor, experts_per_rank: int, N: int,
                         out: Optional[torch.Tensor] = None, status: Optional[torch.Tensor] = None, stream=None):
     """``vp_demand_from_routing``: ``expert_idx`` is ``[n_src, T, topk]`` int32 on device; returns
     (``[n_src, N]`` int64 demand rows, status int32[1])."""
-    assert expert_idx.is_cuda and expert_idx.dtype == torch.int32 and expert_idx.is_contiguous() and expert_idx.dim() == 3
-    n_src, T, topk = expert_idx.shape
     if out is None:
-        out = torch.empty((n_src, N), dtype=torch.int64, device=expert_idx.device)
+        out = torch.empty((expert_idx.shape[0], N), dtype=torch.int64, device=expert_idx.device)
     if status is None:
         status = torch.empty(1, dtype=torch.int32, device=expert_idx.device)
-    _check(_load().vp_demand_from_routing(_ptr(expert_idx), int(n_src), int(T), int(topk), int(experts_per_rank), int(N),
-                                          int(src0), int(row_bytes), _ptr(out), _ptr(status), _stream(stream)),
-           "vp_demand_from_routing")
+    rc = (_calls or _load_calls()).demand_from_routing(expert_idx, experts_per_rank, N, row_bytes, src0, out, status, stream)
+    if rc:
+        _check(rc, "vp_demand_from_routing")
     return out, status
 
 
@@ -421,17 +428,14 @@ def pack(plan: Plan, b: int, rank: int, expert_idx: torch.Tensor, experts_per_ra
          workspace: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """``vp_pack`` for matrix ``b`` of a device plan.  ``rows`` is ``[T, H]`` (any dtype), ``staged`` a
     pre-allocated device buffer; returns the device status tensor (int32[1])."""
-    N = plan.lane_dst.shape[2]
-    assert expert_idx.is_cuda and expert_idx.dtype == torch.int32 and expert_idx.is_contiguous()
-    assert rows.is_cuda and rows.is_contiguous() and staged.is_cuda and staged.is_contiguous()
-    T, topk = expert_idx.shape
-    row_bytes = rows.shape[1] * rows.element_size()
     if status is None:
         status = torch.empty(1, dtype=torch.int32, device=rows.device)
     if workspace is None:
-        workspace = torch.empty(pack_workspace_bytes(N, T, topk, plan.k_max), dtype=torch.uint8, device=rows.device)
-    _check(_pack_call(_load().vp_pack, plan, b, N, rank, expert_idx, experts_per_rank, rows, row_bytes, staged,
-                      src_map, status, workspace, stream), "vp_pack")
+        T, topk = expert_idx.shape
+        workspace = torch.empty(pack_workspace_bytes(plan.lane_dst.shape[2], T, topk, plan.k_max), dtype=torch.uint8, device=rows.device)
+    rc = (_calls or _load_calls()).pack(plan, b, rank, expert_idx, experts_per_rank, rows, staged, src_map, status, workspace, stream)
+    if rc:
+        _check(rc, "vp_pack")
     return status
 
 
@@ -446,18 +450,11 @@ def pack_static(plan: Plan, b: int, rank: int, expert_idx: torch.Tensor, experts
     uses its own fixed 4 MiB device block instead of a workspace, so the problem has to fit it
     (``VpError`` with ``E_WORKSPACE`` otherwise) and calls that may overlap on the GPU must be ordered.
     ``status`` must be passed in by such callers; it is allocated here only when omitted."""
-    N = plan.lane_dst.shape[2]
-    assert expert_idx.is_cuda and expert_idx.dtype == torch.int32 and expert_idx.is_contiguous()
-    assert rows.is_cuda and rows.is_contiguous() and staged.is_cuda and staged.is_contiguous()
-    T, topk = expert_idx.shape
-    row_bytes = rows.shape[1] * rows.element_size()
     if status is None:
         status = torch.empty(1, dtype=torch.int32, device=rows.device)
-    rc = _load().vp_pack_static(_ptr(plan.n_steps[b:b + 1]), _ptr(plan.lane_dst[b]), _ptr(plan.lane_bytes[b]),
-                                _ptr(plan.send_off[b]), int(N), int(rank), int(plan.k_max), _ptr(expert_idx), int(T),
-                                int(topk), int(experts_per_rank), _ptr(rows), int(row_bytes), _ptr(staged),
-                                staged.numel() * staged.element_size(), _ptr(src_map), _ptr(status), _stream(stream))
-    _check(rc, "vp_pack_static")
+    rc = (_calls or _load_calls()).pack(plan, b, rank, expert_idx, experts_per_rank, rows, staged, src_map, status, None, stream)
+    if rc:
+        _check(rc, "vp_pack_static")
     return status
 
 
@@ -491,26 +488,19 @@ def unpack(plan: Plan, b: int, rank: int, recv: torch.Tensor, recv_expert: torch
     """``vp_unpack`` for matrix ``b`` of a device plan: ``recv`` ``[capacity_rows, H]`` is rank ``rank``'s
     receive buffer, ``recv_expert`` the local expert of each received row, ``out`` ``[capacity_rows, H]`` the
     expert-major output.  Returns ``(expert_off, status)`` (device int32 ``[experts_per_rank + 1]`` and ``[1]``)."""
-    N = plan.lane_dst.shape[2]
-    assert recv.is_cuda and recv.is_contiguous() and recv.dim() == 2 and out.is_cuda and out.is_contiguous()
-    assert recv_expert.is_cuda and recv_expert.dtype == torch.int32 and recv_expert.is_contiguous()
-    cap = recv.shape[0]
-    assert recv_expert.numel() >= cap and out.numel() * out.element_size() >= recv.numel() * recv.element_size()
-    row_bytes = recv.shape[1] * recv.element_size()
     if expert_off is None:
         expert_off = torch.empty(experts_per_rank + 1, dtype=torch.int32, device=recv.device)
     if status is None:
         status = torch.empty(1, dtype=torch.int32, device=recv.device)
     if workspace is None:
-        need = unpack_workspace_bytes(N, cap, experts_per_rank, plan.k_max)
+        need = unpack_workspace_bytes(plan.lane_dst.shape[2], recv.shape[0], experts_per_rank, plan.k_max)
         if need == 0:
             raise VpError(E_UNSUPPORTED, "vp_unpack_workspace_bytes")
         workspace = torch.empty(need, dtype=torch.uint8, device=recv.device)
-    rc = _load().vp_unpack(_ptr(plan.n_steps[b:b + 1]), _ptr(plan.lane_dst[b]), _ptr(plan.recv_off[b]), int(N), int(rank),
-                           int(plan.k_max), _ptr(recv), int(row_bytes), int(cap), _ptr(recv_expert), int(experts_per_rank),
-                           _ptr(out), _ptr(expert_off), _ptr(out_src), _ptr(out_map), _ptr(status), _ptr(workspace),
-                           workspace.numel(), _stream(stream))
-    _check(rc, "vp_unpack")
+    rc = (_calls or _load_calls()).unpack(plan, b, rank, recv, recv_expert, experts_per_rank, out, expert_off, out_src, out_map, status,
+                                          workspace, stream)
+    if rc:
+        _check(rc, "vp_unpack")
     return expert_off, status
 
 
@@ -520,25 +510,18 @@ def unpack_tokens(plan: Plan, b: int, rank: int, expert_idx: torch.Tensor, exper
     """``vp_unpack_tokens`` for matrix ``b`` of the RETURN call's device plan: ``recv`` ``[capacity_rows, H]`` is rank
     ``rank``'s return receive buffer, ``expert_idx`` ``[T, topk]`` its routing, ``out`` ``[T*topk, H]`` the token
     layout.  Returns the device status tensor (int32[1])."""
-    N = plan.lane_dst.shape[2]
-    assert expert_idx.is_cuda and expert_idx.dtype == torch.int32 and expert_idx.is_contiguous() and expert_idx.dim() == 2
-    assert recv.is_cuda and recv.is_contiguous() and recv.dim() == 2 and out.is_cuda and out.is_contiguous()
-    T, topk = expert_idx.shape
-    cap = recv.shape[0]
-    row_bytes = recv.shape[1] * recv.element_size()
-    assert out.numel() * out.element_size() >= T * topk * row_bytes
     if status is None:
         status = torch.empty(1, dtype=torch.int32, device=recv.device)
     if workspace is None:
-        need = int(_load().vp_unpack_tokens_workspace_bytes(int(N), int(T), int(topk), int(experts_per_rank), int(cap), int(plan.k_max)))
+        T, topk = expert_idx.shape
+        need = int(_load().vp_unpack_tokens_workspace_bytes(int(plan.lane_dst.shape[2]), int(T), int(topk), int(experts_per_rank),
+                                                            int(recv.shape[0]), int(plan.k_max)))
         if need == 0:
             raise VpError(E_UNSUPPORTED, "vp_unpack_tokens_workspace_bytes")
         workspace = torch.empty(need, dtype=torch.uint8, device=recv.device)
-    rc = _load().vp_unpack_tokens(_ptr(plan.n_steps[b:b + 1]), _ptr(plan.lane_dst[b]), _ptr(plan.lane_bytes[b]), _ptr(plan.recv_off[b]),
-                                  int(N), int(rank), int(plan.k_max), _ptr(expert_idx), int(T), int(topk), int(experts_per_rank),
-                                  _ptr(recv), int(row_bytes), int(cap), _ptr(out), _ptr(out_map), _ptr(status), _ptr(workspace),
-                                  workspace.numel(), _stream(stream))
-    _check(rc, "vp_unpack_tokens")
+    rc = (_calls or _load_calls()).unpack_tokens(plan, b, rank, expert_idx, experts_per_rank, recv, out, out_map, status, workspace, stream)
+    if rc:
+        _check(rc, "vp_unpack_tokens")
     return status
 
 
