@@ -76,3 +76,18 @@ def test_pack_mismatch_and_capacity_in_both_forms(vp, oracle_lib, tokens):  # no
     case["expert_idx"][0, 0] = 1 << 20                         # an expert on no rank
     res = tp._run_case(vp, oracle_lib, case)
     assert res[2] == vp.ST_PACK_MISMATCH and res[5] & vp.ST_PACK_MISMATCH
+
+
+@pytest.mark.parametrize("sources,tokens,topk,N", [(1, 1, 1, 8), (1, 2049, 1, 16), (1, 4097, 4, 256), (8, 1024, 8, 8), (8, 1025, 8, 8),
+                                                   (16, 3, 7, 256), (17, 3, 7, 256), (64, 5, 2, 64), (3, 30000, 8, 5)])
+def test_demand_forms(vp, oracle_lib, sources, tokens, topk, N):  # noqa: F811
+    """One cluster for all sources (up to 65,536 copies and 4,096 cells) or one per source, of one to eight CTAs."""
+    epr = 3
+    idx = torch.randint(-1, N * epr, (sources, tokens, topk), dtype=torch.int32, generator=torch.Generator().manual_seed(tokens))
+    src0 = max(0, N - sources) if N >= sources else 0
+    for last in (0, N * epr):                                  # the second time with an expert on no rank
+        idx[-1, -1, -1] = last
+        got, st = vp.demand_from_routing(idx.cuda(), epr, N, 768, src0=src0)
+        want, bad = oracle_lib.demand_from_routing(idx.numpy(), epr, N, 768, src0=src0)
+        assert int(st.item()) == bad == (1 if last else 0)
+        assert np.array_equal(got.cpu().numpy(), want)
