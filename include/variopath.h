@@ -359,12 +359,12 @@ int vp_plan_time(const vp_catalog* catalog, int B, int k_max, const int32_t* n_s
  * recv_bufs[j] + recv_off[k][j].  The plan pointers are one matrix's device arrays (row stride N), as for vp_pack.
  *   recv_bufs            device array [N] of device pointers: the receive buffer of every rank for the current slot.
  *                        Ordinary device memory when ranks share a GPU; peer-mapped memory of the other GPUs otherwise
- *                        (the kernel only issues ordinary loads and stores, never multicast or cluster-scope copies)
+ *                        (the kernel issues bulk copies of its own CTA and ordinary loads and stores, never multicast)
  *   recv_capacity_bytes  device int64 [N]: size of each receive buffer; a chunk that would overrun it is not copied and
  *                        VP_ST_PACK_CAPACITY is set in status
  *   arrived              device array [N] of pointers to uint64 counters (NULL array or NULL entries: no signalling):
- *                        after a part of a chunk has been stored and fenced system-wide its byte count is added to
- *                        *arrived[j] with a system-scope atomic.  A rank's counter ends at base + recv_off[n_steps][rank]
+ *                        after a CTA's parts of the chunks have been stored and fenced system-wide each byte count is added
+ *                        to *arrived[j] with a system-scope atomic.  A rank's counter ends at base + recv_off[n_steps][rank]
  *   status               device int32[1], bits are OR-ed in (not cleared)
  * The call only enqueues one kernel on cuda_stream of the current device; it never waits.
  *

@@ -91,3 +91,39 @@ def test_demand_forms(vp, oracle_lib, sources, tokens, topk, N):  # noqa: F811
         want, bad = oracle_lib.demand_from_routing(idx.numpy(), epr, N, 768, src0=src0)
         assert int(st.item()) == bad == (1 if last else 0)
         assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("nodes,T,topk,row_bytes", [(2, 3, 1, 16), (2, 700, 8, 14336), (2, 700, 8, 4100), (1, 500, 8, 333), (1, 90, 4, 1),
+                                                    (2, 33, 6, 16400), (8, 40, 8, 7392), (8, 40, 8, 4102)])
+def test_put_alignments(vp, oracle_lib, nodes, T, topk, row_bytes):  # noqa: F811
+    """Chunk parts that go as bulk copies (addresses and sizes multiples of 16, more and less than one piece) and parts at every
+    other alignment, into receive buffers at odd addresses, on plans of up to several hundred activations."""
+    case = _case(nodes, T, topk, row_bytes, seed=T)
+    cat, D, w, rank = case["catalog"], case["demand"][0], case["params"], case["rank"]
+    N = cat.topology.N
+    oc = oracle_lib.OracleCatalog(cat.topology.blob(), cat.blob())
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob())
+    plan = vp.schedule_batch(dc, tp._params(vp, w), D.unsqueeze(0).cuda().contiguous())
+    one = {k: (v[0] if isinstance(v, np.ndarray) else v) for k, v in oc.schedule_batch(D.unsqueeze(0).numpy(), w).items()}
+    sent, cap = int(D[rank].sum()), D.sum(0).tolist()
+    staged = torch.randint(0, 256, (sent + 1,), dtype=torch.uint8, generator=torch.Generator().manual_seed(T)).cuda()[:sent]
+    step = 256 if row_bytes % 16 == 0 else 261
+    bufs = torch.full((sum(cap) + N * 600,), 0xAB, dtype=torch.uint8, device="cuda")
+    at = np.concatenate([[0], np.cumsum([(c + 511) // 256 * 256 + step - 256 for c in cap])[:-1]])
+    counters = torch.zeros(N, dtype=torch.int64, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    vp.exchange_put(plan, 0, rank, staged, bufs.data_ptr() + torch.from_numpy(at).cuda(), torch.tensor(cap, device="cuda"),
+                    counters.data_ptr() + 8 * torch.arange(N, device="cuda"), status)
+    torch.cuda.synchronize()
+    want, want_arrived, st = oc.exchange(one, {i: (staged.cpu().numpy() if i == rank else np.zeros(int(D[i].sum()), np.uint8)) for i in range(N)})
+    got = bufs.cpu().numpy()
+    assert int(status.item()) == st == 0 and counters.cpu().tolist() == D[rank].tolist()
+    mask = np.zeros(got.shape, bool)
+    host = plan.cpu()
+    for k in range(int(host["n_steps"][0])):
+        j, n = int(host["lane_dst"][0, k, rank]), int(host["lane_bytes"][0, k, rank])
+        if j >= 0 and n:
+            r = int(host["recv_off"][0, k, j])
+            assert np.array_equal(got[at[j] + r:at[j] + r + n], np.asarray(want[j]).reshape(-1)[r:r + n]), (k, j)
+            mask[at[j] + r:at[j] + r + n] = True
+    assert (got[~mask] == 0xAB).all()                          # nothing else is touched
