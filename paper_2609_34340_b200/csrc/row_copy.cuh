@@ -25,14 +25,14 @@ struct RowCopy {
     const int32_t* flags;      // device: [0] != 0 turns the copy into a no-op; [2] = rows in use when `bounded`
     int n, fanout, gather, bounded;
     long long row_bytes;
-    int pieces, stage_bytes, run;      // bulk form: pieces per row, ring stage, consecutive rows a CTA takes at a time
+    int pieces, stage_bytes;   // bulk form: pieces per row, ring stage
     int32_t* status;
 };
 
-// One warp per CTA.  A "unit" is one piece (<= kPiece bytes) of one source row.  CTAs take runs of `run` consecutive rows,
-// dealt round robin.  Unit m is loaded into stage m % S, S / 2 units ahead of its stores.
+// One warp per CTA.  A "unit" is one piece (<= kPiece bytes) of one source row.  Rows are dealt to the CTAs round robin (with
+// a contiguous range each the copy is 10 % slower).  Unit m is loaded into stage m % S, S / 2 units ahead of its stores.
 //
-// The map entries of a whole run are fetched by one coalesced load while the run before is in flight.  (With one fetch per
+// The map entries of the CTA's next 32 / fan-out rows are fetched by one load while the rows before are in flight.  (With one fetch per
 // unit each unit waited for a trip to L2: 0.85 us a unit and CTA whatever its size, so rows of 4 to 8 KB reached half of
 // the bandwidth with two CTAs per SM.)  Stores carry no L2 policy: marking them evict-first cost 10 % at fan-out 1
 // (32,768 rows of 14,336 B: 157 -> 142 us) and at 4 KB rows (214 -> 195 us), and changed nothing elsewhere.
@@ -50,32 +50,33 @@ __global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
     grid_wait();
     if (c.flags[0]) return;
     const int n = c.bounded ? min(c.n, c.flags[2]) : c.n;
-    const int F = c.fanout, pieces = c.pieces, run = c.run, per_run = run * pieces;
+    const int F = c.fanout, pieces = c.pieces;
     const bool wide = F > 32;                        // destinations of a row are then handled 32 slots at a time
-    const int n_runs = (n + run - 1) / run;
-    const int my_runs = n_runs > (int)blockIdx.x ? (n_runs - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int batch = wide ? 1 : 32 / F;             // rows whose map entries are fetched together
+    const int mine = n > (int)blockIdx.x ? (n - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;   // this CTA's rows
     unsigned phase = 0;                              // parity per stage (bit s)
     unsigned loaded = 0;                             // stage holds a load that was issued (bit s)
     bool failed = false;
-    auto fetch = [&](int q) {                        // map entries of the q-th run: lane = row in run x fan-out + slot
-        const long long e = ((long long)blockIdx.x + (long long)q * gridDim.x) * run * F + lane;
-        return !wide && q < my_runs && lane < run * F && e < (long long)n * F ? c.map[e] : -1;
+    const int f_row = wide ? 0 : lane / F, f_slot = wide ? 0 : lane - f_row * F;
+    auto fetch = [&](int q) {                        // map entries of rows q .. q + batch - 1: lane = row x fan-out + slot
+        const long long r = (long long)blockIdx.x + (long long)(q + f_row) * gridDim.x;
+        return !wide && f_row < batch && r < n ? c.map[r * F + f_slot] : -1;
     };
     int cur = -1, nxt = fetch(0);
-    // position of the next load (run, row in run, piece) and of the next store; s_*: ring stages
-    int lq = 0, li = 0, lp = 0, ls = 0, sq = 0, si = 0, sp = 0, ss = 0;
-    const long long units = (long long)my_runs * per_run;
+    // next load (row, place in its batch, piece) and next store (row, piece); ls, ss: ring stages
+    int lr = 0, lb = 0, lp = 0, ls = 0, sr = 0, sp = 0, ss = 0;
+    const long long units = (long long)mine * pieces;
     for (long long it = 0; it < units + kLook && !failed; it++) {
         if (it < units) {                            // ---- issue the load of unit `it`
-            if (li == 0 && lp == 0) { cur = nxt; nxt = fetch(lq + 1); }
-            const long long r = ((long long)blockIdx.x + (long long)lq * gridDim.x) * run + li;
-            int d = wide ? -1 : __shfl_sync(0xffffffffu, cur, min(li * F + lane, 31));
+            if (lb == 0 && lp == 0) { cur = nxt; nxt = fetch(lr + batch); }
+            const long long r = (long long)blockIdx.x + (long long)lr * gridDim.x;
+            int d = wide ? -1 : __shfl_sync(0xffffffffu, cur, min(lb * F + lane, 31));
             if (lane >= F) d = -1;
             bool any;
             long long src = r;
             if (wide) {
                 any = false;
-                for (int f = lane; f < F && r < n; f += 32) any |= c.map[r * F + f] >= 0;
+                for (int f = lane; f < F; f += 32) any |= c.map[r * F + f] >= 0;
                 any = __any_sync(0xffffffffu, any);
             } else {
                 any = __any_sync(0xffffffffu, d >= 0);
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
             }
             loaded = any ? (loaded | (1u << ls)) : (loaded & ~(1u << ls));
             ls = ls + 1 == S ? 0 : ls + 1;
-            if (++lp == pieces) { lp = 0; if (++li == run) { li = 0; lq++; } }
+            if (++lp == pieces) { lp = 0; lr++; if (++lb == batch) lb = 0; }
         }
         if (it >= kLook) {                           // ---- unit it - kLook: wait for its load, issue its stores
             if (loaded & (1u << ss)) {
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
                         const int d = sdst[ss][lane];
                         if (d >= 0) bulk_store(to + (long long)d * c.row_bytes, from, bytes);
                     } else {
-                        const long long r = ((long long)blockIdx.x + (long long)sq * gridDim.x) * run + si;
+                        const long long r = (long long)blockIdx.x + (long long)sr * gridDim.x;
                         for (int f = lane; f < F; f += 32) {
                             const int d = c.map[r * F + f];
                             if (d >= 0) bulk_store(to + (long long)d * c.row_bytes, from, bytes);
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
             }
             bulk_commit();                           // one group per unit from every lane, empty or not
             ss = ss + 1 == S ? 0 : ss + 1;
-            if (++sp == pieces) { sp = 0; if (++si == run) { si = 0; sq++; } }
+            if (++sp == pieces) { sp = 0; sr++; }
         }
     }
     bulk_wait_all();                                 // stores must finish before shared memory is released
@@ -216,8 +217,18 @@ inline int launch_row_copy(const void* rows, void* out, const int32_t* map, cons
     RowCopy c;
     c.rows = (const char*)rows; c.out = (char*)out; c.map = map; c.flags = flags;
     c.n = n; c.fanout = fanout; c.gather = gather; c.bounded = bounded; c.row_bytes = row_bytes; c.status = status;
-    c.pieces = 1; c.stage_bytes = 0; c.run = 1;
+    c.pieces = 1; c.stage_bytes = 0;
     const int width = copy_width(rows, out, row_bytes);
+    // Many short CTAs rather than one wave of long ones: 64 to 80 KB of stores per CTA (two rows at least in the bulk form).  The
+    // hardware hands out CTAs in order, so the rows in flight stay neighbours, and so do their destinations in every stream;
+    // in one wave the CTAs drift apart and DRAM takes the stores at 5.0 TB/s instead of 5.7.  16,384 rows of 14,336 B,
+    // fan-out 8: 371 us in one wave, 328 so; 8,192 rows of 4,096 B: 98 and 44 us; rows claimed in order from a counter by one
+    // wave: 325 and 53 us.  (Where the rows in use are known on the device only, half of the buffer is expected.)
+    const double row_stores = (double)row_bytes * fanout;
+    const auto ctas = [&](double most_per_cta) {
+        const double want = (double)n * row_stores / most_per_cta * (bounded ? 0.5 : 1.0);
+        return want < sms ? (n < sms ? n : sms) : (want > 1e6 ? 1000000 : (int)want);
+    };
     cudaError_t e;
     if (width == 16 && row_bytes >= kMinBulkRow) {
         if (dev < 0 || dev >= 64 || !s_attr_set[dev]) {
@@ -227,24 +238,13 @@ inline int launch_row_copy(const void* rows, void* out, const int32_t* map, cons
         }
         c.pieces = (int)((row_bytes + kPiece - 1) / kPiece);
         c.stage_bytes = row_bytes < kPiece ? (int)((row_bytes + 127) & ~127ll) : kPiece;
-        // About 170 KB of ring per SM: two CTAs at 14 KB rows, four at 7 KB, eight at most.  With a fan-out the stores are
-        // most of the traffic and more than two CTAs per SM only scatter them (4 KB rows, fan-out 8: 195 us with two, 215
-        // with four and more).
-        int per_sm = 176 * 1024 / (kStages * c.stage_bytes);
-        per_sm = per_sm < 2 ? 2 : (per_sm > 8 ? 8 : per_sm);
-        if (fanout >= 4) per_sm = 2;
-        const int grid = sms * per_sm;
-        int run = fanout <= 32 ? 32 / fanout : 1;
-        if (run > 8) run = 8;
-        while (run > 1 && (long long)n < (long long)grid * run * 8) run >>= 1;   // eight runs per CTA at least: an even last wave
-        c.run = run;
-        e = launch_after(row_copy_bulk_kernel, grid, 32, (size_t)kStages * c.stage_bytes, stream, c);
+        e = launch_after(row_copy_bulk_kernel, ctas(row_stores > 40960 ? 2 * row_stores : 81920), 32, (size_t)kStages * c.stage_bytes, stream, c);
     } else if (width == 16) {
-        e = launch_after(row_copy_plain_kernel<uint4>, sms * 8, 256, 0, stream, c);
+        e = launch_after(row_copy_plain_kernel<uint4>, ctas(65536), 256, 0, stream, c);
     } else if (width == 4) {
-        e = launch_after(row_copy_plain_kernel<uint32_t>, sms * 8, 256, 0, stream, c);
+        e = launch_after(row_copy_plain_kernel<uint32_t>, ctas(65536), 256, 0, stream, c);
     } else {
-        e = launch_after(row_copy_plain_kernel<uint8_t>, sms * 8, 256, 0, stream, c);
+        e = launch_after(row_copy_plain_kernel<uint8_t>, ctas(65536), 256, 0, stream, c);
     }
     return e == cudaSuccess ? VP_OK : VP_E_CUDA;
 }
