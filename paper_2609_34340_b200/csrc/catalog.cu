@@ -406,6 +406,18 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
     if (!rc) rc = upload(c, fam_slot, &dc.fam_slot);
     if (!rc) rc = upload(c, fam_cls, &dc.fam_cls);
     if (!rc) rc = upload(c, fam_in, &dc.fam_in);
+    if (!rc && g == 4 && G <= 64 && dc.sym) {                 // slot words of vp_schedule_big_kernel's tasks
+        const int st = big_stride(big_lanes(G));
+        std::vector<uint32_t> task((size_t)n_fam * G * 8);
+        for (size_t f = 0; f < (size_t)n_fam; f++)
+            for (int d = 0; d < G; d++)
+                for (int q = 0; q < 4; q++) {
+                    const uint32_t w = fam_in[f * N + d * 4 + q], r = w & 0xffu, cls = w >> 8, sg = r >> 2;
+                    task[(f * G + d) * 8 + 4 + q] = (uint32_t)((2 * sg + 1) * st + 4 * d) | sg << 16 | cls << 24 | (6 - 2 * (r & 3u)) << 28;
+                    task[(f * G + sg) * 8 + (r & 3u)] = (uint32_t)(2 * sg * st + 4 * d + 3) | (uint32_t)d << 16 | cls << 24 | (uint32_t)(6 - 2 * q) << 28;
+                }
+        rc = upload(c, task, &dc.fam_task);
+    }
     dc.n_terms = (int)term.size();      // real (unpadded) multiply-adds of one scoring pass
     if (n_shapes < 65536) {             // inverted terms: entry -> (shape, count)
         std::vector<uint32_t> inv_ptr(dc.tbl_size + 1, 0), inv(term.size());

@@ -43,6 +43,7 @@ struct KParams {
     int64_t lambda_ns, granule;
     int k_target, n_start, i_aa, k_max;
     int max_tasks, stage_terms, stage_fam, stage_bucket, drem_in_smem;
+    int big_stage, big_cross, big_task_warps, big_emit_warp;    // vp_schedule_big_kernel: task tables in shared memory, a task is two warps, task warps, first emitting warp
     int incremental;          // keep the shape scores in shared memory and update them after every activation
 };
 
@@ -1133,10 +1134,6 @@ vp_schedule_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, co
 #include "schedule_big.cuh"
 #include "schedule_warp.cuh"
 
-#ifndef VP_BIG_MIN_GROUPS
-#define VP_BIG_MIN_GROUPS 16      // node-symmetric catalogs with at least this many groups of four take vp_schedule_big_kernel
-#endif
-
 namespace {
 
 struct Launch {
@@ -1145,7 +1142,7 @@ struct Launch {
                               // 2: vp_schedule_big_kernel, followed by vp_schedule_kernel on the matrices it left
     size_t smem;
     KParams kp;
-    int big_w, big_threads, big_grid;     // kernel 2: warps per task, threads and CTAs of the first launch
+    int big_split, big_threads, big_grid; // kernel 2: lanes per group, threads and CTAs of the first launch
     size_t big_smem;
     int wave;                 // CTAs of the chosen kernel that are resident at once (the grid is min(B, wave) or less)
 };
@@ -1171,9 +1168,11 @@ KernelFn pick_kernel(int g, int lpg) {
     }
     return nullptr;
 }
-BigKernelFn pick_big_kernel(int w, bool dec) {
-    if (dec) return w == 2 ? vp_schedule_big_kernel<2, true> : vp_schedule_big_kernel<1, true>;
-    return w == 2 ? vp_schedule_big_kernel<2, false> : vp_schedule_big_kernel<1, false>;
+// Kernel for a number of rank groups, with one or two lanes per group (see vp_schedule_big_kernel).
+BigKernelFn pick_big_kernel(int G, int split) {
+    if (split == 2) return G <= 8 ? vp_schedule_big_kernel<16, 2> : G <= 16 ? vp_schedule_big_kernel<32, 2> : vp_schedule_big_kernel<64, 2>;
+    return G <= 8 ? vp_schedule_big_kernel<8, 1> : G <= 16 ? vp_schedule_big_kernel<16, 1>
+         : G <= 32 ? vp_schedule_big_kernel<32, 1> : vp_schedule_big_kernel<64, 1>;
 }
 
 // Raises a kernel's limit of dynamic shared memory on the current device to `bytes` if it is lower.  The limit belongs
@@ -1250,31 +1249,40 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     long long cap = (long long)per_sm * c->sm_count;
     L.wave = (int)cap;
     L.grid = (int)(B < cap ? B : cap);
-#ifndef VP_NO_BIG_KERNEL
-    // Large node-symmetric catalogs (groups of four, more than sixteen groups): 16-bit credits in shared memory and
-    // scores on the per-node-offset table; the general kernel then takes whatever matrices that kernel left.
-    const int big_min_groups = VP_BIG_MIN_GROUPS;
-    if (dc.g == 4 && dc.G >= big_min_groups && dc.G <= 64 && dc.sym && dc.shape_pat && dc.n_patterns < 1024 && dc.n_classes <= 15) {
-        const size_t smem = (size_t)big_smem_layout(dc, L.kp).total;
-        if (smem + 2048 <= (size_t)c->max_smem_optin) {
-            // one lane per group: two warps per task beyond 32 groups, and then sixteen warps for shape scoring and the
-            // emit step; up to 32 groups a task is one warp and four to eight warps per CTA leave room for several CTAs per SM
-            const int w = dc.G > 32 ? 2 : 1;
-            // sixteen groups: two warps, two tasks each (eight CTAs per SM: config 3's 1,024 matrices are one wave)
-            // up to 32 groups: four warps, a task each (256 threads, with four warps idle in Step 2, halve the CTAs per SM:
-            // 6.9 -> 4.6 ms for 1,024 matrices at N = 96)
-            const int threads = w == 2 ? BIG_W2_THREADS : (dc.G > 16 ? 128 : 64);
-            BigKernelFn bf = pick_big_kernel(w, big_use_dec(dc));
+    // Node-symmetric catalogs: 16-bit credits in shared memory and scores on the per-node-offset table; the general kernel then
+    // takes whatever matrices that kernel left.  (Below sixteen groups, where matrices with granules under 256 bytes run in the
+    // general kernel anyway, those go there directly.)
+    if (dc.g == 4 && dc.G <= 64 && dc.sym && dc.shape_pat && dc.n_patterns < 1024 && dc.n_classes <= 15 &&
+        (dc.G >= 16 || p->granule_bytes >= 256)) {
+        // Four tasks as a rule (one family, four starts).  While the batch leaves SMs room, two lanes per group and warps of
+        // their own that emit; then one lane per group and such warps; once the batch exceeds that wave, CTAs of task warps
+        // only, which pack the SMs.  The families' tables are staged where that costs no CTA.  More than 32 groups: one CTA per SM, two
+        // warps per task, which emit as well.
+        for (int option = 0; option < 6; option++) {
+            if (dc.G > 32 && option < 4) continue;
+            const int split = option < 2 ? 2 : 1;
+            const bool apart = option < 4;                       // warps of their own for the emit step
+            const int lanes = big_lanes(dc.G) * split, task_warps = lanes * 4 / 32;
+            KParams kp = L.kp;
+            kp.big_stage = option % 2 == 0;
+            kp.big_cross = lanes == 64;
+            kp.big_task_warps = task_warps;
+            kp.big_emit_warp = apart ? task_warps : 0;
+            const int threads = dc.G > 32 ? 384 : task_warps * 32 + (apart ? (dc.N + 31) / 32 * 32 : 0);
+            const BigKernelFn bf = pick_big_kernel(dc.G, split);
+            const size_t smem = (size_t)big_smem_layout(dc, kp).total;
+            if (smem + 2048 > (size_t)c->max_smem_optin) continue;
             if (raise_dynamic_smem((const void*)bf, smem) != VP_OK) return VP_E_CUDA;
             int bper_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bper_sm, bf, threads, smem) != cudaSuccess || bper_sm < 1) return VP_E_CUDA;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bper_sm, bf, threads, smem) != cudaSuccess) return VP_E_CUDA;
             const long long bcap = (long long)bper_sm * c->sm_count;
-            L.kernel = 2; L.big_w = w; L.big_threads = threads; L.big_smem = smem;
+            if (bper_sm < 1 || (bcap < B && option < 5)) continue;   // (the last option packs the SMs)
+            L.kernel = 2; L.kp = kp; L.big_split = split; L.big_threads = threads; L.big_smem = smem;
             L.big_grid = (int)(B < bcap ? B : bcap);
             L.wave = (int)bcap;
+            break;
         }
     }
-#endif
 #ifndef VP_NO_WARP_KERNEL
     // Small topologies (groups of four, at most four groups, plain D-hat scores): one warp per matrix.  It has no block
     // barriers and less work per activation than a CTA per matrix, and wins at every batch size once the matrices run
@@ -1395,7 +1403,7 @@ extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, 
                     big_rank_kernel<<<(B + 255) / 256, 256, 0, stream>>>(key, B, order);
                     g_vp_launches += 2;
                 }
-                pick_big_kernel(L.big_w, big_use_dec(c->dc))<<<L.big_grid, L.big_threads, L.big_smem, stream>>>(
+                pick_big_kernel(c->dc.G, L.big_split)<<<L.big_grid, L.big_threads, L.big_smem, stream>>>(
                     c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
                     tau_ns_out, status, counter, todo, order);
                 g_vp_launches++;

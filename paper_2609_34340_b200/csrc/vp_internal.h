@@ -49,6 +49,11 @@ struct DevCat {
     const uint8_t* fam_cls;
     // family f, in-slot d*g+q of destination group d: slot index (N <= 256) | rate class << 8
     const uint16_t* fam_in;
+    // groups of four, at most 64 of them, node-symmetric: family f, group a, eight words.  Words 0..3: out-slots of a, each
+    // (word of its cells in the credit matrix when its destination has tag 0, i.e. is row 3 of its group) | destination group << 16 |
+    // rate class << 24 | shift of the destination's tag in its group's byte << 28.  Words 4..7: in-slots of a, each
+    // (word of the row pair of its source when that has tag 0) | source group << 16 | class << 24 | shift of the source's tag << 28
+    const uint32_t* fam_task;
     int n_terms;
     // inverted terms, for keeping the scores up to date instead of recomputing them: the shapes that use table
     // entry e are inv[inv_ptr[e] .. inv_ptr[e+1]) = shape | count << 16 (built when n_shapes < 65536)
@@ -71,8 +76,19 @@ struct vp_launch_memo {
     int B_class;                  // min(B, CTAs of one wave + 1): batches of one class launch alike up to the grid size
     int32_t k_target, n_start, i_aa, k_max;
     int64_t lambda_ns, granule;
-    unsigned char launch[160];    // the scheduler's Launch record
+    unsigned char launch[192];    // the scheduler's Launch record
 };
+
+// Lanes per task (over lanes per group) of vp_schedule_big_kernel for a number of rank groups, and the stride of its credit
+// matrix, in words per row pair: rows of 128-bit reads, and 2 x stride = 8 modulo 16, so that neighbouring groups start in
+// different banks.
+#ifdef __CUDACC__
+#define VP_HD __host__ __device__
+#else
+#define VP_HD
+#endif
+VP_HD inline constexpr int big_lanes(int G) { return G <= 8 ? 8 : (G <= 16 ? 16 : (G <= 32 ? 32 : 64)); }
+VP_HD inline constexpr int big_stride(int lanes) { return lanes * 4 + 4; }
 
 struct vp_catalog {
     int device;
