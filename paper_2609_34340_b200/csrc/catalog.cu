@@ -406,17 +406,39 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
     if (!rc) rc = upload(c, fam_slot, &dc.fam_slot);
     if (!rc) rc = upload(c, fam_cls, &dc.fam_cls);
     if (!rc) rc = upload(c, fam_in, &dc.fam_in);
-    if (!rc && g == 4 && G <= 64 && dc.sym) {                 // slot words of vp_schedule_big_kernel's tasks
+    if (!rc && g == 4 && (dc.sym ? G <= 64 : G <= 4)) {       // slot words of the (family, start) tasks
         const int st = big_stride(big_lanes(G));
         std::vector<uint32_t> task((size_t)n_fam * G * 8);
         for (size_t f = 0; f < (size_t)n_fam; f++)
             for (int d = 0; d < G; d++)
                 for (int q = 0; q < 4; q++) {
                     const uint32_t w = fam_in[f * N + d * 4 + q], r = w & 0xffu, cls = w >> 8, sg = r >> 2;
-                    task[(f * G + d) * 8 + 4 + q] = (uint32_t)((2 * sg + 1) * st + 4 * d) | sg << 16 | cls << 24 | (6 - 2 * (r & 3u)) << 28;
-                    task[(f * G + sg) * 8 + (r & 3u)] = (uint32_t)(2 * sg * st + 4 * d + 3) | (uint32_t)d << 16 | cls << 24 | (uint32_t)(6 - 2 * q) << 28;
+                    const uint32_t in_at = dc.sym ? (2 * sg + 1) * st + 4 * d : (sg * 4 + 3) * N + 4 * d;
+                    const uint32_t out_at = dc.sym ? 2 * sg * st + 4 * d + 3 : (d * 4 + 3) * N + 4 * sg;
+                    task[(f * G + d) * 8 + 4 + q] = in_at | sg << 16 | cls << 24 | (6 - 2 * (r & 3u)) << 28;
+                    task[(f * G + sg) * 8 + (r & 3u)] = out_at | (uint32_t)d << 16 | cls << 24 | (uint32_t)(6 - 2 * q) << 28;
                 }
         rc = upload(c, task, &dc.fam_task);
+    }
+    if (!rc && g == 4 && G <= 4 && !dc.sym) {                 // row patterns of plain tables
+        std::map<std::vector<uint32_t>, int> ids;
+        std::vector<uint32_t> row_term(32 * 4, 0), shape_rows((size_t)((n_shapes + 31) & ~31), 0);
+        bool fits = true;
+        for (int s = 0; s < n_shapes && fits; s++)
+            for (int a = 0; a < 4 && fits; a++) {
+                std::vector<uint32_t> row;
+                for (uint32_t e = term_ptr[s]; e < term_ptr[s + 1]; e++) {
+                    const uint32_t cell = (term[e] & 0xffffu) / 8;
+                    if ((int)cell / G == a) row.push_back(cell | (term[e] & 0xffff0000u));
+                }
+                const int id = ids.emplace(row, (int)ids.size()).first->second;
+                fits = id < 32 && row.size() <= 4;
+                if (!fits) break;
+                std::copy(row.begin(), row.end(), row_term.begin() + id * 4);
+                shape_rows[s] |= (uint32_t)id << (8 * a);
+            }
+        if (fits) rc = upload(c, row_term, &dc.row_term);
+        if (fits && !rc) rc = upload(c, shape_rows, &dc.shape_rows);
     }
     dc.n_terms = (int)term.size();      // real (unpadded) multiply-adds of one scoring pass
     if (n_shapes < 65536) {             // inverted terms: entry -> (shape, count)

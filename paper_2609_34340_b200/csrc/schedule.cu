@@ -33,8 +33,10 @@
 #include <cstring>
 #include <mutex>
 #include <utility>
+#include <vector>
 
 #include "bulk_copy.cuh"
+#include "route_index.cuh"
 #include "vp_internal.h"
 
 namespace {
@@ -1153,6 +1155,9 @@ typedef void (*KernelFn)(DevCat, KParams, const int64_t*, const int64_t*, int, i
 typedef void (*BigKernelFn)(DevCat, KParams, const int64_t*, const int64_t*, int, int32_t*, int32_t*, int16_t*, uint16_t*,
                             int64_t*, int64_t*, int64_t*, int64_t*, int32_t*, unsigned int*, int*, const int*);
 
+typedef void (*WarpKernelFn)(DevCat, KParams, const int64_t*, const int64_t*, int, int32_t*, int32_t*, int16_t*, uint16_t*,
+                             int64_t*, int64_t*, int64_t*, int64_t*, int32_t*, unsigned int*, unsigned long long*);
+
 KernelFn pick_kernel(int g, int lpg) {
     switch (g) {
         case 1: return vp_schedule_kernel<1, 1>;
@@ -1290,12 +1295,14 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     // granule decides here); with smaller granules only when the batch exceeds the CTAs of one wave.  Up to four
     // matrices per SM get a CTA of one warp each (a scheduler to themselves), larger batches two or four warps per CTA.
     if (dc.g == 4 && dc.G <= 4 && !dc.sym && (B > cap || p->granule_bytes >= 256)) {
+        const bool units = p->granule_bytes >= 256;
+        const WarpKernelFn wf = units ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;
         const int warps = B <= 4 * c->sm_count ? 1 : (B <= 8 * c->sm_count ? 2 : 4);
-        const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps).total;
+        const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
         if (smem + 2048 <= (size_t)c->max_smem_optin) {
-            if (raise_dynamic_smem((const void*)vp_schedule_warp_kernel, smem) != VP_OK) return VP_E_CUDA;
+            if (raise_dynamic_smem((const void*)wf, smem) != VP_OK) return VP_E_CUDA;
             int wper_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper_sm, vp_schedule_warp_kernel, warps * 32, smem) != cudaSuccess || wper_sm < 1)
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper_sm, wf, warps * 32, smem) != cudaSuccess || wper_sm < 1)
                 return VP_E_CUDA;
             const long long wcap = (long long)wper_sm * c->sm_count, want = ((long long)B + warps - 1) / warps;
             L.kernel = 1; L.lpg = 8; L.threads = warps * 32; L.smem = smem;
@@ -1337,15 +1344,17 @@ int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* o
     return VP_OK;
 }
 
-// Workspace: 256 bytes of counters; one residual slot per CTA of the general kernel when it keeps the residual outside
+// Workspace: 256 bytes of counters (work counter, list length, -, warps with counters of their own; sums for
+// vp_schedule_read_stats); the warp kernel's counters per warp; one residual slot per CTA of the general kernel when it keeps the residual outside
 // shared memory; with the kernel for large node-symmetric catalogs also the list of matrices left to the general
 // kernel, the work order and its keys.
-struct WsLayout { size_t drem, todo, order, key, total; };
+struct WsLayout { size_t drem, slots, todo, order, key, total; };
 WsLayout ws_layout(const vp_catalog* c, const Launch& L, int B) {
     WsLayout w;
     const size_t slot_bytes = !L.kp.drem_in_smem ? (size_t)L.grid * c->dc.N * c->dc.N * 8 : 0;
-    w.drem = 256;
-    w.todo = vp_align256(256 + slot_bytes);
+    w.drem = w.slots = 256;
+    const size_t warp_slots = L.kernel == 1 ? (size_t)L.grid * (L.threads / 32) * 24 : 0;
+    w.todo = vp_align256(256 + slot_bytes + warp_slots);
     const size_t list = L.kernel == 2 ? vp_align256((size_t)B * 4) : 0;
     w.order = w.todo + list;
     w.key = w.order + list;
@@ -1385,13 +1394,20 @@ extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, 
         cudaStream_t stream = (cudaStream_t)cuda_stream;
         unsigned int* counter = (unsigned int*)workspace;
         int64_t* ws_drem = (int64_t*)((char*)workspace + 256);
-        if (cudaMemsetAsync(counter, 0, 256, stream) != cudaSuccess) rc = VP_E_CUDA;
+        // a warp for every matrix: nothing is counted across warps, so nothing has to be zeroed
+        const bool warp_each = L.kernel == 1 && (long long)L.grid * (L.threads / 32) >= B;
+#ifndef VP_PHASE_TIMING
+        if (!warp_each)
+#endif
+            if (cudaMemsetAsync(counter, 0, 256, stream) != cudaSuccess) rc = VP_E_CUDA;
         if (!rc) {
             vp_prof_mark(0, 0, stream);
             if (L.kernel == 1) {
-                vp_schedule_warp_kernel<<<L.grid, L.threads, L.smem, stream>>>(
-                    c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
-                    tau_ns_out, status, counter);
+                const WarpKernelFn wf = p->granule_bytes >= 256 ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;
+                unsigned long long* slots = warp_each ? (unsigned long long*)((char*)workspace + ws_layout(c, L, B).slots) : nullptr;
+                if (launch_after(wf, L.grid, L.threads, L.smem, stream, c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst,
+                                 lane_inst, lane_bytes, send_off, recv_off, tau_ns_out, status, counter, slots) != cudaSuccess)
+                    rc = VP_E_CUDA;
             } else if (L.kernel == 2) {
                 const WsLayout w = ws_layout(c, L, B);
                 int* todo = (int*)((char*)workspace + w.todo);
@@ -1410,12 +1426,13 @@ extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, 
                 pick_kernel(c->dc.g, L.lpg)<<<L.grid, L.threads, L.smem, stream>>>(
                     c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
                     tau_ns_out, status, ws_drem, counter, todo);
+                g_vp_launches++;
             } else {
                 pick_kernel(c->dc.g, L.lpg)<<<L.grid, L.threads, L.smem, stream>>>(
                     c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
                     tau_ns_out, status, ws_drem, counter, nullptr);
+                g_vp_launches++;
             }
-            g_vp_launches++;
             if (cudaGetLastError() != cudaSuccess) rc = VP_E_CUDA;
             vp_prof_mark(0, 1, stream);
         }
@@ -1443,6 +1460,15 @@ extern "C" int vp_schedule_launch_info(const vp_catalog* c, int B, const vp_sche
 extern "C" int vp_schedule_read_stats(const void* workspace, void* cuda_stream, uint64_t* out3) {
     if (!workspace || !out3) return VP_E_BAD_ARG;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    if (cudaMemcpyAsync(out3, (const char*)workspace + 16, 24, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return VP_E_CUDA;
-    return cudaStreamSynchronize(stream) == cudaSuccess ? VP_OK : VP_E_CUDA;
+    uint64_t head[32];
+    if (cudaMemcpyAsync(head, workspace, 256, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return VP_E_CUDA;
+    if (cudaStreamSynchronize(stream) != cudaSuccess) return VP_E_CUDA;
+    const uint32_t warps = (uint32_t)(head[1] >> 32);            // warps with counters of their own
+    for (int i = 0; i < 3; i++) out3[i] = warps ? 0 : head[2 + i];
+    if (!warps) return VP_OK;
+    std::vector<uint64_t> slots((size_t)warps * 3);
+    if (cudaMemcpyAsync(slots.data(), (const char*)workspace + 256, slots.size() * 8, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return VP_E_CUDA;
+    if (cudaStreamSynchronize(stream) != cudaSuccess) return VP_E_CUDA;
+    for (size_t i = 0; i < slots.size(); i++) out3[i % 3] += slots[i];
+    return VP_OK;
 }

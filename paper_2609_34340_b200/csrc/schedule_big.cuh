@@ -228,7 +228,6 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     constexpr int WL = CROSS ? 32 : LANES;                // a task's lanes in one warp
     constexpr int TPW = 32 / WL, QN = 4 / SPLIT;          // tasks per warp, columns per lane
     constexpr int ST = big_stride(LANES / SPLIT);         // words per row pair of the credit matrix
-    constexpr unsigned WLM = WL == 32 ? 0xffffffffu : (1u << (WL & 31)) - 1u;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = dc.N, G = dc.G, tid = threadIdx.x, NT = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, n_warps = NT >> 5;
@@ -255,7 +254,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     __shared__ int64_t s_tscale[VP_MAX_CLASSES];
     __shared__ uint32_t s_cap[VP_MAX_CLASSES];
     __shared__ __align__(8) unsigned long long s_stage_bar;
-    unsigned long long n_act = 0, n_tasks_done = 0, n_sweeps = 0;
+    unsigned long long n_act = 0, n_tasks_done = 0;
     Counters cnt;                                         // phase cycle counts (only with VP_PHASE_TIMING)
     cnt.t_mark = 0;
     for (int i = 0; i < 6; i++) cnt.cyc[i] = 0;
@@ -326,6 +325,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     // this thread's place in Step 2: task group (warp, or pair of warps), lane of the task, rank group and columns
     const int wg = CROSS ? warp >> 1 : warp, sub = CROSS ? warp & 1 : 0, n_tg = CROSS ? n_task_warps >> 1 : n_task_warps;
     const int tl = CROSS ? sub * 32 + lane : lane & (WL - 1), tsub = CROSS ? 0 : lane / WL, a = tl / SPLIT, part = tl - a * SPLIT;
+    const unsigned tmask = WL == 32 ? 0xffffffffu : ((1u << (WL & 31)) - 1u) << (tsub * WL);   // the task's lanes
+    unsigned my_sweeps = 0;
     const int ag = a < G ? a : 0;                         // (spare lanes repeat group 0 and are ignored)
     uint8_t* const ex_src = smem_raw + L.exchange + wg * BIG_EXCHANGE;
     uint8_t* const ex_dst = ex_src + 64;
@@ -567,10 +568,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             int p_fam = 0;
             uint32_t p_bind = 0, p_x = 0;
             uint2* const record = (uint2*)(smem_raw + L.record);
-            auto write_slot = [&](int kk, int r, int fam, uint32_t bind, uint32_t x) {
+            auto write_slot = [&](int kk, int r, int fam, uint32_t bind, uint32_t x, uint32_t inst) {
                 const int i = (int)(bind & 0xffu), j = (int)(bind >> 8);
                 const size_t row = (size_t)kk * N, orow = (size_t)(kk + 1) * N;
-                const uint32_t inst = __ldg(dc.fam_slot + (size_t)fam * N + r);
                 const int64_t bytes = (int64_t)x * kp.granule;
                 const int64_t sa = send_acc[i] + bytes, ra = recv_acc[j] + bytes;
                 send_acc[i] = sa;                             // (src and dst are permutations: every rank is written once)
@@ -582,12 +582,14 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 lane_inst_b[row + i] = x ? (uint16_t)inst : (uint16_t)0xFFFF;
                 if (r == 0) chan_id_b[kk] = fam;
             };
-            auto write_row = [&](int kk) {
+            auto write_row = [&](int kk, uint32_t inst) {
                 if (RECORD) {
                     const int fam = (int)record[N].x;
-                    for (int r = tid - n_task_warps * 32; r < N; r += NT - n_task_warps * 32) write_slot(kk, r, fam, record[r].x, record[r].y);
+                    for (int r = tid - n_task_warps * 32; r < N; r += NT - n_task_warps * 32)
+                        write_slot(kk, r, fam, record[r].x, record[r].y, __ldg(dc.fam_slot + (size_t)fam * N + r));
                 } else {
-                    write_slot(kk, r_emit, p_fam, p_bind, p_x);
+                    if (emit_warp > 0) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
+                    write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
                 }
                 pend = false;
             };
@@ -596,6 +598,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             for (;;) {
                 if (left == 0) break;
                 if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
+                // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
+                const uint32_t inst = !RECORD && emit_warp == 0 && pend ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
                 // (A) Eq. (6).  A score is at most four times what is left, so below 2^34, and there are fewer than 2^16
                 // shapes: key = score << 16 | (65535 - shape) orders by score first and lower shape index second, and the first
                 // maximum of Eq. (6) is a plain maximum of keys.
@@ -709,7 +713,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 VP_TICK(1);
 
                 // ---- rows of the last activation, where warps without a task write them, and a block of the fill
-                if (warp >= n_task_warps && pend) write_row(k - 1);
+                if (warp >= n_task_warps && pend) write_row(k - 1, inst);
                 if (fills && warp == fill_warp) {
                     if (fill_lo <= k + 1) {                    // the activations have reached filled rows: those copies must be over
                         bulk_wait_all();
@@ -746,7 +750,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 ui[0] = i.x; ui[1] = i.y;
                             }
                         }
-                        if (!RECORD && pend) write_row(k - 1); // (while the tables travel)
+                        if (!RECORD && pend) write_row(k - 1, inst); // (while the tables travel)
                         // start t binds in-slot q to row (q + t) mod 4
                         uint32_t dst = 0, src = 0;
 #pragma unroll
@@ -811,19 +815,13 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         }
                         fetch_dst();
                         uint32_t src_new = source_half();
-                        int F_old[TPW], F_new[TPW];
-                        unsigned alive = 0;                    // tasks still running, a bit each; the same in all their lanes, as F is
-#pragma unroll
-                        for (int s = 0; s < TPW; s++) {
-                            F_old[s] = F_new[s] = -1;
-                            if (task0 + s < n_tasks) alive |= 1u << s;
-                        }
+                        int F_old = -1, F_new = -1;            // this lane's task; the same in all its lanes, as alive is
+                        bool alive = task0 + tsub < n_tasks;
                         for (int sweep = 0; ; sweep++) {
-                            const bool on = (alive >> tsub) & 1u;
                             // If no source binding of a task moved, the destination half would see what it saw last sweep and
                             // return the same binding and the same F: the run ends here exactly as it would after computing that.
-                            const bool smoved = on && act && (sweep == 0 || src_new != src);
-                            if (on) src = src_new;
+                            const bool smoved = alive && act && (sweep == 0 || src_new != src);
+                            if (alive) src = src_new;
                             unsigned who = __ballot_sync(0xffffffffu, smoved);
                             if (CROSS) {
                                 if (SPLIT == 1 || part == 0) ex_src[a] = (uint8_t)src;
@@ -831,14 +829,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 task_sync();
                                 who = ex_word[0] | ex_word[1];
                             }
-#pragma unroll
-                            for (int s = 0; s < TPW; s++)
-                                if ((alive >> s & 1u) && !(CROSS ? who : who >> (s * WL) & WLM)) {
-                                    if (tl == 0 && tsub == s) n_sweeps++;
-                                    F_new[s] = F_old[s];
-                                    alive &= ~(1u << s);
-                                }
-                            if (!alive) break;
+                            if (alive && !(who & tmask)) { F_new = F_old; my_sweeps++; alive = false; }
+                            if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
                             // destination half: the tags of the in-slots' sources, the cells of their rows
                             uint32_t v[4][QN];
                             unsigned tag[QN];
@@ -862,44 +854,37 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                     }
                             }
                             const uint32_t key = best_key(v);
-                            const bool still = (alive >> tsub) & 1u;
-                            const bool dmoved = still && act && ((key ^ dst) & 0xffu) != 0;
-                            if (still) dst = key & 0xffu;
-                            const uint32_t credit = act && (SPLIT == 1 || part == 0) ? key >> 8 : 0u;
+                            const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
+                            if (alive) dst = key & 0xffu;
                             unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
-                            // Eq. (8): at most 2^8 lanes of less than 2^22 granules.
-                            uint32_t F[TPW];
-#pragma unroll
-                            for (int s = 0; s < TPW; s++) F[s] = __reduce_add_sync(0xffffffffu, TPW == 1 || tsub == s ? credit : 0u);
+                            // Eq. (8): at most 2^8 lanes of less than 2^22 granules.  The next sweep's source half needs no F: it runs while
+                            // the sum is under way and is dropped if the run ends.
+                            const bool more = sweep + 1 < kp.i_aa;
+                            uint32_t F = act ? key >> 8 : 0u;
+                            if constexpr (TPW == 1) F = __reduce_add_sync(0xffffffffu, SPLIT == 1 || part == 0 ? F : 0u);
                             if (CROSS) {
                                 if (SPLIT == 1 || part == 0) ex_dst[a] = (uint8_t)dst;
-                                if (lane == 0) { ex_word[2 + sub] = who2; ex_word[4 + sub] = F[0]; }
+                                if (lane == 0) { ex_word[2 + sub] = who2; ex_word[4 + sub] = F; }
                                 task_sync();
                                 who2 = ex_word[2] | ex_word[3];
-                                F[0] = ex_word[4] + ex_word[5];
+                                F = ex_word[4] + ex_word[5];
                             }
-                            // the next sweep's source half needs no F: it runs while the sums are under way and is dropped if the run ends
                             fetch_dst();
-                            const bool more = sweep + 1 < kp.i_aa;
                             if (more) src_new = source_half();
+                            if constexpr (TPW > 1) {           // (both lanes of a group hold its credit)
+#pragma unroll
+                                for (int o = SPLIT; o < WL; o <<= 1) F += __shfl_xor_sync(0xffffffffu, F, o);
+                            }
                             // If no destination binding moved, the next sweep would be a repetition of this one (same sources, same
                             // destinations, same F) and would end the run, so it is counted and skipped.
-#pragma unroll
-                            for (int s = 0; s < TPW; s++)
-                                if (alive >> s & 1u) {
-                                    const bool first = tl == 0 && tsub == s;
-                                    F_new[s] = (int)F[s];
-                                    if (first) n_sweeps++;
-                                    if (F_new[s] <= F_old[s] || !more) alive &= ~(1u << s);
-                                    else {
-                                        F_old[s] = F_new[s];
-                                        if (!(CROSS ? who2 : who2 >> (s * WL) & WLM)) {
-                                            if (first) n_sweeps++;
-                                            alive &= ~(1u << s);
-                                        }
-                                    }
-                                }
-                            if (!alive) break;
+                            if (alive) {
+                                F_new = (int)F;
+                                my_sweeps++;
+                                alive = F_new > F_old && more;
+                                F_old = F_new;
+                                if (alive && !(who2 & tmask)) { my_sweeps++; alive = false; }
+                            }
+                            if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
                         }
                         // Eq. (9) volumes of the binding as it stands and the slowest lane of Eq. (10): only needed when several
                         // families compete on utility
@@ -931,16 +916,13 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             if (QN == 4) at[1] = bind[QN - 2] | bind[QN - 1] << 16;
                         }
                         if (tl == 0 && task0 + tsub < n_tasks) {
-                            int Fn = F_new[0];
-#pragma unroll
-                            for (int s = 1; s < TPW; s++) Fn = tsub == s ? F_new[s] : Fn;
                             n_tasks_done++;
-                            task_f[task] = (uint32_t)Fn;
-                            if (H > 1) task_den[task] = Fn > 0 ? kp.lambda_ns * dc.W + tmax : 1;
+                            task_f[task] = (uint32_t)F_new;
+                            if (H > 1) task_den[task] = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
                         }
                     }
                 }
-                if (!RECORD && pend) write_row(k - 1);         // (warps that had no task)
+                if (!RECORD && pend) write_row(k - 1, inst);         // (warps that had no task)
                 __syncthreads();
                 VP_TICK(2);
 
@@ -984,7 +966,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     }
                     p_fam = f0 + (ns_shift >= 0 ? wtask >> ns_shift : wtask / kp.n_start);
                     uint32_t cap = cap0;
-                    if (!one_class) cap = s_cap[(__ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) >> 24) & 0xfu];
+                    if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + r_emit)];
                     if (!hot_mode) {
                         const uint32_t x = min_v(cap, c);
                         p_x = x;
@@ -1016,7 +998,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 __syncthreads();
                 VP_TICK(4);
             }
-            if (pend) write_row(k - 1);                          // the last activation of the matrix
+            if (pend) write_row(k - 1, RECORD ? 0u : __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit));   // the last activation of the matrix
         }
         __syncthreads();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
@@ -1063,7 +1045,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     unsigned long long* stats = (unsigned long long*)(counter + 4);
     if (tid == 0 && n_act) atomicAdd(&stats[0], n_act);
     n_tasks_done = (unsigned long long)warp_sum_i64((int64_t)n_tasks_done);    // (counted by the first lane of every task)
-    n_sweeps = (unsigned long long)warp_sum_i64((int64_t)n_sweeps);
+    const unsigned long long n_sweeps = (unsigned long long)warp_sum_i64(tl == 0 && warp < n_task_warps ? (int64_t)my_sweeps : 0);
     if (lane == 0 && n_tasks_done) { atomicAdd(&stats[1], n_tasks_done); atomicAdd(&stats[2], n_sweeps); }
 #ifdef VP_PHASE_TIMING
     if (tid == 0) for (int i = 0; i < 6; i++) atomicAdd(&stats[3 + i], (unsigned long long)cnt.cyc[i]);

@@ -2,14 +2,20 @@
 //
 // A matrix this small has too little work per phase for a whole CTA: with several warps per matrix most of an
 // iteration is spent in block barriers and in hand-overs through shared memory.  Here a warp owns a matrix from
-// the first to the last activation and nothing but __syncwarp orders its phases:
-//  (A) each lane scores every 32nd shape (Eq. 6); a butterfly of shuffles leaves the first maximum in all lanes;
-//  (B) the (family, start) tasks of the bucket run eight at a time: a team of four lanes per task, one lane per rank
-//      group, and every lane solves its group's exact 4 x 4 assignments (Eq. 7) by itself; the two halves of a sweep
-//      exchange nothing but the bindings; a task that stops improving (Eq. 8) is frozen while the others finish;
-//      Evaluate (Eq. 9, 10) runs when several families compete; best start / best family follow in registers;
-//  (D) sixteen lanes emit the activation and subtract it; D-hat is then re-summed from D_rem by all lanes
-//      (two lanes per cell), which needs no atomics.
+// the first to the last activation and nothing but __syncwarp orders its phases.  Two forms of the main loop:
+//
+//  * decompose_units: capacities below 2^22 granules (granules of at least 256 bytes, so as a rule).  Bound by the chain of
+//    dependent instructions of one activation, so each phase is cut to few of them:
+//    (A) a lane scores one row pattern of the catalog (source group x lane counts per destination group: at most 32), then
+//        every shape is the sum of four looked-up row scores; two warp reductions leave the first maximum (Eq. 6);
+//    (B) four (family, start) tasks at a time, two lanes per rank group: a lane reads two of the four columns of its group's
+//        4 x 4 tile (one 16-byte read each) and the pair joins its halves of the exact assignment (Eq. 7) by six shuffles.  A
+//        binding travels as one byte per group, by shuffle.  The next source half runs while Eq. (8) is summed;
+//    (C) every lane knows every F: best start without communication; Evaluate (Eq. 9, 10) only when families compete;
+//    (D) sixteen lanes take the activation off the residual (kept row-major and transposed) and off D-hat; its plan rows
+//        are written in the shadow of the next activation's tasks.
+//  * decompose_bytes: any other matrix, the same algorithm on 64-bit bytes with a lane per rank group.
+//
 // A CTA is one to four such warps that share only the staged catalog.  Included by schedule.cu.
 #pragma once
 
@@ -17,32 +23,36 @@ namespace {
 
 
 struct WarpSmem {                           // byte offsets; the per-warp block comes first, once per warp
-    int drem, dremT, dhat, send_acc, recv_acc, cred, cap64, tscale, cap32, bind_src, bind_dst, per_warp;
-    int term, fam_in, fam_cls, fam_slot, bucket, lut, total;
+    int drem, dremT, dhat, send_acc, recv_acc, rs, cap64, tscale, cap32, bind, bind_dst, per_warp;
+    int rows, shape_rows, fam_task, term, fam_in, fam_cls, fam_slot, bucket, total;
 };
 
-__host__ __device__ inline WarpSmem warp_smem_layout(const DevCat& dc, const KParams& kp, int n_warps) {
+// units: the tables of decompose_units are staged, otherwise those of decompose_bytes.
+__host__ __device__ inline WarpSmem warp_smem_layout(const DevCat& dc, const KParams& kp, int n_warps, bool units) {
     WarpSmem L;
+    const int ns_pad = (dc.n_shapes + 31) & ~31;
     int o = 0;
-    L.drem = o;      o += align16(dc.N * (dc.N + 1) * 8);      // rows padded by one element: no bank conflicts down a column
-    L.dremT = o;     o += align16(dc.N * dc.N * 4);            // 32-bit granules: the transpose (a column's four credits of a group in 16 bytes)
+    L.drem = o;      o += align16(dc.N * (dc.N + 1) * 8);      // bytes: rows padded by one element, no bank conflicts down a column
+    L.dremT = L.drem + dc.N * dc.N * 4;                        // 32-bit granules: residual and transpose share that space
     L.dhat = o;      o += align16(dc.G * dc.G * 8);
     L.send_acc = o;  o += dc.N * 8;
     L.recv_acc = o;  o += dc.N * 8;
-    L.cred = o;
+    L.rs = o;        o += 144 + 272;                           // row scores: 33 of 32 bits, then 33 of 64 bits
     L.cap64 = o;     o += VP_MAX_CLASSES * 8;
     L.tscale = o;    o += VP_MAX_CLASSES * 8;
     L.cap32 = o;     o += VP_MAX_CLASSES * 4;
-    L.bind_src = o;  o += align16(kp.max_tasks * dc.N);
+    L.bind = o;      o += align16(kp.max_tasks * dc.N);        // bytes: source of every slot; granules: with bind_dst, source | destination << 8
     L.bind_dst = o;  o += align16(kp.max_tasks * dc.N);
     L.per_warp = align16(o);
     o = L.per_warp * n_warps;
-    L.term = o;      o += ((dc.n_shapes + 31) & ~31) * dc.max_terms * 4;
-    L.fam_slot = o;  o += align16(dc.n_families * dc.N * 4);
-    L.fam_in = o;    o += align16(dc.n_families * dc.N * 2);
-    L.fam_cls = o;   o += align16(dc.n_families * dc.N);
-    L.bucket = o;    o += align16((dc.n_shapes + 1) * 4);
-    L.lut = o;       o += 32;
+    L.rows = o;        o += dc.row_term ? 32 * 16 : 0;
+    L.shape_rows = o;  o += dc.row_term ? ns_pad * 4 : 0;
+    L.fam_task = o;    o += units ? dc.n_families * dc.G * 32 : 0;
+    L.term = o;        o += units ? 0 : ns_pad * dc.max_terms * 4;
+    L.fam_slot = o;    o += units ? 0 : align16(dc.n_families * dc.N * 4);
+    L.fam_in = o;      o += units ? 0 : align16(dc.n_families * dc.N * 2);
+    L.fam_cls = o;     o += units ? 0 : align16(dc.n_families * dc.N);
+    L.bucket = o;      o += align16((dc.n_shapes + 1) * 4);
     L.total = o;
     return L;
 }
@@ -50,12 +60,15 @@ __host__ __device__ inline WarpSmem warp_smem_layout(const DevCat& dc, const KPa
 
 extern __shared__ __align__(16) unsigned char vp_wsmem[];   // the CTA's dynamic shared memory
 
-// Shared-memory byte offsets (into vp_wsmem) and output pointers of one warp's matrix.  Offsets rather than
+// Shared-memory byte offsets (into vp_wsmem), table and output pointers of one warp's matrix.  Offsets rather than
 // pointers: every access is then provably a shared-memory access with a 32-bit address.
 struct WCtx {
     int N, G, lane;
-    unsigned o_drem, o_dremT, o_dhat, o_send_acc, o_recv_acc, o_cred, o_cap, o_tscale, o_bind_src, o_bind_dst;
-    unsigned o_term, o_fam_slot, o_fam_in, o_fam_cls, o_bucket, o_lut;
+    unsigned o_drem, o_dremT, o_dhat, o_send_acc, o_recv_acc, o_rs, o_cap64, o_cap32, o_tscale, o_bind, o_bind_dst;
+    unsigned o_rows, o_shape_rows, o_fam_task, o_bucket;
+    const uint32_t *term, *fam_slot;                            // (decompose_bytes: shared or global memory)
+    const uint16_t* fam_in;
+    const uint8_t* fam_cls;
     int32_t* chan_id_b;
     int16_t* lane_dst_b;
     uint16_t* lane_inst_b;
@@ -64,11 +77,7 @@ struct WCtx {
 
 template <typename T> __device__ __forceinline__ T* ws(unsigned off) { return (T*)(vp_wsmem + off); }
 
-// Sum over the four lanes of a team (lane & ~3 .. lane | 3); every lane gets it.
-__device__ __forceinline__ uint32_t team_sum(uint32_t v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    return v + __shfl_xor_sync(0xffffffffu, v, 2);
-}
+// Sum and maximum over the four lanes of a team (lane & ~3 .. lane | 3); every lane gets it.
 __device__ __forceinline__ int64_t team_sum(int64_t v) {
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     return v + __shfl_xor_sync(0xffffffffu, v, 2);
@@ -78,65 +87,317 @@ __device__ __forceinline__ int64_t team_max(int64_t v) {
     return max_v(v, __shfl_xor_sync(0xffffffffu, v, 2));
 }
 
-// Eq. (6) for the R shapes of a lane (shape lane + 32 u) from their lane counts, four bits per D-hat cell (cells 0..7 in
-// the first word, 8..15 in the second), against the cells themselves; S is the score type (32 bits while scores stay
-// below 2^31).  Cells are taken four at a time (a table has 1, 4, 9 or 16 of them; a cell beyond the table has count 0
-// in every shape, so what is read there does not matter).  Leaves the lane's first maximum in (best, best_s).
-template <int R, typename S>
-__device__ __forceinline__ void score_dense(const int64_t* Dhat, int tbl_size, const uint32_t (&smask)[4][2], int lane, int n_shapes,
-                                            int64_t& best, int& best_s) {
-    S sc[R];
+// Eq. (6) by row patterns: this lane's pattern, and the byte offsets of the (32-bit) row scores of its up to four shapes.
+struct RowScores {
+    bool on;
+    unsigned rs;
+    int n_shapes;
+    uint4 row;
+    unsigned so[4][4];
+    __device__ __forceinline__ void load(const DevCat& dc, const WCtx& c) {
+        on = dc.row_term != nullptr && dc.n_shapes <= 128;
+        rs = c.o_rs;
+        n_shapes = dc.n_shapes;
+        if (c.lane == 0) { ws<uint32_t>(rs)[32] = 0u; ws<int64_t>(rs + 144)[32] = 0; }
+        row = make_uint4(0u, 0u, 0u, 0u);
+        if (on) row = *(ws<uint4>(c.o_rows) + c.lane);
 #pragma unroll
-    for (int u = 0; u < R; u++) sc[u] = 0;
+        for (int u = 0; u < 4; u++) {
+            // (shapes beyond the catalog: four times pattern 32, whose score is zero)
+            const uint32_t w = on && c.lane + 32 * u < n_shapes ? ws<uint32_t>(c.o_shape_rows)[c.lane + 32 * u] : 0x20202020u;
 #pragma unroll
-    for (int quad = 0; quad < 4; quad++) {
-        if (quad * 4 < tbl_size) {
-#pragma unroll
-            for (int m = 0; m < 4; m++) {
-                const int cell = quad * 4 + m;
-                const S d = (S)Dhat[cell];
-#pragma unroll
-                for (int u = 0; u < R; u++) sc[u] += d * (S)((smask[u][cell >> 3] >> (4 * (cell & 7))) & 15u);
-            }
+            for (int r = 0; r < 4; r++) so[u][r] = rs + 4 * ((w >> (8 * r)) & 0xffu);
         }
     }
+    // largest score and, in best_s, the lane's first shape that has it (low words of D-hat)
+    __device__ __forceinline__ uint32_t narrow(const uint32_t* dhat32, int lane, int& best_s) const {
+        ws<uint32_t>(rs)[lane] = dhat32[2 * (row.x & 0xffffu)] * (row.x >> 16) + dhat32[2 * (row.y & 0xffffu)] * (row.y >> 16) +
+                                 dhat32[2 * (row.z & 0xffffu)] * (row.z >> 16) + dhat32[2 * (row.w & 0xffffu)] * (row.w >> 16);
+        __syncwarp();
+        uint32_t best = 0;
 #pragma unroll
-    for (int u = 0; u < R; u++)
-        if (lane + 32 * u < n_shapes && (int64_t)sc[u] > best) { best = (int64_t)sc[u]; best_s = lane + 32 * u; }
+        for (int u = 0; u < 4; u++)
+            if (u < 3 || n_shapes > 96) {
+                const uint32_t v = *ws<uint32_t>(so[u][0]) + *ws<uint32_t>(so[u][1]) + *ws<uint32_t>(so[u][2]) + *ws<uint32_t>(so[u][3]);
+                if (v > best) { best = v; best_s = lane + 32 * u; }
+            }
+        return best;
+    }
+    __device__ __forceinline__ void wide(const int64_t* Dhat, int lane, int64_t& best, int& best_s) const {
+        ws<int64_t>(rs + 144)[lane] = Dhat[row.x & 0xffffu] * (int64_t)(row.x >> 16) + Dhat[row.y & 0xffffu] * (int64_t)(row.y >> 16) +
+                                Dhat[row.z & 0xffffu] * (int64_t)(row.z >> 16) + Dhat[row.w & 0xffffu] * (int64_t)(row.w >> 16);
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (lane + 32 * u < n_shapes) {
+                int64_t v = 0;
+#pragma unroll
+                for (int r = 0; r < 4; r++) v += *ws<int64_t>(2 * so[u][r] - rs + 144);
+                if (v > best) { best = v; best_s = lane + 32 * u; }
+            }
+    }
+};
+
+// Eq. (6) from the terms themselves, for catalogs with more patterns or shapes than that: first maximum of this lane's shapes.
+__device__ __forceinline__ void score_terms(const DevCat& dc, const uint32_t* term, const int64_t* Dhat, int lane, int64_t& best, int& best_s) {
+    const int ns_pad = (dc.n_shapes + 31) & ~31;               // row stride of the transposed term table
+    for (int s0 = lane; s0 < dc.n_shapes; s0 += 128) {         // four shapes per lane in flight
+        int64_t score[4] = {0, 0, 0, 0};
+        const uint32_t* tp = term + s0;                        // term e of shape s is at [e][s]: lanes read neighbours
+        const int last = dc.n_shapes - 1 - s0;                 // shapes beyond the catalog re-read the last one
+        int du[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) du[u] = min(32 * u, last);
+#pragma unroll 4
+        for (int e = 0; e < dc.max_terms; e++) {
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const uint32_t w = tp[e * ns_pad + du[u]];
+                score[u] += *(const int64_t*)((const char*)Dhat + (w & 0xffffu)) * (int64_t)(w >> 16);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (s0 + 32 * u < dc.n_shapes && score[u] > best) { best = score[u]; best_s = s0 + 32 * u; }
+    }
 }
 
-template <typename V>
-__device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& kp, const WCtx& c, int64_t unit, int64_t left,
-                                               int& k, int& st, Counters& cnt) {
+// Main loop for a matrix held in 32-bit granules (`left` of them) with capacities below 2^22 granules.
+__device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams& kp, const WCtx& c, int64_t left, int& k, int& st, Counters& cnt) {
     const int N = c.N, G = c.G, lane = c.lane;
-    // row stride of D_rem: N for 32-bit granules (a row's four credits of a group are one 16-byte load), N + 1 for bytes
-    const int ld = sizeof(V) == 4 ? N : N + 1;
-    const int ns_pad = (dc.n_shapes + 31) & ~31;         // row stride of the transposed term table
-    // Step 2 runs eight (family, start) tasks at a time: a team of four lanes per task, one lane per rank group, which
-    // solves its group's exact 4 x 4 assignments on its own (best_assignment) -- no credit tiles, no hand-overs
-    // between lanes except the bindings themselves.
+    uint32_t* const D = ws<uint32_t>(c.o_drem);
+    uint32_t* const DT = ws<uint32_t>(c.o_dremT);              // DT[j * N + i] = D[i * N + j]
+    int64_t* const Dhat = ws<int64_t>(c.o_dhat);
+    const uint32_t* const dhat32 = ws<uint32_t>(c.o_dhat);     // (low words)
+    const uint32_t* const s_cap = ws<uint32_t>(c.o_cap32);
+    uint16_t* const bindings = ws<uint16_t>(c.o_bind);
+    const bool one_class = dc.n_classes == 1;
+    const uint32_t cap0 = s_cap[0];
+    const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
+    // this lane's place in Step 2: task of four, rank group, columns 2 part and 2 part + 1 of the group's tile
+    const int tsub = lane >> 3, a = (lane & 7) >> 1, part = lane & 1, ag = a < G ? a : 0;
+    const unsigned gmask = 0xffu << (8 * tsub);
+    unsigned n_sweeps = 0, n_done = 0;
+    uint32_t tags[3][2];
+#pragma unroll
+    for (int r = 0; r < 3; r++)
+#pragma unroll
+        for (int i = 0; i < 2; i++) tags[r][i] = (uint32_t)(3 - r) << (6 - 2 * (part * 2 + i));
+    RowScores by_rows;
+    by_rows.load(dc, c);
+    // the activation taken off the residual whose rows are still to be written (slot `lane`)
+    bool pend = false;
+    int p_fam = 0;
+    uint32_t p_bind = 0, p_x = 0;
+    auto write_row = [&](int kk, uint32_t inst) {
+        if (lane < N) {
+            const int i = (int)(p_bind & 0xffu), j = (int)(p_bind >> 8);
+            const size_t row = (size_t)kk * N, orow = (size_t)(kk + 1) * N;
+            const int64_t bytes = (int64_t)p_x * kp.granule;
+            const int64_t sa = ws<int64_t>(c.o_send_acc)[i] + bytes, ra = ws<int64_t>(c.o_recv_acc)[j] + bytes;
+            ws<int64_t>(c.o_send_acc)[i] = sa;
+            ws<int64_t>(c.o_recv_acc)[j] = ra;
+            c.lane_dst_b[row + i] = p_x ? (int16_t)j : (int16_t)-1;
+            c.lane_bytes_b[row + i] = bytes;
+            c.send_off_b[orow + i] = sa;
+            if (c.recv_off_b) c.recv_off_b[orow + j] = ra;
+            c.lane_inst_b[row + i] = p_x ? (uint16_t)inst : (uint16_t)0xFFFF;
+            if (lane == 0) c.chan_id_b[kk] = p_fam;
+        }
+        pend = false;
+    };
+
+    for (;;) {
+        if (left == 0) break;
+        if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
+        // path instance of the slot to be written out: a trip to L2 that ends long before write_row needs it
+        const uint32_t inst = pend && lane < N ? __ldg(dc.fam_slot + (size_t)p_fam * N + lane) : 0u;
+        // (A) Eq. (6): shape scores, first maximum
+        const bool narrow = left < ((int64_t)1 << 30);           // every score (at most g x what is left) fits 32 bits
+        int best_s = 0x7fffffff;
+        bool covered;
+        if (by_rows.on && narrow) {
+            const uint32_t best = by_rows.narrow(dhat32, lane, best_s), m = __reduce_max_sync(0xffffffffu, best);
+            covered = m != 0;
+            best_s = (int)__reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 0x7fffffffu);
+        } else {
+            int64_t best = -1;
+            if (by_rows.on) by_rows.wide(Dhat, lane, best, best_s);
+            else score_terms(dc, dc.term_t, Dhat, lane, best, best_s);
+            warp_argmax_first(best, best_s);
+            covered = best > 0;
+        }
+        VP_TICK(0);
+        if (!covered) { st |= VP_ST_UNCOVERED; break; }
+        const int f0 = (int)ws<uint32_t>(c.o_bucket)[best_s], H = (int)ws<uint32_t>(c.o_bucket)[best_s + 1] - f0;
+        const int n_tasks = H * kp.n_start;
+        VP_TICK(1);
+
+        // (B) MultiStartAA, four (family, start) tasks at a time; (C) best start per family, best family
+        int64_t bf = -1, bd = 1, ff = -1, fd = 1;                // best family so far; best start of the current family
+        int bt = -1, ft = -1, cur_h = -1;
+        uint32_t my_bind = 0;                                    // this lane's two slots: (source | destination << 8) x 2
+        for (int task0 = 0; task0 < n_tasks; task0 += 4) {
+            const int task = min(task0 + tsub, n_tasks - 1);
+            const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, f = f0 + h, t = task - h * kp.n_start;
+            const bool act = task0 + tsub < n_tasks && a < G;
+            // slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag
+            const uint32_t* const fam = ws<uint32_t>(c.o_fam_task) + (f * G + ag) * 8 + part * 2;
+            const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
+            if (pend) write_row(k - 1, inst);
+            // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits, of
+            // position 3 in the lowest.  Start t binds in-slot q to row (q + t) mod 4.
+            uint32_t dst = 0, src = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
+            const uint32_t oc0 = one_class ? cap0 : s_cap[(uo.x >> 24) & 0xfu], oc1 = one_class ? cap0 : s_cap[(uo.y >> 24) & 0xfu];
+            const uint32_t ic0 = one_class ? cap0 : s_cap[(ui.x >> 24) & 0xfu], ic1 = one_class ? cap0 : s_cap[(ui.y >> 24) & 0xfu];
+            int dt0, dt1;                                        // tags (3 - row) of the out-slots' destinations
+            // best key of the tile whose columns 2 part, 2 part + 1 are x and y: both columns on every pair of rows; the other lane
+            // of the group has the other two columns
+            auto best_key = [&](const uint4& x, uint32_t cx, const uint4& y, uint32_t cy) {
+                const uint32_t x0 = min_v(x.x, cx) * 256u + tags[0][0], x1 = min_v(x.y, cx) * 256u + tags[1][0];
+                const uint32_t x2 = min_v(x.z, cx) * 256u + tags[2][0], x3 = min_v(x.w, cx) * 256u;
+                const uint32_t y0 = min_v(y.x, cy) * 256u + tags[0][1], y1 = min_v(y.y, cy) * 256u + tags[1][1];
+                const uint32_t y2 = min_v(y.z, cy) * 256u + tags[2][1], y3 = min_v(y.w, cy) * 256u;
+                const uint32_t p01 = add_max(x0, y1, x1 + y0), p02 = add_max(x0, y2, x2 + y0), p03 = add_max(x0, y3, x3 + y0);
+                const uint32_t p12 = add_max(x1, y2, x2 + y1), p13 = add_max(x1, y3, x3 + y1), p23 = add_max(x2, y3, x3 + y2);
+                const uint32_t o01 = __shfl_xor_sync(0xffffffffu, p01, 1), o02 = __shfl_xor_sync(0xffffffffu, p02, 1);
+                const uint32_t o03 = __shfl_xor_sync(0xffffffffu, p03, 1), o12 = __shfl_xor_sync(0xffffffffu, p12, 1);
+                const uint32_t o13 = __shfl_xor_sync(0xffffffffu, p13, 1), o23 = __shfl_xor_sync(0xffffffffu, p23, 1);
+                const uint32_t m0 = add_max(p01, o23, add_max(p02, o13, p03 + o12)), m1 = add_max(p12, o03, add_max(p13, o02, p23 + o01));
+                return max_v(m0, m1);
+            };
+            auto tag_of = [&](uint32_t bytes, uint32_t w) { return (int)((__shfl_sync(0xffffffffu, bytes, (int)(w >> 15), 8) >> (w >> 28)) & 3u); };
+            auto source_half = [&]() {                           // credits of group a towards its out-slots' destinations
+                dt0 = tag_of(dst, uo.x);
+                dt1 = tag_of(dst, uo.y);
+                return best_key(*(const uint4*)(DT + ((int)(uo.x & 0xffffu) - dt0 * N)), oc0, *(const uint4*)(DT + ((int)(uo.y & 0xffffu) - dt1 * N)), oc1) & 0xffu;
+            };
+            uint32_t src_new = source_half();
+            int F_old = -1, F_new = -1;                          // this lane's task; the same in its eight lanes, as alive is
+            bool alive = task0 + tsub < n_tasks;
+            for (int sweep = 0; ; sweep++) {
+                // If no source binding of a task moved, the destination half would see what it saw last sweep and return the same
+                // binding and the same F: the run ends here exactly as it would after computing that.
+                const bool smoved = alive && act && (sweep == 0 || src_new != src);
+                if (alive) src = src_new;
+                if (sweep) {
+                    const unsigned who = __ballot_sync(0xffffffffu, smoved);
+                    if (alive && !(who & gmask)) { F_new = F_old; n_sweeps++; alive = false; }
+                    if (!__any_sync(0xffffffffu, alive)) break;
+                }
+                // destination half: credits into group a from its in-slots' sources
+                const int s0 = tag_of(src, ui.x), s1 = tag_of(src, ui.y);
+                const uint32_t key = best_key(*(const uint4*)(D + ((int)(ui.x & 0xffffu) - s0 * N)), ic0, *(const uint4*)(D + ((int)(ui.y & 0xffffu) - s1 * N)), ic1);
+                const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
+                if (alive) dst = key & 0xffu;
+                // the next sweep's source half needs no F: it runs while that is summed and is dropped if the run ends (the destinations'
+                // tags it looks up are those of the final binding)
+                uint32_t F = act ? key >> 8 : 0u;                // Eq. (8); both lanes of a group hold its credit
+                F += __shfl_xor_sync(0xffffffffu, F, 2);
+                src_new = source_half();
+                F += __shfl_xor_sync(0xffffffffu, F, 4);
+                const unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
+                // If no destination binding moved, the next sweep would be a repetition of this one and would end the run, so it is
+                // counted and skipped.
+                if (alive) {
+                    F_new = (int)F;
+                    n_sweeps++;
+                    alive = F_new > F_old && sweep + 1 < kp.i_aa;
+                    F_old = F_new;
+                    if (alive && !(who2 & gmask)) { n_sweeps++; alive = false; }
+                }
+                if (!__any_sync(0xffffffffu, alive)) break;
+            }
+            VP_TICK(2);
+            my_bind = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
+                      (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
+            n_done += (unsigned)min(4, n_tasks - task0);
+            if (H == 1 && n_tasks <= 4) {                        // one family, one round: largest F, lowest start; bindings stay in registers
+                const uint32_t best = __reduce_max_sync(0xffffffffu, F_new > 0 ? (uint32_t)F_new << 2 | (uint32_t)(3 - tsub) : 0u);
+                bf = (int64_t)(best >> 2); bt = 3 - (int)(best & 3u);      // (F is at most sixteen lanes of 2^22 granules)
+                break;
+            }
+            if (act) *(uint32_t*)(bindings + task * N + a * 4 + part * 2) = my_bind;
+            // Evaluate (Eq. 9, 10), needed only when several families compete: slowest lane under the final bindings
+            int64_t den = 1;
+            if (H > 1) {
+                int64_t tmax = 0;
+                if (act) {
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        const uint32_t bw = my_bind >> (16 * i), cl = ((i ? uo.y : uo.x) >> 24) & 0xfu;
+                        const uint32_t x = min_v(D[(int)(bw & 0xffu) * N + (int)((bw >> 8) & 0xffu)], s_cap[cl]);
+                        tmax = max_v(tmax, (int64_t)x * ws<int64_t>(c.o_tscale)[cl]);
+                    }
+                }
+                tmax = team_max(tmax);
+                tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
+                den = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
+            }
+            // the round's results in task order (every lane follows along)
+#pragma unroll
+            for (int s = 0; s < 4; s++) {
+                const int64_t Fs = __shfl_sync(0xffffffffu, F_new, 8 * s), ds = __shfl_sync(0xffffffffu, den, 8 * s);
+                const int tk = task0 + s, ht = ns_shift >= 0 ? tk >> ns_shift : tk / kp.n_start;
+                if (tk < n_tasks) {
+                    if (ht != cur_h) {                           // a new family starts: settle the previous one
+                        if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }
+                        cur_h = ht; ff = -1; fd = 1; ft = -1;
+                    }
+                    if (Fs > ff) { ff = Fs; fd = ds; ft = tk; }  // largest F, lowest start
+                }
+            }
+        }
+        if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }   // lowest family on ties
+        if (bf <= 0) { st |= VP_ST_NO_PROGRESS; break; }
+        VP_TICK(3);
+
+        // (D) activation k off the residual and off D-hat (Eq. 5)
+        __syncwarp();
+        {
+            const int h = ns_shift >= 0 ? bt >> ns_shift : bt / kp.n_start;
+            p_fam = f0 + h;
+            if (cur_h < 0) p_bind = (__shfl_sync(0xffffffffu, my_bind, (bt << 3 | lane >> 1) & 31) >> (16 * (lane & 1))) & 0xffffu;
+            else p_bind = lane < N ? bindings[bt * N + lane] : 0u;
+            if (lane < N) {
+                const int i = (int)(p_bind & 0xffu), j = (int)(p_bind >> 8);
+                uint32_t cap = cap0;
+                if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + lane)];
+                const uint32_t cell = D[i * N + j], x = min_v(cap, cell);
+                D[i * N + j] = cell - x;
+                DT[j * N + i] = cell - x;
+                int64_t* const sum = &Dhat[(lane >> 2) * G + (j >> 2)];
+                if (narrow) atomicSub((unsigned int*)sum, x);    // (high word is zero, low word >= x)
+                else atomicAdd((unsigned long long*)sum, (unsigned long long)(-(int64_t)x));
+                p_x = x;
+            }
+            pend = true;
+            left -= bf;
+        }
+        k++;
+        __syncwarp();
+        VP_TICK(4);
+    }
+    if (pend) write_row(k - 1, lane < N ? __ldg(dc.fam_slot + (size_t)p_fam * N + lane) : 0u);
+    if (lane == 0) cnt.tasks += n_done;
+    if ((lane & 7) == 0) cnt.sweeps += n_sweeps;
+}
+
+// Main loop for any other matrix, in 64-bit bytes (`left` of them): eight (family, start) tasks at a time, a team of four lanes
+// per task, one lane per rank group, which enumerates its group's 24 permutations.
+__device__ __forceinline__ void decompose_bytes(const DevCat& dc, const KParams& kp, const WCtx& c, int64_t left, int& k, int& st, Counters& cnt) {
+    const int N = c.N, G = c.G, lane = c.lane;
+    const int ld = N + 1;                                // row stride of D_rem
     const int team = lane >> 2, a = lane & 3;
     const bool active = a < G;
     const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
-    V* const Drem = ws<V>(c.o_drem);
-    uint32_t* const DremT = ws<uint32_t>(c.o_dremT);      // (32-bit granules only) DremT[j * N + i] = Drem[i * N + j]
-    const V* const cap = ws<V>(c.o_cap);
+    int64_t* const Drem = ws<int64_t>(c.o_drem);
+    const int64_t* const cap = ws<int64_t>(c.o_cap64);
     int64_t* const Dhat = ws<int64_t>(c.o_dhat);
-    // Plain score tables of at most 16 D-hat cells and at most 128 shapes: a lane keeps the lane counts of its (up to
-    // four) shapes in registers, four bits per cell, and scoring needs no term loads.
-    const bool dense = dc.tbl_size <= 16 && dc.n_shapes <= 128;
-    const int n_rounds = (dc.n_shapes + 31) >> 5;         // shapes per lane (dense: at most four)
-    uint32_t smask[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};     // cells 0..7, cells 8..15
-    if (dense)
-        for (int u = 0; u < 4; u++) {
-            const int s = lane + 32 * u;
-            if (s < dc.n_shapes)
-                for (int e = 0; e < dc.max_terms; e++) {
-                    const uint32_t w = ws<uint32_t>(c.o_term)[e * ns_pad + s];
-                    const uint32_t cell = (w & 0xffffu) >> 3;
-                    smask[u][cell >> 3] |= (w >> 16) << (4 * (cell & 7));
-                }
-        }
+    RowScores by_rows;
+    by_rows.load(dc, c);
 
     for (;;) {
         if (left == 0) break;
@@ -144,40 +405,8 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
         // (A) Eq. (6): shape scores, first maximum
         int64_t best = -1;
         int best_s = 0x7fffffff;
-        const bool narrow_now = left < ((int64_t)1 << 31);       // every D-hat cell fits 32 bits
-        if (dense) {
-            const bool narrow = left * 4 < ((int64_t)1 << 31);   // a score is at most g x (what is left)
-            switch (n_rounds * 2 + (narrow ? 1 : 0)) {
-                case 3: score_dense<1, uint32_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 5: score_dense<2, uint32_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 7: score_dense<3, uint32_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 9: score_dense<4, uint32_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 2: score_dense<1, int64_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 4: score_dense<2, int64_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                case 6: score_dense<3, int64_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-                default: score_dense<4, int64_t>(Dhat, dc.tbl_size, smask, lane, dc.n_shapes, best, best_s); break;
-            }
-        } else {
-            for (int s0 = lane; s0 < dc.n_shapes; s0 += 128) {     // four shapes per lane in flight
-                int64_t score[4] = {0, 0, 0, 0};
-                const uint32_t* tp = ws<uint32_t>(c.o_term) + s0;  // term e of shape s is at [e][s]: lanes read neighbours
-                const int last = dc.n_shapes - 1 - s0;             // shapes beyond the catalog re-read the last one
-                int du[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) du[u] = min(32 * u, last);
-#pragma unroll 4
-                for (int e = 0; e < dc.max_terms; e++) {
-#pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        const uint32_t w = tp[e * ns_pad + du[u]];
-                        score[u] += *(const int64_t*)((const char*)Dhat + (w & 0xffffu)) * (int64_t)(w >> 16);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; u++)
-                    if (s0 + 32 * u < dc.n_shapes && score[u] > best) { best = score[u]; best_s = s0 + 32 * u; }
-            }
-        }
+        if (by_rows.on) by_rows.wide(Dhat, lane, best, best_s);
+        else score_terms(dc, c.term, Dhat, lane, best, best_s);
         VP_TICK(0);
         warp_argmax_first(best, best_s);
         if (best <= 0) { st |= VP_ST_UNCOVERED; break; }
@@ -192,13 +421,13 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
             const int task = min(task0 + team, n_tasks - 1);
             const bool has = task0 + team < n_tasks && active;
             const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, tt = task - h * kp.n_start, f = f0 + h;
-            uint8_t* const srcb = ws<uint8_t>(c.o_bind_src) + task * N;
+            uint8_t* const srcb = ws<uint8_t>(c.o_bind) + task * N;
             uint8_t* const dstb = ws<uint8_t>(c.o_bind_dst) + task * N;
-            V cap_out[4], cap_in[4];
+            int64_t cap_out[4], cap_in[4];
             int rq[4], cls_in[4];
             const int ag = active ? a : 0;                   // (spare lanes read group 0's tables and write nothing)
-            const uint2 fin4 = *(const uint2*)(ws<uint16_t>(c.o_fam_in) + f * N + ag * 4);        // four in-slots, 16 bits each
-            const uint32_t fcls4 = *(const uint32_t*)(ws<uint8_t>(c.o_fam_cls) + f * N + ag * 4);  // four out-slot classes
+            const uint2 fin4 = *(const uint2*)(c.fam_in + f * N + ag * 4);        // four in-slots, 16 bits each
+            const uint32_t fcls4 = *(const uint32_t*)(c.fam_cls + f * N + ag * 4);  // four out-slot classes
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const unsigned w = ((q < 2 ? fin4.x : fin4.y) >> (16 * (q & 1))) & 0xffffu;
@@ -215,70 +444,35 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
             for (int sweep = 0; sweep < kp.i_aa && __any_sync(0xffffffffu, alive); sweep++) {
                 if (alive) {                                  // source half: credits of group a towards its out-slots' destinations
                     const uint32_t d4 = *(const uint32_t*)(dstb + a * 4);
-                    V cm[4][4];
+                    int64_t cm[4][4];
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
                         const int dq = (int)((d4 >> (8 * q)) & 0xffu);
-                        if constexpr (sizeof(V) == 4) {
-                            const uint4 c4 = *(const uint4*)(DremT + dq * N + a * 4);
-                            cm[0][q] = min_v((V)c4.x, cap_out[q]); cm[1][q] = min_v((V)c4.y, cap_out[q]);
-                            cm[2][q] = min_v((V)c4.z, cap_out[q]); cm[3][q] = min_v((V)c4.w, cap_out[q]);
-                        } else {
-                            const V* col = Drem + (a * 4) * ld + dq;
+                        const int64_t* col = Drem + (a * 4) * ld + dq;
 #pragma unroll
-                            for (int i = 0; i < 4; i++) cm[i][q] = min_v(col[i * ld], cap_out[q]);
-                        }
+                        for (int i = 0; i < 4; i++) cm[i][q] = min_v(col[i * ld], cap_out[q]);
                     }
-                    uint32_t rows4;                          // the row bound to position q, in byte q
-                    if constexpr (sizeof(V) == 4) {
-                        uint32_t v[4][4];
-#pragma unroll
-                        for (int i = 0; i < 4; i++)
-#pragma unroll
-                            for (int q = 0; q < 4; q++) v[i][q] = (uint32_t)cm[i][q] * 256u + big_tag(i, q);
-                        const uint32_t pb = ~big_best_key(v) & 255u;      // position 0 in the two highest bits
-                        rows4 = ((pb >> 6) & 3u) | ((pb << 4) & 0x300u) | ((pb << 14) & 0x30000u) | ((pb << 24) & 0x3000000u);
-                    } else {
-                        unsigned bpk;
-                        best_assignment<4, V>(cm, bpk);
-                        rows4 = (bpk & 3u) | ((bpk >> 2) & 3u) << 8 | ((bpk >> 4) & 3u) << 16 | ((bpk >> 6) & 3u) << 24;
-                    }
+                    unsigned bpk;
+                    best_assignment<4, int64_t>(cm, bpk);
+                    const uint32_t rows4 = (bpk & 3u) | ((bpk >> 2) & 3u) << 8 | ((bpk >> 4) & 3u) << 16 | ((bpk >> 6) & 3u) << 24;   // the row bound to position q, in byte q
                     *(uint32_t*)(srcb + a * 4) = (uint32_t)(a * 4) * 0x01010101u + rows4;
                 }
                 __syncwarp();
-                V part = 0;
+                int64_t part = 0;
                 if (alive) {                                  // destination half: credits into group a from its in-slots' sources
-                    V cm[4][4];
+                    int64_t cm[4][4];
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
-                        const V* row = Drem + (int)srcb[rq[q]] * ld + a * 4;
-                        if constexpr (sizeof(V) == 4) {
-                            const uint4 r4 = *(const uint4*)row;
-                            cm[0][q] = min_v((V)r4.x, cap_in[q]); cm[1][q] = min_v((V)r4.y, cap_in[q]);
-                            cm[2][q] = min_v((V)r4.z, cap_in[q]); cm[3][q] = min_v((V)r4.w, cap_in[q]);
-                        } else {
+                        const int64_t* row = Drem + (int)srcb[rq[q]] * ld + a * 4;
 #pragma unroll
-                            for (int i = 0; i < 4; i++) cm[i][q] = min_v(row[i], cap_in[q]);
-                        }
+                        for (int i = 0; i < 4; i++) cm[i][q] = min_v(row[i], cap_in[q]);
                     }
-                    if constexpr (sizeof(V) == 4) {
-                        uint32_t v[4][4];
+                    unsigned bpk;
+                    part = best_assignment<4, int64_t>(cm, bpk);
 #pragma unroll
-                        for (int i = 0; i < 4; i++)
-#pragma unroll
-                            for (int q = 0; q < 4; q++) v[i][q] = (uint32_t)cm[i][q] * 256u + big_tag(i, q);
-                        const uint32_t key = big_best_key(v), pb = ~key & 255u;
-                        part = (V)(key >> 8);
-#pragma unroll
-                        for (int q = 0; q < 4; q++) dstb[rq[q]] = (uint8_t)(a * 4 + ((pb >> (6 - 2 * q)) & 3u));
-                    } else {
-                        unsigned bpk;
-                        part = best_assignment<4, V>(cm, bpk);
-#pragma unroll
-                        for (int q = 0; q < 4; q++) dstb[rq[q]] = (uint8_t)(a * 4 + ((bpk >> (2 * q)) & 3u));
-                    }
+                    for (int q = 0; q < 4; q++) dstb[rq[q]] = (uint8_t)(a * 4 + ((bpk >> (2 * q)) & 3u));
                 }
-                const int64_t Fn = (int64_t)team_sum(part);   // Eq. (8)
+                const int64_t Fn = team_sum(part);   // Eq. (8)
                 if (alive) {
                     F_new = Fn;
                     if (a == 0) cnt.sweeps++;
@@ -296,8 +490,8 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
                 if (has) {
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
-                        const V x = min_v(Drem[(int)srcb[rq[q]] * ld + (int)dstb[rq[q]]], cap_in[q]);
-                        tmax = max_v(tmax, (int64_t)x * ws<int64_t>(c.o_tscale)[cls_in[q]]);
+                        const int64_t x = min_v(Drem[(int)srcb[rq[q]] * ld + (int)dstb[rq[q]]], cap_in[q]);
+                        tmax = max_v(tmax, x * ws<int64_t>(c.o_tscale)[cls_in[q]]);
                     }
                 }
                 tmax = team_max(tmax);
@@ -338,23 +532,17 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
             const size_t row = (size_t)k * N, orow = (size_t)(k + 1) * N;
             if (lane < N) {
                 const int r = lane;
-                const uint32_t w = ws<uint32_t>(c.o_fam_slot)[(f0 + h) * N + r];
-                const int i = ws<uint8_t>(c.o_bind_src)[bt * N + r], j = ws<uint8_t>(c.o_bind_dst)[bt * N + r];
-                const V x = min_v(cap[(w >> 24) & 0xf], Drem[i * ld + j]);
+                const uint32_t w = c.fam_slot[(f0 + h) * N + r];
+                const int i = ws<uint8_t>(c.o_bind)[bt * N + r], j = ws<uint8_t>(c.o_bind_dst)[bt * N + r];
+                const int64_t bytes = min_v(cap[(w >> 24) & 0xf], Drem[i * ld + j]);
                 // straight-line: an idle lane (x = 0) writes the idle values and adds zero
-                const bool busy = x > 0;
-                const int64_t bytes = (int64_t)x * unit;
+                const bool busy = bytes > 0;
                 const int64_t sa = ws<int64_t>(c.o_send_acc)[i] + bytes, ra = ws<int64_t>(c.o_recv_acc)[j] + bytes;
                 c.lane_dst_b[row + i] = busy ? (int16_t)j : (int16_t)-1;
                 c.lane_inst_b[row + i] = busy ? (uint16_t)(w & 0xffffu) : (uint16_t)0xFFFF;
                 c.lane_bytes_b[row + i] = bytes;
-                Drem[i * ld + j] -= x;
-                if constexpr (sizeof(V) == 4) DremT[j * N + i] -= (uint32_t)x;
-                if (busy) {                                   // Eq. (5): the volume leaves its group pair's cell of D-hat
-                    int64_t* cell = &Dhat[(i >> 2) * G + (j >> 2)];
-                    if (narrow_now) atomicSub((unsigned int*)cell, (unsigned int)x);     // high word is zero, low word >= x
-                    else atomicAdd((unsigned long long*)cell, (unsigned long long)(-(int64_t)x));
-                }
+                Drem[i * ld + j] -= bytes;
+                if (busy) atomicAdd((unsigned long long*)&Dhat[(i >> 2) * G + (j >> 2)], (unsigned long long)(-bytes));   // Eq. (5)
                 ws<int64_t>(c.o_send_acc)[i] = sa;
                 ws<int64_t>(c.o_recv_acc)[j] = ra;
                 c.send_off_b[orow + i] = sa;
@@ -370,84 +558,104 @@ __device__ __forceinline__ void decompose_warp(const DevCat& dc, const KParams& 
     }
 }
 
-#ifndef VP_WARP_MIN_BLOCKS
-#define VP_WARP_MIN_BLOCKS 4
-#endif
-__global__ void __launch_bounds__(128, VP_WARP_MIN_BLOCKS)
+// UNITS: the granule is at least 256 bytes, so the matrices run in decompose_units as a rule, whose tables are staged; the odd
+// matrix of larger capacities reads those of decompose_bytes from global memory.  Otherwise decompose_bytes and its tables.
+// `slots`: per warp three counters for vp_schedule_read_stats, given when there is a warp for every matrix: the launch then needs
+// no counter and nothing zeroed.
+template <bool UNITS>
+__global__ void __launch_bounds__(128, 3)
 vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, const int64_t* __restrict__ tau_in, int B,
                         int32_t* __restrict__ n_steps, int32_t* __restrict__ chan_id, int16_t* __restrict__ lane_dst,
                         uint16_t* __restrict__ lane_inst, int64_t* __restrict__ lane_bytes, int64_t* __restrict__ send_off,
                         int64_t* __restrict__ recv_off, int64_t* __restrict__ tau_out, int32_t* __restrict__ status,
-                        unsigned int* counter) {
+                        unsigned int* counter, unsigned long long* slots) {
     unsigned char* const smem_raw = vp_wsmem;
     const int N = dc.N, G = dc.G, tid = threadIdx.x, NT = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, n_warps = NT >> 5;
     const int ld = N + 1;
-    const WarpSmem L = warp_smem_layout(dc, kp, n_warps);
-    if (tid < 32) smem_raw[L.lut + tid] = (uint8_t)(31 - tid < 24 ? perm4_packed_rt(31 - tid) : 0);
+    const WarpSmem L = warp_smem_layout(dc, kp, n_warps, UNITS);
     // ---- stage the catalog (shared by the warps of the CTA): bulk asynchronous copies (TMA) of whole arrays onto one
-    // mbarrier; plain loads if the bounded wait gives up
+    // mbarrier; plain loads if the bounded wait gives up.  The catalog was uploaded when it was loaded: no need to wait for the
+    // kernel ahead.
     {
         const int ns_pad = (dc.n_shapes + 31) & ~31;
-        const unsigned b_term = (unsigned)(ns_pad * dc.max_terms * 4), b_slot = (unsigned)align16(dc.n_families * N * 4),
-                       b_fin = (unsigned)align16(dc.n_families * N * 2), b_fcls = (unsigned)align16(dc.n_families * N),
-                       b_bucket = (unsigned)align16((dc.n_shapes + 1) * 4);
-        const unsigned total = b_term + b_slot + b_fin + b_fcls + b_bucket;
+        const void* from[7] = {dc.bucket_ptr, dc.row_term, dc.shape_rows, dc.fam_task, dc.term_t, dc.fam_slot, dc.fam_in};
+        const int at[7] = {L.bucket, L.rows, L.shape_rows, L.fam_task, L.term, L.fam_slot, L.fam_in};
+        const int bytes[7] = {align16((dc.n_shapes + 1) * 4), dc.row_term ? 32 * 16 : 0, dc.row_term ? ns_pad * 4 : 0, UNITS ? dc.n_families * G * 32 : 0,
+                              UNITS ? 0 : ns_pad * dc.max_terms * 4, UNITS ? 0 : align16(dc.n_families * N * 4), UNITS ? 0 : align16(dc.n_families * N * 2)};
+        const int b_cls = UNITS ? 0 : align16(dc.n_families * N);
         __shared__ __align__(8) unsigned long long s_stage_bar;
-        bool landed = false;
-        if (total < (1u << 20)) {
-            const unsigned bar = smem_u32(&s_stage_bar);
-            if (tid == 0) {
-                mbar_init(bar, 1);
-                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-                mbar_expect_tx(bar, total);
-                bulk_load(smem_u32(smem_raw + L.term), dc.term_t, b_term, bar);
-                bulk_load(smem_u32(smem_raw + L.fam_slot), dc.fam_slot, b_slot, bar);
-                bulk_load(smem_u32(smem_raw + L.fam_in), dc.fam_in, b_fin, bar);
-                bulk_load(smem_u32(smem_raw + L.fam_cls), dc.fam_cls, b_fcls, bar);
-                bulk_load(smem_u32(smem_raw + L.bucket), dc.bucket_ptr, b_bucket, bar);
-            }
-            __syncthreads();
-            landed = __syncthreads_and(mbar_wait_bounded(bar, 0, 1u << 20)) != 0;
+        const unsigned bar = smem_u32(&s_stage_bar);
+        if (tid == 0) {
+            mbar_init(bar, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            unsigned total = (unsigned)b_cls;
+#pragma unroll
+            for (int i = 0; i < 7; i++) total += (unsigned)bytes[i];
+            mbar_expect_tx(bar, total);
+#pragma unroll
+            for (int i = 0; i < 7; i++)
+                if (bytes[i]) bulk_load(smem_u32(smem_raw + at[i]), from[i], (unsigned)bytes[i], bar);
+            if (b_cls) bulk_load(smem_u32(smem_raw + L.fam_cls), dc.fam_cls, (unsigned)b_cls, bar);
         }
-        if (!landed) {
-            uint32_t* t_term = (uint32_t*)(smem_raw + L.term);
-            for (int e = tid; e < ns_pad * dc.max_terms; e += NT) t_term[e] = dc.term_t[e];
-            uint32_t* t_slot = (uint32_t*)(smem_raw + L.fam_slot);
-            uint16_t* t_in = (uint16_t*)(smem_raw + L.fam_in);
-            uint8_t* t_cls = smem_raw + L.fam_cls;
-            for (int e = tid; e < dc.n_families * N; e += NT) {
-                t_slot[e] = dc.fam_slot[e]; t_in[e] = dc.fam_in[e]; t_cls[e] = dc.fam_cls[e];
-            }
-            uint32_t* t_bp = (uint32_t*)(smem_raw + L.bucket);
-            for (int e = tid; e <= dc.n_shapes; e += NT) t_bp[e] = dc.bucket_ptr[e];
+        __syncthreads();
+        if (!__syncthreads_and(mbar_wait_bounded(bar, 0, 1u << 20))) {
+#pragma unroll
+            for (int i = 0; i < 7; i++)
+                for (int e = tid; e < bytes[i] / 4; e += NT) ((uint32_t*)(smem_raw + at[i]))[e] = ((const uint32_t*)from[i])[e];
+            for (int e = tid; e < b_cls / 4; e += NT) ((uint32_t*)(smem_raw + L.fam_cls))[e] = ((const uint32_t*)dc.fam_cls)[e];
         }
     }
+    // quantum rule: the cells that cross this lane's resource (at most sixteen cells and resources), as a mask
+    uint32_t forced = 0, forced_bw = 0;
+    if (lane < dc.n_res) {
+        forced_bw = dc.forced_bw[lane];
+        if (forced_bw)
+            for (uint32_t e = dc.forced_ptr[lane]; e < dc.forced_ptr[lane + 1]; e++) forced |= 1u << dc.forced_cell[e];
+    }
+    const bool masks = dc.n_res <= 32;                     // (else the lists are read for every matrix)
     __syncthreads();
+    grid_wait();
     WCtx c;
     c.N = N; c.G = G; c.lane = lane;
     const unsigned base = (unsigned)warp * (unsigned)L.per_warp;
     c.o_drem = base + L.drem; c.o_dremT = base + L.dremT; c.o_dhat = base + L.dhat; c.o_send_acc = base + L.send_acc; c.o_recv_acc = base + L.recv_acc;
-    c.o_cred = base + L.cred; c.o_tscale = base + L.tscale; c.o_bind_src = base + L.bind_src; c.o_bind_dst = base + L.bind_dst;
-    c.o_cap = base + L.cap64;
-    c.o_term = L.term; c.o_fam_slot = L.fam_slot; c.o_fam_in = L.fam_in; c.o_fam_cls = L.fam_cls; c.o_bucket = L.bucket;
-    c.o_lut = L.lut;
+    c.o_rs = base + L.rs; c.o_cap64 = base + L.cap64; c.o_cap32 = base + L.cap32; c.o_tscale = base + L.tscale;
+    c.o_bind = base + L.bind; c.o_bind_dst = base + L.bind_dst;
+    c.o_rows = L.rows; c.o_shape_rows = L.shape_rows; c.o_fam_task = L.fam_task; c.o_bucket = L.bucket;
+    c.term = UNITS ? dc.term_t : ws<const uint32_t>(L.term);
+    c.fam_slot = UNITS ? dc.fam_slot : ws<const uint32_t>(L.fam_slot);
+    c.fam_in = UNITS ? dc.fam_in : ws<const uint16_t>(L.fam_in);
+    c.fam_cls = UNITS ? dc.fam_cls : ws<const uint8_t>(L.fam_cls);
     int64_t* const Drem = ws<int64_t>(c.o_drem);
+    uint32_t* const D32 = ws<uint32_t>(c.o_drem);
+    uint32_t* const DT32 = ws<uint32_t>(c.o_dremT);
     int64_t* const Dhat = ws<int64_t>(c.o_dhat);
     int64_t* const send_acc = ws<int64_t>(c.o_send_acc);
     int64_t* const recv_acc = ws<int64_t>(c.o_recv_acc);
-    int64_t* const cap64 = ws<int64_t>(base + L.cap64);
+    int64_t* const cap64 = ws<int64_t>(c.o_cap64);
     int64_t* const tscale = ws<int64_t>(c.o_tscale);
-    uint32_t* const cap32 = ws<uint32_t>(base + L.cap32);
+    uint32_t* const cap32 = ws<uint32_t>(c.o_cap32);
+    const RowDiv granule{kp.granule, 1.0 / (double)kp.granule}, bw_max{dc.bw_max, 1.0 / (double)dc.bw_max};
+    auto ceil_div = [](int64_t x, const RowDiv& by) {      // x below 2^52
+        int64_t rem;
+        const int64_t q = by.div(x, rem);
+        return q + (rem > 0);
+    };
+    const unsigned inv_n = 65536u / (unsigned)N + 1u;      // e / N for e < 256
     unsigned long long n_act = 0;
     Counters cnt;
     cnt.tasks = 0; cnt.sweeps = 0; cnt.t_mark = 0;
     for (int i = 0; i < 6; i++) cnt.cyc[i] = 0;
 
-    for (;;) {
-        int b = 0;
-        if (lane == 0) b = (int)atomicAdd(counter, 1u);
-        b = __shfl_sync(0xffffffffu, b, 0);
+    for (int round = 0; ; round++) {
+        int b = (int)blockIdx.x * n_warps + warp;
+        if (slots) {
+            if (round) break;
+        } else {
+            if (lane == 0) b = (int)atomicAdd(counter, 1u);
+            b = __shfl_sync(0xffffffffu, b, 0);
+        }
         if (b >= B) break;
         const int64_t* D = demand + (size_t)b * N * N;
         const size_t lane_base = (size_t)b * kp.k_max * N, off_base = (size_t)b * (kp.k_max + 1) * N;
@@ -458,19 +666,32 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
         c.send_off_b = send_off + off_base;
         c.recv_off_b = recv_off ? recv_off + off_base : nullptr;
 
-        // ---- validate, copy D into D_rem
+        // ---- validate; D in granules and its transpose
         int flags = 0;
-        for (int e = lane; e < N * N; e += 32) {
-            const int64_t v = D[e];
-            if (v < 0) flags |= VP_ST_NEGATIVE;
-            else if (v >= VP_ENTRY_LIMIT) flags |= VP_ST_OVERFLOW_RISK;
-            else {
-                if (e / N == e % N && v != 0) flags |= VP_ST_DIAG_NONZERO;
-                if (v % kp.granule) flags |= VP_ST_NOT_GRANULE;
-            }
-            Drem[(e / N) * ld + e % N] = v;
-        }
+        int64_t v[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) v[u] = lane + 32 * u < N * N ? D[lane + 32 * u] : 0;
         const int64_t tau_given = tau_in ? tau_in[b] : 0;
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int e = lane + 32 * u;
+            if (e >= N * N) continue;
+            const int i = (int)(((unsigned)e * inv_n) >> 16), j = e - i * N;
+            int64_t q = 0, rem = 0;
+            if (v[u] < 0) flags |= VP_ST_NEGATIVE;
+            else if (v[u] >= VP_ENTRY_LIMIT) flags |= VP_ST_OVERFLOW_RISK;
+            else {
+                q = granule.div(v[u], rem);
+                if (i == j && v[u] != 0) flags |= VP_ST_DIAG_NONZERO;
+                if (rem) flags |= VP_ST_NOT_GRANULE;
+            }
+            if (UNITS) {
+                D32[e] = (uint32_t)q;
+                DT32[j * N + i] = (uint32_t)q;
+            } else {
+                Drem[i * ld + j] = v[u];
+            }
+        }
         if (tau_given < 0 || tau_given > VP_ENTRY_LIMIT) flags |= VP_ST_BAD_TAU;
         flags = (int)__reduce_or_sync(0xffffffffu, (unsigned)flags);
         for (int i = lane; i < N; i += 32) {
@@ -485,82 +706,123 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
         cnt.t_mark = clock64();
 #endif
         if (st == 0) {
-            // ---- row / column sums, group sums (Eq. 5), quantum (Section 5)
+            // ---- row sums (lanes 0..), column sums (lanes 16..), group sums (Eq. 5), quantum (Section 5), all in bytes
             int64_t est = 0, tot = 0;
-            for (int i = lane; i < N; i += 32) {
-                int64_t row = 0, col = 0;
-                for (int jj = 0; jj < N; jj++) {
-                    int j = jj + i; if (j >= N) j -= N;
-                    row += Drem[i * ld + j];
-                    col += Drem[j * ld + i];
-                }
-                tot += row;
-                est = max_v(est, max_v(ceil_div_i64(row, dc.bw_max), ceil_div_i64(col, dc.bw_max)));
-            }
-            for (int cell = lane; cell < G * G; cell += 32) {
-                const int ga = cell / G, gd = cell % G;
+            if ((lane & 15) < N) {
+                const int i = lane & 15;
                 int64_t s = 0;
+                if (UNITS) {
+                    const uint4* const x = (const uint4*)((lane < 16 ? D32 : DT32) + i * N);
+                    for (int m = 0; m < N / 4; m++) {
+                        const uint4 w = x[m];
+                        s += (int64_t)w.x + w.y + ((int64_t)w.z + w.w);
+                    }
+                    s *= kp.granule;
+                } else {
+                    for (int m = 0; m < N; m++) s += lane < 16 ? Drem[i * ld + m] : Drem[m * ld + i];
+                }
+                est = ceil_div(s, bw_max);
+                if (lane < 16) tot = s;
+            }
+            if (lane < G * G) {
+                const int ga = lane / G, gd = lane - ga * G;
+                int64_t s = 0;
+                if (UNITS) {
 #pragma unroll
-                for (int i = 0; i < 4; i++)
+                    for (int i = 0; i < 4; i++) {
+                        const uint4 w = *(const uint4*)(D32 + (ga * 4 + i) * N + gd * 4);
+                        s += (int64_t)w.x + w.y + ((int64_t)w.z + w.w);
+                    }
+                } else {
 #pragma unroll
-                    for (int j = 0; j < 4; j++) s += Drem[(ga * 4 + i) * ld + gd * 4 + j];
-                Dhat[cell] = s;
+                    for (int i = 0; i < 4; i++)
+#pragma unroll
+                        for (int j = 0; j < 4; j++) s += Drem[(ga * 4 + i) * ld + gd * 4 + j];
+                }
+                Dhat[lane] = s;                              // (granules or bytes, as the matrix is held)
             }
             __syncwarp();
-            for (int l = lane; l < dc.n_res; l += 32) {
-                const uint32_t bwl = dc.forced_bw[l];
-                if (!bwl) continue;
-                int64_t f = 0;
-                for (uint32_t e = dc.forced_ptr[l]; e < dc.forced_ptr[l + 1]; e++) f += Dhat[dc.forced_cell[e]];
-                est = max_v(est, ceil_div_i64(f, (int64_t)bwl));
+            const int64_t unit = UNITS ? kp.granule : 1;
+            if (masks) {
+                if (forced) {
+                    int64_t f = 0;
+                    for (uint32_t m = forced; m; m &= m - 1) f += Dhat[__ffs((int)m) - 1];
+                    est = max_v(est, ceil_div(f * unit, RowDiv{(int64_t)forced_bw, 1.0 / (double)forced_bw}));
+                }
+            } else {
+                for (int l = lane; l < dc.n_res; l += 32) {
+                    const uint32_t bwl = dc.forced_bw[l];
+                    if (!bwl) continue;
+                    int64_t f = 0;
+                    for (uint32_t e = dc.forced_ptr[l]; e < dc.forced_ptr[l + 1]; e++) f += Dhat[dc.forced_cell[e]];
+                    est = max_v(est, ceil_div(f * unit, RowDiv{(int64_t)bwl, 1.0 / (double)bwl}));
+                }
             }
-            est = warp_max_i64(est);
+            est = (int64_t)big_warp_max64((uint64_t)est);
             tot = warp_sum_i64(tot);
-            const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div_i64(est, (int64_t)kp.k_target));
-            int64_t cap_max = 0;
-            for (int cl = 0; cl < dc.n_classes; cl++) {
-                int64_t cp = (tq * dc.class_bw[cl]) / kp.granule * kp.granule;
-                cp = cp < kp.granule ? kp.granule : cp;
-                cap_max = max_v(cap_max, cp);
-                if (lane == 0) cap64[cl] = cp;
-            }
-            // granule units: capacities below 2^22 granules (four credits and a permutation byte share 32 bits)
-            const bool units = cap_max / kp.granule < ((int64_t)1 << 22) && kp.granule >= 256;
-            __syncwarp();
+            const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div(est, RowDiv{(int64_t)kp.k_target, 1.0 / (double)kp.k_target}));
+            // capacities in granules, at least one (rate x quantum may exceed what the reciprocal divides exactly)
+            int64_t cap_gr = 0;
             if (lane < dc.n_classes) {
-                cap32[lane] = (uint32_t)(units ? cap64[lane] / kp.granule : 0);
+                const int64_t x = tq * dc.class_bw[lane];
+                int64_t rem;
+                cap_gr = x < ((int64_t)1 << 52) ? granule.div(x, rem) : x / kp.granule;
+                cap_gr = max_v(cap_gr, (int64_t)1);
+            }
+            // 32-bit granules: capacities below 2^22 granules (four credits and a permutation byte share 32 bits)
+            const bool units = UNITS && !__any_sync(0xffffffffu, cap_gr >= ((int64_t)1 << 22));
+            if (lane < dc.n_classes) {
+                cap64[lane] = cap_gr * kp.granule;
+                cap32[lane] = (uint32_t)cap_gr;
                 tscale[lane] = dc.class_wdiv[lane] * (units ? kp.granule : 1);
             }
             tau = tq;
             __syncwarp();
             if (units) {
-                // the byte copy is no longer needed: overwrite it with the demand in granules
-                uint32_t* Drem32 = (uint32_t*)Drem;
-                uint32_t* DremT32 = ws<uint32_t>(c.o_dremT);
-                for (int e = lane; e < N * N; e += 32) {                                            // (row stride N, and the transpose)
-                    const uint32_t v = (uint32_t)(D[e] / kp.granule);
-                    const int i = e / N, j = e - i * N;
-                    Drem32[e] = v;
-                    DremT32[j * N + i] = v;
-                }
-                for (int cell = lane; cell < G * G; cell += 32) Dhat[cell] /= kp.granule;
-                __syncwarp();
-                c.o_cap = base + L.cap32;
-                decompose_warp<uint32_t>(dc, kp, c, kp.granule, tot / kp.granule, k, st, cnt);
+                int64_t rem;
+                decompose_units(dc, kp, c, granule.div(tot, rem), k, st, cnt);
             } else {
-                c.o_cap = base + L.cap64;
-                decompose_warp<int64_t>(dc, kp, c, 1, tot, k, st, cnt);
+                if (UNITS) {                                 // (back to bytes)
+                    for (int e = lane; e < N * N; e += 32) {
+                        const int i = (int)(((unsigned)e * inv_n) >> 16);
+                        Drem[i * ld + e - i * N] = D[e];
+                    }
+                    for (int cell = lane; cell < G * G; cell += 32) Dhat[cell] *= kp.granule;
+                    __syncwarp();
+                }
+                decompose_bytes(dc, kp, c, tot, k, st, cnt);
             }
         }
         __syncwarp();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
-        for (size_t e = (size_t)k * N + lane; e < (size_t)kp.k_max * N; e += 32) {
-            c.lane_dst_b[e] = -1;
-            c.lane_inst_b[e] = 0xFFFF;
-            c.lane_bytes_b[e] = 0;
-            const int i = (int)(e % N);
-            c.send_off_b[N + e] = send_acc[i];
-            if (c.recv_off_b) c.recv_off_b[N + e] = recv_acc[i];
+        const size_t rows = (size_t)(kp.k_max - k) * N;      // elements per array
+        if ((((uintptr_t)c.lane_dst_b | (uintptr_t)c.lane_inst_b | (uintptr_t)c.lane_bytes_b | (uintptr_t)c.send_off_b |
+              (uintptr_t)(c.recv_off_b ? c.recv_off_b : c.send_off_b)) & 15) == 0 && (32 % N) == 0 && N >= 8) {
+            // whole rows of 2 N bytes and 8 N bytes in 16-byte vectors (N = 8 or 16: a warp's stride keeps a lane's ranks)
+            const uint4 ones = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+            uint4* const ld4 = (uint4*)(c.lane_dst_b + (size_t)k * N);
+            uint4* const li4 = (uint4*)(c.lane_inst_b + (size_t)k * N);
+            for (size_t e = lane; e < rows / 8; e += 32) { ld4[e] = ones; li4[e] = ones; }
+            const int i2 = (2 * lane) & (N - 1);
+            const longlong2 sa = *(const longlong2*)(send_acc + i2), ra = *(const longlong2*)(recv_acc + i2);
+            longlong2* const lb2 = (longlong2*)(c.lane_bytes_b + (size_t)k * N);
+            longlong2* const so2 = (longlong2*)(c.send_off_b + (size_t)(k + 1) * N);
+            longlong2* const ro2 = c.recv_off_b ? (longlong2*)(c.recv_off_b + (size_t)(k + 1) * N) : nullptr;
+#pragma unroll 4
+            for (size_t e = lane; e < rows / 2; e += 32) {
+                lb2[e] = make_longlong2(0, 0);
+                so2[e] = sa;
+                if (ro2) ro2[e] = ra;
+            }
+        } else {
+            for (size_t e = (size_t)k * N + lane; e < (size_t)kp.k_max * N; e += 32) {
+                c.lane_dst_b[e] = -1;
+                c.lane_inst_b[e] = 0xFFFF;
+                c.lane_bytes_b[e] = 0;
+                const int i = (int)(e % N);
+                c.send_off_b[N + e] = send_acc[i];
+                if (c.recv_off_b) c.recv_off_b[N + e] = recv_acc[i];
+            }
         }
         for (int kk = k + lane; kk < kp.k_max; kk += 32) c.chan_id_b[kk] = -1;
         if (lane == 0) {
@@ -571,14 +833,20 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
         }
         __syncwarp();
     }
-    unsigned long long* stats = (unsigned long long*)(counter + 4);
-    cnt.tasks = (unsigned long long)warp_sum_i64((int64_t)cnt.tasks);      // (counted by the first lane of every team)
+    cnt.tasks = (unsigned long long)warp_sum_i64((int64_t)cnt.tasks);      // (counted by one lane, or the first lane of every team)
     cnt.sweeps = (unsigned long long)warp_sum_i64((int64_t)cnt.sweeps);
     if (lane == 0) {
-        if (n_act) atomicAdd(&stats[0], n_act);
-        if (cnt.tasks) { atomicAdd(&stats[1], cnt.tasks); atomicAdd(&stats[2], cnt.sweeps); }
+        if (slots) {
+            unsigned long long* const mine = slots + 3 * ((size_t)blockIdx.x * n_warps + warp);
+            mine[0] = n_act; mine[1] = cnt.tasks; mine[2] = cnt.sweeps;
+            if (blockIdx.x == 0 && warp == 0) counter[3] = gridDim.x * (unsigned)n_warps;
+        } else {
+            unsigned long long* const stats = (unsigned long long*)(counter + 4);
+            if (n_act) atomicAdd(&stats[0], n_act);
+            if (cnt.tasks) { atomicAdd(&stats[1], cnt.tasks); atomicAdd(&stats[2], cnt.sweeps); }
+        }
 #ifdef VP_PHASE_TIMING
-        for (int i = 0; i < 6; i++) atomicAdd(&stats[3 + i], (unsigned long long)cnt.cyc[i]);
+        for (int i = 0; i < 6; i++) atomicAdd((unsigned long long*)(counter + 4) + 3 + i, (unsigned long long)cnt.cyc[i]);
 #endif
     }
 }

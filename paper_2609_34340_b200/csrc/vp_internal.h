@@ -49,10 +49,16 @@ struct DevCat {
     const uint8_t* fam_cls;
     // family f, in-slot d*g+q of destination group d: slot index (N <= 256) | rate class << 8
     const uint16_t* fam_in;
-    // groups of four, at most 64 of them, node-symmetric: family f, group a, eight words.  Words 0..3: out-slots of a, each
+    // Row patterns of plain tables (not node-symmetric, at most four groups of four): the terms of a shape from one source group
+    // are one of at most 32 rows of at most four terms.  row_term[p * 4 + t] = D-hat cell | count << 16 (zero padded);
+    // shape_rows[s] = the patterns of the shape's four source groups, a byte each (missing groups: an empty pattern).  Null otherwise
+    const uint32_t *row_term, *shape_rows;
+    // Groups of four, at most 64 of them when node-symmetric, at most four otherwise: family f, group a, eight words.  Words 0..3: out-slots of a, each
     // (word of its cells in the credit matrix when its destination has tag 0, i.e. is row 3 of its group) | destination group << 16 |
     // rate class << 24 | shift of the destination's tag in its group's byte << 28.  Words 4..7: in-slots of a, each
     // (word of the row pair of its source when that has tag 0) | source group << 16 | class << 24 | shift of the source's tag << 28
+    // The credit matrix of the plain case is two N x N arrays of 32-bit cells: column j of a group's rows at word j * N + 4 * group of
+    // the transposed one, row i of a group's columns at word i * N + 4 * group of the other.
     const uint32_t* fam_task;
     int n_terms;
     // inverted terms, for keeping the scores up to date instead of recomputing them: the shapes that use table

@@ -1,0 +1,73 @@
+"""GPU parity of the scheduler where its kernels change form: one warp per matrix (up to four groups of four) in 32-bit granules
+and in bytes, one and two lanes per rank group, tasks of a part of a warp up to two warps, scores within and beyond 32 bits,
+other numbers of starts and sweeps than four and three, plans cut short."""
+import numpy as np
+import pytest
+
+import tests.test_gpu_schedule as ts
+from tests.test_gpu_schedule import vp  # noqa: F401  (fixture)
+from workloads import SchedParams as WParams, complete_catalog, node_template_catalog, tree_topology
+from workloads.topology import ring_topology
+
+pytestmark = pytest.mark.gpu
+
+CATALOGS = {
+    "one_node": lambda: complete_catalog(tree_topology(1)),
+    "ring_of_three": lambda: complete_catalog(ring_topology(1, switches_per_node=3, g=4)),
+    "two_nodes_64_50": lambda: complete_catalog(tree_topology(2, nic_bw=50)),
+    "template_1": lambda: node_template_catalog(tree_topology(1)),
+    "template_5_64_50": lambda: node_template_catalog(tree_topology(5, nic_bw=50)),
+    "template_8": lambda: node_template_catalog(tree_topology(8)),
+    "template_9": lambda: node_template_catalog(tree_topology(9)),
+    "template_17": lambda: node_template_catalog(tree_topology(17)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CATALOGS))
+def test_magnitudes_starts_and_sweeps(vp, oracle_lib, name):  # noqa: F811
+    cat = CATALOGS[name]()
+    N = cat.topology.N
+    rng = np.random.default_rng(len(name) + N)
+    B = 6
+    # largest entry (granules of 256 bytes): ordinary, beyond 16 bits, scores beyond 32 bits, capacities beyond 2^22 granules
+    for hi, kt, n_start, i_aa, k_max in [(900, 2 * N, 4, 3, 10 * N), (70000, N, 3, 2, 10 * N), (1 << 24, 2 * N, 4, 1, 10 * N),
+                                         ((1 << 32) - 1, 8, 4, 3, 40), (5000, N, 5, 4, N // 2), (300, 3 * N, 1, 3, 10 * N)]:
+        D = rng.integers(0, hi + 1, size=(B, N, N)) * (rng.random((B, N, N)) < (0.6 if N < 64 else 0.15)) * 256
+        D[1] = 0
+        D[2] //= 512
+        D[2] *= 256
+        D[3][:, 0] = hi * 256                                  # one popular destination
+        for b in range(B):
+            np.fill_diagonal(D[b], 0)
+        w = WParams(granule_bytes=256, k_target=kt, n_start=n_start, i_aa=i_aa, k_max=k_max).resolved(N)
+        got, want, *_ = ts._both(vp, oracle_lib, cat, D.astype(np.int64), w)
+        ts._assert_same(got, want)
+
+
+@pytest.mark.parametrize("name,batches", [("one_node", (1, 593, 1185)), ("two_nodes_64_50", (1, 593, 1185)), ("template_8", (296, 297, 593)),
+                                          ("template_5_64_50", (593, 700)), ("template_9", (149, 297))])
+def test_work_counters_and_batches(vp, oracle_lib, name, batches):  # noqa: F811
+    """Batches on both sides of the launch shapes' limits give the same plans, and the work counters add up."""
+    import torch
+    cat = CATALOGS[name]()
+    N = cat.topology.N
+    rng = np.random.default_rng(N)
+    base = (rng.integers(0, 60, size=(3, N, N)) * (rng.random((3, N, N)) < 0.5) * 4096).astype(np.int64)
+    for b in range(3):
+        np.fill_diagonal(base[b], 0)
+    w = WParams(granule_bytes=4096).resolved(N)
+    oc = oracle_lib.OracleCatalog(cat.topology.blob(), cat.blob())
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob())
+    want = oc.schedule_batch(base, w, threads=3)
+    p = ts._params(vp, w)
+    for B in batches:
+        D = torch.from_numpy(np.tile(base, ((B + 2) // 3, 1, 1))[:B].copy()).cuda()
+        ws = torch.full((vp.schedule_workspace_bytes(dc, B, p),), 0x5A, dtype=torch.uint8, device="cuda")
+        got = vp.schedule_batch(dc, p, D, workspace=ws)
+        stats = vp.schedule_read_stats(ws)
+        got = got.cpu()
+        for key in ts.KEYS:
+            for r in range(0, B, 3):
+                n = min(3, B - r)
+                assert np.array_equal(got[key][r:r + n], want[key][:n]), (B, key, r)
+        assert stats["activations"] == int(got["n_steps"].sum()) and stats["tasks"] >= 4 * stats["activations"] and stats["sweeps"] >= stats["tasks"]
