@@ -321,7 +321,9 @@ int vp_schedule_batch_host(const vp_catalog* catalog, const vp_sched_params* par
  * rows k < n_steps[b] of chan_id, lane_dst, lane_inst and lane_bytes and the rows k <= n_steps[b] of send_off / recv_off
  * (row n_steps[b] holds the totals).  Rows beyond keep whatever the host buffers held.  With k_max sized for the
  * longest plan this is a small part of the arrays (config 4: 26 GB instead of 122 GB per 4096 matrices).  Same
- * arguments, scratch and errors as vp_schedule_batch_host; it synchronises the stream once more (to read n_steps).
+ * arguments, scratch and errors as vp_schedule_batch_host.  Page-locked output buffers are written by the scheduler itself
+ * while it decomposes; into pageable ones the rows are copied afterwards, which synchronises the stream once more (to read
+ * n_steps).
  */
 int vp_schedule_batch_host_used(const vp_catalog* catalog, const vp_sched_params* params,
                                 const int64_t* demand, const int64_t* tau_ns_in, int B,

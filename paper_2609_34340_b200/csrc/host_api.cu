@@ -101,59 +101,9 @@ int copy_plan_out(const SchedBufs& s, size_t N, size_t K, size_t lo, size_t n, i
     return VP_OK;
 }
 
-// Used plan rows straight into pinned host memory.  Per matrix six copies of a few KB to a few 100 KB each are needed, of lengths
-// that only the device knows: as cudaMemcpyAsync calls they cost a wait for n_steps and 3 us of host time each (128 matrices of
-// 64 ranks: 768 calls).  One kernel of posted 16-byte writes keeps PCIe as busy as the copy engine does.
-struct UsedRows {
-    const int32_t *n_steps, *status, *chan_id;
-    const int16_t* lane_dst;
-    const uint16_t* lane_inst;
-    const int64_t *lane_bytes, *send_off, *recv_off, *tau;
-    int32_t *h_n_steps, *h_status, *h_chan_id;               // device addresses of the host buffers, from the chunk's first matrix on
-    int16_t* h_lane_dst;
-    uint16_t* h_lane_inst;
-    int64_t *h_lane_bytes, *h_send_off, *h_recv_off, *h_tau;
-    int B, N, K;
-};
-constexpr int kUsedPieces = 4;                               // CTAs' units per matrix
-
-template <typename V>
-__device__ __forceinline__ void copy_units(void* dst, const void* src, size_t lo, size_t hi) {
-    constexpr int T = 256;
-    size_t e = lo + threadIdx.x;
-    for (; e + 3 * T < hi; e += 4 * T) {                     // four loads in flight per thread
-        const V a = ((const V*)src)[e], b = ((const V*)src)[e + T], c = ((const V*)src)[e + 2 * T], d = ((const V*)src)[e + 3 * T];
-        ((V*)dst)[e] = a; ((V*)dst)[e + T] = b; ((V*)dst)[e + 2 * T] = c; ((V*)dst)[e + 3 * T] = d;
-    }
-    for (; e < hi; e += T) ((V*)dst)[e] = ((const V*)src)[e];
-}
-__device__ __forceinline__ void copy_part(void* dst, const void* src, size_t bytes, int piece) {
-    const uintptr_t mix = (uintptr_t)dst | (uintptr_t)src | bytes;
-    const size_t n = mix % 16 == 0 ? bytes / 16 : (mix % 4 == 0 ? bytes / 4 : bytes / 2);      // (every array's rows are whole 16-bit words)
-    const size_t lo = n * piece / kUsedPieces, hi = n * (piece + 1) / kUsedPieces;
-    if (mix % 16 == 0) copy_units<uint4>(dst, src, lo, hi);
-    else if (mix % 4 == 0) copy_units<uint32_t>(dst, src, lo, hi);
-    else copy_units<uint16_t>(dst, src, lo, hi);
-}
-__global__ void __launch_bounds__(256) copy_used_rows_kernel(UsedRows u) {
-    const size_t N = (size_t)u.N, K = (size_t)u.K;
-    for (int unit = blockIdx.x; unit < u.B * kUsedPieces; unit += gridDim.x) {
-        const size_t m = (size_t)(unit / kUsedPieces);
-        const int piece = unit % kUsedPieces, n = u.n_steps[m];
-        const size_t k = n < 0 ? 0 : ((size_t)n > K ? K : (size_t)n);
-        copy_part(u.h_lane_bytes + m * K * N, u.lane_bytes + m * K * N, k * N * 8, piece);
-        copy_part(u.h_send_off + m * (K + 1) * N, u.send_off + m * (K + 1) * N, (k + 1) * N * 8, piece);
-        if (u.h_recv_off) copy_part(u.h_recv_off + m * (K + 1) * N, u.recv_off + m * (K + 1) * N, (k + 1) * N * 8, piece);
-        copy_part(u.h_lane_dst + m * K * N, u.lane_dst + m * K * N, k * N * 2, piece);
-        copy_part(u.h_lane_inst + m * K * N, u.lane_inst + m * K * N, k * N * 2, piece);
-        copy_part(u.h_chan_id + m * K, u.chan_id + m * K, k * 4, piece);
-        if (piece == 0 && threadIdx.x == 0) {
-            u.h_n_steps[m] = n;
-            u.h_status[m] = u.status[m];
-            if (u.h_tau) u.h_tau[m] = u.tau[m];
-        }
-    }
-}
+// Batches of at least this many matrices are copied back in chunks, two of them in flight: while one chunk is
+// decomposed on the caller's stream, the results of the chunk before it travel to the host on a second stream.
+constexpr int kPipeMinBatch = 64;
 
 // Device address of `bytes` of page-locked host memory, or null if the device cannot write there.
 template <typename T>
@@ -186,42 +136,38 @@ int schedule_host(const vp_catalog* cc, const vp_sched_params* p, const int64_t*
     DeviceScope scope(c->device);
     if (!scope.ok) return VP_E_CUDA;
 
-    // Large batches are worked through in chunks, two of them in flight: while one chunk is decomposed on the caller's stream,
-    // the results of the chunk before it travel to the host on a second stream.  About one matrix per SM each: a chunk lasts as
-    // long as its longest matrix's chain however few it holds, so smaller batches are one chunk.  Two chunks' buffers must fit
-    // the scratch of the whole batch.
+    // Only rows in use, into page-locked buffers: the scheduler writes its rows straight into them, over PCIe while it decomposes.
+    // Copied afterwards they would be six pieces per matrix, of lengths that only the device knows: 128 matrices of 64 ranks took
+    // 6.1 ms with cudaMemcpyAsync calls in chunks, 2.3 with a copy kernel behind the scheduler, 1.7 so (69 MB, 1.3 ms of PCIe).
+    if (used_only) {
+        const size_t b = (size_t)B;
+        int32_t *h_steps = pinned_address(n_steps, b * 4), *h_status = pinned_address(status, b * 4), *h_chan = pinned_address(chan_id, b * K * 4);
+        int16_t* h_dst = pinned_address(lane_dst, b * K * N * 2);
+        uint16_t* h_inst = pinned_address(lane_inst, b * K * N * 2);
+        int64_t *h_bytes = pinned_address(lane_bytes, b * K * N * 8), *h_send = pinned_address(send_off, b * (K + 1) * N * 8);
+        int64_t *h_recv = pinned_address(recv_off, b * (K + 1) * N * 8), *h_tau = pinned_address(tau_ns_out, b * 8);
+        if (h_steps && h_status && h_chan && h_dst && h_inst && h_bytes && h_send && (h_recv || !recv_off) && (h_tau || !tau_ns_out)) {
+            const SchedBufs s = carve_sched(device_scratch, c, B, p);
+            VP_COPY(s.demand, demand, b * N * N * 8, cudaMemcpyHostToDevice);
+            if (tau_ns_in) VP_COPY(s.tau_in, tau_ns_in, b * 8, cudaMemcpyHostToDevice);
+            const int rc = vp_schedule_launch(c, p, s.demand, tau_ns_in ? s.tau_in : nullptr, B, h_steps, h_chan, h_dst, h_inst, h_bytes,
+                                              h_send, h_recv, h_tau, h_status, s.ws, s.ws_bytes, cuda_stream, true);
+            if (rc) return rc;
+            return cudaStreamSynchronize(stream) == cudaSuccess ? VP_OK : VP_E_CUDA;
+        }
+    }
+    // chunks: about one matrix per SM each, at least three, and two chunks' buffers must fit the scratch of the whole batch
     int n_chunks = 1, chunk = B;
-    if (c->sm_count > 0 && B >= 2 * c->sm_count) {
-        n_chunks = B / c->sm_count;
+    if (B >= kPipeMinBatch) {
+        n_chunks = B / (c->sm_count > 0 ? c->sm_count : 128);
+        if (n_chunks < 3) n_chunks = 3;
         chunk = (B + n_chunks - 1) / n_chunks;
         n_chunks = (B + chunk - 1) / chunk;
         const SchedBufs one = carve_sched(nullptr, c, chunk, p);
         if (!one.ws_bytes || 2 * one.total > device_scratch_bytes) { n_chunks = 1; chunk = B; }
     }
-    // Used rows by a kernel where every host buffer is page-locked.  From 128 ranks on a matrix's rows are MBs: the copy engine
-    // then needs few enough calls, and no SM has to have room beside the scheduler's CTAs.
-    UsedRows host;
-    bool by_kernel = false;
-    if (used_only && N < 128) {
-        const size_t b = (size_t)B;
-        host.h_n_steps = pinned_address(n_steps, b * 4);
-        host.h_status = pinned_address(status, b * 4);
-        host.h_chan_id = pinned_address(chan_id, b * K * 4);
-        host.h_lane_dst = pinned_address(lane_dst, b * K * N * 2);
-        host.h_lane_inst = pinned_address(lane_inst, b * K * N * 2);
-        host.h_lane_bytes = pinned_address(lane_bytes, b * K * N * 8);
-        host.h_send_off = pinned_address(send_off, b * (K + 1) * N * 8);
-        host.h_recv_off = pinned_address(recv_off, b * (K + 1) * N * 8);
-        host.h_tau = pinned_address(tau_ns_out, b * 8);
-        by_kernel = host.h_n_steps && host.h_status && host.h_chan_id && host.h_lane_dst && host.h_lane_inst && host.h_lane_bytes &&
-                    host.h_send_off && (host.h_recv_off || !recv_off) && (host.h_tau || !tau_ns_out);
-    }
     if (n_chunks > 1 && !c->host_pipe_ready) {
-        // (highest priority: the copy kernel's CTAs go ahead of the next chunk's)
-        int least = 0, greatest = 0;
-        if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&c->copy_stream, cudaStreamNonBlocking, greatest) != cudaSuccess)
-            return VP_E_CUDA;
+        if (cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking) != cudaSuccess) return VP_E_CUDA;
         for (cudaEvent_t& e : c->host_ev)
             if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return VP_E_CUDA;
         c->host_pipe_ready = 1;
@@ -253,19 +199,7 @@ int schedule_host(const vp_catalog* cc, const vp_sched_params* p, const int64_t*
             const SchedBufs& s = slot[j & 1];
             const size_t lo = (size_t)j * chunk, n = (size_t)(B - (int)lo < chunk ? B - (int)lo : chunk);
             if (n_chunks > 1 && cudaStreamWaitEvent(copy, done[j & 1], 0) != cudaSuccess) return VP_E_CUDA;
-            if (by_kernel) {
-                UsedRows u = host;
-                u.n_steps = s.n_steps; u.status = s.status; u.chan_id = s.chan_id; u.lane_dst = s.lane_dst; u.lane_inst = s.lane_inst;
-                u.lane_bytes = s.lane_bytes; u.send_off = s.send_off; u.recv_off = s.recv_off; u.tau = s.tau_out;
-                u.h_n_steps += lo; u.h_status += lo; u.h_chan_id += lo * K; u.h_lane_dst += lo * K * N; u.h_lane_inst += lo * K * N;
-                u.h_lane_bytes += lo * K * N; u.h_send_off += lo * (K + 1) * N;
-                if (u.h_recv_off) u.h_recv_off += lo * (K + 1) * N;
-                if (u.h_tau) u.h_tau += lo;
-                u.B = (int)n; u.N = (int)N; u.K = (int)K;
-                copy_used_rows_kernel<<<(int)(n * kUsedPieces < 256 ? n * kUsedPieces : 256), 256, 0, copy>>>(u);
-                g_vp_launches++;
-                if (cudaGetLastError() != cudaSuccess) return VP_E_CUDA;
-            } else {
+            {
                 cudaStream_t stream = copy;  // (VP_COPY issues on `stream`)
                 VP_COPY(n_steps + lo, s.n_steps, n * 4, cudaMemcpyDeviceToHost);
                 if (tau_ns_out) VP_COPY(tau_ns_out + lo, s.tau_out, n * 8, cudaMemcpyDeviceToHost);

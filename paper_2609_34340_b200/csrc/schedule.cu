@@ -46,6 +46,7 @@ struct KParams {
     int k_target, n_start, i_aa, k_max;
     int max_tasks, stage_terms, stage_fam, stage_bucket, drem_in_smem;
     int big_stage, big_cross, big_task_warps, big_emit_warp;    // vp_schedule_big_kernel: task tables in shared memory, a task is two warps, task warps, first emitting warp
+    int host_rows;            // the plan arrays are page-locked host memory: only rows in use are written
     int incremental;          // keep the shape scores in shared memory and update them after every activation
 };
 
@@ -1105,7 +1106,7 @@ vp_schedule_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, co
         }
         __syncthreads();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
-        for (size_t e = (size_t)k * N + tid; e < (size_t)kp.k_max * N; e += NT) {
+        for (size_t e = (size_t)k * N + tid; e < (size_t)kp.k_max * N && !kp.host_rows; e += NT) {
             c.lane_dst_b[e] = -1;
             c.lane_inst_b[e] = 0xFFFF;
             c.lane_bytes_b[e] = 0;
@@ -1113,7 +1114,7 @@ vp_schedule_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, co
             c.send_off_b[N + e] = c.send_acc[i];
             if (c.recv_off_b) c.recv_off_b[N + e] = c.recv_acc[i];
         }
-        for (int kk = k + tid; kk < kp.k_max; kk += NT) c.chan_id_b[kk] = -1;
+        for (int kk = k + tid; kk < kp.k_max && !kp.host_rows; kk += NT) c.chan_id_b[kk] = -1;
         if (tid == 0) {
             n_act += (unsigned long long)k;
             n_steps[b] = k;
@@ -1376,11 +1377,11 @@ extern "C" size_t vp_schedule_workspace_bytes(const vp_catalog* c, int B, const 
     return rc == VP_OK ? workspace_bytes(c, L, B) : 0;
 }
 
-extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, const int64_t* demand,
-                                 const int64_t* tau_ns_in, int B, int32_t* n_steps, int32_t* chan_id,
-                                 int16_t* lane_dst, uint16_t* lane_inst, int64_t* lane_bytes, int64_t* send_off,
-                                 int64_t* recv_off, int64_t* tau_ns_out, int32_t* status, void* workspace,
-                                 size_t workspace_bytes_given, void* cuda_stream) {
+int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int64_t* demand,
+                       const int64_t* tau_ns_in, int B, int32_t* n_steps, int32_t* chan_id,
+                       int16_t* lane_dst, uint16_t* lane_inst, int64_t* lane_bytes, int64_t* send_off,
+                       int64_t* recv_off, int64_t* tau_ns_out, int32_t* status, void* workspace,
+                       size_t workspace_bytes_given, void* cuda_stream, bool host_rows) {
     if (!c || !p) return VP_E_BAD_ARG;
     if (B <= 0 || !demand || !n_steps || !chan_id || !lane_dst || !lane_inst || !lane_bytes || !send_off || !status)
         return VP_E_BAD_ARG;
@@ -1389,6 +1390,7 @@ extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, 
     if (prev != c->device && cudaSetDevice(c->device) != cudaSuccess) return VP_E_CUDA;
     Launch L;
     int rc = plan_launch(c, B, p, &L);
+    L.kp.host_rows = host_rows;
     if (!rc && (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes_given < workspace_bytes(c, L, B))) rc = VP_E_WORKSPACE;
     if (!rc) {
         cudaStream_t stream = (cudaStream_t)cuda_stream;
@@ -1439,6 +1441,15 @@ extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, 
     }
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return rc;
+}
+
+extern "C" int vp_schedule_batch(const vp_catalog* c, const vp_sched_params* p, const int64_t* demand,
+                                 const int64_t* tau_ns_in, int B, int32_t* n_steps, int32_t* chan_id,
+                                 int16_t* lane_dst, uint16_t* lane_inst, int64_t* lane_bytes, int64_t* send_off,
+                                 int64_t* recv_off, int64_t* tau_ns_out, int32_t* status, void* workspace,
+                                 size_t workspace_bytes_given, void* cuda_stream) {
+    return vp_schedule_launch(c, p, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
+                              tau_ns_out, status, workspace, workspace_bytes_given, cuda_stream, false);
 }
 
 extern "C" int vp_schedule_launch_info(const vp_catalog* c, int B, const vp_sched_params* p, int32_t* out4) {

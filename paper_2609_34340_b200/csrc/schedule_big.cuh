@@ -321,7 +321,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     const bool one_class = dc.n_classes == 1;
     const int n_task_warps = kp.big_task_warps, emit_warp = kp.big_emit_warp;
     const int r_emit = tid - emit_warp * 32;              // this thread's slot when it emits
-    const bool emits = r_emit >= 0 && r_emit < N;
+    const int emit_threads = (N + 31) & ~31;              // whole warps
+    const bool emits = r_emit >= 0 && r_emit < N, emit_warps = r_emit >= 0 && r_emit < emit_threads;
     // this thread's place in Step 2: task group (warp, or pair of warps), lane of the task, rank group and columns
     const int wg = CROSS ? warp >> 1 : warp, sub = CROSS ? warp & 1 : 0, n_tg = CROSS ? n_task_warps >> 1 : n_task_warps;
     const int tl = CROSS ? sub * 32 + lane : lane & (WL - 1), tsub = CROSS ? 0 : lane / WL, a = tl / SPLIT, part = tl - a * SPLIT;
@@ -483,7 +484,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         }
         // Idle rows are filled from the end of the plan towards the activations while the matrix is decomposed (fill_warp,
         // a block of 4 fill_rows rows per iteration): fill_lo is the first row already filled.
-        const bool fills = L.fill_rows > 0 && st == 0 &&
+        const bool fills = L.fill_rows > 0 && st == 0 && !kp.host_rows &&
             (((uintptr_t)lane_dst_b | (uintptr_t)lane_inst_b | (uintptr_t)lane_bytes_b | (uintptr_t)send_off_b |
               (uintptr_t)(recv_off_b ? recv_off_b : send_off_b)) & 15) == 0;
         const unsigned chunk = (unsigned)(L.fill_rows * N * 8);
@@ -578,7 +579,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 lane_dst_b[row + i] = x ? (int16_t)j : (int16_t)-1;
                 lane_bytes_b[row + i] = bytes;
                 send_off_b[orow + i] = sa;
-                if (recv_off_b) recv_off_b[orow + j] = ra;
+                if (recv_off_b && !kp.host_rows) recv_off_b[orow + j] = ra;
                 lane_inst_b[row + i] = x ? (uint16_t)inst : (uint16_t)0xFFFF;
                 if (r == 0) chan_id_b[kk] = fam;
             };
@@ -588,8 +589,15 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     for (int r = tid - n_task_warps * 32; r < N; r += NT - n_task_warps * 32)
                         write_slot(kk, r, fam, record[r].x, record[r].y, __ldg(dc.fam_slot + (size_t)fam * N + r));
                 } else {
-                    if (emit_warp > 0) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
-                    write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
+                    if (emit_warp > 0 && emits) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
+                    if (emits) write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
+                }
+                if (kp.host_rows && recv_off_b) {             // (in rank order: whole lines for PCIe)
+                    // (every lane of the writing warps comes here once per activation: pend is the same in a warp)
+                    const int first = RECORD ? n_task_warps * 32 : emit_warp * 32, threads = RECORD ? NT - first : emit_threads;
+                    asm volatile("bar.sync 9, %0;" ::"r"(threads) : "memory");
+                    for (int r = tid - first; r < N; r += threads) recv_off_b[(size_t)(kk + 1) * N + r] = recv_acc[r];
+                    asm volatile("bar.sync 9, %0;" ::"r"(threads) : "memory");
                 }
                 pend = false;
             };
@@ -599,7 +607,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 if (left == 0) break;
                 if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
                 // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
-                const uint32_t inst = !RECORD && emit_warp == 0 && pend ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
+                const uint32_t inst = !RECORD && emit_warp == 0 && pend && emits ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
                 // (A) Eq. (6).  A score is at most four times what is left, so below 2^34, and there are fewer than 2^16
                 // shapes: key = score << 16 | (65535 - shape) orders by score first and lower shape index second, and the first
                 // maximum of Eq. (6) is a plain maximum of keys.
@@ -992,20 +1000,20 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         if (r_emit == 0) record[N] = make_uint2((uint32_t)p_fam, 0u);
                     }
                 }
-                pend = RECORD ? warp >= n_task_warps : emits;     // plan rows and offset sums follow (write_row)
+                pend = RECORD ? warp >= n_task_warps : emit_warps;   // plan rows and offset sums follow (write_row)
                 left -= wF;
                 k++;
                 __syncthreads();
                 VP_TICK(4);
             }
-            if (pend) write_row(k - 1, RECORD ? 0u : __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit));   // the last activation of the matrix
+            if (pend) write_row(k - 1, RECORD || !emits ? 0u : __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit));   // the last activation of the matrix
         }
         __syncthreads();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
         if (fills && st == 0) {
             if (warp == fill_warp)                               // (the copies go on while the next matrix is decomposed)
                 for (int hi = fill_lo; hi > k; hi -= 4 * L.fill_rows) fill_block(max(hi - 4 * L.fill_rows, k), hi);
-        } else {
+        } else if (!kp.host_rows) {
             if (fills && warp == fill_warp) {                    // incomplete plan: the totals are not the demand's, fill again
                 bulk_wait_all();
                 asm volatile("fence.proxy.async;" ::: "memory");
@@ -1031,7 +1039,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 }
             }
         }
-        for (int kk = k + tid; kk < kp.k_max; kk += NT) chan_id_b[kk] = -1;
+        for (int kk = k + tid; kk < kp.k_max && !kp.host_rows; kk += NT) chan_id_b[kk] = -1;
         if (tid == 0) {
             n_act += (unsigned long long)k;
             n_steps[b] = k;

@@ -795,7 +795,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
         }
         __syncwarp();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
-        const size_t rows = (size_t)(kp.k_max - k) * N;      // elements per array
+        const size_t rows = kp.host_rows ? 0 : (size_t)(kp.k_max - k) * N;      // elements per array
         if ((((uintptr_t)c.lane_dst_b | (uintptr_t)c.lane_inst_b | (uintptr_t)c.lane_bytes_b | (uintptr_t)c.send_off_b |
               (uintptr_t)(c.recv_off_b ? c.recv_off_b : c.send_off_b)) & 15) == 0 && (32 % N) == 0 && N >= 8) {
             // whole rows of 2 N bytes and 8 N bytes in 16-byte vectors (N = 8 or 16: a warp's stride keeps a lane's ranks)
@@ -815,7 +815,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
                 if (ro2) ro2[e] = ra;
             }
         } else {
-            for (size_t e = (size_t)k * N + lane; e < (size_t)kp.k_max * N; e += 32) {
+            for (size_t e = (size_t)k * N + lane; e < (size_t)k * N + rows; e += 32) {
                 c.lane_dst_b[e] = -1;
                 c.lane_inst_b[e] = 0xFFFF;
                 c.lane_bytes_b[e] = 0;
@@ -824,7 +824,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
                 if (c.recv_off_b) c.recv_off_b[N + e] = recv_acc[i];
             }
         }
-        for (int kk = k + lane; kk < kp.k_max; kk += 32) c.chan_id_b[kk] = -1;
+        for (int kk = k + lane; kk < kp.k_max && !kp.host_rows; kk += 32) c.chan_id_b[kk] = -1;
         if (lane == 0) {
             n_act += (unsigned long long)k;
             n_steps[b] = k;

@@ -112,6 +112,13 @@ struct vp_catalog {
     int host_pipe_ready;
 };
 
+// vp_schedule_batch; with host_rows the plan arrays are device addresses of page-locked host memory, and what lies beyond a
+// matrix's n_steps is not written.
+int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int64_t* demand, const int64_t* tau_ns_in, int B,
+                       int32_t* n_steps, int32_t* chan_id, int16_t* lane_dst, uint16_t* lane_inst, int64_t* lane_bytes,
+                       int64_t* send_off, int64_t* recv_off, int64_t* tau_ns_out, int32_t* status, void* workspace,
+                       size_t workspace_bytes, void* cuda_stream, bool host_rows);
+
 extern std::atomic<long long> g_vp_launches;
 
 // Profiling hook: when enabled, records a CUDA event on `stream` before (edge 0) / after (edge 1)

@@ -71,3 +71,35 @@ def test_work_counters_and_batches(vp, oracle_lib, name, batches):  # noqa: F811
                 n = min(3, B - r)
                 assert np.array_equal(got[key][r:r + n], want[key][:n]), (B, key, r)
         assert stats["activations"] == int(got["n_steps"].sum()) and stats["tasks"] >= 4 * stats["activations"] and stats["sweeps"] >= stats["tasks"]
+
+
+@pytest.mark.parametrize("name,B", [("two_nodes_64_50", 70), ("template_5_64_50", 7), ("template_8", 5), ("template_17", 3)])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_rows_in_use(vp, oracle_lib, name, B, pinned):  # noqa: F811
+    """Rows in use come back the same through page-locked buffers (written by the scheduler) and pageable ones (copied), with
+    receive offsets and without a matrix's idle rows being touched; one invalid matrix, one cut short."""
+    import torch
+    cat = CATALOGS[name]()
+    N = cat.topology.N
+    rng = np.random.default_rng(B)
+    D = (rng.integers(0, 90, size=(B, N, N)) * (rng.random((B, N, N)) < (0.5 if N < 64 else 0.1)) * 512).astype(np.int64)
+    D[0] *= (rng.random((N, N)) < 0.05)
+    for b in range(B):
+        np.fill_diagonal(D[b], 0)
+    D[1, 3, 3] = 512
+    w = WParams(granule_bytes=512, k_max=3 * N).resolved(N)
+    oc = oracle_lib.OracleCatalog(cat.topology.blob(), cat.blob())
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob())
+    p = ts._params(vp, w)
+    plan = vp.Plan.empty(B, N, p.k_max, "cpu", pin=pinned)
+    for key in ("chan_id", "lane_dst", "lane_inst", "lane_bytes", "send_off", "recv_off"):
+        getattr(plan, key).fill_(77)
+    demand = torch.from_numpy(D)
+    vp.schedule_batch_host(dc, p, demand.pin_memory() if pinned else demand, plan=plan, used_only=True)
+    want, got = oc.schedule_batch(D, w, threads=B), plan.cpu()
+    for key in ("n_steps", "status", "tau_ns"):
+        assert np.array_equal(got[key], want[key]), key
+    for b in range(B):
+        K = int(want["n_steps"][b])
+        for key, n in (("chan_id", K), ("lane_dst", K), ("lane_inst", K), ("lane_bytes", K), ("send_off", K + 1), ("recv_off", K + 1)):
+            assert np.array_equal(got[key][b][:n], want[key][b][:n]) and (got[key][b][n:] == 77).all(), (key, b)
