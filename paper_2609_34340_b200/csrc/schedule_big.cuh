@@ -155,6 +155,16 @@ __device__ __forceinline__ void big_fill_bytes(unsigned char* dst, size_t lo, si
 __device__ __noinline__ bool big_not_multiple(int64_t x, int64_t granule) { return x % granule != 0; }
 __device__ __noinline__ uint32_t big_div_granule(int64_t x, int64_t granule) { return (uint32_t)(x / granule); }
 
+// An offset row in rank order, whole lines for PCIe, once all of it is up to date: `threads` threads, numbered from 0, whole warps (out of
+// line: for page-locked plans only, and inlined it costs the other case registers).  The barrier's number counts: an SM has 64, and a
+// kernel reserves all up to its highest one (with number 9 eight small CTAs no longer fit an SM: 1.64 -> 2.43 ms).
+template <int BARRIER>
+__device__ __noinline__ void big_write_in_order(int64_t* row, const int64_t* acc, int N, int thread, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"n"(BARRIER), "r"(threads) : "memory");
+    for (int r = thread; r < N; r += threads) row[r] = acc[r];
+    asm volatile("bar.sync %0, %1;" ::"n"(BARRIER), "r"(threads) : "memory");
+}
+
 // Step 3 when several families compete (kept out of line: most shapes have one family, and the main loop should
 // stay small for the instruction cache): best start per family (largest F, lowest start), then the family of largest
 // utility F / duration by exact cross-multiplication, lowest family first among equals.  Whole warp.
@@ -225,6 +235,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     // `order` (may be null) lists the matrices in the order in which the CTAs should take them: longest first.
     constexpr bool CROSS = LANES == 64;                   // a task is two warps
     constexpr bool RECORD = CROSS && SPLIT == 1;          // task warps emit, the others write the rows
+    constexpr bool IN_ORDER = CROSS || SPLIT == 2;        // page-locked plans: receive offsets in rank order (the kernels that pack SMs
+                                                          // have no register to spare: there it cost every plan 6 %)
     constexpr int WL = CROSS ? 32 : LANES;                // a task's lanes in one warp
     constexpr int TPW = 32 / WL, QN = 4 / SPLIT;          // tasks per warp, columns per lane
     constexpr int ST = big_stride(LANES / SPLIT);         // words per row pair of the credit matrix
@@ -579,7 +591,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 lane_dst_b[row + i] = x ? (int16_t)j : (int16_t)-1;
                 lane_bytes_b[row + i] = bytes;
                 send_off_b[orow + i] = sa;
-                if (recv_off_b && !kp.host_rows) recv_off_b[orow + j] = ra;
+                if (recv_off_b && !(IN_ORDER && kp.host_rows)) recv_off_b[orow + j] = ra;
                 lane_inst_b[row + i] = x ? (uint16_t)inst : (uint16_t)0xFFFF;
                 if (r == 0) chan_id_b[kk] = fam;
             };
@@ -592,12 +604,10 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     if (emit_warp > 0 && emits) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
                     if (emits) write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
                 }
-                if (kp.host_rows && recv_off_b) {             // (in rank order: whole lines for PCIe)
-                    // (every lane of the writing warps comes here once per activation: pend is the same in a warp)
-                    const int first = RECORD ? n_task_warps * 32 : emit_warp * 32, threads = RECORD ? NT - first : emit_threads;
-                    asm volatile("bar.sync 9, %0;" ::"r"(threads) : "memory");
-                    for (int r = tid - first; r < N; r += threads) recv_off_b[(size_t)(kk + 1) * N + r] = recv_acc[r];
-                    asm volatile("bar.sync 9, %0;" ::"r"(threads) : "memory");
+                // (every lane of the writing warps comes here once per activation: pend is the same in a warp)
+                if (IN_ORDER && kp.host_rows && recv_off_b) {
+                    const int first = RECORD ? n_task_warps * 32 : emit_warp * 32;
+                    big_write_in_order<CROSS ? 5 : 1>(recv_off_b + (size_t)(kk + 1) * N, recv_acc, N, tid - first, RECORD ? NT - first : emit_threads);
                 }
                 pend = false;
             };
