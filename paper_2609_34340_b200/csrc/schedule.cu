@@ -1175,10 +1175,14 @@ KernelFn pick_kernel(int g, int lpg) {
     return nullptr;
 }
 // Kernel for a number of rank groups, with one or two lanes per group (see vp_schedule_big_kernel).
-BigKernelFn pick_big_kernel(int G, int split) {
-    if (split == 2) return G <= 8 ? vp_schedule_big_kernel<16, 2> : G <= 16 ? vp_schedule_big_kernel<32, 2> : vp_schedule_big_kernel<64, 2>;
-    return G <= 8 ? vp_schedule_big_kernel<8, 1> : G <= 16 ? vp_schedule_big_kernel<16, 1>
-         : G <= 32 ? vp_schedule_big_kernel<32, 1> : vp_schedule_big_kernel<64, 1>;
+template <bool ONE>
+BigKernelFn pick_big_kernel_for(int G, int split) {
+    if (split == 2) return G <= 8 ? vp_schedule_big_kernel<16, 2, ONE> : G <= 16 ? vp_schedule_big_kernel<32, 2, ONE> : vp_schedule_big_kernel<64, 2, ONE>;
+    return G <= 8 ? vp_schedule_big_kernel<8, 1, ONE> : G <= 16 ? vp_schedule_big_kernel<16, 1, ONE>
+         : G <= 32 ? vp_schedule_big_kernel<32, 1, ONE> : vp_schedule_big_kernel<64, 1, ONE>;
+}
+BigKernelFn pick_big_kernel(const DevCat& dc, int split) {
+    return dc.n_classes == 1 ? pick_big_kernel_for<true>(dc.G, split) : pick_big_kernel_for<false>(dc.G, split);
 }
 
 // Raises a kernel's limit of dynamic shared memory on the current device to `bytes` if it is lower.  The limit belongs
@@ -1275,7 +1279,7 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
             kp.big_task_warps = task_warps;
             kp.big_emit_warp = apart ? task_warps : 0;
             const int threads = dc.G > 32 ? 384 : task_warps * 32 + (apart ? (dc.N + 31) / 32 * 32 : 0);
-            const BigKernelFn bf = pick_big_kernel(dc.G, split);
+            const BigKernelFn bf = pick_big_kernel(dc, split);
             const size_t smem = (size_t)big_smem_layout(dc, kp).total;
             if (smem + 2048 > (size_t)c->max_smem_optin) continue;
             if (raise_dynamic_smem((const void*)bf, smem) != VP_OK) return VP_E_CUDA;
@@ -1421,7 +1425,7 @@ int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int6
                     big_rank_kernel<<<(B + 255) / 256, 256, 0, stream>>>(key, B, order);
                     g_vp_launches += 2;
                 }
-                pick_big_kernel(c->dc.G, L.big_split)<<<L.big_grid, L.big_threads, L.big_smem, stream>>>(
+                pick_big_kernel(c->dc, L.big_split)<<<L.big_grid, L.big_threads, L.big_smem, stream>>>(
                     c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst, lane_inst, lane_bytes, send_off, recv_off,
                     tau_ns_out, status, counter, todo, order);
                 g_vp_launches++;

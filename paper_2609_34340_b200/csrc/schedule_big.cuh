@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(256) big_rank_kernel(const int* __restrict__ k
 // a quarter more in all, so it is taken while the batch leaves SMs room.  Up to 32 lanes a task is part of a warp, 64 lanes
 // are two warps that meet at a barrier of their own.  Task warps are the first warps of the CTA (kp.big_task_warps),
 // the threads from warp kp.big_emit_warp on emit, a slot each.
-template <int LANES, int SPLIT>
+// ONE: all paths have one rate, so every slot the same capacity (selected per slot at run time it cost 3 %: 1,024 matrices of 64 ranks 1,636 -> 1,580 us).
+template <int LANES, int SPLIT, bool ONE>
 __global__ void __launch_bounds__(LANES == 64 ? 384 : (SPLIT == 2 ? LANES * 6 : LANES * 8), LANES == 64 ? 1 : 64 / LANES)
 vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, const int64_t* __restrict__ tau_in, int B,
                        int32_t* __restrict__ n_steps, int32_t* __restrict__ chan_id, int16_t* __restrict__ lane_dst,
@@ -330,7 +331,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             if (tid + u * NT < dc.n_shapes) my_pat[u] = spat[tid + u * NT];
     }
     const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
-    const bool one_class = dc.n_classes == 1;
+    constexpr bool one_class = ONE;
     const int n_task_warps = kp.big_task_warps, emit_warp = kp.big_emit_warp;
     const int r_emit = tid - emit_warp * 32;              // this thread's slot when it emits
     const int emit_threads = (N + 31) & ~31;              // whole warps
