@@ -488,8 +488,8 @@ int vp_unpack_tokens(const int32_t* n_steps_b, const int16_t* lane_dst_b, const 
  * warp per matrix (one, two or four warps per CTA as B grows), chosen for topologies of at most four groups of four
  * ranks when granule_bytes >= 256, and with smaller granules once B exceeds the number of CTAs that fit the GPU at
  * once; kernel 2 = one CTA per matrix with 16-bit saturating credits in shared memory, chosen
- * for node-symmetric catalogs of more than sixteen groups of four ranks (a second launch of kernel 0 then takes the
- * matrices whose capacities or totals do not fit that representation).  All kernels produce identical plans.
+ * for node-symmetric catalogs of two to sixty-four groups of four ranks, below sixteen groups when granule_bytes >= 256
+ * (a second launch of kernel 0 then takes the matrices whose capacities or totals do not fit that representation).  All kernels produce identical plans.
  * CTAs is also the number of matrices in flight at once: a caller that splits a large batch into sub-batches
  * wastes least when each sub-batch is several times this number (the CTAs pull matrices from a shared counter, so
  * only the last matrix of each CTA can leave the others waiting).
