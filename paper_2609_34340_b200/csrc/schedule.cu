@@ -1421,7 +1421,7 @@ int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int6
                 if (B > L.big_grid && B <= 16384) {          // more matrices than CTAs: longest first (see big_rank_kernel)
                     order = (int*)((char*)workspace + w.order);
                     int* key = (int*)((char*)workspace + w.key);
-                    big_count_nonzero_kernel<<<(B + 7) / 8, 256, 0, stream>>>(demand, B, c->dc.N * c->dc.N, key);
+                    big_length_kernel<<<B, BIG_KEY_THREADS, 0, stream>>>(c->dc, L.kp, demand, tau_ns_in, key);
                     big_rank_kernel<<<(B + 255) / 256, 256, 0, stream>>>(key, B, order);
                     g_vp_launches += 2;
                 }

@@ -103,3 +103,29 @@ def test_host_rows_in_use(vp, oracle_lib, name, B, pinned):  # noqa: F811
         K = int(want["n_steps"][b])
         for key, n in (("chan_id", K), ("lane_dst", K), ("lane_inst", K), ("lane_bytes", K), ("send_off", K + 1), ("recv_off", K + 1)):
             assert np.array_equal(got[key][b][:n], want[key][b][:n]) and (got[key][b][n:] == 77).all(), (key, b)
+
+
+@pytest.mark.parametrize("name,tau", [("template_8", 0), ("template_9", 500), ("template_17", 0), ("template_17", 700)])
+def test_work_order(vp, oracle_lib, name, tau):  # noqa: F811
+    """More matrices than CTAs at once, of very different lengths (one empty, one invalid): the order in which they are taken
+    changes no plan."""
+    import torch
+    cat = CATALOGS[name]()
+    N = cat.topology.N
+    rng = np.random.default_rng(N + tau)
+    base = (rng.integers(1, 60, size=(5, N, N)) * 4096).astype(np.int64)
+    for b, keep in enumerate((0.0, 0.02, 0.2, 0.05, 0.1)):
+        base[b] *= rng.random((N, N)) < keep
+        np.fill_diagonal(base[b], 0)
+    base[4, 1, 0] = -4096
+    w = WParams(granule_bytes=4096).resolved(N)
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob())
+    p = ts._params(vp, w)
+    B = vp.schedule_launch_info(dc, 1 << 14, p)["ctas"] + 3
+    given = np.full(5, tau, dtype=np.int64) if tau else None
+    want = oracle_lib.OracleCatalog(cat.topology.blob(), cat.blob()).schedule_batch(base, w, tau_in=given, threads=5)
+    pick = np.arange(B) % 5
+    got = vp.schedule_batch(dc, p, torch.from_numpy(base[pick]).cuda(), tau_ns_in=torch.from_numpy(given[pick]).cuda() if tau else None).cpu()
+    for key in ts.KEYS:
+        for r in range(5):
+            assert (got[key][r::5] == want[key][r]).all(), (key, r)
