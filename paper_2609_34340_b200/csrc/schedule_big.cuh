@@ -27,8 +27,10 @@
 //  * Large capacities.  When a lane capacity reaches 2^16 granules (skewed MoE matrices with many tokens), the few
 //    columns that hold cells of 65,535 granules or more -- the destinations of the popular experts -- become "hot
 //    columns": their cells are kept exactly, low 16 bits in the credit matrix and high 16 bits in a side array of up
-//    to 32 columns, and the credits that touch them are patched after the ordinary 16-bit pass.  Every other cell of
-//    such a matrix is below 65,535 granules, so its 16-bit copy is exact.  No L2 traffic is needed in this mode.
+//    to 32 columns, and the credits that touch them are patched after the ordinary 16-bit pass (above 32 groups, where such
+//    matrices are the longest of a batch: from the words already read, and until no cell of the column is beyond 16 bits any more;
+//    5.65 -> 4.2 us an activation with 256 ranks).  Every other cell of such a matrix is below 65,535 granules, so its 16-bit
+//    copy is exact.  No L2 traffic is needed in this mode.
 //
 // A matrix that does not meet the conditions (granule below 256 bytes, a capacity of 2^22 granules or more, 2^32
 // granules or more in total, more than 32 hot columns, more big cells than the side list holds) is appended to a list that
@@ -37,7 +39,8 @@
 
 namespace {
 
-constexpr int BIG_HOT_MAX = 32;       // columns whose cells are kept beyond 16 bits
+constexpr int BIG_HOT_MAX = 32;       // columns whose cells are kept beyond 16 bits; as a column's index: none
+constexpr uint32_t BIG_HOT_NONE = 0x01010101u * BIG_HOT_MAX;  // a group without a hot column
 constexpr int BIG_EXCHANGE = 192;     // bytes per pair of warps: 64 source tags, 64 destination tags, words
 constexpr int BIG_SMEM_LIMIT = 227 * 1024 - 2048;   // dynamic shared memory of one CTA, less room for the static variables
 
@@ -60,8 +63,8 @@ __host__ __device__ inline BigSmem big_smem_layout(const DevCat& dc, const KPara
     int o = 0;
     const int wd_bytes = dc.N / 2 * big_stride(big_lanes(dc.G)) * 4, setup_bytes = dc.G * dc.G * 8 + dc.N * 24;
     L.wd = o;        o += align16(wd_bytes > setup_bytes ? wd_bytes : setup_bytes);   // set-up: D-hat, row and column sums
-    L.hi = o;        o += BIG_HOT_MAX * dc.N * 2;                  // high halves of the hot columns' cells, or the side list
-    L.colmap = o;    o += align16(dc.N);                          // hot-column index of every rank, 0xFF = none
+    L.hi = o;        o += (BIG_HOT_MAX + (dc.G > 32)) * dc.N * 2;   // high halves of the hot columns' cells (and of none of them), or the side list
+    L.colmap = o;    o += align16(dc.N);                          // hot-column index of every rank
     L.tbl = o;       o += align16(dc.tbl_size * 4);
     L.rs = o;        o += dec ? 0 : align16(dc.n_patterns * 8);   // row scores
     L.pat = o;       o += dec ? 0 : align16(dc.n_patterns * dc.max_row_terms * 4);
@@ -134,7 +137,7 @@ struct BigCredits {
     // exact value of a cell as far as the matrix keeps it (a big cell yields its code, at least the capacity)
     __device__ __forceinline__ uint32_t cell(int i, int j) const {
         uint32_t c = ((const uint16_t*)wd)[((i >> 1) * stride + j) * 2 + (i & 1)];
-        if (hot && colmap[j] != 0xFF) c |= (uint32_t)hi[(int)colmap[j] * N + i] << 16;
+        if (hot && colmap[j] != BIG_HOT_MAX) c |= (uint32_t)hi[(int)colmap[j] * N + i] << 16;
         return c;
     }
 };
@@ -308,6 +311,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     // `order` (may be null) lists the matrices in the order in which the CTAs should take them: longest first.
     constexpr bool CROSS = LANES == 64;                   // a task is two warps
     constexpr bool RECORD = CROSS && SPLIT == 1;          // task warps emit, the others write the rows
+    constexpr bool EXACT = RECORD;                        // credits of hot columns from the words at hand (the other kernels lost 1 to 3 % on every matrix by it)
     constexpr bool IN_ORDER = CROSS || SPLIT == 2;        // page-locked plans: receive offsets in rank order (the kernels that pack SMs
                                                           // have no register to spare: there it cost every plan 6 %)
     constexpr int WL = CROSS ? 32 : LANES;                // a task's lanes in one warp
@@ -334,6 +338,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     uint32_t* const side = (uint32_t*)(smem_raw + L.hi);
     const int big_max = min(BIG_HOT_MAX * N / 2, 4096), big_floor = 65536 - big_max;
     __shared__ int s_b, s_flags, s_mode, s_nhot, s_nbig;           // s_mode: 0 leave to the general kernel, 1 plain, 2 hot columns
+    __shared__ int s_hot, s_beyond[BIG_HOT_MAX];          // cells that are 2^16 granules or more still, in all and per hot column
     __shared__ int64_t s_tau, s_left;
     __shared__ int2 s_pick;                               // first family and families of the shape chosen (none: nothing is covered)
     __shared__ int64_t s_tscale[VP_MAX_CLASSES];
@@ -452,8 +457,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         int64_t* rowsum = Dhat + G * G;
         int64_t* colsum = rowsum + N;
         int64_t* colmax = colsum + N;
-        for (int i = tid; i < N; i += NT) { colsum[i] = 0; colmax[i] = 0; rowsum[i] = 0; send_acc[i] = 0; recv_acc[i] = 0; colmap[i] = 0xFF; }
-        if (tid == 0) { s_nhot = 0; s_nbig = 0; }
+        for (int i = tid; i < N; i += NT) { colsum[i] = 0; colmax[i] = 0; rowsum[i] = 0; send_acc[i] = 0; recv_acc[i] = 0; colmap[i] = BIG_HOT_MAX; if (EXACT) Hi[BIG_HOT_MAX * N + i] = 0; }
+        if (EXACT) for (int i = tid; i < BIG_HOT_MAX; i += NT) s_beyond[i] = 0;
+        if (tid == 0) { s_nhot = 0; s_nbig = 0; if (EXACT) s_hot = 0; }
         for (int e = tid; e < G * G; e += NT) Dhat[e] = 0;
         __syncthreads();
         int flags = 0;
@@ -633,8 +639,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             code = (uint32_t)big_floor + (uint32_t)min_v(at, big_max - 1);
                             if (at < big_max) side[at] = v;
                         }
-                    } else if (colmap[j] != 0xFF) {              // exact: 32 bits in a hot column, below 65,535 elsewhere
+                    } else if (colmap[j] != BIG_HOT_MAX) {       // exact: 32 bits in a hot column, below 65,535 elsewhere
                         Hi[(int)colmap[j] * N + i] = (uint16_t)(v >> 16);
+                        if (EXACT && v >> 16) { atomicAdd(&s_beyond[colmap[j]], 1); atomicAdd(&s_hot, 1); }
                     }
                     cells[((i >> 1) * ST + j) * 2 + (i & 1)] = (uint16_t)code;
                 }
@@ -815,6 +822,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     }
                 }
 
+                const bool hot = EXACT && hot_mode && s_hot > 0;            // (none beyond 16 bits left: the 16-bit credits are exact)
                 // (B) MultiStartAA: LANES lanes per (family, start), SPLIT of them per rank group.
                 //
                 // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits,
@@ -877,6 +885,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         };
                         auto cap_of = [&](uint32_t w) { return one_class ? cap0 : s_cap[(w >> 24) & 0xfu]; };
                         auto cap2_of = [&](uint32_t w) { return one_class ? cap2 : min_v(s_cap[(w >> 24) & 0xfu], 65535u) * 0x00010001u; };
+                        // exact credit in place of the 16-bit one (the tag byte stays)
+                        auto hot_credit = [&](uint32_t& key, uint32_t cell, uint32_t cap) { key = __byte_perm(key, min_v(cell, cap), 0x6540); };
                         // source half: one exact assignment per source group
                         auto source_half = [&]() {
                             uint32_t v[4][QN];
@@ -886,14 +896,29 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 const uint32_t c2 = cap2_of(uo[i]);
                                 tile_column(v, i, __vminu2(at[0], c2), __vminu2(at[ST], c2));
                             }
-                            if (hot_mode) {                    // out-slots bound to a hot column: exact 32-bit cells
+                            if (!EXACT && hot_mode) {          // out-slots bound to a hot column: exact 32-bit cells
 #pragma unroll
                                 for (int i = 0; i < QN; i++) {
                                     const int j = (int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i];
-                                    if (colmap[j] != 0xFF) {
+                                    if (colmap[j] != BIG_HOT_MAX) {
 #pragma unroll
                                         for (int r = 0; r < 4; r++)
                                             v[r][i] = min_v(cr.cell(ag * 4 + r, j), cap_of(uo[i])) * 256u + (v[r][i] & 0xffu);
+                                    }
+                                }
+                            }
+                            if (hot) {                         // the same from the words at hand
+#pragma unroll
+                                for (int i = 0; i < QN; i++) {
+                                    const int col = colmap[((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]];
+                                    if (col != BIG_HOT_MAX) {
+                                        const uint2 h = *(const uint2*)(Hi + col * N + ag * 4);
+                                        const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
+                                        const uint32_t lo = at[0], hi = at[ST], cap = cap_of(uo[i]);
+                                        hot_credit(v[0][i], __byte_perm(lo, h.x, 0x5410), cap);
+                                        hot_credit(v[1][i], __byte_perm(lo, h.x, 0x7632), cap);
+                                        hot_credit(v[2][i], __byte_perm(hi, h.y, 0x5410), cap);
+                                        hot_credit(v[3][i], __byte_perm(hi, h.y, 0x7632), cap);
                                     }
                                 }
                             }
@@ -934,15 +959,29 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 const uint32_t c2 = cap2_of(ui[i]);
                                 tile_column(v, i, __vminu2(__byte_perm(w.x, w.y, sel), c2), __vminu2(__byte_perm(w.z, w.w, sel), c2));
                             }
-                            if (hot_mode && *((const uint32_t*)colmap + ag) != 0xffffffffu) {  // some rank of this group is a hot column
+                            if (!EXACT && hot_mode && *((const uint32_t*)colmap + ag) != BIG_HOT_NONE) {
 #pragma unroll
                                 for (int r = 0; r < 4; r++)
-                                    if (colmap[ag * 4 + r] != 0xFF) {
+                                    if (colmap[ag * 4 + r] != BIG_HOT_MAX) {
 #pragma unroll
                                         for (int i = 0; i < QN; i++)
                                             v[r][i] = min_v(cr.cell((int)((ui[i] >> 16) & 0xffu) * 4 + 3 - (int)(tag[i] & 3u), ag * 4 + r), cap_of(ui[i])) * 256u +
                                                       (v[r][i] & 0xffu);
                                     }
+                            }
+                            uint32_t cols;                     // hot columns among the ranks of this group
+                            if (hot && (cols = *((const uint32_t*)colmap + ag)) != BIG_HOT_NONE) {
+#pragma unroll
+                                for (int i = 0; i < QN; i++) {
+                                    const uint16_t* const h = Hi + ((ui[i] >> 16) & 0xffu) * 4 + 3 - (tag[i] & 3u);
+                                    const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
+                                    const unsigned sel = 0x5410u + (~tag[i] & 1u) * 0x0022u;   // its half, then the high half from the side array
+                                    const uint32_t cap = cap_of(ui[i]);
+                                    hot_credit(v[0][i], __byte_perm(w.x, h[(cols & 0xffu) * N], sel), cap);
+                                    hot_credit(v[1][i], __byte_perm(w.y, h[(cols >> 8 & 0xffu) * N], sel), cap);
+                                    hot_credit(v[2][i], __byte_perm(w.z, h[(cols >> 16 & 0xffu) * N], sel), cap);
+                                    hot_credit(v[3][i], __byte_perm(w.w, h[(cols >> 24) * N], sel), cap);
+                                }
                             }
                             const uint32_t key = best_key(v);
                             const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
@@ -1070,11 +1109,16 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         }
                         *cell = (uint16_t)now_cell;
                     } else {
-                        uint16_t* const hcell = colmap[j] != 0xFF ? Hi + (int)colmap[j] * N + i : nullptr;
+                        const int col = colmap[j];
+                        uint16_t* const hcell = col != BIG_HOT_MAX ? Hi + col * N + i : nullptr;
                         if (hcell) c |= (uint32_t)*hcell << 16;   // a hot column: the exact 32-bit cell
                         p_x = min_v(cap, c);
                         *cell = (uint16_t)(c - p_x);
                         if (hcell) *hcell = (uint16_t)((c - p_x) >> 16);
+                        if (EXACT && c >= 65536u && c - p_x < 65536u) {   // one less; a column without any is like the others from here on
+                            atomicSub(&s_hot, 1);                 // (this column is this thread's for this activation)
+                            if (--s_beyond[col] == 0) colmap[j] = BIG_HOT_MAX;
+                        }
                     }
                     atomicSub(&tbl[entry], p_x);                  // (an idle lane takes zero)
                     p_bind = bw;
