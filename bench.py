@@ -594,8 +594,8 @@ def finish(args, world, run, sched, pk, T, topk, R, pack_bytes, copy_bytes, stat
     p_now = extras.get("peaks") or {}
     int_peak = p_now.get("int32_add_min_tops")
     sched_tops = ops / (sched_per_step * 1e-3) / 1e12
-    pack_counters = (counters.get("pack_copy_bulk_kernel") or {}) if args.pack_tokens == 16384 else {}
-    roof_pack = dict(kernel="pack_copy_bulk_kernel", bound="hbm", achieved=round(pack_gbs, 1), peak=peaks["hbm_gbs"],
+    pack_counters = (counters.get("row_copy_bulk_kernel") or {}) if args.pack_tokens == 16384 else {}
+    roof_pack = dict(kernel="row_copy_bulk_kernel", bound="hbm", achieved=round(pack_gbs, 1), peak=peaks["hbm_gbs"],
                      unit="GB/s", frac=round(pack_gbs / peaks["hbm_gbs"], 4), traffic=pack_counters.get("dram_bytes_per_launch"),
                      peak_source=peaks["source"] + " copy peak (MEASURED_PEAKS.json)", ms_per_launch=round(copy_avg, 4),
                      algorithmic_bytes_per_launch=copy_bytes,
