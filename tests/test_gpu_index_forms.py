@@ -93,6 +93,18 @@ def test_demand_forms(vp, oracle_lib, sources, tokens, topk, N):  # noqa: F811
         assert np.array_equal(got.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("sources,tokens,topk,N", [(1, 1, 1, 8), (1, 4099, 3, 16), (200, 331, 7, 256), (256, 1100, 3, 256), (5, 9999, 3, 256)])
+def test_demand_alignments(vp, oracle_lib, sources, tokens, topk, N):  # noqa: F811
+    """Indices that start at any word: copies before, in and after the 16-byte loads; up to and beyond one wave of CTAs."""
+    n = sources * tokens * topk
+    for off in range(4):
+        flat = torch.randint(-1, N * 2, (n + 3,), dtype=torch.int32, generator=torch.Generator().manual_seed(n + off))
+        idx = flat[off:off + n].view(sources, tokens, topk)
+        got, st = vp.demand_from_routing(flat.cuda()[off:off + n].view(sources, tokens, topk), 2, N, 4096)
+        want, bad = oracle_lib.demand_from_routing(idx.numpy(), 2, N, 4096)
+        assert int(st.item()) == bad == 0 and np.array_equal(got.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("nodes,T,topk,row_bytes", [(2, 3, 1, 16), (2, 700, 8, 14336), (2, 700, 8, 4100), (1, 500, 8, 333), (1, 90, 4, 1),
                                                     (2, 33, 6, 16400), (8, 40, 8, 7392), (8, 40, 8, 4102)])
 def test_put_alignments(vp, oracle_lib, nodes, T, topk, row_bytes):  # noqa: F811
