@@ -3,8 +3,8 @@
 // A rank's staged send buffer holds one contiguous chunk per activation; the chunk of step k goes to the step's
 // destination j = lane_dst[k][rank] and lands at j's running receive offset recv_off[k][j].  vp_exchange_put is the
 // sender side: stores through pointers to the receivers' buffers -- ordinary device memory when the ranks share
-// a GPU, peer-mapped memory of other GPUs over NVLink otherwise -- followed by a system-wide fence and, per chunk part, an
-// addition to the receiver's device-resident arrival counter.  vp_exchange_wait is the receiver side: a bounded
+// a GPU, peer-mapped memory of other GPUs over NVLink otherwise -- followed by a system-wide fence and, per CTA and destination,
+// an addition to the receiver's device-resident arrival counter.  vp_exchange_wait is the receiver side: a bounded
 // wait until the counter has reached the bytes the plan sends this rank, which is what replaces a global barrier.
 // Double buffering is the caller's: two receive buffers and two counters per rank, alternated between invocations.
 //
@@ -12,6 +12,7 @@
 // the same code is valid for local and for peer destinations.
 #include <cuda_runtime.h>
 
+#include "announce.h"
 #include "row_copy.cuh"
 #include "vp_internal.h"
 
@@ -139,7 +140,7 @@ __device__ __forceinline__ void put_any(unsigned char* dst, const unsigned char*
 // CTA c moves the bytes [c, c + 1) x total / CTAs of the send buffer (rounded to 16 bytes), chunk part by chunk part.  (Pieces
 // dealt round robin copy 2 % faster, but every CTA then walks the whole plan: 10 us on the 290 activations of 64 ranks.)
 // Parts whose addresses and size are multiples of 16 go through shared memory as bulk asynchronous copies that one thread of
-// warp 0 issues (pieces of up to 16 KB, six stages); others are moved by all warps.  One system fence by one thread per CTA
+// warp 0 issues (pieces of up to 16 KB, six stages); others are moved by all warps.  One system fence by one warp per CTA
 // announces all its parts: fences by every thread, and a second walk over the plan behind them, took 12 us of any call.
 // Bound by HBM.  On one GPU 2,048 tokens x top-8 of 14,336 B (440 MB read and written) took 95.6 us with plain 16-byte loads
 // and stores, now 81; 32 tokens 19.1 us, now 7.9.
@@ -208,15 +209,11 @@ __global__ void __launch_bounds__(kPutThreads) exchange_put_kernel(PutArgs a) {
         if (failed) atomicOr(a.status, VP_ST_INTERNAL_TIMEOUT);
     }
     if (a.arrived) {
-        // every thread's stores become visible system-wide before the counts that announce them: the barrier orders them
-        // before the one thread whose fence covers them all
+        // every thread's stores become visible system-wide before the counts that announce them
         if (__syncthreads_or(failed)) return;
-        if (warp == 0) {
-            if (tid == 0) __threadfence_system();
-            __syncwarp();
-            for (int j = tid; j < a.N; j += 32)
-                if (s_count[j] && s_counter[j]) atomicAdd_system(s_counter[j], s_count[j]);
-        }
+        if (warp == 0)
+            announce_counts(tid, a.N, s_count, [] { __threadfence_system(); },
+                            [&](int j, unsigned long long bytes) { if (s_counter[j]) atomicAdd_system(s_counter[j], bytes); });
     }
 }
 
