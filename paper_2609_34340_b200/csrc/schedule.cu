@@ -31,12 +31,12 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
-#include <mutex>
 #include <utility>
 #include <vector>
 
 #include "bulk_copy.cuh"
 #include "route_index.cuh"
+#include "smem_limit.h"
 #include "vp_internal.h"
 
 namespace {
@@ -1185,27 +1185,6 @@ BigKernelFn pick_big_kernel(const DevCat& dc, int split) {
     return dc.n_classes == 1 ? pick_big_kernel_for<true>(dc.G, split) : pick_big_kernel_for<false>(dc.G, split);
 }
 
-// Raises a kernel's limit of dynamic shared memory on the current device to `bytes` if it is lower.  The limit belongs
-// to the function, not to a launch: launches are planned once and replayed from a memo, several catalogs share the
-// kernels, and one kernel is launched with different sizes, so the limit must never be lowered by a later plan.
-int raise_dynamic_smem(const void* fn, size_t bytes) {
-    struct Mark { int device; const void* fn; size_t bytes; };
-    static Mark marks[64];
-    static int n_marks = 0;
-    static std::mutex lock;
-    std::lock_guard<std::mutex> hold(lock);
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return VP_E_CUDA;
-    Mark* m = nullptr;
-    for (int i = 0; i < n_marks; i++)
-        if (marks[i].device == dev && marks[i].fn == fn) m = &marks[i];
-    if (m && m->bytes >= bytes) return VP_OK;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return VP_E_CUDA;
-    if (m) m->bytes = bytes;
-    else if (n_marks < 64) marks[n_marks++] = Mark{dev, fn, bytes};
-    return VP_OK;
-}
-
 int resolve_params(const vp_catalog* c, const vp_sched_params* p, KParams* kp) {
     if (!c || !p || c->device < 0) return VP_E_BAD_ARG;         // (a host-only handle launches nothing)
     if (p->k_max <= 0 || p->granule_bytes <= 0 || p->lambda_ns < 0 || p->lambda_ns >= VP_ENTRY_LIMIT) return VP_E_BAD_ARG;
@@ -1243,16 +1222,16 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     if (L.kp.incremental) {
         const int staged = L.kp.stage_terms;
         L.kp.stage_terms = 0;
-        if ((size_t)smem_layout(dc, L.kp, L.threads / 32, L.lpg).total + 2048 > (size_t)c->max_smem_optin) {
+        if (smem_layout(dc, L.kp, L.threads / 32, L.lpg).total > dynamic_smem_limit(c->max_smem_optin)) {
             L.kp.incremental = 0;
             L.kp.stage_terms = staged;
         }
     }
     L.smem = (size_t)smem_layout(dc, L.kp, L.threads / 32, L.lpg).total;
-    if (L.smem + 2048 > (size_t)c->max_smem_optin) return VP_E_UNSUPPORTED;
+    if (L.smem > (size_t)dynamic_smem_limit(c->max_smem_optin)) return VP_E_UNSUPPORTED;
     KernelFn fn = pick_kernel(dc.g, L.lpg);
     if (!fn) return VP_E_UNSUPPORTED;
-    if (raise_dynamic_smem((const void*)fn, L.smem) != VP_OK) return VP_E_CUDA;
+    if (set_dynamic_smem_limit((const void*)fn, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, L.threads, L.smem) != cudaSuccess || per_sm < 1)
         return VP_E_CUDA;
@@ -1281,8 +1260,8 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
             const int threads = dc.G > 32 ? 384 : task_warps * 32 + (apart ? (dc.N + 31) / 32 * 32 : 0);
             const BigKernelFn bf = pick_big_kernel(dc, split);
             const size_t smem = (size_t)big_smem_layout(dc, kp).total;
-            if (smem + 2048 > (size_t)c->max_smem_optin) continue;
-            if (raise_dynamic_smem((const void*)bf, smem) != VP_OK) return VP_E_CUDA;
+            if (smem > (size_t)dynamic_smem_limit(c->max_smem_optin)) continue;
+            if (set_dynamic_smem_limit((const void*)bf, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
             int bper_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bper_sm, bf, threads, smem) != cudaSuccess) return VP_E_CUDA;
             const long long bcap = (long long)bper_sm * c->sm_count;
@@ -1304,8 +1283,8 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
         const WarpKernelFn wf = units ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;
         const int warps = B <= 4 * c->sm_count ? 1 : (B <= 8 * c->sm_count ? 2 : 4);
         const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
-        if (smem + 2048 <= (size_t)c->max_smem_optin) {
-            if (raise_dynamic_smem((const void*)wf, smem) != VP_OK) return VP_E_CUDA;
+        if (smem <= (size_t)dynamic_smem_limit(c->max_smem_optin)) {
+            if (set_dynamic_smem_limit((const void*)wf, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
             int wper_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper_sm, wf, warps * 32, smem) != cudaSuccess || wper_sm < 1)
                 return VP_E_CUDA;

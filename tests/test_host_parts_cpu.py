@@ -35,3 +35,38 @@ int main() {
     }
 }
 ''')
+
+
+def test_no_plan_lowers_a_kernels_shared_memory_limit(tmp_path):
+    """Launches are planned once and replayed: with many kernels on several devices, planned in any order and with any sizes, each
+    launch planned so far stays within its kernel's limit."""
+    _run(tmp_path, r'''
+#include "smem_limit.h"
+#include <map>
+#include <utility>
+#include <vector>
+constexpr int kOptin = 232448;
+static int device = 0;
+static std::map<std::pair<int, const void*>, int> limit;
+extern "C" cudaError_t cudaGetDevice(int* d) { *d = device; return cudaSuccess; }
+extern "C" cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute a, int value) {
+    assert(a == cudaFuncAttributeMaxDynamicSharedMemorySize && value <= kOptin);
+    limit[{device, fn}] = value;
+    return cudaSuccess;
+}
+int main() {
+    static char kernel[30];
+    struct Planned { int device; const void* fn; int bytes; };
+    std::vector<Planned> planned;
+    unsigned x = 1;
+    for (int i = 0; i < 4000; i++) {
+        x = x * 1664525u + 1013904223u;
+        device = (x >> 8) % 4;
+        const void* fn = &kernel[(x >> 16) % 30];
+        const int bytes = (int)((x >> 4) % (unsigned)(dynamic_smem_limit(kOptin) + 1));
+        assert(set_dynamic_smem_limit(fn, kOptin) == VP_OK);
+        planned.push_back({device, fn, bytes});
+        for (const Planned& p : planned) assert(p.bytes <= (limit[{p.device, p.fn}]));
+    }
+}
+''')
