@@ -518,7 +518,8 @@ int vp_memset_probe(void* device_buffer, size_t bytes, void* cuda_stream);
  * Work counters of the last vp_schedule_batch that used `workspace` (device): copies three
  * uint64 to host `out3` after synchronising the stream: activations emitted, (family, start)
  * binding tasks run, AA sweeps run over all tasks.  Used to count the algorithmic operations
- * of Section 4.2 "Planning complexity" for a measured batch.
+ * of Section 4.2 "Planning complexity" for a measured batch.  They mean nothing for a workspace that no batch
+ * has used; nothing beyond its first 256 bytes is read then.
  */
 int vp_schedule_read_stats(const void* workspace, void* cuda_stream, uint64_t* out3);
 

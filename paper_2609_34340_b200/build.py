@@ -11,7 +11,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libvariopath.so")
 CALLS = os.path.join(PKG, "_calls.so")
-SOURCES = ["catalog.cu", "schedule.cu", "pack.cu", "host_api.cu", "profile.cu", "plan_tools.cu", "analyzer.cu", "unpack.cu", "microbench.cu", "exchange.cu"]
+SOURCES = ["catalog.cu", "schedule.cu", "read_stats.cu", "pack.cu", "host_api.cu", "profile.cu", "plan_tools.cu", "analyzer.cu", "unpack.cu", "microbench.cu", "exchange.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC"]
 

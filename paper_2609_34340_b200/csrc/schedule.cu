@@ -32,7 +32,6 @@
 
 #include <cstring>
 #include <utility>
-#include <vector>
 
 #include "bulk_copy.cuh"
 #include "route_index.cuh"
@@ -1328,10 +1327,10 @@ int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* o
     return VP_OK;
 }
 
-// Workspace: 256 bytes of counters (work counter, list length, -, warps with counters of their own; sums for
-// vp_schedule_read_stats); the warp kernel's counters per warp; one residual slot per CTA of the general kernel when it keeps the residual outside
-// shared memory; with the kernel for large node-symmetric catalogs also the list of matrices left to the general
-// kernel, the work order and its keys.
+// Workspace: 256 bytes of counters (work counter, list length, and what vp_schedule_read_stats reads: see vp_stats_tag); the warp
+// kernel's counters per warp; one residual slot per CTA of the general kernel when it keeps the residual outside shared memory;
+// with the kernel for large node-symmetric catalogs also the list of matrices left to the general kernel, the work order and
+// its keys.
 struct WsLayout { size_t drem, slots, todo, order, key, total; };
 WsLayout ws_layout(const vp_catalog* c, const Launch& L, int B) {
     WsLayout w;
@@ -1448,21 +1447,5 @@ extern "C" int vp_schedule_launch_info(const vp_catalog* c, int B, const vp_sche
     out4[1] = L.kernel == 2 ? L.big_grid : L.grid;
     out4[2] = L.kernel == 2 ? L.big_threads : L.threads;
     out4[3] = (int32_t)(L.kernel == 2 ? L.big_smem : L.smem);
-    return VP_OK;
-}
-
-extern "C" int vp_schedule_read_stats(const void* workspace, void* cuda_stream, uint64_t* out3) {
-    if (!workspace || !out3) return VP_E_BAD_ARG;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    uint64_t head[32];
-    if (cudaMemcpyAsync(head, workspace, 256, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) return VP_E_CUDA;
-    const uint32_t warps = (uint32_t)(head[1] >> 32);            // warps with counters of their own
-    for (int i = 0; i < 3; i++) out3[i] = warps ? 0 : head[2 + i];
-    if (!warps) return VP_OK;
-    std::vector<uint64_t> slots((size_t)warps * 3);
-    if (cudaMemcpyAsync(slots.data(), (const char*)workspace + 256, slots.size() * 8, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return VP_E_CUDA;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) return VP_E_CUDA;
-    for (size_t i = 0; i < slots.size(); i++) out3[i % 3] += slots[i];
     return VP_OK;
 }

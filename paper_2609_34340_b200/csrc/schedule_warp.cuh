@@ -839,7 +839,11 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
         if (slots) {
             unsigned long long* const mine = slots + 3 * ((size_t)blockIdx.x * n_warps + warp);
             mine[0] = n_act; mine[1] = cnt.tasks; mine[2] = cnt.sweeps;
-            if (blockIdx.x == 0 && warp == 0) counter[3] = gridDim.x * (unsigned)n_warps;
+            if (blockIdx.x == 0 && warp == 0) {
+                const uint32_t warps = gridDim.x * (uint32_t)n_warps;
+                counter[3] = warps;
+                ((uint64_t*)counter)[kStatsTagWord] = vp_stats_tag((uint64_t)(uintptr_t)counter, warps);
+            }
         } else {
             unsigned long long* const stats = (unsigned long long*)(counter + 4);
             if (n_act) atomicAdd(&stats[0], n_act);

@@ -85,14 +85,25 @@ struct vp_launch_memo {
     unsigned char launch[192];    // the scheduler's Launch record
 };
 
-// Lanes per task (over lanes per group) of vp_schedule_big_kernel for a number of rank groups, and the stride of its credit
-// matrix, in words per row pair: rows of 128-bit reads, and 2 x stride = 8 modulo 16, so that neighbouring groups start in
-// different banks.
 #ifdef __CUDACC__
 #define VP_HD __host__ __device__
 #else
 #define VP_HD
 #endif
+
+// Work counters in the first 256 bytes of a scheduler workspace (32 words of 64 bits): sums in words 2 to 4 -- or, where every warp has
+// counters of its own behind the 256 bytes, three words each, the number of these warps in the upper half of word 1 and a tag in
+// word 31.  The launches that keep sums zero the 256 bytes; the tag holds the workspace's address and the number of warps, so that
+// whatever else may be in memory that no launch has used is not taken for a number of counters.
+constexpr int kStatsTagWord = 31;
+constexpr uint32_t kStatsMaxWarps = 16384;      // (at most the warps that are resident at once)
+VP_HD inline uint64_t vp_stats_tag(uint64_t workspace, uint32_t warps) {
+    return (workspace ^ 0x7661726970617468ull) + ((uint64_t)warps << 40) + warps;
+}
+
+// Lanes per task (over lanes per group) of vp_schedule_big_kernel for a number of rank groups, and the stride of its credit
+// matrix, in words per row pair: rows of 128-bit reads, and 2 x stride = 8 modulo 16, so that neighbouring groups start in
+// different banks.
 VP_HD inline constexpr int big_lanes(int G) { return G <= 8 ? 8 : (G <= 16 ? 16 : (G <= 32 ? 32 : 64)); }
 VP_HD inline constexpr int big_stride(int lanes) { return lanes * 4 + 4; }
 

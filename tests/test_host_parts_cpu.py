@@ -70,3 +70,60 @@ int main() {
     }
 }
 ''')
+
+
+def test_work_counters_of_any_workspace(tmp_path):
+    """vp_schedule_read_stats gets no workspace size: whatever a workspace holds that no launch has used, nothing beyond its first
+    256 bytes is read and nothing is allocated.  Sums, and counters of every warp, are read as they were written."""
+    _run(tmp_path, r'''
+#include <string.h>
+#include <vector>
+#include "vp_internal.h"
+static const char *lo, *hi;                      // the workspace
+static cudaError_t copy_result = cudaSuccess;
+extern "C" cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t) {
+    if (copy_result != cudaSuccess) return copy_result;
+    assert((const char*)src >= lo && n <= (size_t)(hi - (const char*)src));
+    memcpy(dst, src, n);
+    return cudaSuccess;
+}
+extern "C" cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+static void read(const std::vector<uint64_t>& ws, uint64_t* out, int want = VP_OK) {
+    lo = (const char*)ws.data(); hi = lo + ws.size() * 8;
+    out[0] = out[1] = out[2] = 99;
+    assert(vp_schedule_read_stats(ws.data(), nullptr, out) == want);
+}
+int main() {
+    uint64_t out[3], x = 1;
+    std::vector<uint64_t> ws(32);
+    auto zeros = [&] { return out[0] == 0 && out[1] == 0 && out[2] == 0; };
+    for (uint64_t fill : {~0ull, 0x0000040000000400ull, 0x5a5a5a5a5a5a5a5aull, 0x0000000100000001ull, 0ull}) {
+        ws.assign(32, fill);
+        read(ws, out);
+        assert(zeros());
+    }
+    for (int i = 0; i < 1000; i++) {             // random bytes, and a small number of warps beside them
+        for (uint64_t& w : ws) { x = x * 6364136223846793005ull + 1442695040888963407ull; w = x; }
+        if (i & 1) ws[1] = (uint64_t)(1 + i) << 32;
+        read(ws, out);
+        assert(zeros());
+    }
+    ws.assign(32, 0);                            // sums
+    ws[0] = 7; ws[2] = 11; ws[3] = 12; ws[4] = 13;
+    read(ws, out);
+    assert(out[0] == 11 && out[1] == 12 && out[2] == 13);
+    for (uint32_t warps : {1u, 255u, 256u, 257u, 9472u, kStatsMaxWarps}) {       // counters of every warp
+        ws.assign(32 + 3 * (size_t)warps, 0x5a5a5a5a5a5a5a5aull);
+        ws[1] = (uint64_t)warps << 32 | 0x5a5a5a5a;
+        ws[kStatsTagWord] = vp_stats_tag((uint64_t)(uintptr_t)ws.data(), warps);
+        for (uint32_t w = 0; w < warps; w++) { ws[32 + 3 * w] = 1; ws[33 + 3 * w] = w; ws[34 + 3 * w] = 3ull << 40; }
+        read(ws, out);
+        assert(out[0] == warps && out[1] == (uint64_t)warps * (warps - 1) / 2 && out[2] == (3ull << 40) * warps);
+        std::vector<uint64_t> moved(ws.begin(), ws.begin() + 32);                // the same bytes in another, shorter workspace
+        read(moved, out);
+        assert(zeros());
+    }
+    copy_result = cudaErrorInvalidValue;
+    read(ws, out, VP_E_CUDA);
+}
+''', "read_stats.cu")
