@@ -170,12 +170,12 @@ __global__ void __launch_bounds__(kIdxThreads) pack_count_kernel(PackArgs a, Pac
         }
         return;
     }
-    const long long E = (long long)a.T * a.topk, e0 = (long long)blockIdx.x * chunk, e1 = min(e0 + chunk, E);
+    const ChunkRange mine = chunk_range(blockIdx.x, chunk, (long long)a.T * a.topk);
     for (int j = tid; j < N; j += kIdxThreads) sm[j] = 0;
     __syncthreads();
     int bad = 0;
 #pragma unroll 4
-    for (long long e = e0 + tid; e < e1; e += kIdxThreads) {
+    for (long long e = mine.lo + tid; e < mine.hi; e += kIdxThreads) {
         const int j = dest_of(a.idx[e], a, bad);
         if (j >= 0) atomicAdd(&sm[j], 1);
     }
@@ -197,8 +197,8 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
     int* const next = sm + N + warp * N;
     for (int j = tid; j < N * (kIdxWarps + 1); j += kIdxThreads) sm[j] = 0;
     __syncthreads();
-    const long long E = (long long)a.T * a.topk, e0 = (long long)blockIdx.x * chunk, e1 = min(e0 + chunk, E);
-    const long long s0 = min(e0 + (long long)warp * (chunk / kIdxWarps), e1), s1 = min(s0 + chunk / kIdxWarps, e1);
+    const ChunkRange mine = chunk_range(blockIdx.x, chunk, (long long)a.T * a.topk);
+    const long long s0 = min(mine.lo + (long long)warp * (chunk / kIdxWarps), mine.hi), s1 = min(s0 + chunk / kIdxWarps, mine.hi);
     int ignore = 0;
     for (long long e = s0 + lane; e < s1; e += 32) {
         const int j = dest_of(a.idx[e], a, ignore);
@@ -283,7 +283,7 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
         }
     }
     const PackWs w = carve(workspace, N, T, topk, k_max);
-    const int chunk = chunk_items(E, N), n_chunks = (int)((E + chunk - 1) / chunk);
+    const int chunk = chunk_items(E, N), n_chunks = chunks_of((unsigned)E, chunk);
     vp_prof_mark(1, 0, stream);
     cudaError_t e = launch_after(pack_count_kernel, n_chunks + 1, kIdxThreads, (size_t)(N + runs_scratch_ints(N)) * 4, stream, a, w, chunk, n_chunks);
     if (e == cudaSuccess) e = launch_after(pack_map_kernel, n_chunks, kIdxThreads, (size_t)pack_map_ints(N, k_max) * 4, stream, a, w, chunk);

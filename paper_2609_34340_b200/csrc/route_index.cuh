@@ -15,11 +15,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chunks.h"
 #include "vp_internal.h"
 
 namespace {
 
-constexpr int kIdxThreads = 512;                    // threads of every index CTA
 constexpr int kIdxWarps = kIdxThreads / 32;
 constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
 // Items up to which one self-contained launch is used.  Its last CTA counts every item itself, and the rows move by plain loads
@@ -27,7 +27,6 @@ constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
 constexpr int kSmallItems = 8192;
 constexpr int kSmallSteps = 1024;                   // plan arrays longer than this do not fit its run table
 constexpr int kSmallOwn = 1024;                     // rows or copies one CTA may own there
-constexpr int kMinChunk = kIdxThreads;              // items per histogram of the chunked form, at least: one per thread
 
 // Division by the row size and by the experts per rank without a divide sequence: plan offsets are below 2^52, so the
 // product with the rounded reciprocal is off by one at most; expert ids are below 2^31 (multiply-high and shift, exact).
@@ -276,17 +275,6 @@ __device__ __forceinline__ void warp_positions(long long lo, long long hi, int* 
         __syncwarp();
         if (i < hi) put(i, k, p);
     }
-}
-
-// Items per chunk and chunks of the chunked form: a map CTA adds up the histograms of all chunks, so their number times the
-// keys is kept within 16 K words (16 chunks at least, however many keys there are).
-inline int chunk_items(long long items, int keys) {
-    long long most = 16384 / keys;
-    if (most > 512) most = 512;
-    if (most < 16) most = 16;
-    long long c = (items + most - 1) / most;
-    if (c < kMinChunk) c = kMinChunk;
-    return (int)((c + kIdxThreads - 1) / kIdxThreads * kIdxThreads);
 }
 
 // ---- moving the rows a CTA owns (the one-launch form) ------------------------------------------------------------

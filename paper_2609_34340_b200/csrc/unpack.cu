@@ -47,8 +47,7 @@ UnpackWs carve(void* base, int N, int keys, long long items, int k_max) {
     UnpackWs w;
     size_t o = 0;
     auto take = [&](size_t n) { size_t at = o; o += vp_align256(n); return (int32_t*)((char*)base + at); };
-    const long long chunk = chunk_items(items, keys);
-    const size_t n_chunks = (size_t)((items + chunk - 1) / chunk);
+    const size_t n_chunks = (size_t)chunks_of((unsigned)items, chunk_items(items, keys));
     w.flags = take(256);
     w.bad = take(n_chunks * 4);
     w.step_row = take((size_t)(k_max + 1) * 4);
@@ -293,9 +292,7 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_steps_kernel(UnpackArgs a,
     if (k0 + (int)threadIdx.x < k1) w.step_peer[k0 + threadIdx.x] = peer[threadIdx.x];
 }
 
-// Chunks in use: those that hold one of the R rows received (return direction: all of them).
-__device__ __forceinline__ int chunks_of(int items, int chunk) { return (items + chunk - 1) / chunk; }
-
+// (Chunks in use are those that hold one of the R rows received; return direction: all of them.)
 // steps: 0 the plan is read here, 1 its senders come from unpack_steps_kernel, 2 the same, and the tables stay in the
 // workspace because they exceed shared memory (every CTA then writes the same values there).
 __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a, UnpackWs w, int chunk, int steps) {
@@ -322,9 +319,9 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
         peer[k] = p;
     }
     __syncthreads();
-    const int r0 = blockIdx.x * chunk, r1 = min(r0 + chunk, R);
-    for (int r = r0 + tid; r < r1; r += kIdxThreads) {
-        const int key = row_key_of(a, r, a.item_expert[r], K, step_row, peer);
+    const ChunkRange mine = chunk_range(blockIdx.x, chunk, R);
+    for (long long r = mine.lo + tid; r < mine.hi; r += kIdxThreads) {
+        const int key = row_key_of(a, (int)r, a.item_expert[r], K, step_row, peer);
         w.item_key[r] = key;
         if (key >= 0) atomicAdd(&hist[key], 1);
         else bad = VP_ST_PACK_MISMATCH;
@@ -354,9 +351,9 @@ __global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a,
     }
     for (int j = tid; j < a.keys; j += kIdxThreads) sm[j] = 0;
     __syncthreads();
-    const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)a.items);
+    const ChunkRange mine = chunk_range(blockIdx.x, chunk, a.items);
 #pragma unroll 4
-    for (long long i = i0 + tid; i < i1; i += kIdxThreads) {
+    for (long long i = mine.lo + tid; i < mine.hi; i += kIdxThreads) {
         const int key = copy_key_of(a, a.item_expert[i]);
         if (key >= 0) atomicAdd(&sm[key], 1);
     }
@@ -386,9 +383,9 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, U
     auto key_of = [&](long long i) { return TOKENS ? copy_key_of(a, a.item_expert[i]) : w.item_key[i]; };
     long long s0, s1;
     auto count_slice = [&](int items) {
-        const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)items);
-        s0 = min(i0 + (long long)warp * (chunk / kIdxWarps), i1);
-        s1 = min(s0 + chunk / kIdxWarps, i1);
+        const ChunkRange own = chunk_range(blockIdx.x, chunk, items);
+        s0 = min(own.lo + (long long)warp * (chunk / kIdxWarps), own.hi);
+        s1 = min(s0 + chunk / kIdxWarps, own.hi);
         for (long long i = s0 + lane; i < s1; i += 32) {
             const int key = key_of(i);
             if (key >= 0) atomicAdd(&next[key], 1);
@@ -487,7 +484,7 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
         }
     }
     const UnpackWs w = carve(workspace, a.N, a.keys, items, a.k_max);
-    const int chunk = chunk_items(items, a.keys), n_chunks = (int)((items + chunk - 1) / chunk);
+    const int chunk = chunk_items(items, a.keys), n_chunks = chunks_of((unsigned)items, chunk);
     if (!inline_steps) e = launch_after(unpack_steps_kernel, (a.k_max + kStepTile - 1) / kStepTile, kIdxThreads, 0, stream, a, w);
     if (e == cudaSuccess) {
         if constexpr (TOKENS) {

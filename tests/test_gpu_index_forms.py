@@ -139,3 +139,35 @@ def test_put_alignments(vp, oracle_lib, nodes, T, topk, row_bytes):  # noqa: F81
             assert np.array_equal(got[at[j] + r:at[j] + r + n], np.asarray(want[j]).reshape(-1)[r:r + n]), (k, j)
             mask[at[j] + r:at[j] + r + n] = True
     assert (got[~mask] == 0xAB).all()                          # nothing else is touched
+
+
+@pytest.fixture
+def large():
+    """Gives the memory of a large test back to the device."""
+    yield
+    torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("tokens", [False, True])
+def test_unpack_at_the_accepted_limit(vp, large, tokens):  # noqa: F811
+    """2^31 - 1 rows of one byte, all of them in use: the last chunk ends where 32-bit indices do."""
+    R, dev = 2 ** 31 - 1, "cuda"
+    plan = vp.Plan.empty(1, 2, 1, dev)                         # one step: rank 0 sends to rank 1, or rank 1 returns to rank 0
+    plan.n_steps.fill_(1)
+    plan.lane_dst.copy_(torch.tensor([[[-1, 0] if tokens else [1, -1]]]))
+    plan.lane_bytes.copy_(torch.tensor([[[0, R] if tokens else [R, 0]]]))
+    plan.recv_off.copy_(torch.tensor([[[0, 0], [R, 0] if tokens else [0, R]]]))
+    recv = torch.randint(-2 ** 63, 2 ** 63 - 1, (2 ** 28,), device=dev).view(torch.uint8)[:R].view(R, 1)
+    expert = torch.randint(-2 ** 63, 2 ** 63 - 1, (2 ** 28,), device=dev).view(torch.uint8)[:R].to(torch.int32) & 1
+    out = torch.zeros_like(recv)
+    if tokens:                                                 # experts 2 and 3 live on rank 1
+        st = vp.unpack_tokens(plan, 0, 0, (expert + 2).view(R, 1), 2, recv, out)
+    else:
+        off, st = vp.unpack(plan, 0, 1, recv, expert, 2, out)
+    first = expert == 0
+    n = int(first.sum())
+    if not tokens:
+        assert off.tolist() == [0, n, R]
+    assert int(st.item()) == 0
+    a, b = (out, recv) if tokens else (recv, out)              # a in the order of the routing, b sorted by expert
+    assert torch.equal(a[first], b[:n]) and torch.equal(a[~first], b[n:])

@@ -127,3 +127,31 @@ int main() {
     read(ws, out, VP_E_CUDA);
 }
 ''', "read_stats.cu")
+
+
+def test_chunks_cover_every_item_up_to_the_accepted_limit(tmp_path):
+    """The chunked index forms accept up to 2^31 - 1 items: the chunks cover all of them once, in order, however many of them a
+    call turns out to use."""
+    _run(tmp_path, r'''
+#include "chunks.h"
+int main() {
+    const long long most = (1ll << 31) - 1;
+    for (long long items : {1ll, 511ll, 512ll, 8193ll, 1ll << 20, (1ll << 20) + 1, 1ll << 27, most - (1 << 20), most - 512, most - 1, most})
+        for (int keys : {1, 2, 16, 33, 256, 1000, 1024}) {
+            const int chunk = chunk_items(items, keys);
+            assert(chunk > 0 && chunk % kIdxThreads == 0);
+            for (long long used : {items, items - 1, items / 2, 1ll}) {
+                if (used < 1) continue;
+                const int n = chunks_of((unsigned)used, chunk);
+                assert(n >= 1 && n <= 512 && n <= chunks_of((unsigned)items, chunk));
+                long long at = 0;
+                for (int b = 0; b < n; b++) {
+                    const ChunkRange c = chunk_range(b, chunk, used);
+                    assert(c.lo == at && c.hi > c.lo && c.hi - c.lo <= chunk);
+                    at = c.hi;
+                }
+                assert(at == used);
+            }
+        }
+}
+''')
