@@ -267,7 +267,7 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
                      expert_idx, row_div(row_bytes), staged_capacity_bytes, src_map, status};
     const int sms = sm_count_of_device();
     if (!sms) return VP_E_CUDA;
-    if (E <= kSmallItems && k_max <= kSmallSteps) {
+    if (E <= kSmallItems && k_max <= kSmallSteps && row_bytes <= kSmallRow) {
         const SmallSplit s = small_split(T, sms);
         const int n_cta = s.grid / s.pieces;
         if ((long long)((T + n_cta - 1) / n_cta) * topk <= kSmallOwn) {

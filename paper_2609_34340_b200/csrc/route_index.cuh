@@ -27,6 +27,7 @@ constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
 constexpr int kSmallItems = 8192;
 constexpr int kSmallSteps = 1024;                   // plan arrays longer than this do not fit its run table
 constexpr int kSmallOwn = 1024;                     // rows or copies one CTA may own there
+constexpr int64_t kSmallRow = (int64_t)1 << 30;     // bytes per row: up to here 32 bits number the vectors of a row
 
 // Division by the row size and by the experts per rank without a divide sequence: plan offsets are below 2^52, so the
 // product with the rounded reciprocal is off by one at most; expert ids are below 2^31 (multiply-high and shift, exact).

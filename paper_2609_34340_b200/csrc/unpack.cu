@@ -466,7 +466,7 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
     const bool steps_fit = ((long long)a.keys + 2ll * a.k_max) * 4 <= (long long)kSmemLimit;
     const bool inline_steps = (long long)a.k_max * a.N <= kInlineCells && steps_fit;
     cudaError_t e = cudaSuccess;
-    if (items <= kSmallItems && a.k_max <= kSmallSteps && inline_steps) {
+    if (items <= kSmallItems && a.k_max <= kSmallSteps && inline_steps && a.row.d <= kSmallRow) {
         const SmallSplit s = small_split(a.items, sms);
         const int n_cta = s.grid / s.pieces;
         const size_t smem = (size_t)unpack_small_layout(a.N, a.keys, a.k_max, TOKENS).ints * 4;

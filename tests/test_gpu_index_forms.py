@@ -171,3 +171,31 @@ def test_unpack_at_the_accepted_limit(vp, large, tokens):  # noqa: F811
     assert int(st.item()) == 0
     a, b = (out, recv) if tokens else (recv, out)              # a in the order of the routing, b sorted by expert
     assert torch.equal(a[first], b[:n]) and torch.equal(a[~first], b[n:])
+
+
+@pytest.mark.parametrize("row_bytes,topk", [(2 ** 31 + 3, 1), (2 ** 31 + 3, 8193), (2 ** 33 + 4, 1)])
+def test_rows_of_more_than_2_gb(vp, large, row_bytes, topk):  # noqa: F811
+    """A row of more vectors (of one and four bytes) than 32 bits number: packed, unpacked and returned whole, by calls of few
+    copies and of many (most of them dropped)."""
+    plan = vp.Plan.empty(1, 2, 1, "cuda")
+    row = torch.randint(-2 ** 63, 2 ** 63 - 1, (row_bytes // 8 + 1,), device="cuda").view(torch.uint8)[:row_bytes].view(1, row_bytes)
+    idx = torch.full((1, topk), -1, dtype=torch.int32, device="cuda")
+    idx[0, -1] = 1                                             # one copy, to rank 1
+
+    def set_plan(src, dst):
+        plan.n_steps.fill_(1)
+        plan.lane_dst.fill_(-1)[0, 0, src] = dst
+        plan.lane_bytes.zero_()[0, 0, src] = row_bytes
+        plan.send_off.zero_()[0, 1, src] = row_bytes
+        plan.recv_off.zero_()[0, 1, dst] = row_bytes
+
+    set_plan(0, 1)
+    out = torch.zeros_like(row)
+    assert int(vp.pack(plan, 0, 0, idx, 1, row, out).item()) == 0 and torch.equal(out, row)
+    out.zero_()
+    off, st = vp.unpack(plan, 0, 1, row, torch.zeros(1, dtype=torch.int32, device="cuda"), 1, out)
+    assert int(st.item()) == 0 and off.tolist() == [0, 1] and torch.equal(out, row)
+    if topk == 1:
+        set_plan(1, 0)
+        out.zero_()
+        assert int(vp.unpack_tokens(plan, 0, 0, idx, 1, row, out).item()) == 0 and torch.equal(out, row)
