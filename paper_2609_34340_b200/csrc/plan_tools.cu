@@ -63,11 +63,16 @@ plan_time_kernel(const uint32_t* __restrict__ inst_wdiv, int n_inst, int64_t W, 
 // Many sources: bound by the additions in shared memory; a loop of its own for a single source (no division), 16-byte loads and one wave of
 // CTAs took 256 sources x 12,833 tokens x 8 from 103 to 41 us, one source x 16,384 x 8 from 10.9 to 6.3.
 constexpr int kDemandCells = 4096;                 // group x N at most
+// WIDE: a CTA has more than 2^kDemandCarry copies of one source; it moves the high bits of its counts on after every so many, and the
+// row is a 64-bit sum.  (As a case at run time it cost one source of a few thousand copies 4.5 -> 4.8 us.)
+constexpr int kDemandCarry = 28;
+template <bool WIDE>
 __global__ void __launch_bounds__(kIdxThreads)
 demand_kernel(const int32_t* __restrict__ idx, int n_src, int group, long long per_src, SmallDiv by_epr, int N, int src0,
               long long row_bytes, int64_t* __restrict__ demand_rows, int32_t* __restrict__ status) {
     namespace cg = cooperative_groups;
     __shared__ unsigned int cnt[kDemandCells];
+    __shared__ unsigned int carried[WIDE ? VP_MAX_N : 1];     // counts in units of 2^kDemandCarry
     __shared__ int s_bad;
     const cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, rank = (int)cluster.block_rank(), n_cta = (int)cluster.num_blocks();
@@ -84,9 +89,8 @@ demand_kernel(const int32_t* __restrict__ idx, int n_src, int group, long long p
         if (j >= N) { bad = 1; return; }
         atomicAdd(&cnt[first + j], 1u);
     };
-    if (ns == 1) {                                 // one source: 16 bytes at a time between the first and the last aligned address
-        const int32_t* const from = x0 + lo;
-        const long long n = hi - lo, head = min(n, (long long)((16 - ((uintptr_t)from & 15)) & 15) / 4), quads = (n - head) / 4;
+    auto count_run = [&](const int32_t* from, long long n) {   // 16 bytes at a time between the first and the last aligned address
+        const long long head = min(n, (long long)((16 - ((uintptr_t)from & 15)) & 15) / 4), quads = (n - head) / 4;
         const int4* const v = (const int4*)(from + head);
         if (tid < head) count(from[tid], 0);
 #pragma unroll 4
@@ -96,6 +100,17 @@ demand_kernel(const int32_t* __restrict__ idx, int n_src, int group, long long p
         }
         const long long e = head + quads * 4 + tid;
         if (e < n) count(from[e], 0);
+    };
+    if (WIDE) {
+        for (int j = tid; j < N; j += kIdxThreads) carried[j] = 0;
+        for (long long at = lo; at < hi; at += 1ll << kDemandCarry) {
+            count_run(x0 + at, min(1ll << kDemandCarry, hi - at));
+            __syncthreads();
+            for (int j = tid; j < N; j += kIdxThreads) { carried[j] += cnt[j] >> kDemandCarry; cnt[j] &= (1u << kDemandCarry) - 1; }
+            __syncthreads();
+        }
+    } else if (ns == 1) {
+        count_run(x0 + lo, hi - lo);
     } else {                                       // (a 64-bit division per copy)
 #pragma unroll 8
         for (long long e = lo + tid; e < hi; e += kIdxThreads) count(x0[e], (int)(e / per_src) * N);
@@ -106,8 +121,11 @@ demand_kernel(const int32_t* __restrict__ idx, int n_src, int group, long long p
     for (int j = rank * kIdxThreads + tid; j < cells; j += n_cta * kIdxThreads) {
         unsigned int n = 0;
         for (int c = 0; c < n_cta; c++) n += cluster.map_shared_rank(cnt, c)[j];
+        long long copies = n;
+        if (WIDE)
+            for (int c = 0; c < n_cta; c++) copies += (long long)cluster.map_shared_rank(carried, c)[j] << kDemandCarry;
         const int s = s0 + j / N, d = j % N;       // D_ii = 0: self traffic is handled locally (Section 3)
-        demand_rows[(size_t)s * N + d] = d == src0 + s ? 0 : (int64_t)n * row_bytes;
+        demand_rows[(size_t)s * N + d] = d == src0 + s ? 0 : copies * row_bytes;
     }
     if (rank == 0 && tid == 0) {
         for (int c = 1; c < n_cta; c++) bad |= *cluster.map_shared_rank(&s_bad, c);
@@ -166,7 +184,8 @@ extern "C" int vp_demand_from_routing(const int32_t* expert_idx, int n_src, int 
     cfg.attrs = at;
     cfg.numAttrs = ctas > 1 ? 2 : 1;
     g_vp_launches++;
-    return cudaLaunchKernelEx(&cfg, demand_kernel, expert_idx, n_src, group, per_src, small_div(experts_per_rank), N, src0,
+    const auto kernel = items > (long long)ctas << kDemandCarry ? demand_kernel<true> : demand_kernel<false>;
+    return cudaLaunchKernelEx(&cfg, kernel, expert_idx, n_src, group, per_src, small_div(experts_per_rank), N, src0,
                               (long long)row_bytes, demand_rows, status) == cudaSuccess ? VP_OK : VP_E_CUDA;
 }
 

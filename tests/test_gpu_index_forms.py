@@ -199,3 +199,11 @@ def test_rows_of_more_than_2_gb(vp, large, row_bytes, topk):  # noqa: F811
         set_plan(1, 0)
         out.zero_()
         assert int(vp.unpack_tokens(plan, 0, 0, idx, 1, row, out).item()) == 0 and torch.equal(out, row)
+
+
+def test_demand_of_more_copies_than_32_bits_count(vp, large):  # noqa: F811
+    """More than 2^32 copies from one source to one rank."""
+    idx = torch.zeros((1, 2 ** 29 + 1, 8), dtype=torch.int32, device="cuda")
+    idx[0, 7, :3], idx[0, -1, 0] = 1, -1                       # three copies to the source itself, one dropped
+    got, st = vp.demand_from_routing(idx, 1, 2, 3, src0=1)
+    assert int(st.item()) == 0 and got.tolist() == [[3 * (2 ** 32 + 8 - 4), 0]]
