@@ -1,6 +1,7 @@
 """Build the CUDA library in-tree for sm_100a: ``python -m paper_2609_34340_b200.build``."""
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -24,6 +25,16 @@ def _stale(target: str, sources) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _built_for() -> str:
+    """What the extension module depends on besides its sources: torch's C++ interface and Python's."""
+    return f"torch {importlib.metadata.version('torch')}, python {sysconfig.get_config_var('SOABI')}"
+
+
+def _calls_stale() -> bool:
+    stamp = CALLS + ".built_for"
+    return _stale(CALLS, ["calls.cpp"]) or not os.path.exists(stamp) or open(stamp).read() != _built_for()
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile ``csrc/*.cu`` into ``libvariopath.so`` (no GPU needed: nvcc cross-compiles) and ``csrc/calls.cpp``, the
     binding's frequent calls, into ``_calls.so``."""
@@ -36,7 +47,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas=-v")
             print(" ".join(cmd))
         subprocess.check_call(cmd)
-    if force or _stale(CALLS, ["calls.cpp"]):
+    if force or _calls_stale():
         import torch
         at = os.path.dirname(torch.__file__)
         cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
@@ -48,6 +59,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd += [os.path.join(CSRC, "calls.cpp"), "-o", CALLS, "-L" + os.path.join(at, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10",
                 "-lc10_cuda", "-L" + PKG, "-l:libvariopath.so", "-Wl,-rpath,$ORIGIN"]
         subprocess.check_call(cmd)
+        with open(CALLS + ".built_for", "w") as f:
+            f.write(_built_for())
     return LIB
 
 

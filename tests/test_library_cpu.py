@@ -186,3 +186,27 @@ def test_argmax_classes_reproduce_every_shape(nodes, nic_bw):
                 assert rows_of_shape[run_start + place] == (p0, p1), (cl, run_start, place)
                 seen[run_start + place] += 1
     assert (seen == 1).all()
+
+
+def test_extension_is_built_again_for_another_torch_or_python(monkeypatch, tmp_path):
+    """The binding's extension module is compiled against one torch and one Python: a build under others compiles it again, a
+    build under the same does not."""
+    import importlib.metadata
+    import sysconfig
+    import paper_2609_34340_b200.build as b
+    b.build()
+    compiled = []
+    monkeypatch.setattr(b, "CALLS", str(tmp_path / "_calls.so"))
+    monkeypatch.setattr(b.subprocess, "check_call", lambda cmd: (compiled.append(cmd[0]), open(b.CALLS, "w").close()))
+    b.build()
+    b.build()
+    assert compiled == ["g++"]                                # not there, then up to date
+    version, soabi = importlib.metadata.version, sysconfig.get_config_var
+    monkeypatch.setattr(importlib.metadata, "version", lambda name: "99.0" if name == "torch" else version(name))
+    b.build()
+    b.build()
+    assert compiled == ["g++"] * 2
+    monkeypatch.setattr(sysconfig, "get_config_var", lambda name: "cpython-399" if name == "SOABI" else soabi(name))
+    b.build()
+    b.build()
+    assert compiled == ["g++"] * 3
