@@ -71,6 +71,7 @@ def _load():
         raise RuntimeError(f"{_LIB_PATH} is missing: build it with `python -m paper_2609_34340_b200.build` "
                            "(there is no CPU fallback)")
     lib = C.CDLL(_LIB_PATH)
+    # (no signatures for the calls of a step: those go through the extension module)
     vp, i32, i64, sz, P = C.c_void_p, C.c_int, C.c_int64, C.c_size_t, C.c_void_p
     lib.vp_load_catalog.argtypes = [P, sz, P, sz, i32, C.POINTER(vp)]
     lib.vp_free_catalog.argtypes = [vp]
@@ -79,39 +80,30 @@ def _load():
     lib.vp_catalog_argmax_classes.argtypes = [vp, P, sz, C.POINTER(sz)]
     lib.vp_schedule_workspace_bytes.argtypes = [vp, i32, C.POINTER(_Params)]
     lib.vp_schedule_workspace_bytes.restype = sz
-    sched_args = [vp, C.POINTER(_Params), P, P, i32] + [P] * 9
-    lib.vp_schedule_batch.argtypes = sched_args + [P, sz, P]
     lib.vp_schedule_host_scratch_bytes.argtypes = [vp, i32, C.POINTER(_Params)]
     lib.vp_schedule_host_scratch_bytes.restype = sz
-    lib.vp_schedule_batch_host.argtypes = sched_args + [P, sz, P]
-    lib.vp_schedule_batch_host_used.argtypes = sched_args + [P, sz, P]
     lib.vp_pack_workspace_bytes.argtypes = [i32, i32, i32, i32]
     lib.vp_pack_workspace_bytes.restype = sz
     pack_args = [P, P, P, P, i32, i32, i32, P, i32, i32, i32, P, i64, P, i64, P, P]
-    lib.vp_pack.argtypes = pack_args + [P, sz, P]
     lib.vp_pack_static.argtypes = pack_args + [P]
     lib.vp_pack_host_scratch_bytes.argtypes = [i32, i32, i32, i32, i64, i64]
     lib.vp_pack_host_scratch_bytes.restype = sz
     lib.vp_pack_host.argtypes = pack_args + [P, sz, P]
     lib.vp_unpack_workspace_bytes.argtypes = [i32, i64, i32, i32]
     lib.vp_unpack_workspace_bytes.restype = sz
-    lib.vp_unpack.argtypes = [P, P, P, i32, i32, i32, P, i64, i64, P, i32, P, P, P, P, P, P, sz, P]
     lib.vp_unpack_tokens_workspace_bytes.argtypes = [i32, i32, i32, i32, i64, i32]
     lib.vp_unpack_tokens_workspace_bytes.restype = sz
-    lib.vp_unpack_tokens.argtypes = [P, P, P, P, i32, i32, i32, P, i32, i32, i32, P, i64, i64, P, P, P, P, sz, P]
     lib.vp_kernel_launch_count.restype = i64
     lib.vp_build_catalog.argtypes = [P, sz, P, sz, C.POINTER(sz), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     lib.vp_build_template_catalog.argtypes = [P, sz, P, sz, C.POINTER(sz), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     lib.vp_prune_paths.argtypes = [P, sz, P, sz, C.POINTER(sz), C.POINTER(C.c_int32)]
     lib.vp_plan_time.argtypes = [vp, i32, i32, P, P, P, i64, P, P]
-    lib.vp_demand_from_routing.argtypes = [P, i32, i32, i32, i32, i32, i32, i64, P, P, P]
     lib.vp_sweep_workspace_bytes.argtypes = [vp, i32, C.POINTER(_Params)]
     lib.vp_sweep_workspace_bytes.restype = sz
     lib.vp_sweep_plan_time.argtypes = [vp, C.POINTER(_Params), P, i32, P, i32, P, i32, P, P, P, P, sz, P]
     lib.vp_schedule_read_stats.argtypes = [P, P, P]
     lib.vp_schedule_launch_info.argtypes = [vp, i32, C.POINTER(_Params), P]
     lib.vp_microbench.argtypes = [i32, i32, P, C.POINTER(i64), P]
-    lib.vp_exchange_put.argtypes = [P, P, P, P, i32, i32, i32, P, P, P, P, P, P]
     lib.vp_exchange_wait.argtypes = [P, P, i32, i32, i32, P, C.c_uint64, C.c_uint32, P, P]
     lib.vp_memset_probe.argtypes = [P, sz, P]
     lib.vp_profile_enable.argtypes = [i32]
