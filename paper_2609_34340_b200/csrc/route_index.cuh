@@ -29,8 +29,8 @@ constexpr int kSmallSteps = 1024;                   // plan arrays longer than t
 constexpr int kSmallOwn = 1024;                     // rows or copies one CTA may own there
 constexpr int64_t kSmallRow = (int64_t)1 << 30;     // bytes per row: up to here 32 bits number the vectors of a row
 
-// Division by the row size and by the experts per rank without a divide sequence: plan offsets are below 2^52, so the
-// product with the rounded reciprocal is off by one at most; expert ids are below 2^31 (multiply-high and shift, exact).
+// Division by the row size without a divide sequence: plan offsets are below 2^52, so the product with the rounded
+// reciprocal is off by one at most.
 struct RowDiv {
     int64_t d;
     double inv;
@@ -43,6 +43,9 @@ struct RowDiv {
     }
 };
 inline RowDiv row_div(int64_t d) { return RowDiv{d, 1.0 / (double)d}; }
+// Division by the experts per rank: unsigned division by an invariant integer after Granlund and Montgomery ("Division by Invariant
+// Integers using Multiplication", PLDI 1994, Section 4).  With l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1 the quotient is
+// (mulhi(m, x) + x) >> l; the sum needs 33 bits in general, 32 for the expert ids here, which are below 2^31.
 struct SmallDiv {
     uint32_t m;
     int shift;
