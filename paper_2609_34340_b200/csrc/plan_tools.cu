@@ -161,6 +161,8 @@ extern "C" int vp_demand_from_routing(const int32_t* expert_idx, int n_src, int 
         src0 + n_src > N || row_bytes <= 0 || row_bytes >= VP_ENTRY_LIMIT)
         return VP_E_BAD_ARG;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
+    const int sms = sm_count_of_device();
+    if (!sms) return VP_E_CUDA;
     const long long per_src = (long long)T * topk, total = per_src * n_src;
     // Few copies from few sources: one cluster counts them all and writes the status itself.  Otherwise a cluster per source,
     // which share the status word.
@@ -169,9 +171,9 @@ extern "C" int vp_demand_from_routing(const int32_t* expert_idx, int n_src, int 
     if (group < n_src && cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess) return VP_E_CUDA;
     const long long items = group * per_src;
     int ctas = 1;
-    // four copies per thread, then more CTAs, up to one wave of them: every further wave is another launch latency and trip to memory
+    // four copies per thread, then more CTAs, up to one wave of them (four per SM): every further wave is another launch latency and trip to memory
     const int groups = (n_src + group - 1) / group;
-    while (ctas < 8 && (long long)ctas * 4 * kIdxThreads < items && (ctas == 1 || groups * ctas * 2 <= 148 * 4)) ctas *= 2;
+    while (ctas < 8 && (long long)ctas * 4 * kIdxThreads < items && (ctas == 1 || groups * ctas * 2 <= 4 * sms)) ctas *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(groups * ctas));
     cfg.blockDim = dim3(kIdxThreads);

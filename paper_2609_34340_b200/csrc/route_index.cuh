@@ -57,6 +57,20 @@ inline SmallDiv small_div(int d) {
     return SmallDiv{(uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << l) - (uint64_t)d)) / (uint64_t)d + 1), l};
 }
 
+// SMs of the current device, asked once per device.
+inline int sm_count_of_device() {
+    static int s_sms[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const bool cached = dev >= 0 && dev < 64;
+    int sms = cached ? __atomic_load_n(&s_sms[dev], __ATOMIC_RELAXED) : 0;
+    if (!sms) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        if (cached) __atomic_store_n(&s_sms[dev], sms, __ATOMIC_RELAXED);
+    }
+    return sms;
+}
+
 // Launch that may start while the kernel ahead of it in the stream drains (its griddepcontrol.wait holds it back).
 template <typename... P, typename... A>
 inline cudaError_t launch_after(void (*fn)(P...), int grid, int threads, size_t smem, cudaStream_t stream, A... args) {

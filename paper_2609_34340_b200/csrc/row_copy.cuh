@@ -187,20 +187,6 @@ __global__ void __launch_bounds__(256) row_copy_plain_kernel(RowCopy c) {
     }
 }
 
-// SMs of the current device, asked once per device.
-inline int sm_count_of_device() {
-    static int s_sms[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    const bool cached = dev >= 0 && dev < 64;
-    int sms = cached ? __atomic_load_n(&s_sms[dev], __ATOMIC_RELAXED) : 0;
-    if (!sms) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-        if (cached) __atomic_store_n(&s_sms[dev], sms, __ATOMIC_RELAXED);
-    }
-    return sms;
-}
-
 // Widest vector (bytes) that source, destination and row size allow.
 inline int copy_width(const void* rows, const void* out, long long row_bytes) {
     const uintptr_t mix = (uintptr_t)rows | (uintptr_t)out | (uintptr_t)row_bytes;

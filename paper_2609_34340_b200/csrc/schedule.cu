@@ -1299,16 +1299,14 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     return VP_OK;
 }
 
-// plan_launch_uncached through the catalog's memo.  A launch depends on B only through min(B, one wave) -- except for
-// the switch to the warp kernel, which happens exactly when B exceeds the general kernel's wave -- so batches are
-// keyed by min(B, 65536) and a cached launch is reused when its own grid rule gives the same answer.  The memo is not
-// locked: calls that share a catalog handle from several host threads must be serialised by the caller (as must
-// anything else that shares a workspace).
+// plan_launch_uncached through the catalog's memo of the last four launches, by batch size and parameters.  A hit saves what the
+// attributes and occupancies cost: 0.5 us of host time, 1.6 at the most.  The memo is not locked: calls that share a catalog
+// handle from several host threads must be serialised by the caller (as must anything else that shares a workspace).
 int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* out) {
     vp_catalog* c = const_cast<vp_catalog*>(cc);
     if (!c || !p) return VP_E_BAD_ARG;
     for (vp_launch_memo& m : c->memo) {
-        if (!m.valid || m.B_class != B || m.k_target != p->k_target || m.n_start != p->n_start || m.i_aa != p->i_aa ||
+        if (!m.valid || m.B != B || m.k_target != p->k_target || m.n_start != p->n_start || m.i_aa != p->i_aa ||
             m.k_max != p->k_max || m.lambda_ns != p->lambda_ns || m.granule != p->granule_bytes)
             continue;
         memcpy(out, m.launch, sizeof(Launch));
@@ -1319,7 +1317,7 @@ int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* o
     if (rc) return rc;
     vp_launch_memo& m = c->memo[c->memo_next];
     c->memo_next = (c->memo_next + 1) % (int)(sizeof(c->memo) / sizeof(c->memo[0]));
-    m.valid = 1; m.B_class = B;
+    m.valid = 1; m.B = B;
     m.k_target = p->k_target; m.n_start = p->n_start; m.i_aa = p->i_aa; m.k_max = p->k_max;
     m.lambda_ns = p->lambda_ns; m.granule = p->granule_bytes;
     memcpy(m.launch, &L, sizeof(Launch));

@@ -76,10 +76,10 @@ struct DevCat {
     int64_t bw_max, W;
 };
 
-// A launch shape worked out once per (catalog, batch class, parameters) and reused by later calls.
+// A launch shape worked out once per (catalog, batch size, parameters) and reused by later calls.
 struct vp_launch_memo {
     int valid;
-    int B_class;                  // min(B, CTAs of one wave + 1): batches of one class launch alike up to the grid size
+    int B;
     int32_t k_target, n_start, i_aa, k_max;
     int64_t lambda_ns, granule;
     unsigned char launch[192];    // the scheduler's Launch record
