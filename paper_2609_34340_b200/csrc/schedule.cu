@@ -1242,29 +1242,43 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     // general kernel anyway, those go there directly.)
     if (dc.g == 4 && dc.G <= 64 && dc.sym && dc.shape_pat && dc.n_patterns < 1024 && dc.n_classes <= 15 &&
         (dc.G >= 16 || p->granule_bytes >= 256)) {
-        // Four tasks as a rule (one family, four starts).  While the batch leaves SMs room, two lanes per group and warps of
-        // their own that emit; then one lane per group and such warps; once the batch exceeds that wave, CTAs of task warps
-        // only, which pack the SMs.  The families' tables are staged where that costs no CTA.  More than 32 groups: one CTA per SM, two
-        // warps per task, which emit as well.
-        for (int option = 0; option < 6; option++) {
-            if (dc.G > 32 && option < 4) continue;
-            const int split = option < 2 ? 2 : 1;
-            const bool apart = option < 4;                       // warps of their own for the emit step
+        // Four tasks as a rule (one family, four starts).  The first of these shapes whose wave holds the batch is taken:
+        //   0  two lanes per group, warps of their own that emit, the families' tables staged
+        //   1  the same, tables in L2
+        //   2  one lane per group and emit warps (9 to 32 groups)
+        //   3  one lane per group, task warps only: these CTAs pack the SMs and take any batch
+        // Above 32 groups a CTA has its SM to itself, two warps per task, which emit as well: 3, with the tables staged if they fit and
+        // the batch is one wave.
+        // Measured on both sides of each line, microseconds for a batch of MoE matrices, last batch in the wave and one more:
+        //   0 | 1:  64 ranks 148: 820 | 838, 149: 1,328 | 838.  Staging gives 1 to 2 % at 40 to 64 ranks and nothing at 24 and 32; with one
+        //           lane per group it was never faster (32 ranks, 741 and 1,184: 535 and 628 staged, 525 and 619 not)
+        //   1 | 2:  64 ranks 296: 890 | 1,053, 297: 1,384 | 1,063;  96 ranks 148: 1,460 | 1,436, 149: 2,480 | 1,509 (17 to 32 groups: two
+        //           lanes are two warps per task, 5 % faster on sequence-parallel matrices, 1 to 6 % slower on MoE ones)
+        //   2 | 3:  64 ranks 297: 1,063 | 1,088, 592: 1,243 | 1,239, 593: 1,781 | 1,272;  96 ranks 296: 1,665 | 1,746, 297: 2,652 | 1,829
+        //   1 | 3 up to 8 groups:  32 ranks 740: 468 | 516, 741: 644 | 512;  1,184 by shape 2: 619, by 3: 534
+        for (int shape = dc.G > 32 ? 3 : 0; shape < 4; shape++) {
+            if (shape == 2 && dc.G <= 8) continue;
+            const int split = shape < 2 ? 2 : 1;
+            const bool apart = shape < 3;                        // warps of their own for the emit step
             const int lanes = big_lanes(dc.G) * split, task_warps = lanes * 4 / 32;
             KParams kp = L.kp;
-            kp.big_stage = option % 2 == 0;
+            kp.big_stage = shape == 0 || (dc.G > 32 && B <= c->sm_count);
             kp.big_cross = lanes == 64;
             kp.big_task_warps = task_warps;
             kp.big_emit_warp = apart ? task_warps : 0;
             const int threads = dc.G > 32 ? 384 : task_warps * 32 + (apart ? (dc.N + 31) / 32 * 32 : 0);
             const BigKernelFn bf = pick_big_kernel(dc, split);
-            const size_t smem = (size_t)big_smem_layout(dc, kp).total;
+            size_t smem = (size_t)big_smem_layout(dc, kp).total;
+            if (shape == 3 && kp.big_stage && smem > (size_t)dynamic_smem_limit(c->max_smem_optin)) {
+                kp.big_stage = 0;
+                smem = (size_t)big_smem_layout(dc, kp).total;
+            }
             if (smem > (size_t)dynamic_smem_limit(c->max_smem_optin)) continue;
             if (set_dynamic_smem_limit((const void*)bf, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
             int bper_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bper_sm, bf, threads, smem) != cudaSuccess) return VP_E_CUDA;
             const long long bcap = (long long)bper_sm * c->sm_count;
-            if (bper_sm < 1 || (bcap < B && option < 5)) continue;   // (the last option packs the SMs)
+            if (bper_sm < 1 || (bcap < B && shape < 3)) continue;
             L.kernel = 2; L.kp = kp; L.big_split = split; L.big_threads = threads; L.big_smem = smem;
             L.big_grid = (int)(B < bcap ? B : bcap);
             L.wave = (int)bcap;
@@ -1275,8 +1289,11 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     // Small topologies (groups of four, at most four groups, plain D-hat scores): one warp per matrix.  It has no block
     // barriers and less work per activation than a CTA per matrix, and wins at every batch size once the matrices run
     // in 32-bit granule units (granule >= 256 bytes; the choice between units and bytes is made per matrix, so the
-    // granule decides here); with smaller granules only when the batch exceeds the CTAs of one wave.  Up to four
-    // matrices per SM get a CTA of one warp each (a scheduler to themselves), larger batches two or four warps per CTA.
+    // granule decides here); with smaller granules when the batch exceeds the CTAs of one wave (16 ranks, granule 64, CTA | warp
+    // per matrix: 296 matrices 224 | 234 us, 592 275 | 232, 593 362 | 257: between two and four matrices per SM a warp is already
+    // the faster one).  Up to four matrices per SM get a CTA of one warp each (a scheduler to themselves: 64 matrices of 16 ranks
+    // 114.8 us, in pairs 117.6; 592 and 593 the same), larger batches two warps per CTA and beyond eight per SM four, which
+    // measure the same (1,185 matrices 134 and 136 us; CTAs of one warp 189: an SM holds eight of them).
     if (dc.g == 4 && dc.G <= 4 && !dc.sym && (B > cap || p->granule_bytes >= 256)) {
         const bool units = p->granule_bytes >= 256;
         const WarpKernelFn wf = units ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;

@@ -300,7 +300,9 @@ __global__ void __launch_bounds__(256) big_rank_kernel(const int* __restrict__ k
 // a quarter more in all, so it is taken while the batch leaves SMs room.  Up to 32 lanes a task is part of a warp, 64 lanes
 // are two warps that meet at a barrier of their own.  Task warps are the first warps of the CTA (kp.big_task_warps),
 // the threads from warp kp.big_emit_warp on emit, a slot each.
-// ONE: all paths have one rate, so every slot the same capacity (selected per slot at run time it cost 3 %: 1,024 matrices of 64 ranks 1,636 -> 1,580 us).
+// ONE: all paths have one rate, so every slot the same capacity.  Selected per slot at run time it costs 5 to 9 %: 16 and 1,024 matrices
+// of 64 ranks 791 -> 830 and 1,589 -> 1,724 us, 512 of 256 ranks 12.6 -> 13.8 ms (two rates, links of 64 and NICs of 50 B/ns: 832 us,
+// 1,718 us, 14.2 ms, the last with 3 % more activations).
 template <int LANES, int SPLIT, bool ONE>
 __global__ void __launch_bounds__(LANES == 64 ? 384 : (SPLIT == 2 ? LANES * 6 : LANES * 8), LANES == 64 ? 1 : 64 / LANES)
 vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, const int64_t* __restrict__ tau_in, int B,

@@ -16,6 +16,8 @@ CATALOGS = {
     "ring_of_three": lambda: complete_catalog(ring_topology(1, switches_per_node=3, g=4)),
     "two_nodes_64_50": lambda: complete_catalog(tree_topology(2, nic_bw=50)),
     "template_1": lambda: node_template_catalog(tree_topology(1)),
+    "template_3_64_50": lambda: node_template_catalog(tree_topology(3, nic_bw=50)),
+    "template_4": lambda: node_template_catalog(tree_topology(4)),
     "template_5_64_50": lambda: node_template_catalog(tree_topology(5, nic_bw=50)),
     "template_8": lambda: node_template_catalog(tree_topology(8)),
     "template_9": lambda: node_template_catalog(tree_topology(9)),
@@ -129,3 +131,11 @@ def test_work_order(vp, oracle_lib, name, tau):  # noqa: F811
     for key in ts.KEYS:
         for r in range(5):
             assert (got[key][r::5] == want[key][r]).all(), (key, r)
+
+
+@pytest.mark.parametrize("name,batches", [("template_3_64_50", (740, 741, 1185)), ("template_4", (740, 741, 1184, 1185, 2369)),
+                                          ("template_8", (148, 149, 592, 1185)), ("template_9", (296, 593))])
+def test_launch_shapes_of_node_symmetric_catalogs(vp, oracle_lib, name, batches):  # noqa: F811
+    """Up to eight groups CTAs of two lanes per group are followed by CTAs of one that pack the SMs, above by CTAs of one and warps
+    that emit: the last batch of a shape and the first of the next, and batches beyond one wave."""
+    test_work_counters_and_batches(vp, oracle_lib, name, batches)
