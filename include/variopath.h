@@ -57,10 +57,11 @@ extern "C" {
 #define VP_ST_PACK_MISMATCH 256   /* vp_pack: routed copies disagree with the plan's byte counts  */
 #define VP_ST_PACK_CAPACITY 512   /* vp_pack: staged buffer smaller than the plan's send volume   */
 #define VP_ST_EXCHANGE_TIMEOUT 2048 /* vp_exchange_wait: the arrival counter did not reach the plan's byte count in max_polls polls */
-/* Row-copy kernels (vp_pack, vp_pack_static, vp_unpack, vp_unpack_tokens): a bounded wait for an asynchronous
- * copy into shared memory gave up (2^22 polls; never seen in practice).  The kernel then issues no further
- * loads, lets the stores it already issued finish and returns; the output buffer is INCOMPLETE and the call
- * must be repeated.  Nothing faults and the context stays usable. */
+/* Kernels that copy through shared memory (vp_pack, vp_pack_static, vp_unpack, vp_unpack_tokens, vp_exchange_put): a
+ * bounded wait for an asynchronous copy into shared memory gave up (2^22 polls; never seen in practice).  The kernel
+ * then issues no further loads, lets the stores it already issued finish and returns; the output buffer is INCOMPLETE
+ * and the call must be repeated (vp_exchange_put: what the CTA that gave up has stored is not counted in arrived).
+ * Nothing faults and the context stays usable. */
 #define VP_ST_INTERNAL_TIMEOUT (1 << 30)
 /* Bits 1..16 reject the matrix before scheduling: n_steps[b] = 0 and an empty plan. */
 
@@ -279,7 +280,7 @@ int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, const int64_t* 
  * Arguments, results and status bits are those of vp_pack; inputs and outputs are still the caller's.
  * Limits and rules:
  *  - vp_pack_workspace_bytes(N, T, topk, k_max) must not exceed VP_PACK_STATIC_SCRATCH_BYTES (4 MiB; about
- *    0.9 million routed copies at N = 16); a larger problem is refused with VP_E_WORKSPACE before anything
+ *    1 million routed copies at N = 16); a larger problem is refused with VP_E_WORKSPACE before anything
  *    is launched.  Use vp_pack with your own workspace for those.
  *  - The first call on each device looks up the block's device address (a cudaGetSymbolAddress query made
  *    with that device current).  Make that first call outside any stream capture.
@@ -367,7 +368,7 @@ int vp_plan_time(const vp_catalog* catalog, int B, int k_max, const int32_t* n_s
  *   arrived              device array [N] of pointers to uint64 counters (NULL array or NULL entries: no signalling):
  *                        after a CTA's parts of the chunks have been stored and fenced system-wide each byte count is added
  *                        to *arrived[j] with a system-scope atomic.  A rank's counter ends at base + recv_off[n_steps][rank]
- *   status               device int32[1], bits are OR-ed in (not cleared)
+ *   status               device int32[1], bits are OR-ed in (not cleared): VP_ST_PACK_CAPACITY, VP_ST_INTERNAL_TIMEOUT
  * The call only enqueues one kernel on cuda_stream of the current device; it never waits.
  *
  * vp_exchange_wait, the receiver side: one thread polls *arrived_counter (acquire, system scope) until it is at least

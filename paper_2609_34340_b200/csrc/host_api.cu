@@ -138,7 +138,7 @@ int schedule_host(const vp_catalog* cc, const vp_sched_params* p, const int64_t*
 
     // Only rows in use, into page-locked buffers: the scheduler writes its rows straight into them, over PCIe while it decomposes.
     // Copied afterwards they would be six pieces per matrix, of lengths that only the device knows: 128 matrices of 64 ranks took
-    // 6.1 ms with cudaMemcpyAsync calls in chunks, 2.3 with a copy kernel behind the scheduler, 1.7 so (69 MB, 1.3 ms of PCIe).
+    // 6.1 ms with cudaMemcpyAsync calls in chunks, 2.3 with a copy kernel behind the scheduler, 1.54 so (69 MB, 1.3 ms of PCIe).
     if (used_only) {
         const size_t b = (size_t)B;
         int32_t *h_steps = pinned_address(n_steps, b * 4), *h_status = pinned_address(status, b * 4), *h_chan = pinned_address(chan_id, b * K * 4);

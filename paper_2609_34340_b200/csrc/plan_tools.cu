@@ -59,9 +59,10 @@ plan_time_kernel(const uint32_t* __restrict__ inst_wdiv, int n_inst, int64_t W, 
 // Histogram of (source rank, destination rank) pairs of routed copies.  One cluster of one to eight CTAs takes the `group`
 // sources from blockIdx / cluster size on, every CTA a slice of their copies; the counts meet in distributed shared memory,
 // so a demand row is written once, by plain stores, and nothing has to be zeroed before the launch.  Bound by latency: with two
-// memsets ahead of it and global atomics behind, the row of one rank with 128 tokens took 7.0 us of GPU time, now 2.3.
-// Many sources: bound by the additions in shared memory; a loop of its own for a single source (no division), 16-byte loads and one wave of
-// CTAs took 256 sources x 12,833 tokens x 8 from 103 to 41 us, one source x 16,384 x 8 from 10.9 to 6.3.
+// memsets ahead of it and global atomics behind, the row of one rank with 128 tokens took 6.4 us of GPU time, now 2.0.
+// Many copies: bound by the additions in shared memory; a loop of its own for a single source (no division), 16-byte loads and one wave
+// of CTAs.  16,384 tokens x top-8 from 1, 64 and 256 sources: 16.4, 24.6 and 69.5 us by slices of 16,384 copies and global atomics,
+// now 5.5, 18.6 and 47.1 (GPU time in a graph).
 constexpr int kDemandCells = 4096;                 // group x N at most
 // WIDE: a CTA has more than 2^kDemandCarry copies of one source; it moves the high bits of its counts on after every so many, and the
 // row is a 64-bit sum.  (As a case at run time it cost one source of a few thousand copies 4.5 -> 4.8 us.)
@@ -161,8 +162,6 @@ extern "C" int vp_demand_from_routing(const int32_t* expert_idx, int n_src, int 
         src0 + n_src > N || row_bytes <= 0 || row_bytes >= VP_ENTRY_LIMIT)
         return VP_E_BAD_ARG;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    const int sms = sm_count_of_device();
-    if (!sms) return VP_E_CUDA;
     const long long per_src = (long long)T * topk, total = per_src * n_src;
     // Few copies from few sources: one cluster counts them all and writes the status itself.  Otherwise a cluster per source,
     // which share the status word.
@@ -173,7 +172,7 @@ extern "C" int vp_demand_from_routing(const int32_t* expert_idx, int n_src, int 
     int ctas = 1;
     // four copies per thread, then more CTAs, up to one wave of them (four per SM): every further wave is another launch latency and trip to memory
     const int groups = (n_src + group - 1) / group;
-    while (ctas < 8 && (long long)ctas * 4 * kIdxThreads < items && (ctas == 1 || groups * ctas * 2 <= 4 * sms)) ctas *= 2;
+    while (ctas < 8 && (long long)ctas * 4 * kIdxThreads < items && (ctas == 1 || groups * ctas * 2 <= 4 * sm_count_of_device())) ctas *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(groups * ctas));
     cfg.blockDim = dim3(kIdxThreads);

@@ -23,7 +23,8 @@ namespace {
 constexpr int kIdxWarps = kIdxThreads / 32;
 constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
 // Items up to which one self-contained launch is used.  Its last CTA counts every item itself, and the rows move by plain loads
-// and stores (10 % behind the bulk copy).  At 8,192 items the two forms cost the same: index work of 10 and 11 us.
+// and stores (10 % behind the bulk copy).  Pack of 16 ranks, top-8, one launch | chunked, us: rows of 256 B 6,144 copies 15.4 | 17.4,
+// 8,192 17.4 | 17.4, 16,384 21.5 | 19.4; rows of 14,336 B 6,144 copies 28.7 | 33.8, 8,192 33.9 | 35.9, 12,288 48.1 | 46.1.
 constexpr int kSmallItems = 8192;
 constexpr int kSmallSteps = 1024;                   // plan arrays longer than this do not fit its run table
 constexpr int kSmallOwn = 1024;                     // rows or copies one CTA may own there

@@ -206,8 +206,8 @@ inline int launch_row_copy(const void* rows, void* out, const int32_t* map, cons
     c.n = n; c.fanout = fanout; c.gather = gather; c.bounded = bounded; c.row_bytes = row_bytes; c.status = status;
     c.pieces = 1; c.stage_bytes = 0;
     const int width = copy_width(rows, out, row_bytes);
-    // Many short CTAs rather than one wave of long ones: 64 to 80 KB of stores per CTA (two rows at least in the bulk form).  The
-    // hardware hands out CTAs in order, so the rows in flight stay neighbours, and so do their destinations in every stream;
+    // Many short CTAs rather than one wave of long ones: 64 KB of stores per CTA in the plain form, 80 KB or two rows, whichever is
+    // more, in the bulk form (14,336 B at fan-out 8: two rows, 229 KB).  The hardware hands out CTAs in order, so the rows in flight stay neighbours, and so do their destinations in every stream;
     // in one wave the CTAs drift apart and DRAM takes the stores at 5.0 TB/s instead of 5.7.  16,384 rows of 14,336 B,
     // fan-out 8: 371 us in one wave, 328 so; 8,192 rows of 4,096 B: 98 and 44 us; rows claimed in order from a counter by one
     // wave: 325 and 53 us.  (Where the rows in use are known on the device only, half of the buffer is expected.)

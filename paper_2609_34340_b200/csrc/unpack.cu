@@ -278,7 +278,9 @@ tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
 // ---- chunked form -----------------------------------------------------------------------------------------------
 
 // A count CTA reads the plan's lane_dst itself up to this many cells (64 KB, five 16-byte loads per thread for the 300 of
-// 512 activations a 64-rank plan uses); larger plans have their steps resolved by steps_kernel first.
+// 512 activations a 64-rank plan uses); larger plans have their steps resolved by steps_kernel first.  Unpack of 2,000 tokens x
+// top-8, 4,096 B, in place | by steps_kernel, us: 16 ranks, 2,048 plan rows 50.1 | 50.2, 4,096 48.1 | 50.2; 64 ranks, 512 rows
+// 56.3 | 54.3, 1,024 56.3 | 53.3; 256 ranks, 128 rows 21.5 | 19.5, 1,024 72.7 | 35.9.
 constexpr int kInlineCells = 32768;
 constexpr int kStepTile = 32;                        // steps per CTA of steps_kernel
 
