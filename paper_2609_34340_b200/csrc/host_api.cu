@@ -1,6 +1,7 @@
 // Host-buffer variants of the two entry points: copy in, run the device path, copy out.
 #include <cuda_runtime.h>
 
+#include "pinned.h"
 #include "vp_internal.h"
 
 namespace {
@@ -104,19 +105,6 @@ int copy_plan_out(const SchedBufs& s, size_t N, size_t K, size_t lo, size_t n, i
 // Batches of at least this many matrices are copied back in chunks, two of them in flight: while one chunk is
 // decomposed on the caller's stream, the results of the chunk before it travel to the host on a second stream.
 constexpr int kPipeMinBatch = 64;
-
-// Device address of `bytes` of page-locked host memory, or null if the device cannot write there.
-template <typename T>
-T* pinned_address(T* host, size_t bytes) {
-    cudaPointerAttributes a, z;
-    if (!host || !bytes) return nullptr;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&z, (const char*)host + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer || !z.devicePointer) return nullptr;
-    return (const char*)z.devicePointer - (const char*)a.devicePointer == (ptrdiff_t)(bytes - 1) ? (T*)a.devicePointer : nullptr;
-}
 
 // Both host-buffer scheduler calls: copy in, run vp_schedule_batch, copy out.
 int schedule_host(const vp_catalog* cc, const vp_sched_params* p, const int64_t* demand, const int64_t* tau_ns_in, int B,

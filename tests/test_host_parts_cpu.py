@@ -155,3 +155,65 @@ int main() {
         }
 }
 ''')
+
+
+def test_a_buffer_counts_as_page_locked_only_as_a_whole(tmp_path):
+    """Plan rows are written straight into page-locked buffers: a buffer may be page-locked in pieces, but not have a gap."""
+    _run(tmp_path, r'''
+#include <string.h>
+#include "pinned.h"
+#include <cuda.h>
+struct Range { char *host, *device; size_t bytes; };
+static Range ranges[8];
+static int n_ranges = 0;
+static const Range* find(const void* p) {
+    for (int i = 0; i < n_ranges; i++)
+        if ((const char*)p >= ranges[i].host && (const char*)p < ranges[i].host + ranges[i].bytes) return &ranges[i];
+    return nullptr;
+}
+extern "C" cudaError_t cudaGetLastError() { return cudaSuccess; }
+extern "C" cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+    memset(a, 0, sizeof(*a));
+    const Range* r = find(p);
+    if (!r) { a->type = cudaMemoryTypeUnregistered; return cudaSuccess; }
+    a->type = cudaMemoryTypeHost;
+    a->hostPointer = (void*)p;
+    a->devicePointer = r->device + ((const char*)p - r->host);
+    return cudaSuccess;
+}
+static CUresult attribute(void* data, CUpointer_attribute what, CUdeviceptr p) {
+    for (int i = 0; i < n_ranges; i++) {
+        const Range& r = ranges[i];
+        if ((char*)p < r.device || (char*)p >= r.device + r.bytes) continue;
+        if (what == CU_POINTER_ATTRIBUTE_RANGE_START_ADDR) *(CUdeviceptr*)data = (CUdeviceptr)r.device;
+        else if (what == CU_POINTER_ATTRIBUTE_RANGE_SIZE) *(size_t*)data = r.bytes;
+        else return CUDA_ERROR_INVALID_VALUE;
+        return CUDA_SUCCESS;
+    }
+    return CUDA_ERROR_INVALID_VALUE;
+}
+extern "C" cudaError_t cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long long, cudaDriverEntryPointQueryResult* found) {
+    assert(!strcmp(name, "cuPointerGetAttribute"));
+    *fn = (void*)attribute;
+    if (found) *found = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
+int main() {
+    static char mem[9 << 16];
+    char* const p = mem;
+    const size_t K = 1 << 16;
+    auto set = [&](std::initializer_list<Range> rs) { n_ranges = 0; for (const Range& r : rs) ranges[n_ranges++] = r; };
+    set({{p, p, 9 * K}});
+    assert(pinned_address(p, 9 * K) == p && pinned_address(p + 5, 1) == p + 5 && pinned_address(p + K, 8 * K) == p + K);
+    assert(!pinned_address(p, 9 * K + 1) && !pinned_address(p, 0) && !pinned_address((char*)nullptr, 4));
+    set({{p, p, K}, {p + K, p + K, K}, {p + 2 * K, p + 2 * K, 7 * K}});           // in pieces
+    assert(pinned_address(p, 9 * K) == p && pinned_address(p + K - 1, 2) == p + K - 1);
+    set({{p, p, K}, {p + 8 * K, p + 8 * K, K}});                                  // both ends, nothing between
+    assert(!pinned_address(p, 9 * K));
+    assert(pinned_address(p, K) == p && !pinned_address(p, K + 1) && !pinned_address(p + 4 * K, K));
+    set({{p, p, K}, {p + 2 * K, p + 2 * K, K}, {p + 8 * K, p + 8 * K, K}});
+    assert(!pinned_address(p, 3 * K) && !pinned_address(p, 9 * K));
+    set({{p, p, K}, {p + K, p + 4 * K, K}});                                      // device addresses that do not follow on
+    assert(!pinned_address(p, 2 * K));
+}
+''')
