@@ -142,8 +142,8 @@ __device__ __forceinline__ void put_any(unsigned char* dst, const unsigned char*
 // Parts whose addresses and size are multiples of 16 go through shared memory as bulk asynchronous copies that one thread of
 // warp 0 issues (pieces of up to 16 KB, six stages); others are moved by all warps.  One system fence by one warp per CTA
 // announces all its parts: fences by every thread, and a second walk over the plan behind them, took 12 us of any call.
-// Bound by HBM.  On one GPU 2,048 tokens x top-8 of 14,336 B (440 MB read and written) took 95.6 us with plain 16-byte loads
-// and stores, now 81; 32 tokens 19.1 us, now 7.9.
+// Bound by HBM.  On one GPU 2,048 tokens x top-8 of 14,336 B (440 MB read and written) took 92 us with plain 16-byte loads
+// and stores, now 81; 32 tokens take 12 us less.
 __global__ void __launch_bounds__(kPutThreads) exchange_put_kernel(PutArgs a) {
     extern __shared__ __align__(128) unsigned char ring[];
     __shared__ __align__(8) unsigned long long bars[kPutStages];
