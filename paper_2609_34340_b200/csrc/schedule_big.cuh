@@ -32,6 +32,12 @@
 //    5.65 -> 4.2 us an activation with 256 ranks).  Every other cell of such a matrix is below 65,535 granules, so its 16-bit
 //    copy is exact.  No L2 traffic is needed in this mode.
 //
+//  * Code size.  Instructions come from caches of about 8 KB per scheduler and 32 KB per SM; straight-line code costs 2.2
+//    cycles an instruction from the first, 4 at 32 KB and 6.5 beyond, and more at every jump.  So what an ordinary
+//    activation does not execute is kept out of its loop: the loop exists twice, with and without hot columns, and the 64-bit
+//    scores are functions of their own.  As one loop of 65 KB with all cases inside: 16 x 64 ranks 774 -> 659 us,
+//    1,024 x 64 ranks 1,591 -> 1,455, 512 x 256 ranks 12,560 -> 11,760.
+//
 // A matrix that does not meet the conditions (granule below 256 bytes, a capacity of 2^22 granules or more, 2^32
 // granules or more in total, more than 32 hot columns, more big cells than the side list holds) is appended to a list that
 // the general kernel works through afterwards.
@@ -43,6 +49,8 @@ constexpr int BIG_HOT_MAX = 32;       // columns whose cells are kept beyond 16 
 constexpr uint32_t BIG_HOT_NONE = 0x01010101u * BIG_HOT_MAX;  // a group without a hot column
 constexpr int BIG_EXCHANGE = 192;     // bytes per pair of warps: 64 source tags, 64 destination tags, words
 constexpr int BIG_SMEM_LIMIT = 227 * 1024 - 2048;   // dynamic shared memory of one CTA, less room for the static variables
+
+template <bool V> struct BigConst { static constexpr bool value = V; };
 
 struct BigSmem {
     int wd, hi, colmap, tbl, rs, pat, dec, gnode, send_acc, recv_acc, red, task_f, task_den, bind, exchange, record, term, bucket, fam_task, total;
@@ -166,6 +174,50 @@ __device__ __noinline__ void big_write_in_order(int64_t* row, const int64_t* acc
     asm volatile("bar.sync %0, %1;" ::"n"(BARRIER), "r"(threads) : "memory");
     for (int r = thread; r < N; r += threads) row[r] = acc[r];
     asm volatile("bar.sync %0, %1;" ::"n"(BARRIER), "r"(threads) : "memory");
+}
+
+// Eq. (6) by the general route, in 64 bits (out of line, as the loop should stay small for the instruction caches): scores beyond
+// 32 bits, catalogs whose rows have more than three terms or whose groups are more than two rails.  All threads of the CTA; every
+// warp gets the key of the first maximum, score << 16 | (65535 - shape): a score is at most four times what is left, so below 2^34,
+// and there are fewer than 2^16 shapes.
+__device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t* rs, uint64_t* red, const uint32_t* pat, const uint32_t* spat,
+                                                   int n_patterns, int row_terms, int n_shapes, int S) {
+    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, ns_pad = (n_shapes + 31) & ~31;
+#pragma unroll 1
+    for (int p = tid; p < n_patterns; p += NT) {
+        uint64_t v = 0;
+#pragma unroll 1
+        for (int t = 0; t < row_terms; t++) {
+            const uint32_t tw = pat[p * row_terms + t];
+            v += (uint64_t)tbl[tw & 0xffffu] * (tw >> 16);
+        }
+        rs[p] = v << 16;
+    }
+    __syncthreads();
+    uint64_t best = 0;
+#pragma unroll 1
+    for (int s = tid; s < n_shapes; s += NT) {
+        uint64_t key = (uint64_t)(65535 - s);
+#pragma unroll 1
+        for (int q = 0; q < S; q += 2) {
+            const uint32_t pw = spat[q / 2 * ns_pad + s];
+            key += rs[pw & 0xffffu];
+            if (q + 1 < S) key += rs[pw >> 16];
+        }
+        best = max_v(best, key);
+    }
+    best = big_warp_max64(best);
+    if (lane == 0) red[tid >> 5] = best;
+    __syncthreads();
+    return big_warp_max64(lane < NT / 32 ? red[lane] : 0ull);
+}
+// One chunk of the class-wise arg-max in 64 bits (see the loop): its key score << 16 | (65535 - tie-break word).  Whole warp.
+__device__ __noinline__ uint64_t big_chunk_key(const uint32_t* tbl, const uint32_t* ent, int ent_words) {
+    uint64_t v = 0;
+#pragma unroll 1
+    for (int t = 0; t < ent_words - 1; t++) v += (uint64_t)tbl[ent[t] & 0xffffu] * (ent[t] >> 16);
+    const uint32_t meta = ent[ent_words - 1];
+    return big_warp_max64(meta == 0xffffffffu ? 0ull : (v << 16 | (uint64_t)(65535u - (meta & 0xffffu))));
 }
 
 // Step 3 when several families compete (kept out of line: most shapes have one family, and the main loop should
@@ -577,7 +629,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         }
         // Idle rows are filled from the end of the plan towards the activations while the matrix is decomposed (fill_warp,
         // a block of 4 fill_rows rows per iteration): fill_lo is the first row already filled.
-        const bool fills = L.fill_rows > 0 && st == 0 && !kp.host_rows &&
+        const bool fills = RECORD && L.fill_rows > 0 && st == 0 && !kp.host_rows &&
             (((uintptr_t)lane_dst_b | (uintptr_t)lane_inst_b | (uintptr_t)lane_bytes_b | (uintptr_t)send_off_b |
               (uintptr_t)(recv_off_b ? recv_off_b : send_off_b)) & 15) == 0;
         const unsigned chunk = (unsigned)(L.fill_rows * N * 8);
@@ -654,488 +706,464 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                 __syncthreads();
                 continue;
             }
-            int64_t left = s_left;
-            const BigCredits cr{wd, Hi, colmap, ST, N, hot_mode};
-            const uint32_t cap0 = s_cap[0], cap2 = min_v(cap0, 65535u) * 0x00010001u;
-            // An activation is first taken off the residual; its rows are written while the next one's tasks run: by the thread
-            // that emitted the slot (p_*), or (RECORD) by the warps without a task, from the record of the slot.
-            bool pend = false;
-            int p_fam = 0;
-            uint32_t p_bind = 0, p_x = 0;
-            uint2* const record = (uint2*)(smem_raw + L.record);
-            auto write_slot = [&](int kk, int r, int fam, uint32_t bind, uint32_t x, uint32_t inst) {
-                const int i = (int)(bind & 0xffu), j = (int)(bind >> 8);
-                const size_t row = (size_t)kk * N, orow = (size_t)(kk + 1) * N;
-                const int64_t bytes = (int64_t)x * kp.granule;
-                const int64_t sa = send_acc[i] + bytes, ra = recv_acc[j] + bytes;
-                send_acc[i] = sa;                             // (src and dst are permutations: every rank is written once)
-                recv_acc[j] = ra;
-                lane_dst_b[row + i] = x ? (int16_t)j : (int16_t)-1;
-                lane_bytes_b[row + i] = bytes;
-                send_off_b[orow + i] = sa;
-                if (recv_off_b && !(IN_ORDER && kp.host_rows)) recv_off_b[orow + j] = ra;
-                lane_inst_b[row + i] = x ? (uint16_t)inst : (uint16_t)0xFFFF;
-                if (r == 0) chan_id_b[kk] = fam;
+            // The loop, with and without hot columns: two copies, each with a short path (see "Code size" above).
+            auto decompose = [&](auto hot_columns) {
+                constexpr bool HOT = decltype(hot_columns)::value;
+                int64_t left = s_left;
+                const BigCredits cr{wd, Hi, colmap, ST, N, HOT};
+                const uint32_t cap0 = s_cap[0], cap2 = min_v(cap0, 65535u) * 0x00010001u;
+                // An activation is first taken off the residual; its rows are written while the next one's tasks run: by the thread
+                // that emitted the slot (p_*), or (RECORD) by the warps without a task, from the record of the slot.
+                bool pend = false;
+                int p_fam = 0;
+                uint32_t p_bind = 0, p_x = 0;
+                uint2* const record = (uint2*)(smem_raw + L.record);
+                auto write_slot = [&](int kk, int r, int fam, uint32_t bind, uint32_t x, uint32_t inst) {
+                    const int i = (int)(bind & 0xffu), j = (int)(bind >> 8);
+                    const size_t row = (size_t)kk * N, orow = (size_t)(kk + 1) * N;
+                    const int64_t bytes = (int64_t)x * kp.granule;
+                    const int64_t sa = send_acc[i] + bytes, ra = recv_acc[j] + bytes;
+                    send_acc[i] = sa;                             // (src and dst are permutations: every rank is written once)
+                    recv_acc[j] = ra;
+                    lane_dst_b[row + i] = x ? (int16_t)j : (int16_t)-1;
+                    lane_bytes_b[row + i] = bytes;
+                    send_off_b[orow + i] = sa;
+                    if (recv_off_b && !(IN_ORDER && kp.host_rows)) recv_off_b[orow + j] = ra;
+                    lane_inst_b[row + i] = x ? (uint16_t)inst : (uint16_t)0xFFFF;
+                    if (r == 0) chan_id_b[kk] = fam;
             };
-            auto write_row = [&](int kk, uint32_t inst) {
-                if (RECORD) {
-                    const int fam = (int)record[N].x;
-                    for (int r = tid - n_task_warps * 32; r < N; r += NT - n_task_warps * 32)
-                        write_slot(kk, r, fam, record[r].x, record[r].y, __ldg(dc.fam_slot + (size_t)fam * N + r));
-                } else {
-                    if (emit_warp > 0 && emits) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
-                    if (emits) write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
-                }
-                // (every lane of the writing warps comes here once per activation: pend is the same in a warp)
-                if (IN_ORDER && kp.host_rows && recv_off_b) {
-                    const int first = RECORD ? n_task_warps * 32 : emit_warp * 32;
-                    big_write_in_order<CROSS ? 5 : 1>(recv_off_b + (size_t)(kk + 1) * N, recv_acc, N, tid - first, RECORD ? NT - first : emit_threads);
-                }
-                pend = false;
+                auto write_row = [&](int kk, uint32_t inst) {
+                    if (RECORD) {
+                        const int fam = (int)record[N].x;
+                        for (int r = tid - n_task_warps * 32; r < N; r += NT - n_task_warps * 32)
+                            write_slot(kk, r, fam, record[r].x, record[r].y, __ldg(dc.fam_slot + (size_t)fam * N + r));
+                    } else {
+                        if (emit_warp > 0 && emits) inst = __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit);
+                        if (emits) write_slot(kk, r_emit, p_fam, p_bind, p_x, inst);
+                    }
+                    // (every lane of the writing warps comes here once per activation: pend is the same in a warp)
+                    if (IN_ORDER && kp.host_rows && recv_off_b) {
+                        const int first = RECORD ? n_task_warps * 32 : emit_warp * 32;
+                        big_write_in_order<CROSS ? 5 : 1>(recv_off_b + (size_t)(kk + 1) * N, recv_acc, N, tid - first, RECORD ? NT - first : emit_threads);
+                    }
+                    pend = false;
             };
-            VP_TICK(0);
+                VP_TICK(0);
 
-            for (;;) {
-                if (left == 0) break;
-                if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
-                // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
-                const uint32_t inst = !RECORD && emit_warp == 0 && pend && emits ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
-                // (A) Eq. (6).  A score is at most four times what is left, so below 2^34, and there are fewer than 2^16
-                // shapes: key = score << 16 | (65535 - shape) orders by score first and lower shape index second, and the first
-                // maximum of Eq. (6) is a plain maximum of keys.
-                const bool narrow = left < ((int64_t)1 << 30);        // every score fits 32 bits
-                uint64_t bkey = 0;
-                if (use_dec) {
-                    // Class by class (two rails).  A shape is a first row p0 and a second row p1 from the list of p0's
-                    // class, and its index grows with p0's place in shape order first, p1's place in the list second.
-                    // So within a class the first maximum is (first maximal p0, first maximal p1 of the list): two
-                    // independent maxima.  One warp per chunk of 32 rows, in shape order: each lane scores its row from the
-                    // table and the first lane with the chunk's largest score leaves score << 16 | (65535 - tie-break word)
-                    // (the word is the run start for a first row, the place in the list for a second row: both grow in shape order).
-                    for (int c = warp; c < n_chunks; c += n_warps) {
-                        if (narrow && ent_words == 4) {
-                            const uint4 e = *((const uint4*)ents + c * 32 + lane);
-                            const uint32_t v = tbl[e.x & 0xffffu] * (e.x >> 16) + tbl[e.y & 0xffffu] * (e.y >> 16) + tbl[e.z & 0xffffu] * (e.z >> 16);
-                            const uint32_t mine = e.w == 0xffffffffu ? 0u : v + 1u;       // (+ 1: any row beats padding)
-                            const uint32_t m = __reduce_max_sync(0xffffffffu, mine);
-                            const unsigned who = __ballot_sync(0xffffffffu, mine == m);
-                            if (lane == __ffs(who) - 1) red[c] = (uint64_t)(m - 1u) << 16 | (uint64_t)(65535u - (e.w & 0xffffu));
-                        } else {
-                            const uint32_t* ent = ents + (size_t)(c * 32 + lane) * ent_words;
-                            uint64_t v = 0;
-#pragma unroll 1
-                            for (int t = 0; t < ent_words - 1; t++) v += (uint64_t)tbl[ent[t] & 0xffffu] * (ent[t] >> 16);
-                            const uint32_t meta = ent[ent_words - 1];
-                            const uint64_t key = big_warp_max64(meta == 0xffffffffu ? 0ull : (v << 16 | (uint64_t)(65535u - (meta & 0xffffu))));
-                            if (lane == 0) red[c] = key;
+                for (;;) {
+                    if (left == 0) break;
+                    if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
+                    // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
+                    const uint32_t inst = !RECORD && emit_warp == 0 && pend && emits ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
+                    // (A) Eq. (6).  A score is at most four times what is left, so below 2^34, and there are fewer than 2^16
+                    // shapes: key = score << 16 | (65535 - shape) orders by score first and lower shape index second, and the first
+                    // maximum of Eq. (6) is a plain maximum of keys.
+                    const bool narrow = left < ((int64_t)1 << 30);        // every score fits 32 bits
+                    uint64_t bkey = 0;
+                    if (use_dec) {
+                        // Class by class (two rails).  A shape is a first row p0 and a second row p1 from the list of p0's
+                        // class, and its index grows with p0's place in shape order first, p1's place in the list second.
+                        // So within a class the first maximum is (first maximal p0, first maximal p1 of the list): two
+                        // independent maxima.  One warp per chunk of 32 rows, in shape order: each lane scores its row from the
+                        // table and the first lane with the chunk's largest score leaves score << 16 | (65535 - tie-break word)
+                        // (the word is the run start for a first row, the place in the list for a second row: both grow in shape order).
+                        for (int c = warp; c < n_chunks; c += n_warps) {
+                            if (narrow && ent_words == 4) {
+                                const uint4 e = *((const uint4*)ents + c * 32 + lane);
+                                const uint32_t v = tbl[e.x & 0xffffu] * (e.x >> 16) + tbl[e.y & 0xffffu] * (e.y >> 16) + tbl[e.z & 0xffffu] * (e.z >> 16);
+                                const uint32_t mine = e.w == 0xffffffffu ? 0u : v + 1u;       // (+ 1: any row beats padding)
+                                const uint32_t m = __reduce_max_sync(0xffffffffu, mine);
+                                const unsigned who = __ballot_sync(0xffffffffu, mine == m);
+                                if (lane == __ffs(who) - 1) red[c] = (uint64_t)(m - 1u) << 16 | (uint64_t)(65535u - (e.w & 0xffffu));
+                            } else {
+                                const uint64_t key = big_chunk_key(tbl, ents + (size_t)(c * 32 + lane) * ent_words, ent_words);
+                                if (lane == 0) red[c] = key;
+                            }
                         }
-                    }
-                    __syncthreads();
-                    if (warp < n_task_warps) {
-                        uint64_t u = lane < n_chunks ? red[lane] : 0ull;       // chunks, then (in each unit's first chunk) units
-                        for (int s = 1; s < unit_span; s++) {
-                            const uint64_t next = __shfl_down_sync(0xffffffffu, u, 1);
-                            if (ch_more) u = max_v(u, next);
+                        __syncthreads();
+                        if (warp < n_task_warps) {
+                            uint64_t u = lane < n_chunks ? red[lane] : 0ull;       // chunks, then (in each unit's first chunk) units
+                            for (int s = 1; s < unit_span; s++) {
+                                const uint64_t next = __shfl_down_sync(0xffffffffu, u, 1);
+                                if (ch_more) u = max_v(u, next);
+                            }
+                            const uint64_t k0 = __shfl_sync(0xffffffffu, u, ch0), k1 = __shfl_sync(0xffffffffu, u, ch1);   // lane's class: first row, second row
+                            uint64_t cand = 0;
+                            if (lane < dec_n) {
+                                const uint32_t shape = (65535u - (uint32_t)(k0 & 0xffffu)) + (65535u - (uint32_t)(k1 & 0xffffu));   // run start + place
+                                cand = ((k0 >> 16) + (k1 >> 16)) << 16 | (uint64_t)(65535u - shape);
+                            }
+                            bkey = big_warp_max64(cand);
                         }
-                        const uint64_t k0 = __shfl_sync(0xffffffffu, u, ch0), k1 = __shfl_sync(0xffffffffu, u, ch1);   // lane's class: first row, second row
-                        uint64_t cand = 0;
-                        if (lane < dec_n) {
-                            const uint32_t shape = (65535u - (uint32_t)(k0 & 0xffffu)) + (65535u - (uint32_t)(k1 & 0xffffu));   // run start + place
-                            cand = ((k0 >> 16) + (k1 >> 16)) << 16 | (uint64_t)(65535u - shape);
+                    } else if (narrow && simple_scan) {
+                        // Row scores (one per thread as a rule), then every shape is the sum of its rows' scores.
+                        for (int p = tid; p < dc.n_patterns; p += NT) {
+                            if (p != tid)
+                                for (int t = 0; t < 3; t++) my_row[t] = t < dc.max_row_terms ? pat[p * dc.max_row_terms + t] : 0u;
+                            rs32[p] = tbl[my_row[0] & 0xffffu] * (my_row[0] >> 16) + tbl[my_row[1] & 0xffffu] * (my_row[1] >> 16) +
+                                      tbl[my_row[2] & 0xffffu] * (my_row[2] >> 16);
                         }
-                        bkey = big_warp_max64(cand);
-                    }
-                } else if (narrow && simple_scan) {
-                    // Row scores (one per thread as a rule), then every shape is the sum of its rows' scores.
-                    for (int p = tid; p < dc.n_patterns; p += NT) {
-                        if (p != tid)
-                            for (int t = 0; t < 3; t++) my_row[t] = t < dc.max_row_terms ? pat[p * dc.max_row_terms + t] : 0u;
-                        rs32[p] = tbl[my_row[0] & 0xffffu] * (my_row[0] >> 16) + tbl[my_row[1] & 0xffffu] * (my_row[1] >> 16) +
-                                  tbl[my_row[2] & 0xffffu] * (my_row[2] >> 16);
-                    }
-                    if (dc.n_patterns > NT && tid < dc.n_patterns)
-                        for (int t = 0; t < dc.max_row_terms; t++) my_row[t] = pat[tid * dc.max_row_terms + t];
-                    __syncthreads();
-                    uint32_t best = 0;
-                    int best_s = 65535;
-#pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        const int s = tid + u * NT;
-                        if (s < dc.n_shapes) {
-                            const uint32_t v = rs32[my_pat[u] & 0xffffu] + (S > 1 ? rs32[my_pat[u] >> 16] : 0u);
+                        if (dc.n_patterns > NT && tid < dc.n_patterns)
+                            for (int t = 0; t < dc.max_row_terms; t++) my_row[t] = pat[tid * dc.max_row_terms + t];
+                        __syncthreads();
+                        uint32_t best = 0;
+                        int best_s = 65535;
+    #pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            const int s = tid + u * NT;
+                            if (s < dc.n_shapes) {
+                                const uint32_t v = rs32[my_pat[u] & 0xffffu] + (S > 1 ? rs32[my_pat[u] >> 16] : 0u);
+                                if (v > best) { best = v; best_s = s; }
+                            }
+                        }
+                        for (int s = tid + 4 * NT; s < dc.n_shapes; s += NT) {
+                            const uint32_t pw = spat[s], v = rs32[pw & 0xffffu] + (S > 1 ? rs32[pw >> 16] : 0u);
                             if (v > best) { best = v; best_s = s; }
                         }
+                        const uint32_t m = __reduce_max_sync(0xffffffffu, best);
+                        const uint32_t s1 = __reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 65535u);
+                        bkey = (uint64_t)m << 16 | (uint64_t)(65535u - s1);
+                        if (lane == 0) red[warp] = bkey;           // the warps' candidates
+                        __syncthreads();
+                        if (warp < n_task_warps) bkey = big_warp_max64(lane < n_warps ? red[lane] : 0ull);
+                    } else {
+                        bkey = big_first_maximum(tbl, rs64, red, pat, spat, dc.n_patterns, dc.max_row_terms, dc.n_shapes, S);
                     }
-                    for (int s = tid + 4 * NT; s < dc.n_shapes; s += NT) {
-                        const uint32_t pw = spat[s], v = rs32[pw & 0xffffu] + (S > 1 ? rs32[pw >> 16] : 0u);
-                        if (v > best) { best = v; best_s = s; }
+                    int f0 = 0, H = 0;                             // (warps without a task learn them after Step 2)
+                    if (warp < n_task_warps && (bkey >> 16) != 0) {
+                        const int best_s = 65535 - (int)(bkey & 0xffffu);
+                        f0 = (int)bucket[best_s]; H = (int)bucket[best_s + 1] - f0;
                     }
-                    const uint32_t m = __reduce_max_sync(0xffffffffu, best);
-                    const uint32_t s1 = __reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 65535u);
-                    bkey = (uint64_t)m << 16 | (uint64_t)(65535u - s1);
-                } else {
-                    for (int p = tid; p < dc.n_patterns; p += NT) {
-                        uint64_t v = 0;
-#pragma unroll 1
-                        for (int t = 0; t < dc.max_row_terms; t++) {
-                            const uint32_t tw = pat[p * dc.max_row_terms + t];
-                            v += (uint64_t)tbl[tw & 0xffffu] * (tw >> 16);
+                    if (tid == 0) s_pick = make_int2(f0, H);
+                    const int n_tasks = H * kp.n_start;
+                    VP_TICK(1);
+
+                    // ---- rows of the last activation, where warps without a task write them, and a block of the fill
+                    if (warp >= n_task_warps && pend) write_row(k - 1, inst);
+                    if (RECORD && fills && warp == fill_warp) {
+                        if (fill_lo <= k + 1) {                    // the activations have reached filled rows: those copies must be over
+                            bulk_wait_all();
+                            asm volatile("fence.proxy.async;" ::: "memory");
+                        } else if (fill_lo - 4 * L.fill_rows >= k + 64) {
+                            fill_block(fill_lo - 4 * L.fill_rows, fill_lo);
+                            fill_lo -= 4 * L.fill_rows;
                         }
-                        rs64[p] = v << 16;
                     }
-                    __syncthreads();
-                    for (int s = tid; s < dc.n_shapes; s += NT) {
-                        uint64_t key = (uint64_t)(65535 - s);
-                        for (int w = 0; w < L.pat_words; w++) {
-                            const uint32_t pw = spat[w * ns_pad + s];
-                            key += rs64[pw & 0xffffu];
-                            if (2 * w + 1 < S) key += rs64[pw >> 16];
-                        }
-                        bkey = max_v(bkey, key);
-                    }
-                    bkey = big_warp_max64(bkey);
-                }
-                if (!use_dec && n_warps > 1) {                 // the warps' candidates
-                    if (lane == 0) red[warp] = bkey;
-                    __syncthreads();
+
+                    const bool hot = EXACT && HOT && s_hot > 0;            // (none beyond 16 bits left: the 16-bit credits are exact)
+                    // (B) MultiStartAA: LANES lanes per (family, start), SPLIT of them per rank group.
+                    //
+                    // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits,
+                    // of position 3 in the lowest.  An in-slot finds the tag of its slot in the byte of the slot's source group, an
+                    // out-slot the tag of its destination likewise: by a shuffle inside a warp, through shared memory between two.
                     if (warp < n_task_warps) {
-                        if (n_warps == 2) bkey = max_v(red[0], red[1]);
-                        else bkey = big_warp_max64(lane < n_warps ? red[lane] : 0ull);
-                    }
-                }
-                int f0 = 0, H = 0;                             // (warps without a task learn them after Step 2)
-                if (warp < n_task_warps && (bkey >> 16) != 0) {
-                    const int best_s = 65535 - (int)(bkey & 0xffffu);
-                    f0 = (int)bucket[best_s]; H = (int)bucket[best_s + 1] - f0;
-                }
-                if (tid == 0) s_pick = make_int2(f0, H);
-                const int n_tasks = H * kp.n_start;
-                VP_TICK(1);
-
-                // ---- rows of the last activation, where warps without a task write them, and a block of the fill
-                if (warp >= n_task_warps && pend) write_row(k - 1, inst);
-                if (fills && warp == fill_warp) {
-                    if (fill_lo <= k + 1) {                    // the activations have reached filled rows: those copies must be over
-                        bulk_wait_all();
-                        asm volatile("fence.proxy.async;" ::: "memory");
-                    } else if (fill_lo - 4 * L.fill_rows >= k + 64) {
-                        fill_block(fill_lo - 4 * L.fill_rows, fill_lo);
-                        fill_lo -= 4 * L.fill_rows;
-                    }
-                }
-
-                const bool hot = EXACT && hot_mode && s_hot > 0;            // (none beyond 16 bits left: the 16-bit credits are exact)
-                // (B) MultiStartAA: LANES lanes per (family, start), SPLIT of them per rank group.
-                //
-                // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits,
-                // of position 3 in the lowest.  An in-slot finds the tag of its slot in the byte of the slot's source group, an
-                // out-slot the tag of its destination likewise: by a shuffle inside a warp, through shared memory between two.
-                if (warp < n_task_warps) {
-                    for (int task0 = wg * TPW; task0 < n_tasks; task0 += n_tg * TPW) {
-                        const int task = min(task0 + tsub, n_tasks - 1);
-                        const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, f = f0 + h, t = task - h * kp.n_start;
-                        const bool act = task0 + tsub < n_tasks && a < G;
-                        // Slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag.
-                        uint32_t uo[QN], ui[QN];
-                        {
-                            const uint32_t* const row = (kp.big_stage ? (const uint32_t*)(smem_raw + L.fam_task) : dc.fam_task) + ((size_t)f * G + ag) * 8;
-                            if (SPLIT == 1) {
-                                const uint4 o = kp.big_stage ? *(const uint4*)row : __ldg((const uint4*)row);
-                                const uint4 i = kp.big_stage ? *((const uint4*)row + 1) : __ldg((const uint4*)row + 1);
-                                uo[0] = o.x; uo[1] = o.y; uo[QN - 2] = o.z; uo[QN - 1] = o.w;
-                                ui[0] = i.x; ui[1] = i.y; ui[QN - 2] = i.z; ui[QN - 1] = i.w;
-                            } else {
-                                const uint2 o = kp.big_stage ? *((const uint2*)row + part) : __ldg((const uint2*)row + part);
-                                const uint2 i = kp.big_stage ? *((const uint2*)row + 2 + part) : __ldg((const uint2*)row + 2 + part);
-                                uo[0] = o.x; uo[1] = o.y;
-                                ui[0] = i.x; ui[1] = i.y;
-                            }
-                        }
-                        if (!RECORD && pend) write_row(k - 1, inst); // (while the tables travel)
-                        // start t binds in-slot q to row (q + t) mod 4
-                        uint32_t dst = 0, src = 0;
-#pragma unroll
-                        for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
-                        int dt[QN];                            // tag (3 - row) each out-slot's destination has
-                        auto fetch_dst = [&]() {
-#pragma unroll
-                            for (int i = 0; i < QN; i++) {
-                                if (CROSS) dt[i] = (int)(((unsigned)ex_dst[(uo[i] >> 16) & 0xffu] >> (uo[i] >> 28)) & 3u);
-                                else dt[i] = (int)((__shfl_sync(0xffffffffu, dst, (int)(uo[i] >> (17 - SPLIT)), WL) >> (uo[i] >> 28)) & 3u);
-                            }
-                        };
-                        // best key of the group's 4 x 4 tile: v holds this lane's columns
-                        auto best_key = [&](const uint32_t (&v)[4][QN]) {
-                            if constexpr (SPLIT == 1) {
-                                return big_best_key(v);
-                            } else {                           // both columns of a pair of rows; the other lane has the other two columns
-                                const uint32_t p01 = add_max(v[0][0], v[1][1], v[1][0] + v[0][1]), p02 = add_max(v[0][0], v[2][1], v[2][0] + v[0][1]);
-                                const uint32_t p03 = add_max(v[0][0], v[3][1], v[3][0] + v[0][1]), p12 = add_max(v[1][0], v[2][1], v[2][0] + v[1][1]);
-                                const uint32_t p13 = add_max(v[1][0], v[3][1], v[3][0] + v[1][1]), p23 = add_max(v[2][0], v[3][1], v[3][0] + v[2][1]);
-                                const uint32_t o01 = __shfl_xor_sync(0xffffffffu, p01, 1), o02 = __shfl_xor_sync(0xffffffffu, p02, 1);
-                                const uint32_t o03 = __shfl_xor_sync(0xffffffffu, p03, 1), o12 = __shfl_xor_sync(0xffffffffu, p12, 1);
-                                const uint32_t o13 = __shfl_xor_sync(0xffffffffu, p13, 1), o23 = __shfl_xor_sync(0xffffffffu, p23, 1);
-                                const uint32_t m0 = add_max(p01, o23, add_max(p02, o13, p03 + o12)), m1 = add_max(p12, o03, add_max(p13, o02, p23 + o01));
-                                return max_v(m0, m1);
-                            }
-                        };
-                        auto tile_column = [&](uint32_t (&v)[4][QN], int i, uint32_t lo, uint32_t hi) {
-                            v[0][i] = __byte_perm(lo, SPLIT == 1 ? big_tag(0, i) : tags[0][i], 0x5104);      // (low half) << 8 | tag
-                            v[1][i] = __byte_perm(lo, SPLIT == 1 ? big_tag(1, i) : tags[1][i], 0x5324);      // (high half) << 8 | tag
-                            v[2][i] = __byte_perm(hi, SPLIT == 1 ? big_tag(2, i) : tags[2][i], 0x5104);
-                            v[3][i] = __byte_perm(hi, 0u, 0x5324);                                           // (row 3 has tag 0)
-                        };
-                        auto cap_of = [&](uint32_t w) { return one_class ? cap0 : s_cap[(w >> 24) & 0xfu]; };
-                        auto cap2_of = [&](uint32_t w) { return one_class ? cap2 : min_v(s_cap[(w >> 24) & 0xfu], 65535u) * 0x00010001u; };
-                        // exact credit in place of the 16-bit one (the tag byte stays)
-                        auto hot_credit = [&](uint32_t& key, uint32_t cell, uint32_t cap) { key = __byte_perm(key, min_v(cell, cap), 0x6540); };
-                        // source half: one exact assignment per source group
-                        auto source_half = [&]() {
-                            uint32_t v[4][QN];
-#pragma unroll
-                            for (int i = 0; i < QN; i++) {
-                                const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
-                                const uint32_t c2 = cap2_of(uo[i]);
-                                tile_column(v, i, __vminu2(at[0], c2), __vminu2(at[ST], c2));
-                            }
-                            if (!EXACT && hot_mode) {          // out-slots bound to a hot column: exact 32-bit cells
-#pragma unroll
-                                for (int i = 0; i < QN; i++) {
-                                    const int j = (int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i];
-                                    if (colmap[j] != BIG_HOT_MAX) {
-#pragma unroll
-                                        for (int r = 0; r < 4; r++)
-                                            v[r][i] = min_v(cr.cell(ag * 4 + r, j), cap_of(uo[i])) * 256u + (v[r][i] & 0xffu);
-                                    }
+                        for (int task0 = wg * TPW; task0 < n_tasks; task0 += n_tg * TPW) {
+                            const int task = min(task0 + tsub, n_tasks - 1);
+                            const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, f = f0 + h, t = task - h * kp.n_start;
+                            const bool act = task0 + tsub < n_tasks && a < G;
+                            // Slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag.
+                            uint32_t uo[QN], ui[QN];
+                            {
+                                const uint32_t* const row = (kp.big_stage ? (const uint32_t*)(smem_raw + L.fam_task) : dc.fam_task) + ((size_t)f * G + ag) * 8;
+                                if (SPLIT == 1) {
+                                    const uint4 o = kp.big_stage ? *(const uint4*)row : __ldg((const uint4*)row);
+                                    const uint4 i = kp.big_stage ? *((const uint4*)row + 1) : __ldg((const uint4*)row + 1);
+                                    uo[0] = o.x; uo[1] = o.y; uo[QN - 2] = o.z; uo[QN - 1] = o.w;
+                                    ui[0] = i.x; ui[1] = i.y; ui[QN - 2] = i.z; ui[QN - 1] = i.w;
+                                } else {
+                                    const uint2 o = kp.big_stage ? *((const uint2*)row + part) : __ldg((const uint2*)row + part);
+                                    const uint2 i = kp.big_stage ? *((const uint2*)row + 2 + part) : __ldg((const uint2*)row + 2 + part);
+                                    uo[0] = o.x; uo[1] = o.y;
+                                    ui[0] = i.x; ui[1] = i.y;
                                 }
                             }
-                            if (hot) {                         // the same from the words at hand
-#pragma unroll
+                            if (!RECORD && pend) write_row(k - 1, inst); // (while the tables travel)
+                            // start t binds in-slot q to row (q + t) mod 4
+                            uint32_t dst = 0, src = 0;
+    #pragma unroll
+                            for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
+                            int dt[QN];                            // tag (3 - row) each out-slot's destination has
+                            auto fetch_dst = [&]() {
+    #pragma unroll
                                 for (int i = 0; i < QN; i++) {
-                                    const int col = colmap[((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]];
-                                    if (col != BIG_HOT_MAX) {
-                                        const uint2 h = *(const uint2*)(Hi + col * N + ag * 4);
-                                        const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
-                                        const uint32_t lo = at[0], hi = at[ST], cap = cap_of(uo[i]);
-                                        hot_credit(v[0][i], __byte_perm(lo, h.x, 0x5410), cap);
-                                        hot_credit(v[1][i], __byte_perm(lo, h.x, 0x7632), cap);
-                                        hot_credit(v[2][i], __byte_perm(hi, h.y, 0x5410), cap);
-                                        hot_credit(v[3][i], __byte_perm(hi, h.y, 0x7632), cap);
+                                    if (CROSS) dt[i] = (int)(((unsigned)ex_dst[(uo[i] >> 16) & 0xffu] >> (uo[i] >> 28)) & 3u);
+                                    else dt[i] = (int)((__shfl_sync(0xffffffffu, dst, (int)(uo[i] >> (17 - SPLIT)), WL) >> (uo[i] >> 28)) & 3u);
+                                }
+                            };
+                            // best key of the group's 4 x 4 tile: v holds this lane's columns
+                            auto best_key = [&](const uint32_t (&v)[4][QN]) {
+                                if constexpr (SPLIT == 1) {
+                                    return big_best_key(v);
+                                } else {                           // both columns of a pair of rows; the other lane has the other two columns
+                                    const uint32_t p01 = add_max(v[0][0], v[1][1], v[1][0] + v[0][1]), p02 = add_max(v[0][0], v[2][1], v[2][0] + v[0][1]);
+                                    const uint32_t p03 = add_max(v[0][0], v[3][1], v[3][0] + v[0][1]), p12 = add_max(v[1][0], v[2][1], v[2][0] + v[1][1]);
+                                    const uint32_t p13 = add_max(v[1][0], v[3][1], v[3][0] + v[1][1]), p23 = add_max(v[2][0], v[3][1], v[3][0] + v[2][1]);
+                                    const uint32_t o01 = __shfl_xor_sync(0xffffffffu, p01, 1), o02 = __shfl_xor_sync(0xffffffffu, p02, 1);
+                                    const uint32_t o03 = __shfl_xor_sync(0xffffffffu, p03, 1), o12 = __shfl_xor_sync(0xffffffffu, p12, 1);
+                                    const uint32_t o13 = __shfl_xor_sync(0xffffffffu, p13, 1), o23 = __shfl_xor_sync(0xffffffffu, p23, 1);
+                                    const uint32_t m0 = add_max(p01, o23, add_max(p02, o13, p03 + o12)), m1 = add_max(p12, o03, add_max(p13, o02, p23 + o01));
+                                    return max_v(m0, m1);
+                                }
+                            };
+                            auto tile_column = [&](uint32_t (&v)[4][QN], int i, uint32_t lo, uint32_t hi) {
+                                v[0][i] = __byte_perm(lo, SPLIT == 1 ? big_tag(0, i) : tags[0][i], 0x5104);      // (low half) << 8 | tag
+                                v[1][i] = __byte_perm(lo, SPLIT == 1 ? big_tag(1, i) : tags[1][i], 0x5324);      // (high half) << 8 | tag
+                                v[2][i] = __byte_perm(hi, SPLIT == 1 ? big_tag(2, i) : tags[2][i], 0x5104);
+                                v[3][i] = __byte_perm(hi, 0u, 0x5324);                                           // (row 3 has tag 0)
+                            };
+                            auto cap_of = [&](uint32_t w) { return one_class ? cap0 : s_cap[(w >> 24) & 0xfu]; };
+                            auto cap2_of = [&](uint32_t w) { return one_class ? cap2 : min_v(s_cap[(w >> 24) & 0xfu], 65535u) * 0x00010001u; };
+                            // exact credit in place of the 16-bit one (the tag byte stays)
+                            auto hot_credit = [&](uint32_t& key, uint32_t cell, uint32_t cap) { key = __byte_perm(key, min_v(cell, cap), 0x6540); };
+                            // source half: one exact assignment per source group
+                            auto source_half = [&]() {
+                                uint32_t v[4][QN];
+    #pragma unroll
+                                for (int i = 0; i < QN; i++) {
+                                    const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
+                                    const uint32_t c2 = cap2_of(uo[i]);
+                                    tile_column(v, i, __vminu2(at[0], c2), __vminu2(at[ST], c2));
+                                }
+                                if (!EXACT && HOT) {          // out-slots bound to a hot column: exact 32-bit cells
+    #pragma unroll
+                                    for (int i = 0; i < QN; i++) {
+                                        const int j = (int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i];
+                                        if (colmap[j] != BIG_HOT_MAX) {
+    #pragma unroll
+                                            for (int r = 0; r < 4; r++)
+                                                v[r][i] = min_v(cr.cell(ag * 4 + r, j), cap_of(uo[i])) * 256u + (v[r][i] & 0xffu);
+                                        }
                                     }
                                 }
-                            }
-                            return best_key(v) & 0xffu;
-                        };
-                        if (CROSS) {
-                            task_sync();                       // (the last task's bytes have been read)
-                            ex_dst[tl] = (uint8_t)dst;
-                            task_sync();
-                        }
-                        fetch_dst();
-                        uint32_t src_new = source_half();
-                        int F_old = -1, F_new = -1;            // this lane's task; the same in all its lanes, as alive is
-                        bool alive = task0 + tsub < n_tasks;
-                        for (int sweep = 0; ; sweep++) {
-                            // If no source binding of a task moved, the destination half would see what it saw last sweep and
-                            // return the same binding and the same F: the run ends here exactly as it would after computing that.
-                            const bool smoved = alive && act && (sweep == 0 || src_new != src);
-                            if (alive) src = src_new;
-                            unsigned who = __ballot_sync(0xffffffffu, smoved);
+                                if (hot) {                         // the same from the words at hand
+    #pragma unroll
+                                    for (int i = 0; i < QN; i++) {
+                                        const int col = colmap[((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]];
+                                        if (col != BIG_HOT_MAX) {
+                                            const uint2 h = *(const uint2*)(Hi + col * N + ag * 4);
+                                            const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
+                                            const uint32_t lo = at[0], hi = at[ST], cap = cap_of(uo[i]);
+                                            hot_credit(v[0][i], __byte_perm(lo, h.x, 0x5410), cap);
+                                            hot_credit(v[1][i], __byte_perm(lo, h.x, 0x7632), cap);
+                                            hot_credit(v[2][i], __byte_perm(hi, h.y, 0x5410), cap);
+                                            hot_credit(v[3][i], __byte_perm(hi, h.y, 0x7632), cap);
+                                        }
+                                    }
+                                }
+                                return best_key(v) & 0xffu;
+                            };
                             if (CROSS) {
-                                if (SPLIT == 1 || part == 0) ex_src[a] = (uint8_t)src;
-                                if (lane == 0) ex_word[sub] = who;
+                                task_sync();                       // (the last task's bytes have been read)
+                                ex_dst[tl] = (uint8_t)dst;
                                 task_sync();
-                                who = ex_word[0] | ex_word[1];
-                            }
-                            if (alive && !(who & tmask)) { F_new = F_old; my_sweeps++; alive = false; }
-                            if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
-                            // destination half: the tags of the in-slots' sources, the cells of their rows
-                            uint32_t v[4][QN];
-                            unsigned tag[QN];
-#pragma unroll
-                            for (int i = 0; i < QN; i++) {
-                                if (CROSS) tag[i] = (unsigned)ex_src[(ui[i] >> 16) & 0xffu] >> (ui[i] >> 28);
-                                else tag[i] = __shfl_sync(0xffffffffu, src, (int)(ui[i] >> (17 - SPLIT)), WL) >> (ui[i] >> 28);
-                                const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
-                                const unsigned sel = 0x7632u - (tag[i] & 1u) * 0x2222u;        // high or low halves
-                                const uint32_t c2 = cap2_of(ui[i]);
-                                tile_column(v, i, __vminu2(__byte_perm(w.x, w.y, sel), c2), __vminu2(__byte_perm(w.z, w.w, sel), c2));
-                            }
-                            if (!EXACT && hot_mode && *((const uint32_t*)colmap + ag) != BIG_HOT_NONE) {
-#pragma unroll
-                                for (int r = 0; r < 4; r++)
-                                    if (colmap[ag * 4 + r] != BIG_HOT_MAX) {
-#pragma unroll
-                                        for (int i = 0; i < QN; i++)
-                                            v[r][i] = min_v(cr.cell((int)((ui[i] >> 16) & 0xffu) * 4 + 3 - (int)(tag[i] & 3u), ag * 4 + r), cap_of(ui[i])) * 256u +
-                                                      (v[r][i] & 0xffu);
-                                    }
-                            }
-                            uint32_t cols;                     // hot columns among the ranks of this group
-                            if (hot && (cols = *((const uint32_t*)colmap + ag)) != BIG_HOT_NONE) {
-#pragma unroll
-                                for (int i = 0; i < QN; i++) {
-                                    const uint16_t* const h = Hi + ((ui[i] >> 16) & 0xffu) * 4 + 3 - (tag[i] & 3u);
-                                    const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
-                                    const unsigned sel = 0x5410u + (~tag[i] & 1u) * 0x0022u;   // its half, then the high half from the side array
-                                    const uint32_t cap = cap_of(ui[i]);
-                                    hot_credit(v[0][i], __byte_perm(w.x, h[(cols & 0xffu) * N], sel), cap);
-                                    hot_credit(v[1][i], __byte_perm(w.y, h[(cols >> 8 & 0xffu) * N], sel), cap);
-                                    hot_credit(v[2][i], __byte_perm(w.z, h[(cols >> 16 & 0xffu) * N], sel), cap);
-                                    hot_credit(v[3][i], __byte_perm(w.w, h[(cols >> 24) * N], sel), cap);
-                                }
-                            }
-                            const uint32_t key = best_key(v);
-                            const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
-                            if (alive) dst = key & 0xffu;
-                            unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
-                            // Eq. (8): at most 2^8 lanes of less than 2^22 granules.  The next sweep's source half needs no F: it runs while
-                            // the sum is under way and is dropped if the run ends.
-                            const bool more = sweep + 1 < kp.i_aa;
-                            uint32_t F = act ? key >> 8 : 0u;
-                            if constexpr (TPW == 1) F = __reduce_add_sync(0xffffffffu, SPLIT == 1 || part == 0 ? F : 0u);
-                            if (CROSS) {
-                                if (SPLIT == 1 || part == 0) ex_dst[a] = (uint8_t)dst;
-                                if (lane == 0) { ex_word[2 + sub] = who2; ex_word[4 + sub] = F; }
-                                task_sync();
-                                who2 = ex_word[2] | ex_word[3];
-                                F = ex_word[4] + ex_word[5];
                             }
                             fetch_dst();
-                            if (more) src_new = source_half();
-                            if constexpr (TPW > 1) {           // (both lanes of a group hold its credit)
-#pragma unroll
-                                for (int o = SPLIT; o < WL; o <<= 1) F += __shfl_xor_sync(0xffffffffu, F, o);
-                            }
-                            // If no destination binding moved, the next sweep would be a repetition of this one (same sources, same
-                            // destinations, same F) and would end the run, so it is counted and skipped.
-                            if (alive) {
-                                F_new = (int)F;
-                                my_sweeps++;
-                                alive = F_new > F_old && more;
-                                F_old = F_new;
-                                if (alive && !(who2 & tmask)) { my_sweeps++; alive = false; }
-                            }
-                            if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
-                        }
-                        // Eq. (9) volumes of the binding as it stands and the slowest lane of Eq. (10): only needed when several
-                        // families compete on utility
-                        int64_t tmax = 0;
-                        uint32_t bind[QN];                     // source and destination rank of every out-slot
-#pragma unroll
-                        for (int i = 0; i < QN; i++)
-                            bind[i] = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 2 * (part * QN + i))) & 3u)) |
-                                      (uint32_t)((int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]) << 8;
-                        if (H > 1) {
-                            if (act) {
-#pragma unroll
+                            uint32_t src_new = source_half();
+                            int F_old = -1, F_new = -1;            // this lane's task; the same in all its lanes, as alive is
+                            bool alive = task0 + tsub < n_tasks;
+                            for (int sweep = 0; ; sweep++) {
+                                // If no source binding of a task moved, the destination half would see what it saw last sweep and
+                                // return the same binding and the same F: the run ends here exactly as it would after computing that.
+                                const bool smoved = alive && act && (sweep == 0 || src_new != src);
+                                if (alive) src = src_new;
+                                unsigned who = __ballot_sync(0xffffffffu, smoved);
+                                if (CROSS) {
+                                    if (SPLIT == 1 || part == 0) ex_src[a] = (uint8_t)src;
+                                    if (lane == 0) ex_word[sub] = who;
+                                    task_sync();
+                                    who = ex_word[0] | ex_word[1];
+                                }
+                                if (alive && !(who & tmask)) { F_new = F_old; my_sweeps++; alive = false; }
+                                if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
+                                // destination half: the tags of the in-slots' sources, the cells of their rows
+                                uint32_t v[4][QN];
+                                unsigned tag[QN];
+    #pragma unroll
                                 for (int i = 0; i < QN; i++) {
-                                    const uint32_t cl = (uo[i] >> 24) & 0xfu;
-                                    tmax = max_v(tmax, (int64_t)min_v(cr.cell((int)(bind[i] & 0xffu), (int)(bind[i] >> 8)), s_cap[cl]) * s_tscale[cl]);
+                                    if (CROSS) tag[i] = (unsigned)ex_src[(ui[i] >> 16) & 0xffu] >> (ui[i] >> 28);
+                                    else tag[i] = __shfl_sync(0xffffffffu, src, (int)(ui[i] >> (17 - SPLIT)), WL) >> (ui[i] >> 28);
+                                    const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
+                                    const unsigned sel = 0x7632u - (tag[i] & 1u) * 0x2222u;        // high or low halves
+                                    const uint32_t c2 = cap2_of(ui[i]);
+                                    tile_column(v, i, __vminu2(__byte_perm(w.x, w.y, sel), c2), __vminu2(__byte_perm(w.z, w.w, sel), c2));
+                                }
+                                if (!EXACT && HOT && *((const uint32_t*)colmap + ag) != BIG_HOT_NONE) {
+    #pragma unroll
+                                    for (int r = 0; r < 4; r++)
+                                        if (colmap[ag * 4 + r] != BIG_HOT_MAX) {
+    #pragma unroll
+                                            for (int i = 0; i < QN; i++)
+                                                v[r][i] = min_v(cr.cell((int)((ui[i] >> 16) & 0xffu) * 4 + 3 - (int)(tag[i] & 3u), ag * 4 + r), cap_of(ui[i])) * 256u +
+                                                          (v[r][i] & 0xffu);
+                                        }
+                                }
+                                uint32_t cols;                     // hot columns among the ranks of this group
+                                if (hot && (cols = *((const uint32_t*)colmap + ag)) != BIG_HOT_NONE) {
+    #pragma unroll
+                                    for (int i = 0; i < QN; i++) {
+                                        const uint16_t* const h = Hi + ((ui[i] >> 16) & 0xffu) * 4 + 3 - (tag[i] & 3u);
+                                        const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
+                                        const unsigned sel = 0x5410u + (~tag[i] & 1u) * 0x0022u;   // its half, then the high half from the side array
+                                        const uint32_t cap = cap_of(ui[i]);
+                                        hot_credit(v[0][i], __byte_perm(w.x, h[(cols & 0xffu) * N], sel), cap);
+                                        hot_credit(v[1][i], __byte_perm(w.y, h[(cols >> 8 & 0xffu) * N], sel), cap);
+                                        hot_credit(v[2][i], __byte_perm(w.z, h[(cols >> 16 & 0xffu) * N], sel), cap);
+                                        hot_credit(v[3][i], __byte_perm(w.w, h[(cols >> 24) * N], sel), cap);
+                                    }
+                                }
+                                const uint32_t key = best_key(v);
+                                const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
+                                if (alive) dst = key & 0xffu;
+                                unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
+                                // Eq. (8): at most 2^8 lanes of less than 2^22 granules.  The next sweep's source half needs no F: it runs while
+                                // the sum is under way and is dropped if the run ends.
+                                const bool more = sweep + 1 < kp.i_aa;
+                                uint32_t F = act ? key >> 8 : 0u;
+                                if constexpr (TPW == 1) F = __reduce_add_sync(0xffffffffu, SPLIT == 1 || part == 0 ? F : 0u);
+                                if (CROSS) {
+                                    if (SPLIT == 1 || part == 0) ex_dst[a] = (uint8_t)dst;
+                                    if (lane == 0) { ex_word[2 + sub] = who2; ex_word[4 + sub] = F; }
+                                    task_sync();
+                                    who2 = ex_word[2] | ex_word[3];
+                                    F = ex_word[4] + ex_word[5];
+                                }
+                                fetch_dst();
+                                if (more) src_new = source_half();
+                                if constexpr (TPW > 1) {           // (both lanes of a group hold its credit)
+    #pragma unroll
+                                    for (int o = SPLIT; o < WL; o <<= 1) F += __shfl_xor_sync(0xffffffffu, F, o);
+                                }
+                                // If no destination binding moved, the next sweep would be a repetition of this one (same sources, same
+                                // destinations, same F) and would end the run, so it is counted and skipped.
+                                if (alive) {
+                                    F_new = (int)F;
+                                    my_sweeps++;
+                                    alive = F_new > F_old && more;
+                                    F_old = F_new;
+                                    if (alive && !(who2 & tmask)) { my_sweeps++; alive = false; }
+                                }
+                                if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
+                            }
+                            // Eq. (9) volumes of the binding as it stands and the slowest lane of Eq. (10): only needed when several
+                            // families compete on utility
+                            int64_t tmax = 0;
+                            uint32_t bind[QN];                     // source and destination rank of every out-slot
+    #pragma unroll
+                            for (int i = 0; i < QN; i++)
+                                bind[i] = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 2 * (part * QN + i))) & 3u)) |
+                                          (uint32_t)((int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]) << 8;
+                            if (H > 1) {
+                                if (act) {
+    #pragma unroll
+                                    for (int i = 0; i < QN; i++) {
+                                        const uint32_t cl = (uo[i] >> 24) & 0xfu;
+                                        tmax = max_v(tmax, (int64_t)min_v(cr.cell((int)(bind[i] & 0xffu), (int)(bind[i] >> 8)), s_cap[cl]) * s_tscale[cl]);
+                                    }
+                                }
+    #pragma unroll
+                                for (int o = WL / 2; o; o >>= 1) tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+                                if (CROSS) {
+                                    if (lane == 0) ex_time[sub] = tmax;
+                                    task_sync();
+                                    tmax = max_v(ex_time[0], ex_time[1]);
                                 }
                             }
-#pragma unroll
-                            for (int o = WL / 2; o; o >>= 1) tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-                            if (CROSS) {
-                                if (lane == 0) ex_time[sub] = tmax;
-                                task_sync();
-                                tmax = max_v(ex_time[0], ex_time[1]);
+                            if (act) {
+                                uint32_t* const at = (uint32_t*)(bindings + (size_t)task * N + a * 4 + part * QN);
+                                at[0] = bind[0] | bind[1] << 16;
+                                if (QN == 4) at[1] = bind[QN - 2] | bind[QN - 1] << 16;
+                            }
+                            if (tl == 0 && task0 + tsub < n_tasks) {
+                                n_tasks_done++;
+                                task_f[task] = (uint32_t)F_new;
+                                if (H > 1) task_den[task] = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
                             }
                         }
-                        if (act) {
-                            uint32_t* const at = (uint32_t*)(bindings + (size_t)task * N + a * 4 + part * QN);
-                            at[0] = bind[0] | bind[1] << 16;
-                            if (QN == 4) at[1] = bind[QN - 2] | bind[QN - 1] << 16;
-                        }
-                        if (tl == 0 && task0 + tsub < n_tasks) {
-                            n_tasks_done++;
-                            task_f[task] = (uint32_t)F_new;
-                            if (H > 1) task_den[task] = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
-                        }
                     }
-                }
-                if (!RECORD && pend) write_row(k - 1, inst);         // (warps that had no task)
-                __syncthreads();
-                VP_TICK(2);
+                    if (!RECORD && pend) write_row(k - 1, inst);         // (warps that had no task)
+                    __syncthreads();
+                    VP_TICK(2);
 
-                // (C) best start per family (largest F, lowest t), then largest utility, lowest family
-                f0 = s_pick.x; H = s_pick.y;
-                if (H == 0) { st |= VP_ST_UNCOVERED; break; }
-                int wtask;
-                int64_t wF;
-                if (H == 1 && kp.n_start == 4) {                 // one family, four starts: best start, no utilities to compare
-                    const uint4 f4 = *(const uint4*)task_f;
-                    const uint32_t m01 = max_v(f4.x, f4.y), m23 = max_v(f4.z, f4.w);
-                    wF = (int64_t)max_v(m01, m23);
-                    wtask = m01 >= m23 ? (f4.x >= f4.y ? 0 : 1) : (f4.z >= f4.w ? 2 : 3);
-                } else if (H == 1) {
-                    wtask = 0; wF = (int64_t)task_f[0];
-                    for (int t = 1; t < kp.n_start; t++)
-                        if ((int64_t)task_f[t] > wF) { wF = (int64_t)task_f[t]; wtask = t; }
-                } else {
-                    big_select_family(task_f, task_den, H, kp.n_start, lane, wtask, wF);
-                }
-                if (wF <= 0) { st |= VP_ST_NO_PROGRESS; break; }
-                VP_TICK(3);
-
-                // (D) activation k: its volumes off the residual and off the score table
-                if (emits) {
-                    const uint32_t bw = bindings[(size_t)wtask * N + r_emit];
-                    const int i = (int)(bw & 0xffu), j = (int)(bw >> 8);
-                    uint16_t* const cell = cells + ((i >> 1) * ST + j) * 2 + (i & 1);
-                    uint32_t c = *cell, now_cell;
-                    // the table entry of the slot's group pair
-                    int entry;
-                    if (S == 2) {
-                        int delta = (j >> 3) - (r_emit >> 3);
-                        if (delta < 0) delta += P;
-                        entry = delta * 4 + ((r_emit >> 2) & 1) * 2 + ((j >> 2) & 1);
+                    // (C) best start per family (largest F, lowest t), then largest utility, lowest family
+                    f0 = s_pick.x; H = s_pick.y;
+                    if (H == 0) { st |= VP_ST_UNCOVERED; break; }
+                    int wtask;
+                    int64_t wF;
+                    if (H == 1 && kp.n_start == 4) {                 // one family, four starts: best start, no utilities to compare
+                        const uint4 f4 = *(const uint4*)task_f;
+                        const uint32_t m01 = max_v(f4.x, f4.y), m23 = max_v(f4.z, f4.w);
+                        wF = (int64_t)max_v(m01, m23);
+                        wtask = m01 >= m23 ? (f4.x >= f4.y ? 0 : 1) : (f4.z >= f4.w ? 2 : 3);
+                    } else if (H == 1) {
+                        wtask = 0; wF = (int64_t)task_f[0];
+                        for (int t = 1; t < kp.n_start; t++)
+                            if ((int64_t)task_f[t] > wF) { wF = (int64_t)task_f[t]; wtask = t; }
                     } else {
-                        const int ga = r_emit >> 2, gd = j >> 2;
-                        int delta = (int)gnode[gd] - (int)gnode[ga];
-                        if (delta < 0) delta += P;
-                        entry = (delta * S + gnode[G + ga]) * S + gnode[G + gd];
+                        big_select_family(task_f, task_den, H, kp.n_start, lane, wtask, wF);
                     }
-                    p_fam = f0 + (ns_shift >= 0 ? wtask >> ns_shift : wtask / kp.n_start);
-                    uint32_t cap = cap0;
-                    if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + r_emit)];
-                    if (!hot_mode) {
-                        const uint32_t x = min_v(cap, c);
-                        p_x = x;
-                        if (c >= (uint32_t)big_floor) {           // a big cell: exact value in the side list
-                            const uint32_t now = side[c - big_floor] - x;
-                            if (now >= (uint32_t)big_floor) { side[c - big_floor] = now; now_cell = c; }
-                            else now_cell = now;                  // (an ordinary cell from here on)
+                    if (wF <= 0) { st |= VP_ST_NO_PROGRESS; break; }
+                    VP_TICK(3);
+
+                    // (D) activation k: its volumes off the residual and off the score table
+                    if (emits) {
+                        const uint32_t bw = bindings[(size_t)wtask * N + r_emit];
+                        const int i = (int)(bw & 0xffu), j = (int)(bw >> 8);
+                        uint16_t* const cell = cells + ((i >> 1) * ST + j) * 2 + (i & 1);
+                        uint32_t c = *cell, now_cell;
+                        // the table entry of the slot's group pair
+                        int entry;
+                        if (S == 2) {
+                            int delta = (j >> 3) - (r_emit >> 3);
+                            if (delta < 0) delta += P;
+                            entry = delta * 4 + ((r_emit >> 2) & 1) * 2 + ((j >> 2) & 1);
                         } else {
-                            now_cell = c - x;
+                            const int ga = r_emit >> 2, gd = j >> 2;
+                            int delta = (int)gnode[gd] - (int)gnode[ga];
+                            if (delta < 0) delta += P;
+                            entry = (delta * S + gnode[G + ga]) * S + gnode[G + gd];
                         }
-                        *cell = (uint16_t)now_cell;
-                    } else {
-                        const int col = colmap[j];
-                        uint16_t* const hcell = col != BIG_HOT_MAX ? Hi + col * N + i : nullptr;
-                        if (hcell) c |= (uint32_t)*hcell << 16;   // a hot column: the exact 32-bit cell
-                        p_x = min_v(cap, c);
-                        *cell = (uint16_t)(c - p_x);
-                        if (hcell) *hcell = (uint16_t)((c - p_x) >> 16);
-                        if (EXACT && c >= 65536u && c - p_x < 65536u) {   // one less; a column without any is like the others from here on
-                            atomicSub(&s_hot, 1);                 // (this column is this thread's for this activation)
-                            if (--s_beyond[col] == 0) colmap[j] = BIG_HOT_MAX;
+                        p_fam = f0 + (ns_shift >= 0 ? wtask >> ns_shift : wtask / kp.n_start);
+                        uint32_t cap = cap0;
+                        if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + r_emit)];
+                        if (!HOT) {
+                            const uint32_t x = min_v(cap, c);
+                            p_x = x;
+                            if (c >= (uint32_t)big_floor) {           // a big cell: exact value in the side list
+                                const uint32_t now = side[c - big_floor] - x;
+                                if (now >= (uint32_t)big_floor) { side[c - big_floor] = now; now_cell = c; }
+                                else now_cell = now;                  // (an ordinary cell from here on)
+                            } else {
+                                now_cell = c - x;
+                            }
+                            *cell = (uint16_t)now_cell;
+                        } else {
+                            const int col = colmap[j];
+                            uint16_t* const hcell = col != BIG_HOT_MAX ? Hi + col * N + i : nullptr;
+                            if (hcell) c |= (uint32_t)*hcell << 16;   // a hot column: the exact 32-bit cell
+                            p_x = min_v(cap, c);
+                            *cell = (uint16_t)(c - p_x);
+                            if (hcell) *hcell = (uint16_t)((c - p_x) >> 16);
+                            if (EXACT && HOT && c >= 65536u && c - p_x < 65536u) {   // one less; a column without any is like the others from here on
+                                atomicSub(&s_hot, 1);                 // (this column is this thread's for this activation)
+                                if (--s_beyond[col] == 0) colmap[j] = BIG_HOT_MAX;
+                            }
+                        }
+                        atomicSub(&tbl[entry], p_x);                  // (an idle lane takes zero)
+                        p_bind = bw;
+                        if (RECORD) {
+                            record[r_emit] = make_uint2(bw, p_x);
+                            if (r_emit == 0) record[N] = make_uint2((uint32_t)p_fam, 0u);
                         }
                     }
-                    atomicSub(&tbl[entry], p_x);                  // (an idle lane takes zero)
-                    p_bind = bw;
-                    if (RECORD) {
-                        record[r_emit] = make_uint2(bw, p_x);
-                        if (r_emit == 0) record[N] = make_uint2((uint32_t)p_fam, 0u);
-                    }
+                    pend = RECORD ? warp >= n_task_warps : emit_warps;   // plan rows and offset sums follow (write_row)
+                    left -= wF;
+                    k++;
+                    __syncthreads();
+                    VP_TICK(4);
                 }
-                pend = RECORD ? warp >= n_task_warps : emit_warps;   // plan rows and offset sums follow (write_row)
-                left -= wF;
-                k++;
-                __syncthreads();
-                VP_TICK(4);
-            }
-            if (pend) write_row(k - 1, RECORD || !emits ? 0u : __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit));   // the last activation of the matrix
+                if (pend) write_row(k - 1, RECORD || !emits ? 0u : __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit));   // the last activation of the matrix
+            };
+            if (hot_mode) decompose(BigConst<true>()); else decompose(BigConst<false>());
         }
         __syncthreads();
         // ---- idle rows beyond n_steps; offset rows repeat the totals
