@@ -338,14 +338,17 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
             if (!rc) rc = upload(c, pat_term, &dc.pat_term);
             if (!rc) rc = upload(c, shape_pat, &dc.shape_pat);
             // Two rails: when the shapes that share a first row are consecutive, and first rows fall into few classes
-            // with the same list of second rows, the first maximum of Eq. (6) can be taken class by class.
-            if (S == 2 && !rc) {
+            // with the same list of second rows, the first maximum of Eq. (6) can be taken class by class.  (One rail: every shape's
+            // second row is the empty one, whose number is that of the rows.)
+            const std::vector<uint32_t> no_terms;
+            const auto terms_of = [&](uint32_t id) -> const std::vector<uint32_t>& { return id < rows.size() ? rows[id] : no_terms; };
+            if (S <= 2 && !rc) {
                 std::vector<int> run_row, run_start;                       // first row and first shape of every run
                 std::vector<std::vector<uint32_t>> run_list;               // its second rows, in shape order
                 std::vector<char> seen(rows.size(), 0);
                 bool ok = true;
                 for (int s = 0; s < n_shapes && ok; s++) {
-                    const int p0 = (int)(shape_pat[s] & 0xffffu), p1 = (int)(shape_pat[s] >> 16);
+                    const int p0 = (int)(shape_pat[s] & 0xffffu), p1 = S == 2 ? (int)(shape_pat[s] >> 16) : (int)rows.size();
                     if (run_row.empty() || run_row.back() != p0) {
                         if (seen[p0]) ok = false;                           // a first row with two separate runs
                         seen[p0] = 1;
@@ -370,7 +373,7 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
                 }
                 // Units: 2 cl = the first rows of class cl, 2 cl + 1 = its second rows; each unit's entries fill whole
                 // chunks of 32 (one warp each).  An entry carries the row's terms and its place within the unit.
-                const int n = (int)members.size(), stride = (int)max_row + 1;
+                const int n = (int)members.size(), stride = std::max((int)max_row, 3) + 1;
                 size_t n_chunks = 0;
                 for (int cl = 0; cl < n; cl++) n_chunks += (members[cl].size() + 31) / 32 + (lists[cl].size() + 31) / 32;
                 if (ok && n <= 16 && n_chunks <= 32) {
@@ -385,7 +388,7 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
                         for (size_t i = 0; i < padded; i++) {
                             uint32_t* ent = &dec[kHeader + (chunk * 32 + i) * stride];
                             if (i >= src.size()) { ent[stride - 1] = 0xffffffffu; continue; }    // padding: never wins
-                            const std::vector<uint32_t>& row = rows[src[i] & 0xffffu];
+                            const std::vector<uint32_t>& row = terms_of(src[i] & 0xffffu);
                             for (size_t t = 0; t < row.size(); t++) ent[t] = row[t];
                             // tie-break word: the run start for a first row (runs are in shape order), the place for a second row
                             ent[stride - 1] = unit & 1 ? (uint32_t)i : src[i] >> 16;
@@ -396,9 +399,35 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
                     dec[3 + 2 * n] = (uint32_t)chunk;
                     dc.dec_classes = n;
                     dc.dec_words = (int)dec.size();
+                    dc.dec_chunks = (int)n_chunks;
+                    dc.dec_stride = stride;
                     c->dec_host = dec;
                     rc = upload(c, dec, &dc.dec);
                 }
+                // a row per lane (see DevCat::lane_rows)
+                std::vector<uint32_t> second;
+                for (const auto& list : lists)
+                    for (uint32_t p1 : list)
+                        if (std::find(second.begin(), second.end(), p1) == second.end()) second.push_back(p1);
+                bool by_lane = ok && n <= 5 && max_row <= 3 && run_row.size() <= 32 && second.size() <= 32;
+                std::vector<uint32_t> lane_rows(2 * 32 * 4, 0);
+                for (size_t r = run_row.size(); r < 32; r++) lane_rows[4 * r + 3] = 0xffffffffu;
+                for (size_t r = 0; r < run_row.size() && by_lane; r++) {
+                    const std::vector<uint32_t>& row = rows[run_row[r]];
+                    std::copy(row.begin(), row.end(), lane_rows.begin() + 4 * r);
+                    lane_rows[4 * r + 3] = (uint32_t)run_start[r] << 3 | (uint32_t)cls_of[run_list[r]];
+                }
+                for (size_t r = 0; r < second.size() && by_lane; r++) {
+                    const std::vector<uint32_t>& row = terms_of(second[r]);
+                    std::copy(row.begin(), row.end(), lane_rows.begin() + 4 * (32 + r));
+                }
+                for (int cl = 0; cl < n && by_lane; cl++) {
+                    for (size_t place = 0; place < lists[cl].size(); place++) {
+                        const size_t at = std::find(second.begin(), second.end(), lists[cl][place]) - second.begin();
+                        lane_rows[4 * (32 + at) + 3] |= 1u << cl | (uint32_t)place << (5 + 5 * cl);
+                    }
+                }
+                if (by_lane && !rc) rc = upload(c, lane_rows, &dc.lane_rows);
             }
         }
     }

@@ -17,8 +17,10 @@
 //    (P S S entries, 32-bit granules) is kept in shared memory and every activation subtracts its lane volumes from
 //    the entries they fall in, so D-hat itself is needed only once, for the quantum rule and the first table.
 //    The terms of a shape are split by source rail into S rows, and the catalog has few distinct rows (127 per rail
-//    for 4,095 shapes): either every row is scored and every shape is the sum of its S row scores, or the first maximum is
-//    taken class by class (see big_use_dec).  Scores are 32-bit while four times what is left fits.
+//    for 4,095 shapes).  On one and two rails the first maximum is taken class by class (see (A) and big_by_class), the rows'
+//    terms in registers: up to sixteen groups every task warp does it alone, without a barrier, where the block scored rows,
+//    then shapes, then joined its warps behind three barriers.  16 x 64 ranks 659 -> 593 us, 1,024 x 64 ranks 1,455 -> 1,344,
+//    16 x 32 ranks 306 -> 277, 512 x 256 ranks 11,760 -> 11,250.
 //  * Step 2.  A (family, start) task is one or two lanes per rank group: up to four tasks share a warp, the largest are two
 //    warps.  The two halves of a sweep exchange bindings as one byte per group, by shuffles wherever a task fits a warp.
 //  * Emit.  An activation is first taken off the residual and off C; its plan rows and offset sums are written while the next
@@ -53,30 +55,29 @@ constexpr int BIG_SMEM_LIMIT = 227 * 1024 - 2048;   // dynamic shared memory of 
 template <bool V> struct BigConst { static constexpr bool value = V; };
 
 struct BigSmem {
-    int wd, hi, colmap, tbl, rs, pat, dec, gnode, send_acc, recv_acc, red, task_f, task_den, bind, exchange, record, term, bucket, fam_task, total;
+    int wd, hi, colmap, tbl, rs, pat, gnode, send_acc, recv_acc, red, task_f, task_den, bind, exchange, record, term, bucket, fam_task, total;
     int fill, fill_rows;      // source buffers of the asynchronous fill, offset rows per buffer (0: plain stores)
     int pat_words;            // 32-bit words of row-pattern ids per shape (two ids per word)
 };
 
-// The arg-max is taken class by class when the catalog allows it and has enough shapes for that to pay: a few hundred
-// shapes are summed by a few per thread, behind one more barrier.
-#ifndef BIG_DEC_MIN_SHAPES
-#define BIG_DEC_MIN_SHAPES 512
-#endif
-__host__ __device__ inline bool big_use_dec(const DevCat& dc) { return dc.dec != nullptr && dc.n_shapes >= BIG_DEC_MIN_SHAPES; }
+// Is the arg-max taken class by class in 32 bits (see (A) in the kernel)?  Up to sixteen groups every task warp does so by itself, a
+// first and a second row per lane; above, the warps share the chunks of 32 rows, at most BIG_CHUNKS each (of four warps or more).
+constexpr int BIG_CHUNKS = 3;
+__host__ __device__ inline bool big_by_class(const DevCat& dc) {
+    return dc.G <= 16 ? dc.lane_rows != nullptr : dc.dec != nullptr && dc.dec_stride == 4 && dc.dec_chunks <= 4 * BIG_CHUNKS;
+}
 
 __host__ __device__ inline BigSmem big_smem_layout(const DevCat& dc, const KParams& kp) {
     BigSmem L;
-    const bool dec = big_use_dec(dc);
+    const bool by_class = big_by_class(dc);
     int o = 0;
     const int wd_bytes = dc.N / 2 * big_stride(big_lanes(dc.G)) * 4, setup_bytes = dc.G * dc.G * 8 + dc.N * 24;
     L.wd = o;        o += align16(wd_bytes > setup_bytes ? wd_bytes : setup_bytes);   // set-up: D-hat, row and column sums
     L.hi = o;        o += (BIG_HOT_MAX + (dc.G > 32)) * dc.N * 2;   // high halves of the hot columns' cells (and of none of them), or the side list
     L.colmap = o;    o += align16(dc.N);                          // hot-column index of every rank
     L.tbl = o;       o += align16(dc.tbl_size * 4);
-    L.rs = o;        o += dec ? 0 : align16(dc.n_patterns * 8);   // row scores
-    L.pat = o;       o += dec ? 0 : align16(dc.n_patterns * dc.max_row_terms * 4);
-    L.dec = o;       o += dec ? align16(dc.dec_words * 4) : 0;     // class decomposition of the arg-max, if any
+    L.rs = o;        o += align16(dc.n_patterns * 8);             // row scores of the general route, and its tables where it is the usual one
+    L.pat = o;       o += by_class ? 0 : align16(dc.n_patterns * dc.max_row_terms * 4);
     L.gnode = o;     o += align16(dc.G * 2);
     L.send_acc = o;  o += dc.N * 8;
     L.recv_acc = o;  o += dc.N * 8;
@@ -87,7 +88,7 @@ __host__ __device__ inline BigSmem big_smem_layout(const DevCat& dc, const KPara
     L.exchange = o;  o += kp.big_cross ? 4 * BIG_EXCHANGE : 0;     // what the two warps of a task tell each other
     L.record = o;    o += dc.G > 32 ? dc.N * 8 + 16 : 0;           // the activation to be written out: source | destination << 8, volume
     L.pat_words = (dc.S + 1) / 2;
-    L.term = o;      o += dec ? 0 : ((dc.n_shapes + 31) & ~31) * L.pat_words * 4;
+    L.term = o;      o += by_class ? 0 : ((dc.n_shapes + 31) & ~31) * L.pat_words * 4;
     L.bucket = o;    o += align16((dc.n_shapes + 1) * 4);
     // the families' task tables, where a CTA has its SM to itself or they are small: the tables of a new family are otherwise a
     // trip to L2 in the middle of the chain
@@ -177,7 +178,7 @@ __device__ __noinline__ void big_write_in_order(int64_t* row, const int64_t* acc
 }
 
 // Eq. (6) by the general route, in 64 bits (out of line, as the loop should stay small for the instruction caches): scores beyond
-// 32 bits, catalogs whose rows have more than three terms or whose groups are more than two rails.  All threads of the CTA; every
+// 32 bits, and catalogs that have no class structure (see big_by_class).  All threads of the CTA; every
 // warp gets the key of the first maximum, score << 16 | (65535 - shape): a score is at most four times what is left, so below 2^34,
 // and there are fewer than 2^16 shapes.
 __device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t* rs, uint64_t* red, const uint32_t* pat, const uint32_t* spat,
@@ -211,20 +212,11 @@ __device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t
     __syncthreads();
     return big_warp_max64(lane < NT / 32 ? red[lane] : 0ull);
 }
-// One chunk of the class-wise arg-max in 64 bits (see the loop): its key score << 16 | (65535 - tie-break word).  Whole warp.
-__device__ __noinline__ uint64_t big_chunk_key(const uint32_t* tbl, const uint32_t* ent, int ent_words) {
-    uint64_t v = 0;
-#pragma unroll 1
-    for (int t = 0; t < ent_words - 1; t++) v += (uint64_t)tbl[ent[t] & 0xffffu] * (ent[t] >> 16);
-    const uint32_t meta = ent[ent_words - 1];
-    return big_warp_max64(meta == 0xffffffffu ? 0ull : (v << 16 | (uint64_t)(65535u - (meta & 0xffffu))));
-}
-
 // Step 3 when several families compete (kept out of line: most shapes have one family, and the main loop should
 // stay small for the instruction cache): best start per family (largest F, lowest start), then the family of largest
 // utility F / duration by exact cross-multiplication, lowest family first among equals.  Whole warp.
-__device__ __noinline__ void big_select_family(const uint32_t* task_f, const int64_t* task_den, int H, int n_start, int lane,
-                                               int& wtask, int64_t& wF) {
+// (Returns F << 32 | task: by reference the two would live in local memory, also where this is not called.)
+__device__ __noinline__ uint64_t big_select_family(const uint32_t* task_f, const int64_t* task_den, int H, int n_start, int lane) {
     int64_t bf = -1, bd = 1;
     int bt = 0x7fffffff;
     for (int h = lane; h < H; h += 32) {
@@ -245,8 +237,9 @@ __device__ __noinline__ void big_select_family(const uint32_t* task_f, const int
         }
         if (take) { bf = of; bd = od; bt = ot; }
     }
-    wtask = __shfl_sync(0xffffffffu, bt, 0);
-    wF = __shfl_sync(0xffffffffu, bf, 0);
+    bt = __shfl_sync(0xffffffffu, bt, 0);
+    bf = __shfl_sync(0xffffffffu, bf, 0);
+    return (uint64_t)bf << 32 | (uint32_t)bt;
 }
 
 // Work order for a batch whose matrices differ a lot in length: CTAs that take the long matrices first leave a short tail.  An
@@ -398,22 +391,22 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     __shared__ int64_t s_tscale[VP_MAX_CLASSES];
     __shared__ uint32_t s_cap[VP_MAX_CLASSES];
     __shared__ __align__(8) unsigned long long s_stage_bar;
-    unsigned long long n_act = 0, n_tasks_done = 0;
+    unsigned long long n_act = 0;
+    unsigned n_done = 0;
     Counters cnt;                                         // phase cycle counts (only with VP_PHASE_TIMING)
     cnt.t_mark = 0;
     for (int i = 0; i < 6; i++) cnt.cyc[i] = 0;
     const int ns_pad = (dc.n_shapes + 31) & ~31;
     const int S = dc.S, P = dc.P;
-    const bool use_dec = big_use_dec(dc);
-    const uint32_t* const decs = (const uint32_t*)(smem_raw + L.dec);
+    const bool by_class = big_by_class(dc);
 
     // ---- stage the catalog once per CTA: bulk asynchronous copies (TMA) onto one mbarrier; should the bounded wait give
     // up, plain loads fetch the same arrays
     {
-        const void* from[4] = {dc.bucket_ptr, use_dec ? (const void*)dc.dec : dc.shape_pat, dc.pat_term, dc.fam_task};
-        const int at[4] = {L.bucket, use_dec ? L.dec : L.term, L.pat, L.fam_task};
-        const int bytes[4] = {align16((dc.n_shapes + 1) * 4), use_dec ? align16(dc.dec_words * 4) : ns_pad * L.pat_words * 4,
-                              use_dec ? 0 : align16(dc.n_patterns * dc.max_row_terms * 4), kp.big_stage ? dc.n_families * G * 32 : 0};
+        const void* from[4] = {dc.bucket_ptr, dc.shape_pat, dc.pat_term, dc.fam_task};
+        const int at[4] = {L.bucket, L.term, L.pat, L.fam_task};
+        const int bytes[4] = {align16((dc.n_shapes + 1) * 4), by_class ? 0 : ns_pad * L.pat_words * 4,
+                              by_class ? 0 : align16(dc.n_patterns * dc.max_row_terms * 4), kp.big_stage ? dc.n_families * G * 32 : 0};
         const unsigned bar = smem_u32(&s_stage_bar);
         if (tid == 0) {
             mbar_init(bar, 1);
@@ -436,31 +429,33 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         }
         __syncthreads();
     }
-    // ---- what a thread keeps of the catalog for Step 1
-    // class by class: lane = chunk (does the next chunk belong to the same unit?) and lane = class (its two units' first chunks)
-    const int dec_n = use_dec ? dc.dec_classes : 0, n_chunks = use_dec ? (int)decs[0] : 0, ent_words = use_dec ? (int)decs[1] : 0;
-    const uint32_t* const ents = use_dec ? decs + decs[2] : nullptr;
-    int ch0 = 0, ch1 = 0, unit_span = 1;                  // (span: most chunks of a unit)
-    bool ch_more = false;
-    if (use_dec) {
-        if (lane < dec_n) { ch0 = (int)decs[3 + 2 * lane]; ch1 = (int)decs[4 + 2 * lane]; }
-        ch_more = lane + 1 < n_chunks && decs[3 + 2 * dec_n + 1 + lane + 1] == decs[3 + 2 * dec_n + 1 + lane];
-        for (int u = 0; u < 2 * dec_n; u++) unit_span = max(unit_span, (int)(decs[4 + u] - decs[3 + u]));
-    }
-    // scan: this thread's row and its first four shapes
-    uint32_t* const rs32 = (uint32_t*)(smem_raw + L.rs);
-    uint64_t* const rs64 = (uint64_t*)(smem_raw + L.rs);
-    const uint32_t* const pat = (const uint32_t*)(smem_raw + L.pat);
-    const uint32_t* const spat = (const uint32_t*)(smem_raw + L.term);
-    uint32_t my_row[3] = {0u, 0u, 0u}, my_pat[4] = {0u, 0u, 0u, 0u};
-    const bool simple_scan = !use_dec && dc.max_row_terms <= 3 && L.pat_words == 1;
-    if (simple_scan) {
-        if (tid < dc.n_patterns)
-            for (int t = 0; t < dc.max_row_terms; t++) my_row[t] = pat[tid * dc.max_row_terms + t];
+    // ---- what a thread keeps of the catalog for Step 1 (see (A) below)
+    uint64_t* const rs = (uint64_t*)(smem_raw + L.rs);
+    const uint32_t* const pat = by_class ? dc.pat_term : (const uint32_t*)(smem_raw + L.pat);
+    const uint32_t* const spat = by_class ? dc.shape_pat : (const uint32_t*)(smem_raw + L.term);
+    constexpr bool BY_LANE = LANES / SPLIT <= 16;         // a first and a second row per lane, else up to BIG_CHUNKS chunks per warp
+    constexpr int ROWS = BY_LANE ? 2 : BIG_CHUNKS;
+    uint4 row[ROWS];
+    int unit0 = 0, unit0_end = 0, unit1 = 0, unit1_end = 0, unit_span = 1;   // lane = class: chunks of its two units; most chunks of a unit
+    if (by_class) {
+        if constexpr (BY_LANE) {
+            row[0] = __ldg((const uint4*)dc.lane_rows + lane);
+            row[1] = __ldg((const uint4*)dc.lane_rows + 32 + lane);
+        } else {
 #pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (tid + u * NT < dc.n_shapes) my_pat[u] = spat[tid + u * NT];
+            for (int i = 0; i < ROWS; i++) {
+                const int c = warp + i * n_warps;
+                row[i] = __ldg((const uint4*)(dc.dec + dc.dec[2]) + min(c, dc.dec_chunks - 1) * 32 + lane);
+            }
+            if (lane < dc.dec_classes) {
+                unit0 = (int)dc.dec[3 + 2 * lane]; unit0_end = unit1 = (int)dc.dec[4 + 2 * lane]; unit1_end = (int)dc.dec[5 + 2 * lane];
+            }
+            unit_span = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(1, max(unit0_end - unit0, unit1_end - unit1)));
+        }
     }
+    auto row_score = [&](const uint4& w) {
+        return tbl[w.x & 0xffffu] * (w.x >> 16) + tbl[w.y & 0xffffu] * (w.y >> 16) + tbl[w.z & 0xffffu] * (w.z >> 16);
+    };
     const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
     constexpr bool one_class = ONE;
     const int n_task_warps = kp.big_task_warps, emit_warp = kp.big_emit_warp;
@@ -472,6 +467,15 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     const int tl = CROSS ? sub * 32 + lane : lane & (WL - 1), tsub = CROSS ? 0 : lane / WL, a = tl / SPLIT, part = tl - a * SPLIT;
     const unsigned tmask = WL == 32 ? 0xffffffffu : ((1u << (WL & 31)) - 1u) << (tsub * WL);   // the task's lanes
     unsigned my_sweeps = 0;
+    // first task of this lane's and its initial binding: start t binds in-slot q to row (q + t) mod 4 (a byte per group, see (B))
+    auto start_binding = [](int t) {
+        uint32_t dst = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
+        return dst;
+    };
+    const int task_1 = wg * TPW + tsub, h_1 = task_1 / kp.n_start;
+    const uint32_t dst_1 = start_binding(task_1 - h_1 * kp.n_start);
     const int ag = a < G ? a : 0;                         // (spare lanes repeat group 0 and are ignored)
     uint8_t* const ex_src = smem_raw + L.exchange + wg * BIG_EXCHANGE;
     uint8_t* const ex_dst = ex_src + 64;
@@ -709,7 +713,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             // The loop, with and without hot columns: two copies, each with a short path (see "Code size" above).
             auto decompose = [&](auto hot_columns) {
                 constexpr bool HOT = decltype(hot_columns)::value;
-                int64_t left = s_left;
+                uint32_t left = (uint32_t)s_left;                  // (below 2^32 granules, see s_mode)
                 const BigCredits cr{wd, Hi, colmap, ST, N, HOT};
                 const uint32_t cap0 = s_cap[0], cap2 = min_v(cap0, 65535u) * 0x00010001u;
                 // An activation is first taken off the residual; its rows are written while the next one's tasks run: by the thread
@@ -747,93 +751,73 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         big_write_in_order<CROSS ? 5 : 1>(recv_off_b + (size_t)(kk + 1) * N, recv_acc, N, tid - first, RECORD ? NT - first : emit_threads);
                     }
                     pend = false;
-            };
+                };
                 VP_TICK(0);
 
+                int f0 = 0, H = 0;                                 // first family and families of the shape chosen
                 for (;;) {
                     if (left == 0) break;
                     if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
                     // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
                     const uint32_t inst = !RECORD && emit_warp == 0 && pend && emits ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
-                    // (A) Eq. (6).  A score is at most four times what is left, so below 2^34, and there are fewer than 2^16
-                    // shapes: key = score << 16 | (65535 - shape) orders by score first and lower shape index second, and the first
-                    // maximum of Eq. (6) is a plain maximum of keys.
-                    const bool narrow = left < ((int64_t)1 << 30);        // every score fits 32 bits
-                    uint64_t bkey = 0;
-                    if (use_dec) {
-                        // Class by class (two rails).  A shape is a first row p0 and a second row p1 from the list of p0's
-                        // class, and its index grows with p0's place in shape order first, p1's place in the list second.
-                        // So within a class the first maximum is (first maximal p0, first maximal p1 of the list): two
-                        // independent maxima.  One warp per chunk of 32 rows, in shape order: each lane scores its row from the
-                        // table and the first lane with the chunk's largest score leaves score << 16 | (65535 - tie-break word)
-                        // (the word is the run start for a first row, the place in the list for a second row: both grow in shape order).
-                        for (int c = warp; c < n_chunks; c += n_warps) {
-                            if (narrow && ent_words == 4) {
-                                const uint4 e = *((const uint4*)ents + c * 32 + lane);
-                                const uint32_t v = tbl[e.x & 0xffffu] * (e.x >> 16) + tbl[e.y & 0xffffu] * (e.y >> 16) + tbl[e.z & 0xffffu] * (e.z >> 16);
-                                const uint32_t mine = e.w == 0xffffffffu ? 0u : v + 1u;       // (+ 1: any row beats padding)
-                                const uint32_t m = __reduce_max_sync(0xffffffffu, mine);
-                                const unsigned who = __ballot_sync(0xffffffffu, mine == m);
-                                if (lane == __ffs(who) - 1) red[c] = (uint64_t)(m - 1u) << 16 | (uint64_t)(65535u - (e.w & 0xffffu));
-                            } else {
-                                const uint64_t key = big_chunk_key(tbl, ents + (size_t)(c * 32 + lane) * ent_words, ent_words);
-                                if (lane == 0) red[c] = key;
+                    // (A) Eq. (6), class by class (two rails).  A shape is a first row p0 and a second row p1 from the list of p0's class, and
+                    // its index grows with p0's place in shape order first, p1's place in the list second.  So within a class the
+                    // first maximum is (first maximal p0, first maximal p1 of the list): two independent maxima.  32 bits hold every
+                    // score while what is left is below 2^30 (a score is at most four times that); 1 is added so that any row beats none.
+                    int best_s = -1;
+                    if (by_class && left < (1u << 30)) {
+                        if constexpr (BY_LANE) {
+                            // Every task warp by itself, a first and a second row per lane: no barrier.  A first row adds the largest second row
+                            // of its class; among equal sums the lowest run start is the lowest shape, as the runs do not overlap.
+                            if (warp < n_task_warps) {
+                                const uint32_t v0 = row_score(row[0]) + 1u, v1 = row_score(row[1]) + 1u;
+                                uint32_t m1[5], sum = 0;
+#pragma unroll
+                                for (int cl = 0; cl < 5; cl++) {
+                                    m1[cl] = __reduce_max_sync(0xffffffffu, row[1].w >> cl & 1u ? v1 : 0u);
+                                    if ((row[0].w & 7u) == (uint32_t)cl) sum = v0 + m1[cl];
+                                }
+                                const uint32_t best = __reduce_max_sync(0xffffffffu, sum);
+                                const uint32_t first = __reduce_min_sync(0xffffffffu, sum == best ? row[0].w : 0xffffffffu);
+                                const uint32_t cl = first & 7u;
+                                uint32_t most = m1[0];
+#pragma unroll
+                                for (int o = 1; o < 5; o++) if (cl == (uint32_t)o) most = m1[o];
+                                const uint32_t place = __reduce_min_sync(0xffffffffu, (row[1].w >> cl & 1u) && v1 == most ? row[1].w >> (5u + 5u * cl) & 31u : 31u);
+                                if (best > 2u) best_s = (int)((first >> 3) + place);
+                            }
+                        } else {
+                            // A warp per chunk of 32 rows, in shape order: the first lane with the chunk's largest score leaves it with its
+                            // tie-break word (run start or place in the list); every task warp combines them, a class per lane.
+                            uint2* const chunk_best = (uint2*)red;
+#pragma unroll
+                            for (int i = 0; i < ROWS; i++) {
+                                const int c = warp + i * n_warps;
+                                if (c < dc.dec_chunks) {
+                                    const uint32_t v = row[i].w == 0xffffffffu ? 0u : row_score(row[i]) + 1u, m = __reduce_max_sync(0xffffffffu, v);
+                                    const unsigned who = __ballot_sync(0xffffffffu, v == m);
+                                    if (lane == __ffs((int)who) - 1) chunk_best[c] = make_uint2(m, row[i].w);
+                                }
+                            }
+                            __syncthreads();
+                            if (warp < n_task_warps) {
+                                uint2 k0 = chunk_best[unit0], k1 = chunk_best[unit1];
+                                for (int i = 1; i < unit_span; i++) {          // (units of more than 32 rows)
+                                    const uint2 x0 = chunk_best[min(unit0 + i, dc.dec_chunks - 1)], x1 = chunk_best[min(unit1 + i, dc.dec_chunks - 1)];
+                                    if (unit0 + i < unit0_end && x0.x > k0.x) k0 = x0;
+                                    if (unit1 + i < unit1_end && x1.x > k1.x) k1 = x1;
+                                }
+                                const uint32_t sum = lane < dc.dec_classes ? k0.x + k1.x : 0u, best = __reduce_max_sync(0xffffffffu, sum);
+                                const uint32_t s = __reduce_min_sync(0xffffffffu, sum == best ? k0.y + k1.y : 0xffffu);
+                                if (best > 2u) best_s = (int)s;
                             }
                         }
-                        __syncthreads();
-                        if (warp < n_task_warps) {
-                            uint64_t u = lane < n_chunks ? red[lane] : 0ull;       // chunks, then (in each unit's first chunk) units
-                            for (int s = 1; s < unit_span; s++) {
-                                const uint64_t next = __shfl_down_sync(0xffffffffu, u, 1);
-                                if (ch_more) u = max_v(u, next);
-                            }
-                            const uint64_t k0 = __shfl_sync(0xffffffffu, u, ch0), k1 = __shfl_sync(0xffffffffu, u, ch1);   // lane's class: first row, second row
-                            uint64_t cand = 0;
-                            if (lane < dec_n) {
-                                const uint32_t shape = (65535u - (uint32_t)(k0 & 0xffffu)) + (65535u - (uint32_t)(k1 & 0xffffu));   // run start + place
-                                cand = ((k0 >> 16) + (k1 >> 16)) << 16 | (uint64_t)(65535u - shape);
-                            }
-                            bkey = big_warp_max64(cand);
-                        }
-                    } else if (narrow && simple_scan) {
-                        // Row scores (one per thread as a rule), then every shape is the sum of its rows' scores.
-                        for (int p = tid; p < dc.n_patterns; p += NT) {
-                            if (p != tid)
-                                for (int t = 0; t < 3; t++) my_row[t] = t < dc.max_row_terms ? pat[p * dc.max_row_terms + t] : 0u;
-                            rs32[p] = tbl[my_row[0] & 0xffffu] * (my_row[0] >> 16) + tbl[my_row[1] & 0xffffu] * (my_row[1] >> 16) +
-                                      tbl[my_row[2] & 0xffffu] * (my_row[2] >> 16);
-                        }
-                        if (dc.n_patterns > NT && tid < dc.n_patterns)
-                            for (int t = 0; t < dc.max_row_terms; t++) my_row[t] = pat[tid * dc.max_row_terms + t];
-                        __syncthreads();
-                        uint32_t best = 0;
-                        int best_s = 65535;
-    #pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            const int s = tid + u * NT;
-                            if (s < dc.n_shapes) {
-                                const uint32_t v = rs32[my_pat[u] & 0xffffu] + (S > 1 ? rs32[my_pat[u] >> 16] : 0u);
-                                if (v > best) { best = v; best_s = s; }
-                            }
-                        }
-                        for (int s = tid + 4 * NT; s < dc.n_shapes; s += NT) {
-                            const uint32_t pw = spat[s], v = rs32[pw & 0xffffu] + (S > 1 ? rs32[pw >> 16] : 0u);
-                            if (v > best) { best = v; best_s = s; }
-                        }
-                        const uint32_t m = __reduce_max_sync(0xffffffffu, best);
-                        const uint32_t s1 = __reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 65535u);
-                        bkey = (uint64_t)m << 16 | (uint64_t)(65535u - s1);
-                        if (lane == 0) red[warp] = bkey;           // the warps' candidates
-                        __syncthreads();
-                        if (warp < n_task_warps) bkey = big_warp_max64(lane < n_warps ? red[lane] : 0ull);
                     } else {
-                        bkey = big_first_maximum(tbl, rs64, red, pat, spat, dc.n_patterns, dc.max_row_terms, dc.n_shapes, S);
+                        const uint64_t key = big_first_maximum(tbl, rs, red, pat, spat, dc.n_patterns, dc.max_row_terms, dc.n_shapes, S);
+                        if (warp < n_task_warps && (key >> 16) != 0) best_s = 65535 - (int)(key & 0xffffu);
                     }
-                    int f0 = 0, H = 0;                             // (warps without a task learn them after Step 2)
-                    if (warp < n_task_warps && (bkey >> 16) != 0) {
-                        const int best_s = 65535 - (int)(bkey & 0xffffu);
-                        f0 = (int)bucket[best_s]; H = (int)bucket[best_s + 1] - f0;
-                    }
+                    f0 = 0; H = 0;                                 // (warps without a task learn them after Step 2)
+                    if (best_s >= 0) { f0 = (int)bucket[best_s]; H = (int)bucket[best_s + 1] - f0; }
                     if (tid == 0) s_pick = make_int2(f0, H);
                     const int n_tasks = H * kp.n_start;
                     VP_TICK(1);
@@ -859,7 +843,14 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     if (warp < n_task_warps) {
                         for (int task0 = wg * TPW; task0 < n_tasks; task0 += n_tg * TPW) {
                             const int task = min(task0 + tsub, n_tasks - 1);
-                            const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, f = f0 + h, t = task - h * kp.n_start;
+                            int h = h_1;
+                            uint32_t dst = dst_1, src = 0;
+                            if (task0 >= n_tg * TPW) {             // (further families)
+                                h = task / kp.n_start;
+                                dst = start_binding(task - h * kp.n_start);
+                                if (CROSS) task_sync();            // (the last task's bytes have been read)
+                            }
+                            const int f = f0 + min(h, H - 1);      // (a lane without a task repeats another's reads)
                             const bool act = task0 + tsub < n_tasks && a < G;
                             // Slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag.
                             uint32_t uo[QN], ui[QN];
@@ -878,13 +869,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 }
                             }
                             if (!RECORD && pend) write_row(k - 1, inst); // (while the tables travel)
-                            // start t binds in-slot q to row (q + t) mod 4
-                            uint32_t dst = 0, src = 0;
-    #pragma unroll
-                            for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
                             int dt[QN];                            // tag (3 - row) each out-slot's destination has
                             auto fetch_dst = [&]() {
-    #pragma unroll
+#pragma unroll
                                 for (int i = 0; i < QN; i++) {
                                     if (CROSS) dt[i] = (int)(((unsigned)ex_dst[(uo[i] >> 16) & 0xffu] >> (uo[i] >> 28)) & 3u);
                                     else dt[i] = (int)((__shfl_sync(0xffffffffu, dst, (int)(uo[i] >> (17 - SPLIT)), WL) >> (uo[i] >> 28)) & 3u);
@@ -918,25 +905,25 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             // source half: one exact assignment per source group
                             auto source_half = [&]() {
                                 uint32_t v[4][QN];
-    #pragma unroll
+#pragma unroll
                                 for (int i = 0; i < QN; i++) {
                                     const uint32_t* const at = wd + ((int)(uo[i] & 0xffffu) - dt[i]);
                                     const uint32_t c2 = cap2_of(uo[i]);
                                     tile_column(v, i, __vminu2(at[0], c2), __vminu2(at[ST], c2));
                                 }
                                 if (!EXACT && HOT) {          // out-slots bound to a hot column: exact 32-bit cells
-    #pragma unroll
+#pragma unroll
                                     for (int i = 0; i < QN; i++) {
                                         const int j = (int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i];
                                         if (colmap[j] != BIG_HOT_MAX) {
-    #pragma unroll
+#pragma unroll
                                             for (int r = 0; r < 4; r++)
                                                 v[r][i] = min_v(cr.cell(ag * 4 + r, j), cap_of(uo[i])) * 256u + (v[r][i] & 0xffu);
                                         }
                                     }
                                 }
                                 if (hot) {                         // the same from the words at hand
-    #pragma unroll
+#pragma unroll
                                     for (int i = 0; i < QN; i++) {
                                         const int col = colmap[((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]];
                                         if (col != BIG_HOT_MAX) {
@@ -952,12 +939,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 }
                                 return best_key(v) & 0xffu;
                             };
-                            if (CROSS) {
-                                task_sync();                       // (the last task's bytes have been read)
-                                ex_dst[tl] = (uint8_t)dst;
-                                task_sync();
-                            }
-                            fetch_dst();
+#pragma unroll
+                            for (int i = 0; i < QN; i++) dt[i] = (int)((dst >> (uo[i] >> 28)) & 3u);   // (every group starts from the same binding)
                             uint32_t src_new = source_half();
                             int F_old = -1, F_new = -1;            // this lane's task; the same in all its lanes, as alive is
                             bool alive = task0 + tsub < n_tasks;
@@ -978,7 +961,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 // destination half: the tags of the in-slots' sources, the cells of their rows
                                 uint32_t v[4][QN];
                                 unsigned tag[QN];
-    #pragma unroll
+#pragma unroll
                                 for (int i = 0; i < QN; i++) {
                                     if (CROSS) tag[i] = (unsigned)ex_src[(ui[i] >> 16) & 0xffu] >> (ui[i] >> 28);
                                     else tag[i] = __shfl_sync(0xffffffffu, src, (int)(ui[i] >> (17 - SPLIT)), WL) >> (ui[i] >> 28);
@@ -988,10 +971,10 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                     tile_column(v, i, __vminu2(__byte_perm(w.x, w.y, sel), c2), __vminu2(__byte_perm(w.z, w.w, sel), c2));
                                 }
                                 if (!EXACT && HOT && *((const uint32_t*)colmap + ag) != BIG_HOT_NONE) {
-    #pragma unroll
+#pragma unroll
                                     for (int r = 0; r < 4; r++)
                                         if (colmap[ag * 4 + r] != BIG_HOT_MAX) {
-    #pragma unroll
+#pragma unroll
                                             for (int i = 0; i < QN; i++)
                                                 v[r][i] = min_v(cr.cell((int)((ui[i] >> 16) & 0xffu) * 4 + 3 - (int)(tag[i] & 3u), ag * 4 + r), cap_of(ui[i])) * 256u +
                                                           (v[r][i] & 0xffu);
@@ -999,7 +982,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 }
                                 uint32_t cols;                     // hot columns among the ranks of this group
                                 if (hot && (cols = *((const uint32_t*)colmap + ag)) != BIG_HOT_NONE) {
-    #pragma unroll
+#pragma unroll
                                     for (int i = 0; i < QN; i++) {
                                         const uint16_t* const h = Hi + ((ui[i] >> 16) & 0xffu) * 4 + 3 - (tag[i] & 3u);
                                         const uint4 w = *(const uint4*)(wd + ((int)(ui[i] & 0xffffu) - (int)((tag[i] >> 1) & 1u) * ST));
@@ -1030,7 +1013,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 fetch_dst();
                                 if (more) src_new = source_half();
                                 if constexpr (TPW > 1) {           // (both lanes of a group hold its credit)
-    #pragma unroll
+#pragma unroll
                                     for (int o = SPLIT; o < WL; o <<= 1) F += __shfl_xor_sync(0xffffffffu, F, o);
                                 }
                                 // If no destination binding moved, the next sweep would be a repetition of this one (same sources, same
@@ -1048,19 +1031,19 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             // families compete on utility
                             int64_t tmax = 0;
                             uint32_t bind[QN];                     // source and destination rank of every out-slot
-    #pragma unroll
+#pragma unroll
                             for (int i = 0; i < QN; i++)
                                 bind[i] = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 2 * (part * QN + i))) & 3u)) |
                                           (uint32_t)((int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]) << 8;
                             if (H > 1) {
                                 if (act) {
-    #pragma unroll
+#pragma unroll
                                     for (int i = 0; i < QN; i++) {
                                         const uint32_t cl = (uo[i] >> 24) & 0xfu;
                                         tmax = max_v(tmax, (int64_t)min_v(cr.cell((int)(bind[i] & 0xffu), (int)(bind[i] >> 8)), s_cap[cl]) * s_tscale[cl]);
                                     }
                                 }
-    #pragma unroll
+#pragma unroll
                                 for (int o = WL / 2; o; o >>= 1) tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
                                 if (CROSS) {
                                     if (lane == 0) ex_time[sub] = tmax;
@@ -1074,7 +1057,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 if (QN == 4) at[1] = bind[QN - 2] | bind[QN - 1] << 16;
                             }
                             if (tl == 0 && task0 + tsub < n_tasks) {
-                                n_tasks_done++;
+                                n_done++;
                                 task_f[task] = (uint32_t)F_new;
                                 if (H > 1) task_den[task] = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
                             }
@@ -1085,23 +1068,25 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     VP_TICK(2);
 
                     // (C) best start per family (largest F, lowest t), then largest utility, lowest family
-                    f0 = s_pick.x; H = s_pick.y;
+                    if (warp >= n_task_warps) { f0 = s_pick.x; H = s_pick.y; }
                     if (H == 0) { st |= VP_ST_UNCOVERED; break; }
                     int wtask;
-                    int64_t wF;
+                    uint32_t wF;
                     if (H == 1 && kp.n_start == 4) {                 // one family, four starts: best start, no utilities to compare
                         const uint4 f4 = *(const uint4*)task_f;
                         const uint32_t m01 = max_v(f4.x, f4.y), m23 = max_v(f4.z, f4.w);
-                        wF = (int64_t)max_v(m01, m23);
+                        wF = max_v(m01, m23);
                         wtask = m01 >= m23 ? (f4.x >= f4.y ? 0 : 1) : (f4.z >= f4.w ? 2 : 3);
                     } else if (H == 1) {
-                        wtask = 0; wF = (int64_t)task_f[0];
+                        wtask = 0; wF = task_f[0];
+#pragma unroll 1
                         for (int t = 1; t < kp.n_start; t++)
-                            if ((int64_t)task_f[t] > wF) { wF = (int64_t)task_f[t]; wtask = t; }
+                            if (task_f[t] > wF) { wF = task_f[t]; wtask = t; }
                     } else {
-                        big_select_family(task_f, task_den, H, kp.n_start, lane, wtask, wF);
+                        const uint64_t chosen = big_select_family(task_f, task_den, H, kp.n_start, lane);
+                        wtask = (int)(uint32_t)chosen; wF = (uint32_t)(chosen >> 32);
                     }
-                    if (wF <= 0) { st |= VP_ST_NO_PROGRESS; break; }
+                    if (wF == 0) { st |= VP_ST_NO_PROGRESS; break; }
                     VP_TICK(3);
 
                     // (D) activation k: its volumes off the residual and off the score table
@@ -1209,7 +1194,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     bulk_wait_all();
     unsigned long long* stats = (unsigned long long*)(counter + 4);
     if (tid == 0 && n_act) atomicAdd(&stats[0], n_act);
-    n_tasks_done = (unsigned long long)warp_sum_i64((int64_t)n_tasks_done);    // (counted by the first lane of every task)
+    const unsigned long long n_tasks_done = (unsigned long long)warp_sum_i64((int64_t)n_done);   // (counted by the first lane of every task)
     const unsigned long long n_sweeps = (unsigned long long)warp_sum_i64(tl == 0 && warp < n_task_warps ? (int64_t)my_sweeps : 0);
     if (lane == 0 && n_tasks_done) { atomicAdd(&stats[1], n_tasks_done); atomicAdd(&stats[2], n_sweeps); }
 #ifdef VP_PHASE_TIMING

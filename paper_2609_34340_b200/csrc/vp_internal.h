@@ -33,7 +33,7 @@ struct DevCat {
     const uint32_t* pat_term;
     const uint32_t* shape_pat;
     int n_patterns, max_row_terms;
-    // Class decomposition of the arg-max (two rails): the shapes with first row p0 are consecutive, starting at shape
+    // Class decomposition of the arg-max (two rails; one rail counts as two with an empty second row): the shapes with first row p0 are consecutive, starting at shape
     // run_start(p0), and first rows of one class share the list of second rows that complete them, in shape order, so
     // shape(p0, p1) = run_start(p0) + place of p1 in the list of p0's class.  Unit 2 cl holds the first rows of class cl,
     // unit 2 cl + 1 its second rows, each padded to whole chunks of 32 entries.  dec[0] = chunks, dec[1] = words per
@@ -41,7 +41,11 @@ struct DevCat {
     // (table index | count << 16, zero padded) followed by its tie-break word: run_start for a first row, place for a second row (all ones marks padding).  Null
     // when the catalog has no such structure.
     const uint32_t* dec;
-    int dec_classes, dec_words;
+    int dec_classes, dec_words, dec_chunks, dec_stride;
+    // The same for at most 32 first and 32 second rows of at most three terms in at most five classes, a row of each per lane: 32 x
+    // (three terms, run_start << 3 | class; all ones: no row), then 32 x (three terms, a bit for every class whose list holds the row
+    // and, five bits each from bit 5 on, its places in the lists).  Null when the catalog has no such structure.
+    const uint32_t* lane_rows;
     const uint32_t* bucket_ptr;
     // family f, slot r: instance id | destination group << 16 | rate class << 24
     const uint32_t* fam_slot;

@@ -7,7 +7,7 @@ import pytest
 import tests.test_gpu_schedule as ts
 from tests.test_gpu_schedule import vp  # noqa: F401  (fixture)
 from workloads import SchedParams as WParams, complete_catalog, node_template_catalog, tree_topology
-from workloads.topology import ring_topology
+from workloads.topology import _assemble, ring_topology
 
 pytestmark = pytest.mark.gpu
 
@@ -139,3 +139,35 @@ def test_launch_shapes_of_node_symmetric_catalogs(vp, oracle_lib, name, batches)
     """Up to eight groups CTAs of two lanes per group are followed by CTAs of one that pack the SMs, above by CTAs of one and warps
     that emit: the last batch of a shape and the first of the next, and batches beyond one wave."""
     test_work_counters_and_batches(vp, oracle_lib, name, batches)
+
+
+def _one_rail(nodes):
+    """One switch per node: every rank group keeps its four lanes, or sends one to the group `delta` further on."""
+    topo = tree_topology(nodes, switches_per_node=1)
+    by_key = {(r.src_group, r.dst_group): i for i, r in enumerate(topo.instances)}
+    fams = [tuple(sorted(x for a in range(nodes) for x in [by_key[a, a]] * (3 if d else 4) + ([by_key[a, (a + d) % nodes]] if d else [])))
+            for d in range(nodes)]
+    return _assemble(topo, fams)
+
+
+@pytest.mark.parametrize("nodes,rails", [(2, 2), (3, 2), (4, 2), (8, 2), (9, 2), (16, 2), (17, 2), (2, 1), (5, 1), (16, 1), (17, 1), (40, 1)])
+def test_first_maximum_by_class(vp, oracle_lib, nodes, rails):  # noqa: F811
+    """Step 1 class by class, a row per lane (up to sixteen groups) and in chunks, with two rails and one: shape scores that tie
+    massively (every cell equal; inside the switches only; between neighbours only), a single cell, and random ones."""
+    cat = node_template_catalog(tree_topology(nodes)) if rails == 2 else _one_rail(nodes)
+    N = cat.topology.N
+    rng = np.random.default_rng(10 * nodes + rails)
+    D = (rng.integers(0, 900, size=(6, N, N)) * (rng.random((6, N, N)) < 0.3)).astype(np.int64)
+    group = np.arange(N) // 4
+    D[1] = 1000
+    D[2] = 700 * (group[:, None] == group[None, :])
+    D[3] = 500 * ((group[:, None] ^ 1) == group[None, :])
+    D[4] = 0
+    D[4][1, N - 2] = 77
+    D *= 256
+    for b in range(6):
+        np.fill_diagonal(D[b], 0)
+    for extra in ({}, {"k_target": N, "n_start": 3}):
+        w = WParams(granule_bytes=256, k_max=12 * N, **extra).resolved(N)
+        got, want, *_ = ts._both(vp, oracle_lib, cat, D, w)
+        ts._assert_same(got, want)
