@@ -39,6 +39,10 @@
 //    activation does not execute is kept out of its loop: the loop exists twice, with and without hot columns, and the 64-bit
 //    scores are functions of their own.  As one loop of 65 KB with all cases inside: 16 x 64 ranks 774 -> 659 us,
 //    1,024 x 64 ranks 1,591 -> 1,455, 512 x 256 ranks 12,560 -> 11,760.
+//  * Instructions.  A warp that is alone on its scheduler issues one in four to five cycles, whatever it is, and a task warp executes
+//    hundreds per activation.  So integer divisions and further families are out of line, rows are written at one place, a
+//    warp with a single task carries no "alive" flags, the run ends as soon as a ballot says so, and the usual path is laid out
+//    straight: 593 -> 532 us, 1,344 -> 1,275, 11,250 -> 10,630; 16 x 32 ranks 277 -> 247, 16 x 96 ranks 1,296 -> 1,225.
 //
 // A matrix that does not meet the conditions (granule below 256 bytes, a capacity of 2^22 granules or more, 2^32
 // granules or more in total, more than 32 hot columns, more big cells than the side list holds) is appended to a list that
@@ -51,6 +55,11 @@ constexpr int BIG_HOT_MAX = 32;       // columns whose cells are kept beyond 16 
 constexpr uint32_t BIG_HOT_NONE = 0x01010101u * BIG_HOT_MAX;  // a group without a hot column
 constexpr int BIG_EXCHANGE = 192;     // bytes per pair of warps: 64 source tags, 64 destination tags, words
 constexpr int BIG_SMEM_LIMIT = 227 * 1024 - 2048;   // dynamic shared memory of one CTA, less room for the static variables
+
+// Branch weights: the usual path of an activation runs straight through (every jump beyond the nearest instruction cache waits for
+// the next one).
+__device__ __forceinline__ bool usually(bool c) { return __builtin_expect(c, 1); }
+__device__ __forceinline__ bool rarely(bool c) { return __builtin_expect(c, 0); }
 
 template <bool V> struct BigConst { static constexpr bool value = V; };
 
@@ -212,6 +221,16 @@ __device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t
     __syncthreads();
     return big_warp_max64(lane < NT / 32 ? red[lane] : 0ull);
 }
+// Family (of those that compete) and initial binding of a (family, start) task: h << 8 | binding, as a byte per group (see (B)).  Start t
+// binds in-slot q to row (q + t) mod 4.
+__device__ __noinline__ uint32_t big_family_and_start(int task, int n_start) {
+    const int h = task / n_start, t = task - h * n_start;
+    uint32_t dst = (uint32_t)h << 8;
+#pragma unroll
+    for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
+    return dst;
+}
+
 // Step 3 when several families compete (kept out of line: most shapes have one family, and the main loop should
 // stay small for the instruction cache): best start per family (largest F, lowest start), then the family of largest
 // utility F / duration by exact cross-multiplication, lowest family first among equals.  Whole warp.
@@ -456,7 +475,6 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     auto row_score = [&](const uint4& w) {
         return tbl[w.x & 0xffffu] * (w.x >> 16) + tbl[w.y & 0xffffu] * (w.y >> 16) + tbl[w.z & 0xffffu] * (w.z >> 16);
     };
-    const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
     constexpr bool one_class = ONE;
     const int n_task_warps = kp.big_task_warps, emit_warp = kp.big_emit_warp;
     const int r_emit = tid - emit_warp * 32;              // this thread's slot when it emits
@@ -467,15 +485,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     const int tl = CROSS ? sub * 32 + lane : lane & (WL - 1), tsub = CROSS ? 0 : lane / WL, a = tl / SPLIT, part = tl - a * SPLIT;
     const unsigned tmask = WL == 32 ? 0xffffffffu : ((1u << (WL & 31)) - 1u) << (tsub * WL);   // the task's lanes
     unsigned my_sweeps = 0;
-    // first task of this lane's and its initial binding: start t binds in-slot q to row (q + t) mod 4 (a byte per group, see (B))
-    auto start_binding = [](int t) {
-        uint32_t dst = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
-        return dst;
-    };
-    const int task_1 = wg * TPW + tsub, h_1 = task_1 / kp.n_start;
-    const uint32_t dst_1 = start_binding(task_1 - h_1 * kp.n_start);
+    // this lane's first task: its family (of those that compete) and initial binding
+    const uint32_t first_task = big_family_and_start(wg * TPW + tsub, kp.n_start), dst_1 = first_task & 0xffu;
+    const int h_1 = (int)(first_task >> 8);
     const int ag = a < G ? a : 0;                         // (spare lanes repeat group 0 and are ignored)
     uint8_t* const ex_src = smem_raw + L.exchange + wg * BIG_EXCHANGE;
     uint8_t* const ex_dst = ex_src + 64;
@@ -714,6 +726,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             auto decompose = [&](auto hot_columns) {
                 constexpr bool HOT = decltype(hot_columns)::value;
                 uint32_t left = (uint32_t)s_left;                  // (below 2^32 granules, see s_mode)
+                const uint32_t by_class_below = by_class ? 1u << 30 : 0u;
                 const BigCredits cr{wd, Hi, colmap, ST, N, HOT};
                 const uint32_t cap0 = s_cap[0], cap2 = min_v(cap0, 65535u) * 0x00010001u;
                 // An activation is first taken off the residual; its rows are written while the next one's tasks run: by the thread
@@ -756,8 +769,10 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
 
                 int f0 = 0, H = 0;                                 // first family and families of the shape chosen
                 for (;;) {
-                    if (left == 0) break;
-                    if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
+                    if (rarely(left == 0 || k == kp.k_max)) {
+                        if (left != 0) st |= VP_ST_STEP_LIMIT;
+                        break;
+                    }
                     // path instance of the slot to be written out, where task warps write it: a trip to L2 that ends long before then
                     const uint32_t inst = !RECORD && emit_warp == 0 && pend && emits ? __ldg(dc.fam_slot + (size_t)p_fam * N + r_emit) : 0u;
                     // (A) Eq. (6), class by class (two rails).  A shape is a first row p0 and a second row p1 from the list of p0's class, and
@@ -765,7 +780,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     // first maximum is (first maximal p0, first maximal p1 of the list): two independent maxima.  32 bits hold every
                     // score while what is left is below 2^30 (a score is at most four times that); 1 is added so that any row beats none.
                     int best_s = -1;
-                    if (by_class && left < (1u << 30)) {
+                    if (usually(left < by_class_below)) {
                         if constexpr (BY_LANE) {
                             // Every task warp by itself, a first and a second row per lane: no barrier.  A first row adds the largest second row
                             // of its class; among equal sums the lowest run start is the lowest shape, as the runs do not overlap.
@@ -816,14 +831,41 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         const uint64_t key = big_first_maximum(tbl, rs, red, pat, spat, dc.n_patterns, dc.max_row_terms, dc.n_shapes, S);
                         if (warp < n_task_warps && (key >> 16) != 0) best_s = 65535 - (int)(key & 0xffffu);
                     }
-                    f0 = 0; H = 0;                                 // (warps without a task learn them after Step 2)
-                    if (best_s >= 0) { f0 = (int)bucket[best_s]; H = (int)bucket[best_s + 1] - f0; }
+                    f0 = (int)bucket[max(best_s, 0)];              // (warps without a task learn them after Step 2)
+                    H = best_s >= 0 ? (int)bucket[best_s + 1] - f0 : 0;
                     if (tid == 0) s_pick = make_int2(f0, H);
                     const int n_tasks = H * kp.n_start;
                     VP_TICK(1);
 
-                    // ---- rows of the last activation, where warps without a task write them, and a block of the fill
-                    if (warp >= n_task_warps && pend) write_row(k - 1, inst);
+                    const bool hot = EXACT && HOT && s_hot > 0;            // (none beyond 16 bits left: the 16-bit credits are exact)
+                    // (B) MultiStartAA: LANES lanes per (family, start), SPLIT of them per rank group.
+                    //
+                    // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits,
+                    // of position 3 in the lowest.  An in-slot finds the tag of its slot in the byte of the slot's source group, an
+                    // out-slot the tag of its destination likewise: by a shuffle inside a warp, through shared memory between two.
+                    // Slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag.
+                    uint32_t uo[QN], ui[QN];
+                    auto fetch_slots = [&](int f) {
+                        const unsigned at = ((unsigned)f * (unsigned)G + (unsigned)ag) * 32u + (SPLIT == 2 ? 8u * (unsigned)part : 0u);
+                        auto take = [&](const unsigned char* row) {
+                            if constexpr (SPLIT == 1) {
+                                const uint4 o = *(const uint4*)row, i = *(const uint4*)(row + 16);
+                                uo[0] = o.x; uo[1] = o.y; uo[QN - 2] = o.z; uo[QN - 1] = o.w;
+                                ui[0] = i.x; ui[1] = i.y; ui[QN - 2] = i.z; ui[QN - 1] = i.w;
+                            } else {
+                                const uint2 o = *(const uint2*)row, i = *(const uint2*)(row + 16);
+                                uo[0] = o.x; uo[1] = o.y;
+                                ui[0] = i.x; ui[1] = i.y;
+                            }
+                        };
+                        if (SPLIT == 2 ? usually(kp.big_stage) : rarely(kp.big_stage)) take(smem_raw + L.fam_task + at);
+                        else take((const unsigned char*)dc.fam_task + at);
+                    };
+                    int task0 = warp < n_task_warps ? wg * TPW : n_tasks;
+                    uint32_t dst = dst_1;
+                    if (usually(task0 < n_tasks)) fetch_slots(f0 + min(h_1, H - 1));     // (a lane without a task repeats another's reads)
+                    // ---- rows of the last activation, while the tables travel, and a block of the fill
+                    if (SPLIT == 2 || RECORD ? rarely(pend) : usually(pend)) write_row(k - 1, inst);
                     if (RECORD && fills && warp == fill_warp) {
                         if (fill_lo <= k + 1) {                    // the activations have reached filled rows: those copies must be over
                             bulk_wait_all();
@@ -834,41 +876,11 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         }
                     }
 
-                    const bool hot = EXACT && HOT && s_hot > 0;            // (none beyond 16 bits left: the 16-bit credits are exact)
-                    // (B) MultiStartAA: LANES lanes per (family, start), SPLIT of them per rank group.
-                    //
-                    // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits,
-                    // of position 3 in the lowest.  An in-slot finds the tag of its slot in the byte of the slot's source group, an
-                    // out-slot the tag of its destination likewise: by a shuffle inside a warp, through shared memory between two.
-                    if (warp < n_task_warps) {
-                        for (int task0 = wg * TPW; task0 < n_tasks; task0 += n_tg * TPW) {
+                    if (usually(task0 < n_tasks)) {
+                        for (;;) {
                             const int task = min(task0 + tsub, n_tasks - 1);
-                            int h = h_1;
-                            uint32_t dst = dst_1, src = 0;
-                            if (task0 >= n_tg * TPW) {             // (further families)
-                                h = task / kp.n_start;
-                                dst = start_binding(task - h * kp.n_start);
-                                if (CROSS) task_sync();            // (the last task's bytes have been read)
-                            }
-                            const int f = f0 + min(h, H - 1);      // (a lane without a task repeats another's reads)
-                            const bool act = task0 + tsub < n_tasks && a < G;
-                            // Slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag.
-                            uint32_t uo[QN], ui[QN];
-                            {
-                                const uint32_t* const row = (kp.big_stage ? (const uint32_t*)(smem_raw + L.fam_task) : dc.fam_task) + ((size_t)f * G + ag) * 8;
-                                if (SPLIT == 1) {
-                                    const uint4 o = kp.big_stage ? *(const uint4*)row : __ldg((const uint4*)row);
-                                    const uint4 i = kp.big_stage ? *((const uint4*)row + 1) : __ldg((const uint4*)row + 1);
-                                    uo[0] = o.x; uo[1] = o.y; uo[QN - 2] = o.z; uo[QN - 1] = o.w;
-                                    ui[0] = i.x; ui[1] = i.y; ui[QN - 2] = i.z; ui[QN - 1] = i.w;
-                                } else {
-                                    const uint2 o = kp.big_stage ? *((const uint2*)row + part) : __ldg((const uint2*)row + part);
-                                    const uint2 i = kp.big_stage ? *((const uint2*)row + 2 + part) : __ldg((const uint2*)row + 2 + part);
-                                    uo[0] = o.x; uo[1] = o.y;
-                                    ui[0] = i.x; ui[1] = i.y;
-                                }
-                            }
-                            if (!RECORD && pend) write_row(k - 1, inst); // (while the tables travel)
+                            const bool mine = TPW == 1 || task0 + tsub < n_tasks, act = mine && a < G;
+                            uint32_t src = 0x100u;                 // (no binding yet)
                             int dt[QN];                            // tag (3 - row) each out-slot's destination has
                             auto fetch_dst = [&]() {
 #pragma unroll
@@ -942,22 +954,26 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
 #pragma unroll
                             for (int i = 0; i < QN; i++) dt[i] = (int)((dst >> (uo[i] >> 28)) & 3u);   // (every group starts from the same binding)
                             uint32_t src_new = source_half();
-                            int F_old = -1, F_new = -1;            // this lane's task; the same in all its lanes, as alive is
-                            bool alive = task0 + tsub < n_tasks;
+                            int F_old = -1;                        // this lane's task; the same in all its lanes, as alive is
+                            bool alive = mine;                     // (the only task of a warp lives until its loop ends)
                             for (int sweep = 0; ; sweep++) {
                                 // If no source binding of a task moved, the destination half would see what it saw last sweep and
                                 // return the same binding and the same F: the run ends here exactly as it would after computing that.
-                                const bool smoved = alive && act && (sweep == 0 || src_new != src);
+                                // (Spare lanes follow group 0, so they need no mask.)
+                                unsigned who = __ballot_sync(0xffffffffu, alive && src_new != src);
                                 if (alive) src = src_new;
-                                unsigned who = __ballot_sync(0xffffffffu, smoved);
                                 if (CROSS) {
                                     if (SPLIT == 1 || part == 0) ex_src[a] = (uint8_t)src;
                                     if (lane == 0) ex_word[sub] = who;
                                     task_sync();
                                     who = ex_word[0] | ex_word[1];
                                 }
-                                if (alive && !(who & tmask)) { F_new = F_old; my_sweeps++; alive = false; }
-                                if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
+                                if constexpr (TPW == 1) {
+                                    if (who == 0) { my_sweeps++; break; }
+                                } else {
+                                    if (alive && !(who & tmask)) { my_sweeps++; alive = false; }
+                                    if (!__any_sync(0xffffffffu, alive)) break;
+                                }
                                 // destination half: the tags of the in-slots' sources, the cells of their rows
                                 uint32_t v[4][QN];
                                 unsigned tag[QN];
@@ -995,14 +1011,13 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                     }
                                 }
                                 const uint32_t key = best_key(v);
-                                const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
+                                unsigned who2 = __ballot_sync(0xffffffffu, alive && ((key ^ dst) & 0xffu) != 0);
                                 if (alive) dst = key & 0xffu;
-                                unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
                                 // Eq. (8): at most 2^8 lanes of less than 2^22 granules.  The next sweep's source half needs no F: it runs while
                                 // the sum is under way and is dropped if the run ends.
                                 const bool more = sweep + 1 < kp.i_aa;
-                                uint32_t F = act ? key >> 8 : 0u;
-                                if constexpr (TPW == 1) F = __reduce_add_sync(0xffffffffu, SPLIT == 1 || part == 0 ? F : 0u);
+                                uint32_t F = (TPW == 1 ? a < G && (SPLIT == 1 || part == 0) : act) ? key >> 8 : 0u;
+                                if constexpr (TPW == 1) F = __reduce_add_sync(0xffffffffu, F);
                                 if (CROSS) {
                                     if (SPLIT == 1 || part == 0) ex_dst[a] = (uint8_t)dst;
                                     if (lane == 0) { ex_word[2 + sub] = who2; ex_word[4 + sub] = F; }
@@ -1011,21 +1026,28 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                     F = ex_word[4] + ex_word[5];
                                 }
                                 fetch_dst();
-                                if (more) src_new = source_half();
+                                if (more && (TPW > 1 || who2 != 0)) src_new = source_half();
                                 if constexpr (TPW > 1) {           // (both lanes of a group hold its credit)
 #pragma unroll
                                     for (int o = SPLIT; o < WL; o <<= 1) F += __shfl_xor_sync(0xffffffffu, F, o);
                                 }
                                 // If no destination binding moved, the next sweep would be a repetition of this one (same sources, same
                                 // destinations, same F) and would end the run, so it is counted and skipped.
-                                if (alive) {
-                                    F_new = (int)F;
+                                if constexpr (TPW == 1) {
                                     my_sweeps++;
-                                    alive = F_new > F_old && more;
-                                    F_old = F_new;
-                                    if (alive && !(who2 & tmask)) { my_sweeps++; alive = false; }
+                                    const bool up = (int)F > F_old && more;
+                                    F_old = (int)F;
+                                    if (!up) break;
+                                    if (who2 == 0) { my_sweeps++; break; }
+                                } else {
+                                    if (alive) {
+                                        my_sweeps++;
+                                        alive = (int)F > F_old && more;
+                                        F_old = (int)F;
+                                        if (alive && !(who2 & tmask)) { my_sweeps++; alive = false; }
+                                    }
+                                    if (!__any_sync(0xffffffffu, alive)) break;
                                 }
-                                if (!(TPW == 1 ? alive : __any_sync(0xffffffffu, alive))) break;
                             }
                             // Eq. (9) volumes of the binding as it stands and the slowest lane of Eq. (10): only needed when several
                             // families compete on utility
@@ -1035,7 +1057,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             for (int i = 0; i < QN; i++)
                                 bind[i] = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 2 * (part * QN + i))) & 3u)) |
                                           (uint32_t)((int)((uo[i] >> 16) & 0xffu) * 4 + 3 - dt[i]) << 8;
-                            if (H > 1) {
+                            if (rarely(H > 1)) {
                                 if (act) {
 #pragma unroll
                                     for (int i = 0; i < QN; i++) {
@@ -1056,23 +1078,29 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 at[0] = bind[0] | bind[1] << 16;
                                 if (QN == 4) at[1] = bind[QN - 2] | bind[QN - 1] << 16;
                             }
-                            if (tl == 0 && task0 + tsub < n_tasks) {
+                            if (tl == 0 && mine) {
                                 n_done++;
-                                task_f[task] = (uint32_t)F_new;
-                                if (H > 1) task_den[task] = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
+                                task_f[task] = (uint32_t)F_old;
+                                if (H > 1) task_den[task] = F_old > 0 ? kp.lambda_ns * dc.W + tmax : 1;
                             }
+                            task0 += n_tg * TPW;
+                            if (usually(task0 >= n_tasks)) break;
+                            // (further families)
+                            const uint32_t next = big_family_and_start(min(task0 + tsub, n_tasks - 1), kp.n_start);
+                            dst = next & 0xffu;
+                            fetch_slots(f0 + (int)(next >> 8));
+                            if (CROSS) task_sync();                // (the last task's bytes have been read)
                         }
                     }
-                    if (!RECORD && pend) write_row(k - 1, inst);         // (warps that had no task)
                     __syncthreads();
                     VP_TICK(2);
 
                     // (C) best start per family (largest F, lowest t), then largest utility, lowest family
                     if (warp >= n_task_warps) { f0 = s_pick.x; H = s_pick.y; }
-                    if (H == 0) { st |= VP_ST_UNCOVERED; break; }
-                    int wtask;
+                    int wtask, wfam = f0;
                     uint32_t wF;
-                    if (H == 1 && kp.n_start == 4) {                 // one family, four starts: best start, no utilities to compare
+                    if (rarely(H == 0)) { st |= VP_ST_UNCOVERED; break; }
+                    if (usually(H == 1 && kp.n_start == 4)) {                 // one family, four starts: best start, no utilities to compare
                         const uint4 f4 = *(const uint4*)task_f;
                         const uint32_t m01 = max_v(f4.x, f4.y), m23 = max_v(f4.z, f4.w);
                         wF = max_v(m01, m23);
@@ -1085,8 +1113,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     } else {
                         const uint64_t chosen = big_select_family(task_f, task_den, H, kp.n_start, lane);
                         wtask = (int)(uint32_t)chosen; wF = (uint32_t)(chosen >> 32);
+                        wfam += (int)(big_family_and_start(wtask, kp.n_start) >> 8);
                     }
-                    if (wF == 0) { st |= VP_ST_NO_PROGRESS; break; }
+                    if (rarely(wF == 0)) { st |= VP_ST_NO_PROGRESS; break; }
                     VP_TICK(3);
 
                     // (D) activation k: its volumes off the residual and off the score table
@@ -1107,13 +1136,13 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                             if (delta < 0) delta += P;
                             entry = (delta * S + gnode[G + ga]) * S + gnode[G + gd];
                         }
-                        p_fam = f0 + (ns_shift >= 0 ? wtask >> ns_shift : wtask / kp.n_start);
+                        p_fam = wfam;
                         uint32_t cap = cap0;
                         if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + r_emit)];
                         if (!HOT) {
                             const uint32_t x = min_v(cap, c);
                             p_x = x;
-                            if (c >= (uint32_t)big_floor) {           // a big cell: exact value in the side list
+                            if (rarely(c >= (uint32_t)big_floor)) {           // a big cell: exact value in the side list
                                 const uint32_t now = side[c - big_floor] - x;
                                 if (now >= (uint32_t)big_floor) { side[c - big_floor] = now; now_cell = c; }
                                 else now_cell = now;                  // (an ordinary cell from here on)
