@@ -1184,6 +1184,11 @@ BigKernelFn pick_big_kernel(const DevCat& dc, int split) {
     return dc.n_classes == 1 ? pick_big_kernel_for<true>(dc.G, split) : pick_big_kernel_for<false>(dc.G, split);
 }
 
+WarpKernelFn pick_warp_kernel(const DevCat& dc, bool units) {
+    if (!units) return vp_schedule_warp_kernel<false, false>;
+    return dc.n_classes == 1 ? vp_schedule_warp_kernel<true, true> : vp_schedule_warp_kernel<true, false>;
+}
+
 int resolve_params(const vp_catalog* c, const vp_sched_params* p, KParams* kp) {
     if (!c || !p || c->device < 0) return VP_E_BAD_ARG;         // (a host-only handle launches nothing)
     if (p->k_max <= 0 || p->granule_bytes <= 0 || p->lambda_ns < 0 || p->lambda_ns >= VP_ENTRY_LIMIT) return VP_E_BAD_ARG;
@@ -1296,7 +1301,7 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     // measure the same (1,185 matrices 134 and 136 us; CTAs of one warp 189: an SM holds eight of them).
     if (dc.g == 4 && dc.G <= 4 && !dc.sym && (B > cap || p->granule_bytes >= 256)) {
         const bool units = p->granule_bytes >= 256;
-        const WarpKernelFn wf = units ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;
+        const WarpKernelFn wf = pick_warp_kernel(dc, units);
         const int warps = B <= 4 * c->sm_count ? 1 : (B <= 8 * c->sm_count ? 2 : 4);
         const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
         if (smem <= (size_t)dynamic_smem_limit(c->max_smem_optin)) {
@@ -1402,7 +1407,7 @@ int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int6
         if (!rc) {
             vp_prof_mark(0, 0, stream);
             if (L.kernel == 1) {
-                const WarpKernelFn wf = p->granule_bytes >= 256 ? vp_schedule_warp_kernel<true> : vp_schedule_warp_kernel<false>;
+                const WarpKernelFn wf = pick_warp_kernel(c->dc, p->granule_bytes >= 256);
                 unsigned long long* slots = warp_each ? (unsigned long long*)((char*)workspace + ws_layout(c, L, B).slots) : nullptr;
                 if (launch_after(wf, L.grid, L.threads, L.smem, stream, c->dc, L.kp, demand, tau_ns_in, B, n_steps, chan_id, lane_dst,
                                  lane_inst, lane_bytes, send_off, recv_off, tau_ns_out, status, counter, slots) != cudaSuccess)

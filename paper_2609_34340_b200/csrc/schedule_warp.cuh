@@ -5,15 +5,18 @@
 // the first to the last activation and nothing but __syncwarp orders its phases.  Two forms of the main loop:
 //
 //  * decompose_units: capacities below 2^22 granules (granules of at least 256 bytes, so as a rule).  Bound by the chain of
-//    dependent instructions of one activation, so each phase is cut to few of them:
+//    dependent instructions of one activation, so each phase is cut to few of them, and what an ordinary activation does not
+//    execute (families that compete, 64-bit scores) is out of line, because instructions come from small caches:
 //    (A) a lane scores one row pattern of the catalog (source group x lane counts per destination group: at most 32), then
-//        every shape is the sum of four looked-up row scores; two warp reductions leave the first maximum (Eq. 6);
-//    (B) four (family, start) tasks at a time, two lanes per rank group: a lane reads two of the four columns of its group's
-//        4 x 4 tile (one 16-byte read each) and the pair joins its halves of the exact assignment (Eq. 7) by six shuffles.  A
-//        binding travels as one byte per group, by shuffle.  The next source half runs while Eq. (8) is summed;
-//    (C) every lane knows every F: best start without communication; Evaluate (Eq. 9, 10) only when families compete;
-//    (D) sixteen lanes take the activation off the residual (kept row-major and transposed) and off D-hat; its plan rows
+//        every shape is the sum of four row scores; two warp reductions leave the first maximum (Eq. 6);
+//    (B) four starts at a time, two lanes per rank group: a lane reads two of the four columns of its group's 4 x 4 tile (one
+//        16-byte read each, from credits kept ready) and the pair joins its halves of the exact assignment (Eq. 7) by six
+//        shuffles.  A binding travels as one byte per group, by shuffle.  The next source half runs while Eq. (8) is summed;
+//    (C) one warp maximum of F and start leaves the best start;
+//    (D) sixteen lanes take the activation off the residual, the credits (row-major and transposed) and D-hat; its plan rows
 //        are written in the shadow of the next activation's tasks.
+//    One matrix of 8 ranks 40.2 -> 30.4 us, 256 of 16 ranks 104.6 -> 81.1, 4,096 of 8 ranks 147.9 -> 111.5 by the code out of
+//    line, the credits kept ready and the last sweep's source half left out.
 //  * decompose_bytes: any other matrix, the same algorithm on 64-bit bytes with a lane per rank group.
 //
 // A CTA is one to four such warps that share only the staged catalog.  Included by schedule.cu.
@@ -23,7 +26,7 @@ namespace {
 
 
 struct WarpSmem {                           // byte offsets; the per-warp block comes first, once per warp
-    int drem, dremT, dhat, send_acc, recv_acc, rs, cap64, tscale, cap32, bind, bind_dst, per_warp;
+    int drem, dremT, cred, dhat, send_acc, recv_acc, rs, cap64, tscale, cap32, bind, bind_dst, per_warp;
     int rows, shape_rows, fam_task, term, fam_in, fam_cls, fam_slot, bucket, total;
 };
 
@@ -32,12 +35,14 @@ __host__ __device__ inline WarpSmem warp_smem_layout(const DevCat& dc, const KPa
     WarpSmem L;
     const int ns_pad = (dc.n_shapes + 31) & ~31;
     int o = 0;
-    L.drem = o;      o += align16(dc.N * (dc.N + 1) * 8);      // bytes: rows padded by one element, no bank conflicts down a column
-    L.dremT = L.drem + dc.N * dc.N * 4;                        // 32-bit granules: residual and transpose share that space
+    // bytes: rows padded by one element, no bank conflicts down a column; 32-bit granules: residual, credits and their transpose
+    L.drem = o;      o += align16(dc.N * (dc.N + 1) * 8 > 3 * dc.N * dc.N * 4 ? dc.N * (dc.N + 1) * 8 : 3 * dc.N * dc.N * 4);
+    L.dremT = L.drem + dc.N * dc.N * 4;
+    L.cred = L.dremT + dc.N * dc.N * 4;
     L.dhat = o;      o += align16(dc.G * dc.G * 8);
     L.send_acc = o;  o += dc.N * 8;
     L.recv_acc = o;  o += dc.N * 8;
-    L.rs = o;        o += 144 + 272;                           // row scores: 33 of 32 bits, then 33 of 64 bits
+    L.rs = o;        o += 272;                                 // row scores: 33 of 64 bits
     L.cap64 = o;     o += VP_MAX_CLASSES * 8;
     L.tscale = o;    o += VP_MAX_CLASSES * 8;
     L.cap32 = o;     o += VP_MAX_CLASSES * 4;
@@ -64,7 +69,7 @@ extern __shared__ __align__(16) unsigned char vp_wsmem[];   // the CTA's dynamic
 // pointers: every access is then provably a shared-memory access with a 32-bit address.
 struct WCtx {
     int N, G, lane;
-    unsigned o_drem, o_dremT, o_dhat, o_send_acc, o_recv_acc, o_rs, o_cap64, o_cap32, o_tscale, o_bind, o_bind_dst;
+    unsigned o_drem, o_dremT, o_cred, o_dhat, o_send_acc, o_recv_acc, o_rs, o_cap64, o_cap32, o_tscale, o_bind, o_bind_dst;
     unsigned o_rows, o_shape_rows, o_fam_task, o_bucket;
     const uint32_t *term, *fam_slot;                            // (decompose_bytes: shared or global memory)
     const uint16_t* fam_in;
@@ -87,44 +92,41 @@ __device__ __forceinline__ int64_t team_max(int64_t v) {
     return max_v(v, __shfl_xor_sync(0xffffffffu, v, 2));
 }
 
-// Eq. (6) by row patterns: this lane's pattern, and the byte offsets of the (32-bit) row scores of its up to four shapes.
+// Eq. (6) by row patterns: this lane's pattern, and the patterns of its up to four shapes (a byte per source group; pattern 32 scores
+// zero).
 struct RowScores {
     bool on;
     unsigned rs;
     int n_shapes;
     uint4 row;
-    unsigned so[4][4];
+    uint32_t shape[4];
     __device__ __forceinline__ void load(const DevCat& dc, const WCtx& c) {
         on = dc.row_term != nullptr && dc.n_shapes <= 128;
         rs = c.o_rs;
         n_shapes = dc.n_shapes;
-        if (c.lane == 0) { ws<uint32_t>(rs)[32] = 0u; ws<int64_t>(rs + 144)[32] = 0; }
+        if (c.lane == 0) ws<int64_t>(rs)[32] = 0;
         row = make_uint4(0u, 0u, 0u, 0u);
         if (on) row = *(ws<uint4>(c.o_rows) + c.lane);
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            // (shapes beyond the catalog: four times pattern 32, whose score is zero)
-            const uint32_t w = on && c.lane + 32 * u < n_shapes ? ws<uint32_t>(c.o_shape_rows)[c.lane + 32 * u] : 0x20202020u;
-#pragma unroll
-            for (int r = 0; r < 4; r++) so[u][r] = rs + 4 * ((w >> (8 * r)) & 0xffu);
-        }
+        for (int u = 0; u < 4; u++) shape[u] = on && c.lane + 32 * u < n_shapes ? ws<uint32_t>(c.o_shape_rows)[c.lane + 32 * u] : 0x20202020u;
     }
-    // largest score and, in best_s, the lane's first shape that has it (low words of D-hat)
+    // largest score and, in best_s, the lane's first shape that has it (low words of D-hat); the scores travel by shuffles
     __device__ __forceinline__ uint32_t narrow(const uint32_t* dhat32, int lane, int& best_s) const {
-        ws<uint32_t>(rs)[lane] = dhat32[2 * (row.x & 0xffffu)] * (row.x >> 16) + dhat32[2 * (row.y & 0xffffu)] * (row.y >> 16) +
-                                 dhat32[2 * (row.z & 0xffffu)] * (row.z >> 16) + dhat32[2 * (row.w & 0xffffu)] * (row.w >> 16);
-        __syncwarp();
+        const uint32_t mine = dhat32[2 * (row.x & 0xffffu)] * (row.x >> 16) + dhat32[2 * (row.y & 0xffffu)] * (row.y >> 16) +
+                              dhat32[2 * (row.z & 0xffffu)] * (row.z >> 16) + dhat32[2 * (row.w & 0xffffu)] * (row.w >> 16);
         uint32_t best = 0;
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (u < 3 || n_shapes > 96) {
-                const uint32_t v = *ws<uint32_t>(so[u][0]) + *ws<uint32_t>(so[u][1]) + *ws<uint32_t>(so[u][2]) + *ws<uint32_t>(so[u][3]);
-                if (v > best) { best = v; best_s = lane + 32 * u; }
+            if (u == 0 || n_shapes > (u < 3 ? 32 : 96)) {        // (a few shapes: one per lane)
+                const uint32_t w = shape[u];                    // (a shuffle takes the source lane from the low five bits)
+                uint32_t v = __shfl_sync(0xffffffffu, mine, (int)w) + __shfl_sync(0xffffffffu, mine, (int)(w >> 8)) +
+                             __shfl_sync(0xffffffffu, mine, (int)(w >> 16)) + __shfl_sync(0xffffffffu, mine, (int)(w >> 24));
+                if ((w & 0x20u) == 0 && v > best) { best = v; best_s = lane + 32 * u; }
             }
         return best;
     }
     __device__ __forceinline__ void wide(const int64_t* Dhat, int lane, int64_t& best, int& best_s) const {
-        ws<int64_t>(rs + 144)[lane] = Dhat[row.x & 0xffffu] * (int64_t)(row.x >> 16) + Dhat[row.y & 0xffffu] * (int64_t)(row.y >> 16) +
+        ws<int64_t>(rs)[lane] = Dhat[row.x & 0xffffu] * (int64_t)(row.x >> 16) + Dhat[row.y & 0xffffu] * (int64_t)(row.y >> 16) +
                                 Dhat[row.z & 0xffffu] * (int64_t)(row.z >> 16) + Dhat[row.w & 0xffffu] * (int64_t)(row.w >> 16);
         __syncwarp();
 #pragma unroll
@@ -132,24 +134,24 @@ struct RowScores {
             if (lane + 32 * u < n_shapes) {
                 int64_t v = 0;
 #pragma unroll
-                for (int r = 0; r < 4; r++) v += *ws<int64_t>(2 * so[u][r] - rs + 144);
+                for (int r = 0; r < 4; r++) v += ws<int64_t>(rs)[(shape[u] >> (8 * r)) & 0xffu];
                 if (v > best) { best = v; best_s = lane + 32 * u; }
             }
     }
 };
 
 // Eq. (6) from the terms themselves, for catalogs with more patterns or shapes than that: first maximum of this lane's shapes.
-__device__ __forceinline__ void score_terms(const DevCat& dc, const uint32_t* term, const int64_t* Dhat, int lane, int64_t& best, int& best_s) {
-    const int ns_pad = (dc.n_shapes + 31) & ~31;               // row stride of the transposed term table
-    for (int s0 = lane; s0 < dc.n_shapes; s0 += 128) {         // four shapes per lane in flight
+__device__ __forceinline__ void score_terms(int n_shapes, int max_terms, const uint32_t* term, const int64_t* Dhat, int lane, int64_t& best, int& best_s) {
+    const int ns_pad = (n_shapes + 31) & ~31;               // row stride of the transposed term table
+    for (int s0 = lane; s0 < n_shapes; s0 += 128) {         // four shapes per lane in flight
         int64_t score[4] = {0, 0, 0, 0};
         const uint32_t* tp = term + s0;                        // term e of shape s is at [e][s]: lanes read neighbours
-        const int last = dc.n_shapes - 1 - s0;                 // shapes beyond the catalog re-read the last one
+        const int last = n_shapes - 1 - s0;                 // shapes beyond the catalog re-read the last one
         int du[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) du[u] = min(32 * u, last);
 #pragma unroll 4
-        for (int e = 0; e < dc.max_terms; e++) {
+        for (int e = 0; e < max_terms; e++) {
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const uint32_t w = tp[e * ns_pad + du[u]];
@@ -158,33 +160,189 @@ __device__ __forceinline__ void score_terms(const DevCat& dc, const uint32_t* te
         }
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (s0 + 32 * u < dc.n_shapes && score[u] > best) { best = score[u]; best_s = s0 + 32 * u; }
+            if (s0 + 32 * u < n_shapes && score[u] > best) { best = score[u]; best_s = s0 + 32 * u; }
     }
 }
 
-// Main loop for a matrix held in 32-bit granules (`left` of them) with capacities below 2^22 granules.
-__device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams& kp, const WCtx& c, int64_t left, int& k, int& st, Counters& cnt) {
+// Eq. (6) in 64 bits, from the terms (out of line): first maximal shape, -1 if nothing is covered.
+__device__ __noinline__ int warp_first_shape(int n_shapes, int max_terms, const uint32_t* term, const int64_t* Dhat, int lane) {
+    int64_t best = -1;
+    int best_s = 0x7fffffff;
+    score_terms(n_shapes, max_terms, term, Dhat, lane, best, best_s);
+    warp_argmax_first(best, best_s);
+    return best > 0 ? best_s : -1;
+}
+
+// What a warp's tasks read: the residual in granules (row i at D + i * N); the credits min(residual, largest capacity) << 8, row-major
+// (C) and transposed (CT), so that a tile needs no minimum and no shift on one path rate; the capacities.
+struct WarpUnits {
+    const uint32_t *D, *C, *CT, *cap;
+    int N;
+};
+
+// MultiStartAA of four tasks at a time, two lanes per rank group (eight lanes per task).  uo, ui: slot words of the lane's two
+// out-slots and in-slots (see DevCat::fam_task); dst: the task's initial binding; mine: the lane belongs to a task; act: and to a group.
+//
+// A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits, of position 3 in the
+// lowest.  Spare lanes repeat group 0.  Returns the task's F; src, dt0, dt1: its final binding (dt: tags of the out-slots' destinations).
+template <bool ONE>
+__device__ __forceinline__ uint32_t warp_tasks(const WarpUnits& m, const uint2 uo, const uint2 ui, uint32_t dst, bool mine, bool act, int part,
+                                               unsigned gmask, int i_aa, unsigned& n_sweeps, uint32_t& src, int& dt0, int& dt1) {
+    auto cap_of = [&](uint32_t w) { return ONE ? 0xffffffffu : m.cap[(w >> 24) & 0xfu] << 8; };
+    const uint32_t oc0 = cap_of(uo.x), oc1 = cap_of(uo.y), ic0 = cap_of(ui.x), ic1 = cap_of(ui.y);
+    // tags of the lane's two columns: (3 - row) << (6 - 2 column), row 3 has none
+    const uint32_t t10 = part ? 1u << 2 : 1u << 6, t11 = t10 >> 2;
+    // best key of the tile whose columns 2 part, 2 part + 1 are x and y: both columns on every pair of rows; the other lane
+    // of the group has the other two columns
+    auto best_key = [&](const uint4& x, uint32_t cx, const uint4& y, uint32_t cy) {
+        const uint32_t x0 = min_v(x.x, cx) + 3u * t10, x1 = min_v(x.y, cx) + 2u * t10, x2 = min_v(x.z, cx) + t10, x3 = min_v(x.w, cx);
+        const uint32_t y0 = min_v(y.x, cy) + 3u * t11, y1 = min_v(y.y, cy) + 2u * t11, y2 = min_v(y.z, cy) + t11, y3 = min_v(y.w, cy);
+        const uint32_t p01 = add_max(x0, y1, x1 + y0), p02 = add_max(x0, y2, x2 + y0), p03 = add_max(x0, y3, x3 + y0);
+        const uint32_t p12 = add_max(x1, y2, x2 + y1), p13 = add_max(x1, y3, x3 + y1), p23 = add_max(x2, y3, x3 + y2);
+        const uint32_t o01 = __shfl_xor_sync(0xffffffffu, p01, 1), o02 = __shfl_xor_sync(0xffffffffu, p02, 1);
+        const uint32_t o03 = __shfl_xor_sync(0xffffffffu, p03, 1), o12 = __shfl_xor_sync(0xffffffffu, p12, 1);
+        const uint32_t o13 = __shfl_xor_sync(0xffffffffu, p13, 1), o23 = __shfl_xor_sync(0xffffffffu, p23, 1);
+        const uint32_t m0 = add_max(p01, o23, add_max(p02, o13, p03 + o12)), m1 = add_max(p12, o03, add_max(p13, o02, p23 + o01));
+        return max_v(m0, m1);
+    };
+    auto tag_of = [&](uint32_t bytes, uint32_t w) { return (int)((__shfl_sync(0xffffffffu, bytes, (int)(w >> 15), 8) >> (w >> 28)) & 3u); };
+    auto source_half = [&]() {                               // credits of group a towards its out-slots' destinations
+        return best_key(*(const uint4*)(m.CT + ((int)(uo.x & 0xffffu) - dt0 * m.N)), oc0, *(const uint4*)(m.CT + ((int)(uo.y & 0xffffu) - dt1 * m.N)), oc1) & 0xffu;
+    };
+    dt0 = (int)((dst >> (uo.x >> 28)) & 3u);                 // (every group starts from the same binding)
+    dt1 = (int)((dst >> (uo.y >> 28)) & 3u);
+    uint32_t src_new = source_half(), F_old = 0;             // (0: a first F of zero ends the run as -1 would: the sweep after it repeats it)
+    src = 0x100u;                                            // (no binding yet)
+    bool alive = mine;                                       // the same in a task's eight lanes, as F is
+#pragma unroll 1
+    for (int sweep = 1; ; sweep++) {
+        // If no source binding of a task moved, the destination half would see what it saw last sweep and return the same
+        // binding and the same F: the run ends here exactly as it would after computing that.
+        const unsigned who = __ballot_sync(0xffffffffu, alive && src_new != src);
+        if (alive) src = src_new;
+        if (alive && !(who & gmask)) { n_sweeps++; alive = false; }
+        if (who == 0) break;
+        // destination half: credits into group a from its in-slots' sources
+        const int s0 = tag_of(src, ui.x), s1 = tag_of(src, ui.y);
+        const uint32_t key = best_key(*(const uint4*)(m.C + ((int)(ui.x & 0xffffu) - s0 * m.N)), ic0, *(const uint4*)(m.C + ((int)(ui.y & 0xffffu) - s1 * m.N)), ic1);
+        const unsigned who2 = __ballot_sync(0xffffffffu, alive && ((key ^ dst) & 0xffu) != 0);
+        if (alive) dst = key & 0xffu;
+        uint32_t F = act ? key >> 8 : 0u;                    // Eq. (8); both lanes of a group hold its credit
+        F += __shfl_xor_sync(0xffffffffu, F, 2);
+        dt0 = tag_of(dst, uo.x);
+        dt1 = tag_of(dst, uo.y);
+        // the next sweep's source half needs no F: it runs while that is summed and is dropped if the run ends
+        const bool more = sweep < i_aa && who2 != 0;
+        if (more) src_new = source_half();
+        F += __shfl_xor_sync(0xffffffffu, F, 4);
+        // If no destination binding moved, the next sweep would be a repetition of this one and would end the run, so it is
+        // counted and skipped.
+        if (alive) {
+            n_sweeps++;
+            alive = (sweep == 1 || F > F_old) && sweep < i_aa;
+            F_old = F;
+            if (alive && !(who2 & gmask)) { n_sweeps++; alive = false; }
+        }
+        if (!more || !__any_sync(0xffffffffu, alive)) break;
+    }
+    return F_old;
+}
+
+// Steps 2 and 3 by the general route (out of line): any number of families and starts, four tasks at a time.  Returns F << 32 | task
+// of the best start of the best family (F = 0: none), whose binding is at bindings + task * N then (source | destination << 8 per slot).
+template <bool ONE>
+__device__ __noinline__ uint64_t warp_families(const WarpUnits m, const uint32_t* fam_task, const int64_t* tscale, uint16_t* bindings, int f0, int H, int G,
+                                               int n_start, int i_aa, int64_t lambda_w, int lane, unsigned& sweeps_out) {
+    const int tsub = lane >> 3, a = (lane & 7) >> 1, part = lane & 1, ag = a < G ? a : 0, n_tasks = H * n_start;
+    int64_t bf = -1, bd = 1, ff = -1, fd = 1;                // best family so far; best start of the current family
+    int bt = -1, ft = -1, cur_h = -1;
+    unsigned n_sweeps = 0;
+#pragma unroll 1
+    for (int task0 = 0; task0 < n_tasks; task0 += 4) {
+        const int task = min(task0 + tsub, n_tasks - 1), h = task / n_start, t = task - h * n_start;
+        const bool mine = task0 + tsub < n_tasks, act = mine && a < G;
+        const uint32_t* const fam = fam_task + ((f0 + h) * G + ag) * 8 + part * 2;
+        const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
+        uint32_t src;
+        int dt0, dt1;
+        const uint32_t F = warp_tasks<ONE>(m, uo, ui, big_family_and_start(t, n_start) & 0xffu, mine, act, part, 0xffu << (8 * tsub), i_aa, n_sweeps, src, dt0, dt1);
+        const uint32_t bind = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
+                              (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
+        if (act) *(uint32_t*)(bindings + task * m.N + a * 4 + part * 2) = bind;
+        // Evaluate (Eq. 9, 10), needed only when several families compete: slowest lane under the final bindings
+        int64_t den = 1;
+        if (H > 1) {
+            int64_t tmax = 0;
+            if (act) {
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    const uint32_t bw = bind >> (16 * i), cl = ((i ? uo.y : uo.x) >> 24) & 0xfu;
+                    const uint32_t x = min_v(m.D[(int)(bw & 0xffu) * m.N + (int)((bw >> 8) & 0xffu)], m.cap[cl]);
+                    tmax = max_v(tmax, (int64_t)x * tscale[cl]);
+                }
+            }
+            tmax = team_max(tmax);
+            tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
+            den = F > 0 ? lambda_w + tmax : 1;
+        }
+        // the round's results in task order (every lane follows along)
+#pragma unroll 1
+        for (int s = 0; s < 4; s++) {
+            const int64_t Fs = __shfl_sync(0xffffffffu, F, 8 * s), ds = __shfl_sync(0xffffffffu, den, 8 * s);
+            const int tk = task0 + s, ht = tk / n_start;
+            if (tk < n_tasks) {
+                if (ht != cur_h) {                           // a new family starts: settle the previous one
+                    if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }
+                    cur_h = ht; ff = -1; fd = 1; ft = -1;
+                }
+                if (Fs > ff) { ff = Fs; fd = ds; ft = tk; }  // largest F, lowest start
+            }
+        }
+    }
+    if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }   // lowest family on ties
+    sweeps_out = n_sweeps;
+    __syncwarp();
+    return (uint64_t)bf << 32 | (uint32_t)bt;
+}
+
+template <bool NARROW> struct WarpLeft { typedef uint32_t type; };
+template <> struct WarpLeft<false> { typedef int64_t type; };
+
+// Main loop for a matrix held in 32-bit granules (`total` of them) with capacities below 2^22 granules.  Two copies: while scores need
+// 64 bits, and from then on; what an ordinary activation does not execute is out of line (instructions come from small caches, see
+// schedule_big.cuh).  ONE: all paths have one rate.
+template <bool ONE>
+__device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams& kp, const WCtx& c, int64_t total, int& k_out, int& st, Counters& cnt) {
     const int N = c.N, G = c.G, lane = c.lane;
     uint32_t* const D = ws<uint32_t>(c.o_drem);
-    uint32_t* const DT = ws<uint32_t>(c.o_dremT);              // DT[j * N + i] = D[i * N + j]
+    uint32_t* const C = ws<uint32_t>(c.o_cred);
+    uint32_t* const CT = ws<uint32_t>(c.o_dremT);              // CT[j * N + i] = C[i * N + j]
     int64_t* const Dhat = ws<int64_t>(c.o_dhat);
     const uint32_t* const dhat32 = ws<uint32_t>(c.o_dhat);     // (low words)
     const uint32_t* const s_cap = ws<uint32_t>(c.o_cap32);
     uint16_t* const bindings = ws<uint16_t>(c.o_bind);
-    const bool one_class = dc.n_classes == 1;
+    const uint32_t* const fam_task = ws<uint32_t>(c.o_fam_task);
     const uint32_t cap0 = s_cap[0];
-    const int ns_shift = (kp.n_start & (kp.n_start - 1)) == 0 ? 31 - __clz(kp.n_start) : -1;
+    const WarpUnits units{D, C, CT, s_cap, N};
+    uint32_t cap_most = cap0;
+    if (!ONE)
+        for (int cl = 1; cl < dc.n_classes; cl++) cap_most = max_v(cap_most, s_cap[cl]);
+    for (int e = lane; e < N * N; e += 32) {                   // (D and its transpose are given)
+        C[e] = min_v(D[e], cap_most) << 8;
+        CT[e] = min_v(CT[e], cap_most) << 8;
+    }
+    __syncwarp();
     // this lane's place in Step 2: task of four, rank group, columns 2 part and 2 part + 1 of the group's tile
     const int tsub = lane >> 3, a = (lane & 7) >> 1, part = lane & 1, ag = a < G ? a : 0;
     const unsigned gmask = 0xffu << (8 * tsub);
+    const uint32_t dst_1 = big_family_and_start(tsub, 4) & 0xffu;
+    const uint32_t my_fam = (uint32_t)(ag * 8 + part * 2);
+    const bool act = a < G;
+    const int my_slot = lane < N ? lane : 0;
     unsigned n_sweeps = 0, n_done = 0;
-    uint32_t tags[3][2];
-#pragma unroll
-    for (int r = 0; r < 3; r++)
-#pragma unroll
-        for (int i = 0; i < 2; i++) tags[r][i] = (uint32_t)(3 - r) << (6 - 2 * (part * 2 + i));
     RowScores by_rows;
     by_rows.load(dc, c);
+    int k = 0;
     // the activation taken off the residual whose rows are still to be written (slot `lane`)
     bool pend = false;
     int p_fam = 0;
@@ -204,183 +362,94 @@ __device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams&
             c.lane_inst_b[row + i] = p_x ? (uint16_t)inst : (uint16_t)0xFFFF;
             if (lane == 0) c.chan_id_b[kk] = p_fam;
         }
-        pend = false;
     };
 
-    for (;;) {
-        if (left == 0) break;
-        if (k == kp.k_max) { st |= VP_ST_STEP_LIMIT; break; }
-        // path instance of the slot to be written out: a trip to L2 that ends long before write_row needs it
-        const uint32_t inst = pend && lane < N ? __ldg(dc.fam_slot + (size_t)p_fam * N + lane) : 0u;
-        // (A) Eq. (6): shape scores, first maximum
-        const bool narrow = left < ((int64_t)1 << 30);           // every score (at most g x what is left) fits 32 bits
-        int best_s = 0x7fffffff;
-        bool covered;
-        if (by_rows.on && narrow) {
-            const uint32_t best = by_rows.narrow(dhat32, lane, best_s), m = __reduce_max_sync(0xffffffffu, best);
-            covered = m != 0;
-            best_s = (int)__reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 0x7fffffffu);
-        } else {
-            int64_t best = -1;
-            if (by_rows.on) by_rows.wide(Dhat, lane, best, best_s);
-            else score_terms(dc, dc.term_t, Dhat, lane, best, best_s);
-            warp_argmax_first(best, best_s);
-            covered = best > 0;
-        }
-        VP_TICK(0);
-        if (!covered) { st |= VP_ST_UNCOVERED; break; }
-        const int f0 = (int)ws<uint32_t>(c.o_bucket)[best_s], H = (int)ws<uint32_t>(c.o_bucket)[best_s + 1] - f0;
-        const int n_tasks = H * kp.n_start;
-        VP_TICK(1);
+    auto slot_inst = [&]() { return __ldg(dc.fam_slot + (unsigned)(p_fam * N + my_slot)); };
 
-        // (B) MultiStartAA, four (family, start) tasks at a time; (C) best start per family, best family
-        int64_t bf = -1, bd = 1, ff = -1, fd = 1;                // best family so far; best start of the current family
-        int bt = -1, ft = -1, cur_h = -1;
-        uint32_t my_bind = 0;                                    // this lane's two slots: (source | destination << 8) x 2
-        for (int task0 = 0; task0 < n_tasks; task0 += 4) {
-            const int task = min(task0 + tsub, n_tasks - 1);
-            const int h = ns_shift >= 0 ? task >> ns_shift : task / kp.n_start, f = f0 + h, t = task - h * kp.n_start;
-            const bool act = task0 + tsub < n_tasks && a < G;
-            // slot words (see DevCat::fam_task): place of the cells for tag 0, owning group, class, shift of the tag
-            const uint32_t* const fam = ws<uint32_t>(c.o_fam_task) + (f * G + ag) * 8 + part * 2;
-            const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
-            if (pend) write_row(k - 1, inst);
-            // A binding travels as the low byte of a group's best key: the tag 3 - row of position 0 in its two highest bits, of
-            // position 3 in the lowest.  Start t binds in-slot q to row (q + t) mod 4.
-            uint32_t dst = 0, src = 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) dst |= (uint32_t)(3 - ((q + t) & 3)) << (6 - 2 * q);
-            const uint32_t oc0 = one_class ? cap0 : s_cap[(uo.x >> 24) & 0xfu], oc1 = one_class ? cap0 : s_cap[(uo.y >> 24) & 0xfu];
-            const uint32_t ic0 = one_class ? cap0 : s_cap[(ui.x >> 24) & 0xfu], ic1 = one_class ? cap0 : s_cap[(ui.y >> 24) & 0xfu];
-            int dt0, dt1;                                        // tags (3 - row) of the out-slots' destinations
-            // best key of the tile whose columns 2 part, 2 part + 1 are x and y: both columns on every pair of rows; the other lane
-            // of the group has the other two columns
-            auto best_key = [&](const uint4& x, uint32_t cx, const uint4& y, uint32_t cy) {
-                const uint32_t x0 = min_v(x.x, cx) * 256u + tags[0][0], x1 = min_v(x.y, cx) * 256u + tags[1][0];
-                const uint32_t x2 = min_v(x.z, cx) * 256u + tags[2][0], x3 = min_v(x.w, cx) * 256u;
-                const uint32_t y0 = min_v(y.x, cy) * 256u + tags[0][1], y1 = min_v(y.y, cy) * 256u + tags[1][1];
-                const uint32_t y2 = min_v(y.z, cy) * 256u + tags[2][1], y3 = min_v(y.w, cy) * 256u;
-                const uint32_t p01 = add_max(x0, y1, x1 + y0), p02 = add_max(x0, y2, x2 + y0), p03 = add_max(x0, y3, x3 + y0);
-                const uint32_t p12 = add_max(x1, y2, x2 + y1), p13 = add_max(x1, y3, x3 + y1), p23 = add_max(x2, y3, x3 + y2);
-                const uint32_t o01 = __shfl_xor_sync(0xffffffffu, p01, 1), o02 = __shfl_xor_sync(0xffffffffu, p02, 1);
-                const uint32_t o03 = __shfl_xor_sync(0xffffffffu, p03, 1), o12 = __shfl_xor_sync(0xffffffffu, p12, 1);
-                const uint32_t o13 = __shfl_xor_sync(0xffffffffu, p13, 1), o23 = __shfl_xor_sync(0xffffffffu, p23, 1);
-                const uint32_t m0 = add_max(p01, o23, add_max(p02, o13, p03 + o12)), m1 = add_max(p12, o03, add_max(p13, o02, p23 + o01));
-                return max_v(m0, m1);
-            };
-            auto tag_of = [&](uint32_t bytes, uint32_t w) { return (int)((__shfl_sync(0xffffffffu, bytes, (int)(w >> 15), 8) >> (w >> 28)) & 3u); };
-            auto source_half = [&]() {                           // credits of group a towards its out-slots' destinations
-                dt0 = tag_of(dst, uo.x);
-                dt1 = tag_of(dst, uo.y);
-                return best_key(*(const uint4*)(DT + ((int)(uo.x & 0xffffu) - dt0 * N)), oc0, *(const uint4*)(DT + ((int)(uo.y & 0xffffu) - dt1 * N)), oc1) & 0xffu;
-            };
-            uint32_t src_new = source_half();
-            int F_old = -1, F_new = -1;                          // this lane's task; the same in its eight lanes, as alive is
-            bool alive = task0 + tsub < n_tasks;
-            for (int sweep = 0; ; sweep++) {
-                // If no source binding of a task moved, the destination half would see what it saw last sweep and return the same
-                // binding and the same F: the run ends here exactly as it would after computing that.
-                const bool smoved = alive && act && (sweep == 0 || src_new != src);
-                if (alive) src = src_new;
-                if (sweep) {
-                    const unsigned who = __ballot_sync(0xffffffffu, smoved);
-                    if (alive && !(who & gmask)) { F_new = F_old; n_sweeps++; alive = false; }
-                    if (!__any_sync(0xffffffffu, alive)) break;
-                }
-                // destination half: credits into group a from its in-slots' sources
-                const int s0 = tag_of(src, ui.x), s1 = tag_of(src, ui.y);
-                const uint32_t key = best_key(*(const uint4*)(D + ((int)(ui.x & 0xffffu) - s0 * N)), ic0, *(const uint4*)(D + ((int)(ui.y & 0xffffu) - s1 * N)), ic1);
-                const bool dmoved = alive && act && ((key ^ dst) & 0xffu) != 0;
-                if (alive) dst = key & 0xffu;
-                // the next sweep's source half needs no F: it runs while that is summed and is dropped if the run ends (the destinations'
-                // tags it looks up are those of the final binding)
-                uint32_t F = act ? key >> 8 : 0u;                // Eq. (8); both lanes of a group hold its credit
-                F += __shfl_xor_sync(0xffffffffu, F, 2);
-                src_new = source_half();
-                F += __shfl_xor_sync(0xffffffffu, F, 4);
-                const unsigned who2 = __ballot_sync(0xffffffffu, dmoved);
-                // If no destination binding moved, the next sweep would be a repetition of this one and would end the run, so it is
-                // counted and skipped.
-                if (alive) {
-                    F_new = (int)F;
-                    n_sweeps++;
-                    alive = F_new > F_old && sweep + 1 < kp.i_aa;
-                    F_old = F_new;
-                    if (alive && !(who2 & gmask)) { n_sweeps++; alive = false; }
-                }
-                if (!__any_sync(0xffffffffu, alive)) break;
+    auto run = [&](auto scores) {
+        constexpr bool NARROW = decltype(scores)::value;         // every score (at most g x what is left) fits 32 bits
+        typedef typename WarpLeft<NARROW>::type left_t;
+        left_t left = (left_t)total;
+        for (;;) {
+            if (rarely(left == 0 || k == kp.k_max || (!NARROW && left < ((left_t)1 << 30)))) break;
+            // path instance of the slot to be written out: a trip to L2 that ends long before write_row needs it
+            const uint32_t inst = slot_inst();
+            // (A) Eq. (6): shape scores, first maximum
+            int best_s = 0x7fffffff;
+            if (NARROW && usually(by_rows.on)) {
+                const uint32_t best = by_rows.narrow(dhat32, lane, best_s), m = __reduce_max_sync(0xffffffffu, best);
+                best_s = (int)__reduce_min_sync(0xffffffffu, best == m ? (uint32_t)best_s : 0x7fffffffu);
+                if (m == 0) best_s = -1;
+            } else {
+                best_s = warp_first_shape(dc.n_shapes, dc.max_terms, dc.term_t, Dhat, lane);
             }
-            VP_TICK(2);
-            my_bind = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
-                      (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
-            n_done += (unsigned)min(4, n_tasks - task0);
-            if (H == 1 && n_tasks <= 4) {                        // one family, one round: largest F, lowest start; bindings stay in registers
-                const uint32_t best = __reduce_max_sync(0xffffffffu, F_new > 0 ? (uint32_t)F_new << 2 | (uint32_t)(3 - tsub) : 0u);
-                bf = (int64_t)(best >> 2); bt = 3 - (int)(best & 3u);      // (F is at most sixteen lanes of 2^22 granules)
-                break;
-            }
-            if (act) *(uint32_t*)(bindings + task * N + a * 4 + part * 2) = my_bind;
-            // Evaluate (Eq. 9, 10), needed only when several families compete: slowest lane under the final bindings
-            int64_t den = 1;
-            if (H > 1) {
-                int64_t tmax = 0;
-                if (act) {
-#pragma unroll
-                    for (int i = 0; i < 2; i++) {
-                        const uint32_t bw = my_bind >> (16 * i), cl = ((i ? uo.y : uo.x) >> 24) & 0xfu;
-                        const uint32_t x = min_v(D[(int)(bw & 0xffu) * N + (int)((bw >> 8) & 0xffu)], s_cap[cl]);
-                        tmax = max_v(tmax, (int64_t)x * ws<int64_t>(c.o_tscale)[cl]);
-                    }
-                }
-                tmax = team_max(tmax);
-                tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
-                den = F_new > 0 ? kp.lambda_ns * dc.W + tmax : 1;
-            }
-            // the round's results in task order (every lane follows along)
-#pragma unroll
-            for (int s = 0; s < 4; s++) {
-                const int64_t Fs = __shfl_sync(0xffffffffu, F_new, 8 * s), ds = __shfl_sync(0xffffffffu, den, 8 * s);
-                const int tk = task0 + s, ht = ns_shift >= 0 ? tk >> ns_shift : tk / kp.n_start;
-                if (tk < n_tasks) {
-                    if (ht != cur_h) {                           // a new family starts: settle the previous one
-                        if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }
-                        cur_h = ht; ff = -1; fd = 1; ft = -1;
-                    }
-                    if (Fs > ff) { ff = Fs; fd = ds; ft = tk; }  // largest F, lowest start
-                }
-            }
-        }
-        if (cur_h >= 0 && (bt < 0 || util_greater(ff, fd, bf, bd))) { bf = ff; bd = fd; bt = ft; }   // lowest family on ties
-        if (bf <= 0) { st |= VP_ST_NO_PROGRESS; break; }
-        VP_TICK(3);
+            VP_TICK(0);
+            if (rarely(best_s < 0)) { st |= VP_ST_UNCOVERED; break; }
+            const int f0 = (int)ws<uint32_t>(c.o_bucket)[best_s], H = (int)ws<uint32_t>(c.o_bucket)[best_s + 1] - f0;
+            VP_TICK(1);
 
-        // (D) activation k off the residual and off D-hat (Eq. 5)
-        __syncwarp();
-        {
-            const int h = ns_shift >= 0 ? bt >> ns_shift : bt / kp.n_start;
-            p_fam = f0 + h;
-            if (cur_h < 0) p_bind = (__shfl_sync(0xffffffffu, my_bind, (bt << 3 | lane >> 1) & 31) >> (16 * (lane & 1))) & 0xffffu;
-            else p_bind = lane < N ? bindings[bt * N + lane] : 0u;
+            // (B) MultiStartAA, (C) best start per family, best family
+            uint32_t wF, bind;                                   // F of the best start, source | destination << 8 of slot `lane`
+            int wfam = f0;
+            if (usually(H == 1 && kp.n_start == 4)) {            // one family, one round: largest F, lowest start; bindings stay in registers
+                const uint32_t* const fam = fam_task + (uint32_t)(f0 * G) * 8u + my_fam;
+                const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
+                if (usually(pend)) write_row(k - 1, inst);
+                uint32_t src;
+                int dt0, dt1;
+                const uint32_t F = warp_tasks<ONE>(units, uo, ui, dst_1, true, act, part, gmask, kp.i_aa, n_sweeps, src, dt0, dt1);
+                VP_TICK(2);
+                const uint32_t mine = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
+                                      (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
+                n_done += 4;
+                const uint32_t best = __reduce_max_sync(0xffffffffu, F << 2 | (uint32_t)(3 - tsub));     // (F is at most sixteen lanes of 2^22 granules)
+                wF = best >> 2;
+                bind = (__shfl_sync(0xffffffffu, mine, (int)(3u - (best & 3u)) << 3 | ((lane >> 1) & 7)) >> (16 * (lane & 1))) & 0xffffu;
+            } else {
+                if (pend) write_row(k - 1, inst);
+                unsigned more_sweeps;
+                const uint64_t chosen = warp_families<ONE>(units, fam_task, ws<int64_t>(c.o_tscale), bindings, f0, H, G, kp.n_start, kp.i_aa, kp.lambda_ns * dc.W, lane, more_sweeps);
+                n_sweeps += more_sweeps;
+                n_done += (unsigned)(H * kp.n_start);
+                wF = (uint32_t)(chosen >> 32);
+                wfam += (int)(big_family_and_start((int)(uint32_t)chosen, kp.n_start) >> 8);
+                bind = lane < N ? bindings[(int)(uint32_t)chosen * N + lane] : 0u;
+            }
+            pend = false;
+            if (rarely(wF == 0)) { st |= VP_ST_NO_PROGRESS; break; }
+            VP_TICK(3);
+
+            // (D) activation k off the residual and off D-hat (Eq. 5)
+            __syncwarp();
             if (lane < N) {
-                const int i = (int)(p_bind & 0xffu), j = (int)(p_bind >> 8);
+                const int i = (int)(bind & 0xffu), j = (int)(bind >> 8);
                 uint32_t cap = cap0;
-                if (!one_class) cap = s_cap[__ldg(dc.fam_cls + (size_t)p_fam * N + lane)];
+                if (!ONE) cap = s_cap[__ldg(dc.fam_cls + (size_t)wfam * N + lane)];
                 const uint32_t cell = D[i * N + j], x = min_v(cap, cell);
+                const uint32_t credit = min_v(cell - x, cap_most) << 8;
                 D[i * N + j] = cell - x;
-                DT[j * N + i] = cell - x;
+                C[i * N + j] = credit;
+                CT[j * N + i] = credit;
                 int64_t* const sum = &Dhat[(lane >> 2) * G + (j >> 2)];
-                if (narrow) atomicSub((unsigned int*)sum, x);    // (high word is zero, low word >= x)
+                if (NARROW) atomicSub((unsigned int*)sum, x);    // (high word is zero, low word >= x)
                 else atomicAdd((unsigned long long*)sum, (unsigned long long)(-(int64_t)x));
                 p_x = x;
             }
+            p_bind = bind;
+            p_fam = wfam;
             pend = true;
-            left -= bf;
+            left -= wF;
+            k++;
+            __syncwarp();
+            VP_TICK(4);
         }
-        k++;
-        __syncwarp();
-        VP_TICK(4);
-    }
-    if (pend) write_row(k - 1, lane < N ? __ldg(dc.fam_slot + (size_t)p_fam * N + lane) : 0u);
+        total = (int64_t)left;
+    };
+    if (total >= ((int64_t)1 << 30)) run(BigConst<false>());
+    if (st == 0 && k < kp.k_max && total < ((int64_t)1 << 30)) run(BigConst<true>());
+    if (st == 0 && total != 0) st |= VP_ST_STEP_LIMIT;
+    if (pend) write_row(k - 1, slot_inst());
+    k_out = k;
     if (lane == 0) cnt.tasks += n_done;
     if ((lane & 7) == 0) cnt.sweeps += n_sweeps;
 }
@@ -406,7 +475,7 @@ __device__ __forceinline__ void decompose_bytes(const DevCat& dc, const KParams&
         int64_t best = -1;
         int best_s = 0x7fffffff;
         if (by_rows.on) by_rows.wide(Dhat, lane, best, best_s);
-        else score_terms(dc, c.term, Dhat, lane, best, best_s);
+        else score_terms(dc.n_shapes, dc.max_terms, c.term, Dhat, lane, best, best_s);
         VP_TICK(0);
         warp_argmax_first(best, best_s);
         if (best <= 0) { st |= VP_ST_UNCOVERED; break; }
@@ -562,7 +631,7 @@ __device__ __forceinline__ void decompose_bytes(const DevCat& dc, const KParams&
 // matrix of larger capacities reads those of decompose_bytes from global memory.  Otherwise decompose_bytes and its tables.
 // `slots`: per warp three counters for vp_schedule_read_stats, given when there is a warp for every matrix: the launch then needs
 // no counter and nothing zeroed.
-template <bool UNITS>
+template <bool UNITS, bool ONE>
 __global__ void __launch_bounds__(128, 3)
 vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, const int64_t* __restrict__ tau_in, int B,
                         int32_t* __restrict__ n_steps, int32_t* __restrict__ chan_id, int16_t* __restrict__ lane_dst,
@@ -619,7 +688,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
     WCtx c;
     c.N = N; c.G = G; c.lane = lane;
     const unsigned base = (unsigned)warp * (unsigned)L.per_warp;
-    c.o_drem = base + L.drem; c.o_dremT = base + L.dremT; c.o_dhat = base + L.dhat; c.o_send_acc = base + L.send_acc; c.o_recv_acc = base + L.recv_acc;
+    c.o_drem = base + L.drem; c.o_dremT = base + L.dremT; c.o_cred = base + L.cred; c.o_dhat = base + L.dhat; c.o_send_acc = base + L.send_acc; c.o_recv_acc = base + L.recv_acc;
     c.o_rs = base + L.rs; c.o_cap64 = base + L.cap64; c.o_cap32 = base + L.cap32; c.o_tscale = base + L.tscale;
     c.o_bind = base + L.bind; c.o_bind_dst = base + L.bind_dst;
     c.o_rows = L.rows; c.o_shape_rows = L.shape_rows; c.o_fam_task = L.fam_task; c.o_bucket = L.bucket;
@@ -780,7 +849,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
             __syncwarp();
             if (units) {
                 int64_t rem;
-                decompose_units(dc, kp, c, granule.div(tot, rem), k, st, cnt);
+                decompose_units<ONE>(dc, kp, c, granule.div(tot, rem), k, st, cnt);
             } else {
                 if (UNITS) {                                 // (back to bytes)
                     for (int e = lane; e < N * N; e += 32) {
