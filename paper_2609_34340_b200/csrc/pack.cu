@@ -66,89 +66,113 @@ __device__ __forceinline__ int dest_of(int x, const PackArgs& a, int& bad) {
 
 __device__ __forceinline__ int steps_in_use(const PackArgs& a) { return min(max(*a.n_steps, 0), a.k_max); }
 
-__device__ __forceinline__ Step pack_step(const PackArgs& a, int k, int& bad) {
+// A step's figures as the plan has them; pack_step makes rows of them.
+struct RawStep { int j; int64_t bytes, off; };
+__device__ __forceinline__ RawStep raw_step(const PackArgs& a, int k) {
     const size_t at = (size_t)k * a.N + a.rank;
+    return RawStep{a.lane_dst[at], a.lane_bytes[at], a.send_off[at]};
+}
+__device__ __forceinline__ Step pack_step(const PackArgs& a, const RawStep& raw, int& bad) {
     int64_t odd, ignore;
-    const int j = a.lane_dst[at];
-    const int64_t rows = a.row.div(a.lane_bytes[at], odd), row0 = a.row.div(a.send_off[at], ignore);
+    const int j = raw.j;
+    const int64_t rows = a.row.div(raw.bytes, odd), row0 = a.row.div(raw.off, ignore);
     if (j < 0 || j >= a.N) return Step{-1, 0, 0};
     if (odd) bad = VP_ST_PACK_MISMATCH;
     return Step{j, (int)rows, (int)row0};
 }
 
-// Status bits of the run table, the same in every thread.
-__device__ __forceinline__ int pack_runs(const PackArgs& a, int K, Step first, int bad, Runs out, int* cnt, int* scratch) {
+// Status bits of the run table, the same in every thread (left out unless `report`).
+__device__ __forceinline__ int pack_runs(const PackArgs& a, int K, Step first, int bad, Runs out, int* cnt, int* scratch, bool cleared = false, bool report = true) {
     if ((int)threadIdx.x >= K) bad = 0;
-    build_runs(K, a.N, first, [&](int k) { return pack_step(a, k, bad); }, out, cnt, scratch);
+    build_runs(K, a.N, first, [&](int k) { return pack_step(a, raw_step(a, k), bad); }, out, cnt, scratch, cleared);
+    if (!report) return 0;
     if (threadIdx.x == 0 && out.total[a.rank] != 0) bad = VP_ST_PACK_MISMATCH;
     return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
 }
 
 // ---- one launch -------------------------------------------------------------------------------------------------
 
-struct PackSmall { int cnt, hist, total, ptr, start, row, src, dst, scratch, ints; };   // offsets in ints
-__host__ __device__ inline PackSmall pack_small_layout(int N, int k_max) {
+struct PackSmall { int key, cnt, hist, total, ptr, start, row, src, dst, scratch, ints; };   // offsets in ints
+__host__ __device__ inline PackSmall pack_small_layout(int N, int k_max, int own) {
     PackSmall L;
     int o = 0;
+    L.key = o;     o += (own + 3) & ~3;              // (read four at a time)
     L.cnt = o;     o += N;
     L.hist = o;    o += N;
     L.total = o;   o += N;
     L.ptr = o;     o += N + 1;
     L.start = o;   o += k_max;
     L.row = o;     o += k_max;
-    L.src = o;     o += kSmallOwn;
-    L.dst = o;     o += kSmallOwn;
+    L.src = o;     o += own;
+    L.dst = o;     o += own;
     L.scratch = o; o += runs_scratch_ints(N);
     L.ints = o;
     return L;
 }
 
-// Decode steps and prefill chunks of a few thousand tokens.  Bound by latency (launch, two trips to L2 for plan and routing,
-// one for the rows), then by HBM writes.  CTA c owns the tokens [c T / grid, (c + 1) T / grid) -- or one of `pieces` column
+// Decode steps and prefill chunks of a few thousand tokens.  Bound by latency (launch, one trip to L2 for plan and routing, the
+// run table: 3 us), then by HBM writes.  CTA c owns the tokens [c T / grid, (c + 1) T / grid) -- or one of `pieces` column
 // ranges of one token while there are fewer tokens than SMs -- and finds their places by itself: the run table from the
 // plan, and how many copies to each destination come before its own.  The last CTA thereby sees every copy and writes the
-// status.  Replaces two memsets and four kernels: 128 tokens x top-8 of 14,336 B 30 -> 8 us a call.
-template <typename V>
-__global__ void __launch_bounds__(kIdxThreads, 2)
-pack_small_kernel(PackArgs a, const char* __restrict__ rows, char* __restrict__ staged, int pieces) {
-    extern __shared__ int sm[];
-    const PackSmall L = pack_small_layout(a.N, a.k_max);
+// status.  Replaces two memsets and four kernels: 128 tokens x top-8 of 14,336 B 30 -> 6.8 us a call.
+template <typename V, bool BULK>
+__global__ void __launch_bounds__(kIdxThreads, BULK ? 1 : 2)
+pack_small_kernel(PackArgs a, const char* __restrict__ rows, char* __restrict__ staged, SmallLaunch z) {
+    extern __shared__ __align__(128) int sm[];
+    __shared__ __align__(8) unsigned long long bars[kOwnWarps * kOwnStages];
+    const PackSmall L = pack_small_layout(a.N, a.k_max, z.own);
+    const int pieces = z.pieces;
     int* const hist = sm + L.hist;
     const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
     const int t0 = (int)((long long)a.T * c / n_cta), t1 = (int)((long long)a.T * (c + 1) / n_cta);
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V)), v_lo = (int)((long long)vecs * piece / pieces),
+              v_hi = (int)((long long)vecs * (piece + 1) / pieces);
     for (int j = tid; j < a.N; j += kIdxThreads) hist[j] = 0;
-    grid_wait();
-    int bad = 0, bad_step = 0;
-    const Step first = tid < a.k_max ? pack_step(a, tid, bad_step) : Step{-1, 0, 0};
-    const int K = steps_in_use(a);
-    const bool over = a.send_off[(size_t)K * a.N + a.rank] > a.capacity;
+    OwnRing ring;
+    if (BULK && tid < kOwnWarps * 32) ring.init(z, rows, staged, a.row.d, v_lo, v_hi, sm, bars);
+    int *const src = sm + L.src, *const dst = sm + L.dst, *const own_key = sm + L.key;
+    clear_runs_scratch(a.N, sm + L.scratch);
     __syncthreads();
+    grid_wait();
+    // All that the index needs is asked for at once; rows are loaded behind it (ahead of it they keep it waiting).
+    const RawStep raw = tid < a.k_max ? raw_step(a, tid) : RawStep{-1, 0, 0};
+    const int K = steps_in_use(a), own = (t1 - t0) * a.topk;
+    int bad = 0, bad_step = 0;
+    for (int i = tid; i < own; i += kIdxThreads) own_key[i] = dest_of(a.idx[t0 * a.topk + i], a, bad);
     for_each_item(a.idx, 0, t0 * a.topk, [&](int, int x) {
         const int j = dest_of(x, a, bad);
         if (j >= 0) atomicAdd(&hist[j], 1);
     });
+    const int64_t end = a.send_off[(size_t)K * a.N + a.rank];
+    if (BULK && tid < kOwnWarps * 32) ring.start(t1 - t0, [&](int i) { return t0 + i; });
+    const Step first = pack_step(a, raw, bad_step);
     const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
-    const int st = pack_runs(a, K, first, bad_step, runs, sm + L.cnt, sm + L.scratch);   // (ends with a barrier: the histogram is complete, too)
-    int *const src = sm + L.src, *const dst = sm + L.dst;
-    if (tid < 32)
-        warp_positions(t0 * a.topk, t1 * a.topk, hist, [&](long long e) { return dest_of(a.idx[e], a, bad); },
-                       [&](long long e, int j, int p) {
-                           const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
-                           dst[e - t0 * a.topk] = row;
-                           if (row >= 0 && a.src_map && piece == 0) a.src_map[row] = (int)e;
-                       });
-    else
-        for (int i = tid - 32; i < t1 - t0; i += kIdxThreads - 32) src[i] = t0 + i;
+    const bool last = c == n_cta - 1 && piece == 0;
+    const int st = pack_runs(a, K, first, bad_step, runs, sm + L.cnt, sm + L.scratch, true, last);   // (has barriers: the histogram and the own copies are complete, too)
+    const bool over = end > a.capacity;
+    own_positions(own_key, own, hist, [&](int i, int j, int p) {
+        const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
+        dst[i] = row;
+        if (row >= 0 && a.src_map && piece == 0) a.src_map[row] = t0 * a.topk + i;
+    });
+    if (!BULK)
+        for (int i = tid; i < t1 - t0; i += kIdxThreads) src[i] = t0 + i;
     __syncthreads();
-    if (c == n_cta - 1 && piece == 0) {              // every copy has been counted here
+    if (last) {                                      // every copy has been counted here, but for its own
+        for (int i = tid; i < own; i += kIdxThreads)
+            if (own_key[i] >= 0) atomicAdd(&hist[own_key[i]], 1);
+        __syncthreads();
         if (tid < a.N && tid != a.rank && hist[tid] != runs.total[tid]) bad = VP_ST_PACK_MISMATCH;
         const int any = __syncthreads_or(bad);
         if (tid == 0) *a.status = st | (any ? VP_ST_PACK_MISMATCH : 0) | (over ? VP_ST_PACK_CAPACITY : 0);
     }
+    if (BULK) {
+        if (tid < kOwnWarps * 32 && !(over ? ring.drain() : ring.finish(a.topk, dst, [&](int i) { return t0 + i; })) && (tid & 31) == 0)
+            atomicOr(a.status, VP_ST_INTERNAL_TIMEOUT);
+        return;
+    }
     if (over) return;
-    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
-    move_rows<V>(rows, staged, a.row.d, t1 - t0, a.topk, src, dst, (int)((long long)vecs * piece / pieces),
-                 (int)((long long)vecs * (piece + 1) / pieces));
+    move_rows<V>(rows, staged, a.row.d, t1 - t0, a.topk, src, dst, v_lo, v_hi);
 }
 
 // ---- chunked form -----------------------------------------------------------------------------------------------
@@ -160,7 +184,7 @@ __global__ void __launch_bounds__(kIdxThreads) pack_count_kernel(PackArgs a, Pac
     grid_wait();
     if ((int)blockIdx.x == n_chunks) {
         int bad = 0;
-        const Step first = tid < a.k_max ? pack_step(a, tid, bad) : Step{-1, 0, 0};
+        const Step first = pack_step(a, tid < a.k_max ? raw_step(a, tid) : RawStep{-1, 0, 0}, bad);
         const int K = steps_in_use(a);
         const int st = pack_runs(a, K, first, bad, Runs{w.start, w.row, w.ptr, w.total}, sm, sm + N);
         if (tid == 0) {
@@ -268,16 +292,14 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
     const int sms = sm_count_of_device();
     if (!sms) return VP_E_CUDA;
     if (E <= kSmallItems && k_max <= kSmallSteps && row_bytes <= kSmallRow) {
-        const SmallSplit s = small_split(T, sms);
-        const int n_cta = s.grid / s.pieces;
-        if ((long long)((T + n_cta - 1) / n_cta) * topk <= kSmallOwn) {
-            const size_t smem = (size_t)pack_small_layout(N, k_max).ints * 4;
+        const int width = copy_width(rows, staged, row_bytes);
+        const SmallLaunch z = small_launch(T, sms, topk, row_bytes, width, [&](int own) { return pack_small_layout(N, k_max, own * topk).ints; });
+        if (z.own <= kSmallOwn) {
             const char* from = (const char*)rows;
-            const int width = copy_width(rows, staged, row_bytes);
             vp_prof_mark(2, 0, stream);
-            const cudaError_t e = width == 16 ? launch_wide(pack_small_kernel<uint4>, s.grid, smem, stream, a, from, (char*)staged, s.pieces)
-                                : width == 4 ? launch_wide(pack_small_kernel<uint32_t>, s.grid, smem, stream, a, from, (char*)staged, s.pieces)
-                                             : launch_wide(pack_small_kernel<uint8_t>, s.grid, smem, stream, a, from, (char*)staged, s.pieces);
+            const auto go = [&](auto fn) { return launch_wide(fn, z.grid, z.smem, stream, a, from, (char*)staged, z); };
+            const cudaError_t e = z.bulk ? go(pack_small_kernel<uint4, true>) : width == 16 ? go(pack_small_kernel<uint4, false>)
+                                : width == 4 ? go(pack_small_kernel<uint32_t, false>) : go(pack_small_kernel<uint8_t, false>);
             vp_prof_mark(2, 1, stream);
             return e == cudaSuccess ? VP_OK : VP_E_CUDA;
         }

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32) row_copy_bulk_kernel(RowCopy c) {
             if (++sp == pieces) { sp = 0; sr++; }
         }
     }
-    bulk_wait_all();                                 // stores must finish before shared memory is released
+    bulk_wait_read<0>();                             // stores must have read shared memory before it is released
     if (failed) {
         // Give-up path: no further loads were issued.  Loads already in flight must not land in shared memory that
         // the next CTA owns, so each is given one more bounded wait (the stage whose wait gave up had its parity

@@ -11,7 +11,7 @@
 //   copy  : the row copy shared with the pack (each received row read once, written once)
 // vp_unpack_tokens, the return direction, sorts the routed copies by expert id the same way; a copy's position among the
 // copies to its expert's rank is its position in that sender's stream, whose runs give the receive row.
-// Up to kSmallItems rows (copies) each call is one kernel (see route_index.cuh).
+// Up to kSmallItems rows (kSmallReturn copies) each call is one kernel (see route_index.cuh).
 #include <cuda_runtime.h>
 
 #include "row_copy.cuh"
@@ -90,15 +90,25 @@ __device__ __forceinline__ int check_step(int row, bool any, int& peer, int& bad
     return row < 0 ? -1 - row : row;
 }
 
-// Key of a received row r < R: (local expert, sender of its step), -1 if either is missing.
-__device__ __forceinline__ int row_key_of(const UnpackArgs& a, int r, int e, int K, const int* step_row, const int* step_peer) {
-    int lo = 0, hi = K - 1;                                        // last step starting at or before r
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (step_row[mid] <= r) lo = mid; else hi = mid - 1;
+// Keys of the received rows r .. r + n - 1 < R with the experts e[]: (local expert, sender of its step), -1 if either is missing.  The
+// searches for the last step that starts at or before a row run side by side, without branches (one by one 700 cycles each).
+template <int n>
+__device__ __forceinline__ void row_keys_of(const UnpackArgs& a, int r, const int (&e)[n], int K, const int* step_row, const int* step_peer, int (&key)[n]) {
+    int lo[n];
+#pragma unroll
+    for (int q = 0; q < n; q++) lo[q] = 0;
+    for (int w = K > 1 ? 1 << (31 - __clz(K - 1)) : 0; w; w >>= 1) {
+#pragma unroll
+        for (int q = 0; q < n; q++) {
+            const int mid = min(lo[q] + w, K - 1);
+            lo[q] = step_row[mid] <= r + q ? mid : lo[q];
+        }
     }
-    const int src = K > 0 ? step_peer[lo] : -1;
-    return e < 0 || e >= a.epr || src < 0 ? -1 : e * a.N + src;
+#pragma unroll
+    for (int q = 0; q < n; q++) {
+        const int src = K > 0 ? step_peer[lo[q]] : -1;
+        key[q] = e[q] < 0 || e[q] >= a.epr || src < 0 ? -1 : e[q] * a.N + src;
+    }
 }
 
 // Key of a routed copy: its expert id, -1 if it does not travel.
@@ -108,13 +118,15 @@ __device__ __forceinline__ int copy_key_of(const UnpackArgs& a, int e) {
 
 // Run table of the return plan: bucket = sender, runs = its segments in the receive buffer.  peer(k) is the sender of step k;
 // row0 is the first row of step threadIdx.x as return_row gives it.
-__device__ __forceinline__ int return_row(const UnpackArgs& a, int k) {
+__device__ __forceinline__ int return_row(const UnpackArgs& a, int64_t off) {
     int64_t odd;
-    const int row = (int)a.row.div(a.recv_off[(size_t)k * a.N + a.rank], odd);
+    const int row = (int)a.row.div(off, odd);
     return odd ? -1 : row;
 }
+__device__ __forceinline__ int return_row(const UnpackArgs& a, int k) { return return_row(a, a.recv_off[(size_t)k * a.N + a.rank]); }
 template <typename Peer>
-__device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, int row0, Peer peer, Runs out, int* cnt, int* scratch) {
+__device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, int row0, Peer peer, Runs out, int* cnt, int* scratch, bool cleared = false,
+                                           bool report = true) {
     int bad = 0;
     const auto step = [&](int k, int at) {
         const int j = peer(k);
@@ -125,7 +137,8 @@ __device__ __forceinline__ int return_runs(const UnpackArgs& a, int K, int row0,
         return Step{rows > 0 ? j : -1, (int)rows, at};
     };
     const Step first = (int)threadIdx.x < K ? step(threadIdx.x, row0) : Step{-1, 0, 0};
-    build_runs(K, a.N, first, [&](int k) { return step(k, return_row(a, k)); }, out, cnt, scratch);
+    build_runs(K, a.N, first, [&](int k) { return step(k, return_row(a, k)); }, out, cnt, scratch, cleared);
+    if (!report) return 0;
     return __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
 }
 
@@ -143,25 +156,45 @@ __device__ __forceinline__ void scan_keys(const int* total, int* first, int keys
     __syncthreads();
 }
 
+// The same by one warp, of all[key] + next[key]; no barrier.
+__device__ __forceinline__ void warp_scan_keys(const int* all, const int* next, int* first, int keys) {
+    const int lane = threadIdx.x & 31;
+    int run = 0;
+#pragma unroll 4
+    for (int k = lane; k - lane < keys; k += 32) {
+        const int mine = k < keys ? all[k] + next[k] : 0;
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (k < keys) first[k] = run + incl - mine;
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) first[keys] = run;
+}
+
 // ---- one launch -------------------------------------------------------------------------------------------------
 
-struct UnpackSmall { int peer, step_row, all, next, first, wsum, cnt, total, ptr, start, row, src, dst, scratch, ints; };
-__host__ __device__ inline UnpackSmall unpack_small_layout(int N, int keys, int k_max, bool tokens) {
+struct UnpackSmall { int key, peer, step_row, all, next, first, wsum, cnt, total, ptr, start, row, src, dst, scratch, ints; };
+__host__ __device__ inline UnpackSmall unpack_small_layout(int N, int keys, int k_max, int own, bool tokens) {
     UnpackSmall L;
     int o = 0;
+    L.key = o;      o += (own + 3) & ~3;             // (read four at a time)
     L.peer = o;     o += k_max;
     L.step_row = o; o += tokens ? 0 : k_max + 1;
     L.all = o;      o += keys;
     L.next = o;     o += keys;
     L.first = o;    o += keys + 1;
-    L.wsum = o;     o += kIdxWarps + 1;
+    L.wsum = o;     o += tokens ? 0 : kIdxWarps + 1;
     L.cnt = o;      o += tokens ? N : 0;
     L.total = o;    o += tokens ? N : 0;
     L.ptr = o;      o += tokens ? N + 1 : 0;
     L.start = o;    o += tokens ? k_max : 0;
     L.row = o;      o += tokens ? k_max : 0;
-    L.src = o;      o += kSmallOwn;
-    L.dst = o;      o += kSmallOwn;
+    L.src = o;      o += own;
+    L.dst = o;      o += own;
     L.scratch = o;  o += tokens ? runs_scratch_ints(N) : 0;
     L.ints = o;
     return L;
@@ -170,21 +203,45 @@ __host__ __device__ inline UnpackSmall unpack_small_layout(int N, int keys, int 
 // Receive side of small calls.  Every CTA reads the plan and the keys of all received rows, counts them (all of them, and
 // those before its own), and moves its own contiguous range of rows.  Bound by latency, then by HBM.  Replaces two memsets
 // and six kernels.
-template <typename V>
-__global__ void __launch_bounds__(kIdxThreads, 2)
-unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, int pieces) {
-    extern __shared__ int sm[];
-    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, false);
+template <typename V, bool BULK>
+__global__ void __launch_bounds__(kIdxThreads, BULK ? 1 : 2)
+unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, SmallLaunch z) {
+    extern __shared__ __align__(128) int sm[];
+    __shared__ __align__(8) unsigned long long bars[kOwnWarps * kOwnStages];
+    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, z.own, false);
+    const int pieces = z.pieces;
     int *const peer = sm + L.peer, *const step_row = sm + L.step_row, *const all = sm + L.all, *const next = sm + L.next;
     const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V)), v_lo = (int)((long long)vecs * piece / pieces),
+              v_hi = (int)((long long)vecs * (piece + 1) / pieces);
     for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
+    OwnRing ring;
+    if (BULK && tid < kOwnWarps * 32) ring.init(z, recv, out, a.row.d, v_lo, v_hi, sm, bars);
+    for (int k = tid; k < a.k_max; k += kIdxThreads) peer[k] = -1;
+    __syncthreads();
     grid_wait();
+    // what the index needs first is asked for at once, before K is known
+    const uint4 cells = sender_cells(a.lane_dst, a.N, a.k_max);
+    constexpr int kAhead = 4;                        // loads of rows' experts per thread: of one up to 2,048 rows, else of four
+    const bool by4 = ((uintptr_t)a.item_expert & 15) == 0 && a.items > kAhead * kIdxThreads;
+    const int ahead = by4 ? min(a.items / 4, kAhead * kIdxThreads) : min(a.items, kAhead * kIdxThreads);
+    int4 expert[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; u++) {
+        const int v = tid + u * kIdxThreads;
+        expert[u] = make_int4(0, 0, 0, 0);
+        if (v < ahead) {
+            if (by4) expert[u] = __ldg((const int4*)a.item_expert + v);
+            else expert[u].x = __ldg(a.item_expert + v);
+        }
+    }
     bool any0 = false;
-    const int row0 = tid < a.k_max ? step_rows(a, tid, any0) : 0;      // (before K is known: a trip to L2 saved)
+    const int row0 = tid < a.k_max ? step_rows(a, tid, any0) : 0;
     const int K = steps_in_use(a);
     int st, bad = 0;
     const int R = rows_received(a, K, st);
-    find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+    const int r0 = (int)((long long)R * c / n_cta), r1 = (int)((long long)R * (c + 1) / n_cta);
+    find_senders(a.lane_dst, a.N, a.rank, 0, K, cells, peer);
     for (int k = tid; k < K; k += kIdxThreads) {
         bool any = any0;
         const int row = k == tid ? row0 : step_rows(a, k, any);
@@ -193,15 +250,37 @@ unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
         peer[k] = p;
     }
     __syncthreads();
-    const int r0 = (int)((long long)R * c / n_cta), r1 = (int)((long long)R * (c + 1) / n_cta);
-#pragma unroll 4
-    for (int r = tid; r < R; r += kIdxThreads) {
-        const int key = row_key_of(a, r, a.item_expert[r], K, step_row, peer);
-        if (key < 0) { bad = VP_ST_PACK_MISMATCH; continue; }
-        atomicAdd(&all[key], 1);
-        if (r < r0) atomicAdd(&next[key], 1);
+    int* const own_key = sm + L.key;
+    const auto add = [&](int r, int key) {
+        if (r >= r0 && r < r1) own_key[r - r0] = key;
+        if (key < 0) bad = VP_ST_PACK_MISMATCH;
+        else atomicAdd(&sm[(r < r0 ? L.next : L.all) + key], 1);
+    };
+    const auto count = [&](int r, int x) {
+        const int e[1] = {x};
+        int key[1];
+        row_keys_of(a, r, e, K, step_row, peer, key);
+        add(r, key[0]);
+    };
+#pragma unroll
+    for (int u = 0; u < kAhead; u++) {
+        const int v = tid + u * kIdxThreads;
+        if (v >= ahead) break;
+        if (!by4) {
+            if (v < R) count(v, expert[u].x);
+        } else if (4 * v < R) {
+            const int e[4] = {expert[u].x, expert[u].y, expert[u].z, expert[u].w};
+            int key[4];
+            row_keys_of(a, 4 * v, e, K, step_row, peer, key);
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (4 * v + q < R) add(4 * v + q, key[q]);
+        }
     }
+    for_each_item(a.item_expert, min(by4 ? 4 * ahead : ahead, R), R, count);
+    if (BULK && tid < kOwnWarps * 32) ring.start(r1 - r0, [&](int i) { return r0 + i; });
     bad = __syncthreads_or(bad) ? VP_ST_PACK_MISMATCH : 0;
+    for (int j = tid; j < a.keys; j += kIdxThreads) all[j] += next[j];     // (scan_keys reads what the thread wrote)
     int* const first = sm + L.first;
     scan_keys(all, first, a.keys, sm + L.wsum);
     if (blockIdx.x == 0) {
@@ -209,47 +288,60 @@ unpack_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
         if (tid == 0) *a.status = st | bad | (!(st & VP_ST_PACK_CAPACITY) && first[a.keys] != R ? VP_ST_PACK_MISMATCH : 0);
     }
     int *const src = sm + L.src, *const dst = sm + L.dst;
-    if (tid < 32)
-        warp_positions(r0, r1, next, [&](long long r) { return row_key_of(a, (int)r, a.item_expert[r], K, step_row, peer); },
-                       [&](long long r, int key, int p) {
-                           const int o = p >= 0 ? first[key] + p : -1;
-                           src[r - r0] = o >= 0 ? (int)r : -1;
-                           dst[r - r0] = o;
-                           if (o >= 0 && piece == 0) {
-                               if (a.out_src) a.out_src[o] = key % a.N;
-                               if (a.out_map) a.out_map[o] = (int)r;
-                           }
-                       });
+    own_positions(own_key, r1 - r0, next, [&](int i, int key, int p) {
+        const int o = p >= 0 ? first[key] + p : -1;
+        src[i] = o >= 0 ? r0 + i : -1;
+        dst[i] = o;
+        if (o >= 0 && piece == 0) {
+            if (a.out_src) a.out_src[o] = key % a.N;
+            if (a.out_map) a.out_map[o] = r0 + i;
+        }
+    });
     __syncthreads();
-    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
-    move_rows<V>(recv, out, a.row.d, r1 - r0, 1, src, dst, (int)((long long)vecs * piece / pieces),
-                 (int)((long long)vecs * (piece + 1) / pieces));
+    if (BULK) {
+        if (tid < kOwnWarps * 32 && !ring.finish(1, dst, [&](int i) { return r0 + i; }) && (tid & 31) == 0) atomicOr(a.status, VP_ST_INTERNAL_TIMEOUT);
+        return;
+    }
+    move_rows<V>(recv, out, a.row.d, r1 - r0, 1, src, dst, v_lo, v_hi);
 }
 
 // Return direction of small calls, the same way: own range = output rows (routed copies).
-template <typename V>
-__global__ void __launch_bounds__(kIdxThreads, 2)
-tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, int pieces) {
-    extern __shared__ int sm[];
-    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, true);
+template <typename V, bool BULK>
+__global__ void __launch_bounds__(kIdxThreads, BULK ? 1 : 2)
+tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restrict__ out, SmallLaunch z) {
+    extern __shared__ __align__(128) int sm[];
+    __shared__ __align__(8) unsigned long long bars[kOwnWarps * kOwnStages];
+    const UnpackSmall L = unpack_small_layout(a.N, a.keys, a.k_max, z.own, true);
+    const int pieces = z.pieces;
     int *const peer = sm + L.peer, *const all = sm + L.all, *const next = sm + L.next, *const first = sm + L.first;
     const int tid = threadIdx.x, n_cta = gridDim.x / pieces, c = blockIdx.x / pieces, piece = blockIdx.x - c * pieces;
+    const int vecs = (int)(a.row.d / (int64_t)sizeof(V)), v_lo = (int)((long long)vecs * piece / pieces),
+              v_hi = (int)((long long)vecs * (piece + 1) / pieces);
     for (int j = tid; j < a.keys; j += kIdxThreads) { all[j] = 0; next[j] = 0; }
+    OwnRing ring;
+    if (BULK && tid < kOwnWarps * 32) ring.init(z, recv, out, a.row.d, v_lo, v_hi, sm, bars);
+    for (int k = tid; k < a.k_max; k += kIdxThreads) peer[k] = -1;
+    clear_runs_scratch(a.N, sm + L.scratch);
+    __syncthreads();
     grid_wait();
-    const int row0 = tid < a.k_max ? return_row(a, tid) : 0;           // (before K is known: a trip to L2 saved)
+    // all that the index needs first is asked for at once, before K is known
+    const uint4 cells = sender_cells(a.lane_dst, a.N, a.k_max);
+    const int64_t off0 = tid < a.k_max ? a.recv_off[(size_t)tid * a.N + a.rank] : 0;
     const int K = steps_in_use(a);
-    const bool over = a.recv_off[(size_t)K * a.N + a.rank] > a.capacity_rows * a.row.d;      // nothing is unpacked then
-    find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
     const int c0 = (int)((long long)a.items * c / n_cta), c1 = (int)((long long)a.items * (c + 1) / n_cta);
+    int* const own_key = sm + L.key;
+    for (int i = tid; i < c1 - c0; i += kIdxThreads) own_key[i] = copy_key_of(a, a.item_expert[c0 + i]);
     for_each_item(a.item_expert, 0, a.items, [&](int i, int e) {
         const int key = copy_key_of(a, e);
-        if (key < 0) return;
-        atomicAdd(&all[key], 1);
-        if (i < c0) atomicAdd(&next[key], 1);
+        if (key >= 0) atomicAdd(&sm[(i < c0 ? L.next : L.all) + key], 1);
     });
+    const int64_t end = a.recv_off[(size_t)K * a.N + a.rank];
+    find_senders(a.lane_dst, a.N, a.rank, 0, K, cells, peer);         // (ends with a barrier: the counts are complete, too)
+    if (tid >= kIdxThreads - 32) warp_scan_keys(all, next, first, a.keys);   // (while the others fetch the steps' bytes)
+    const int row0 = return_row(a, off0);
     const Runs runs{sm + L.start, sm + L.row, sm + L.ptr, sm + L.total};
-    const int st = return_runs(a, K, row0, [&](int k) { return peer[k]; }, runs, sm + L.cnt, sm + L.scratch);
-    scan_keys(all, first, a.keys, sm + L.wsum);
+    const int st = return_runs(a, K, row0, [&](int k) { return peer[k]; }, runs, sm + L.cnt, sm + L.scratch, true, blockIdx.x == 0);
+    const bool over = end > a.capacity_rows * a.row.d;                // nothing is unpacked then
     if (blockIdx.x == 0) {                           // every sender's stream is used up exactly
         int bad = st;
         if (tid < a.N && tid != a.rank && first[(tid + 1) * a.epr] - first[tid * a.epr] != runs.total[tid]) bad = VP_ST_PACK_MISMATCH;
@@ -257,22 +349,26 @@ tokens_small_kernel(UnpackArgs a, const char* __restrict__ recv, char* __restric
         if (tid == 0) *a.status = over ? VP_ST_PACK_CAPACITY : bad;
     }
     int *const src = sm + L.src, *const dst = sm + L.dst;
-    if (tid < 32)
-        warp_positions(c0, c1, next, [&](long long i) { return copy_key_of(a, a.item_expert[i]); },
-                       [&](long long i, int key, int p) {
-                           int row = -1;
-                           if (p >= 0 && !over) {
-                               const int j = a.by_epr.div(key);
-                               row = run_lookup(runs, j, first[key] + p - first[j * a.epr]);   // position in sender j's stream
-                           }
-                           src[i - c0] = row;
-                           dst[i - c0] = (int)i;
-                           if (a.out_map && piece == 0) a.out_map[i] = row;
-                       });
+    own_positions(own_key, c1 - c0, next, [&](int i, int key, int p) {
+        int row = -1;
+        if (p >= 0 && !over) {
+            const int j = a.by_epr.div(key);
+            row = run_lookup(runs, j, first[key] + p - first[j * a.epr]);      // position in sender j's stream
+        }
+        src[i] = row;
+        dst[i] = c0 + i;
+        if (a.out_map && piece == 0) a.out_map[c0 + i] = row;
+    });
     __syncthreads();
-    const int vecs = (int)(a.row.d / (int64_t)sizeof(V));
-    move_rows<V>(recv, out, a.row.d, c1 - c0, 1, src, dst, (int)((long long)vecs * piece / pieces),
-                 (int)((long long)vecs * (piece + 1) / pieces));
+    if (BULK) {
+        if (tid < kOwnWarps * 32) {
+            const auto from = [&](int i) { return src[i]; };
+            ring.start(c1 - c0, from);
+            if (!ring.finish(1, dst, from) && (tid & 31) == 0) atomicOr(a.status, VP_ST_INTERNAL_TIMEOUT);
+        }
+        return;
+    }
+    move_rows<V>(recv, out, a.row.d, c1 - c0, 1, src, dst, v_lo, v_hi);
 }
 
 // ---- chunked form -----------------------------------------------------------------------------------------------
@@ -323,7 +419,10 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     __syncthreads();
     const ChunkRange mine = chunk_range(blockIdx.x, chunk, R);
     for (long long r = mine.lo + tid; r < mine.hi; r += kIdxThreads) {
-        const int key = row_key_of(a, (int)r, a.item_expert[r], K, step_row, peer);
+        const int e[1] = {a.item_expert[r]};
+        int keys[1];
+        row_keys_of(a, (int)r, e, K, step_row, peer, keys);
+        const int key = keys[0];
         w.item_key[r] = key;
         if (key >= 0) atomicAdd(&hist[key], 1);
         else bad = VP_ST_PACK_MISMATCH;
@@ -339,7 +438,7 @@ __global__ void __launch_bounds__(kIdxThreads) tokens_count_kernel(UnpackArgs a,
     grid_wait();
     if ((int)blockIdx.x == n_chunks) {               // the senders' run table
         int *const cnt = sm, *const scratch = sm + a.N, *const peer = scratch + runs_scratch_ints(a.N);
-        const int row0 = tid < a.k_max ? return_row(a, tid) : 0;
+        const int row0 = tid < a.k_max ? return_row(a, (int)tid) : 0;
         const int K = steps_in_use(a);
         if (inline_steps) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
         const int st = return_runs(a, K, row0, [&](int k) { return inline_steps ? peer[k] : w.step_peer[k]; },
@@ -468,19 +567,19 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
     const bool steps_fit = ((long long)a.keys + 2ll * a.k_max) * 4 <= (long long)kSmemLimit;
     const bool inline_steps = (long long)a.k_max * a.N <= kInlineCells && steps_fit;
     cudaError_t e = cudaSuccess;
-    if (items <= kSmallItems && a.k_max <= kSmallSteps && inline_steps && a.row.d <= kSmallRow) {
-        const SmallSplit s = small_split(a.items, sms);
-        const int n_cta = s.grid / s.pieces;
-        const size_t smem = (size_t)unpack_small_layout(a.N, a.keys, a.k_max, TOKENS).ints * 4;
-        if ((items + n_cta - 1) / n_cta <= kSmallOwn) {
+    if (items <= (TOKENS ? kSmallReturn : kSmallItems) && a.k_max <= kSmallSteps && inline_steps && a.row.d <= kSmallRow) {
+        const int width = copy_width(recv, out, a.row.d);
+        const SmallLaunch z = small_launch(a.items, sms, 1, a.row.d, width, [&](int own) { return unpack_small_layout(a.N, a.keys, a.k_max, own, TOKENS).ints; });
+        if (z.own <= kSmallOwn) {
             const char* from = (const char*)recv;
             vp_prof_mark(3, 0, stream);
-            const auto go = [&](auto fn) { return launch_wide(fn, s.grid, smem, stream, a, from, (char*)out, s.pieces); };
-            const int width = copy_width(recv, out, a.row.d);
+            const auto go = [&](auto fn) { return launch_wide(fn, z.grid, z.smem, stream, a, from, (char*)out, z); };
             if constexpr (TOKENS)
-                e = width == 16 ? go(tokens_small_kernel<uint4>) : width == 4 ? go(tokens_small_kernel<uint32_t>) : go(tokens_small_kernel<uint8_t>);
+                e = z.bulk ? go(tokens_small_kernel<uint4, true>) : width == 16 ? go(tokens_small_kernel<uint4, false>)
+                  : width == 4 ? go(tokens_small_kernel<uint32_t, false>) : go(tokens_small_kernel<uint8_t, false>);
             else
-                e = width == 16 ? go(unpack_small_kernel<uint4>) : width == 4 ? go(unpack_small_kernel<uint32_t>) : go(unpack_small_kernel<uint8_t>);
+                e = z.bulk ? go(unpack_small_kernel<uint4, true>) : width == 16 ? go(unpack_small_kernel<uint4, false>)
+                  : width == 4 ? go(unpack_small_kernel<uint32_t, false>) : go(unpack_small_kernel<uint8_t, false>);
             vp_prof_mark(3, 1, stream);
             return e == cudaSuccess ? VP_OK : VP_E_CUDA;
         }

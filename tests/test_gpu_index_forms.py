@@ -1,5 +1,5 @@
 """GPU parity of the pack and both unpack directions where their index work changes form: one self-contained launch up to
-8,192 items and 1,024 plan rows, chunked histograms beyond; the plan's senders read in place or resolved by a kernel of
+16,384 items (return: 12,288) and 1,024 plan rows, chunked histograms beyond; the plan's senders read in place or resolved by a kernel of
 their own; fewer rows than SMs (a row split over CTAs) and more; every copy width."""
 import numpy as np
 import pytest
@@ -38,7 +38,8 @@ def _case(nodes, tokens, topk, row_bytes, k_max=0, seed=0):
 # are multiples of 16, 4 and 1 bytes on both sides of 2 KB, and rows of more than one 16 KB piece
 CASES = [(2, 1, 1, 4096, 0), (2, 5, 8, 14336, 0), (1, 149, 3, 4100, 0), (2, 700, 6, 333, 0), (2, 1024, 8, 96, 0), (2, 1025, 8, 96, 0),
          (2, 2400, 8, 2064, 0), (2, 2100, 8, 4100, 0), (2, 300, 8, 2048, 1025), (2, 300, 8, 2048, 40000), (8, 40, 6, 7392, 0),
-         (8, 2300, 8, 1536, 0), (16, 30, 4, 4096, 2048), (32, 12, 8, 512, 4096), (2, 2100, 8, 16400, 0)]
+         (2, 1536, 8, 2064, 0), (2, 1537, 8, 2064, 0), (2, 2048, 8, 96, 0), (2, 2049, 8, 96, 0), (2, 600, 8, 33008, 0), (2, 297, 8, 2048, 0),
+         (2, 74, 1, 2064, 0), (2, 75, 1, 16400, 0), (8, 1200, 8, 4096, 0), (8, 2300, 8, 1536, 0), (16, 30, 4, 4096, 2048), (32, 12, 8, 512, 4096), (2, 2100, 8, 16400, 0)]
 
 
 @pytest.mark.parametrize("nodes,tokens,topk,row_bytes,k_max", CASES)
