@@ -224,8 +224,10 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
     const ChunkRange mine = chunk_range(blockIdx.x, chunk, (long long)a.T * a.topk);
     const long long s0 = min(mine.lo + (long long)warp * (chunk / kIdxWarps), mine.hi), s1 = min(s0 + chunk / kIdxWarps, mine.hi);
     int ignore = 0;
-    for (long long e = s0 + lane; e < s1; e += 32) {
-        const int j = dest_of(a.idx[e], a, ignore);
+    const long long own0 = s0 + lane;
+    const int dest0 = own0 < s1 ? dest_of(a.idx[own0], a, ignore) : -1;
+    for (long long e = own0; e < s1; e += 32) {
+        const int j = e == own0 ? dest0 : dest_of(a.idx[e], a, ignore);
         if (j >= 0) atomicAdd(&next[j], 1);
     }
     grid_wait();
@@ -238,14 +240,7 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
     const Runs runs = runs_to_shared(Runs{w.start, w.row, w.ptr, w.total}, N, kMapRuns, sm + N * (kIdxWarps + 1));
     __syncthreads();
     for (int j = tid; j < N; j += kIdxThreads) {     // exclusive prefix over the warps
-        int run = base[j];
-        for (int v = 0; v < kIdxWarps; v++) {
-            int* const at = sm + N + v * N + j;
-            const int x = *at;
-            *at = run;
-            run += x;
-        }
-        base[j] = run;                               // copies up to the end of this chunk
+        base[j] = slices_prefix(sm + N + j, N, base[j]);     // copies up to the end of this chunk
     }
     __syncthreads();
     if (blockIdx.x == gridDim.x - 1) {
@@ -256,7 +251,7 @@ __global__ void __launch_bounds__(kIdxThreads) pack_map_kernel(PackArgs a, PackW
         const int mismatch = __syncthreads_or(bad & VP_ST_PACK_MISMATCH);
         if (tid == 0) *a.status = (bad & VP_ST_PACK_CAPACITY) | (mismatch ? VP_ST_PACK_MISMATCH : 0);
     }
-    warp_positions(s0, s1, next, [&](long long e) { return dest_of(a.idx[e], a, ignore); },
+    warp_positions(s0, s1, next, [&](long long e) { return e == own0 ? dest0 : dest_of(a.idx[e], a, ignore); },
                    [&](long long e, int j, int p) {
                        const int row = p >= 0 && !over ? run_lookup(runs, j, p) : -1;
                        w.dst_row[e] = row;

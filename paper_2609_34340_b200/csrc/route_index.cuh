@@ -375,6 +375,17 @@ __device__ __forceinline__ void for_each_item(const int32_t* __restrict__ x, int
     for (int i = v1 + threadIdx.x; i < hi; i += kIdxThreads) f(i, __ldg(x + i));
 }
 
+// Counts of the warps' slices, count[w * stride], to the first position of each, starting at `run`; returns where the last one ends.
+// (All read before the first is written: one after the other each read waits for the write ahead of it.)
+__device__ __forceinline__ int slices_prefix(int* count, int stride, int run) {
+    int x[kIdxWarps];
+#pragma unroll
+    for (int w = 0; w < kIdxWarps; w++) x[w] = count[w * stride];
+#pragma unroll
+    for (int w = 0; w < kIdxWarps; w++) { count[w * stride] = run; run += x[w]; }
+    return run;
+}
+
 // Stable positions of the items lo <= i < hi, taken 32 at a time by ONE warp: key(i) names an item's key (-1: none),
 // next[] holds the position of the next item of every key and is carried on; put(i, key, position) is called for every
 // item, with position -1 where there is no key.

@@ -400,7 +400,14 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     int* const step_row = steps == 2 ? w.step_row : sm + a.keys + a.k_max;
     const int tid = threadIdx.x;
     for (int j = tid; j < a.keys; j += kIdxThreads) hist[j] = 0;
+    if (steps == 0)
+        for (int k = tid; k < a.k_max; k += kIdxThreads) peer[k] = -1;
+    __syncthreads();
     grid_wait();
+    // plan cells and the first row's expert, before it is known how many there are
+    const uint4 cells = steps == 0 ? sender_cells(a.lane_dst, a.N, a.k_max) : make_uint4(0, 0, 0, 0);
+    const long long own0 = (long long)blockIdx.x * chunk + tid;
+    const int expert0 = own0 < a.items ? __ldg(a.item_expert + own0) : 0;
     bool any0 = false;
     const int row0 = tid < a.k_max ? step_rows(a, tid, any0) : 0;
     const int K = steps_in_use(a);
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     const int R = rows_received(a, K, st);
     if (blockIdx.x == 0 && tid == 0) { w.flags[0] = (st & VP_ST_PACK_CAPACITY) != 0; w.flags[1] = st; w.flags[2] = R; }
     if ((int)blockIdx.x > 0 && (int)blockIdx.x >= chunks_of(R, chunk)) return;     // (CTA 0 always reports on the plan)
-    if (steps == 0) find_senders(a.lane_dst, a.N, a.rank, 0, K, peer);
+    if (steps == 0) find_senders(a.lane_dst, a.N, a.rank, 0, K, cells, peer);
     for (int k = tid; k < K; k += kIdxThreads) {
         bool any = any0;
         const int row = k == tid ? row0 : step_rows(a, k, any);
@@ -419,7 +426,7 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_count_kernel(UnpackArgs a,
     __syncthreads();
     const ChunkRange mine = chunk_range(blockIdx.x, chunk, R);
     for (long long r = mine.lo + tid; r < mine.hi; r += kIdxThreads) {
-        const int e[1] = {a.item_expert[r]};
+        const int e[1] = {r == own0 ? expert0 : a.item_expert[r]};
         int keys[1];
         row_keys_of(a, (int)r, e, K, step_row, peer, keys);
         const int key = keys[0];
@@ -483,17 +490,23 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, U
     __syncthreads();
     auto key_of = [&](long long i) { return TOKENS ? copy_key_of(a, a.item_expert[i]) : w.item_key[i]; };
     long long s0, s1;
+    const long long own0 = (long long)blockIdx.x * chunk + (long long)warp * (chunk / kIdxWarps) + lane;
+    int key0 = -1;                                   // the slice's first 32 keys: asked for with the flags, and read twice
     auto count_slice = [&](int items) {
         const ChunkRange own = chunk_range(blockIdx.x, chunk, items);
         s0 = min(own.lo + (long long)warp * (chunk / kIdxWarps), own.hi);
         s1 = min(s0 + chunk / kIdxWarps, own.hi);
         for (long long i = s0 + lane; i < s1; i += 32) {
-            const int key = key_of(i);
+            const int key = i == own0 ? key0 : key_of(i);
             if (key >= 0) atomicAdd(&next[key], 1);
         }
     };
-    if (TOKENS) count_slice(a.items);
+    if (TOKENS) {
+        if (own0 < a.items) key0 = key_of(own0);
+        count_slice(a.items);
+    }
     grid_wait();
+    if (!TOKENS && own0 < a.items) key0 = key_of(own0);      // (beyond the rows received: not used)
     const bool over = w.flags[0] != 0;
     const int items = TOKENS ? a.items : w.flags[2];
     const int n_chunks = chunks_of(items, chunk);
@@ -530,15 +543,10 @@ __global__ void __launch_bounds__(kIdxThreads) unpack_map_kernel(UnpackArgs a, U
         if (tid == 0) *a.status = w.flags[1] | (TOKENS && over ? 0 : bad);
     }
     for (int j = tid; j < keys; j += kIdxThreads) {  // start of every warp's slice: key, chunks before, warps before
-        int run = first[j] + before[j];
-        for (int v = 0; v < kIdxWarps; v++) {
-            const int x = slices[v * keys + j];
-            slices[v * keys + j] = run;
-            run += x;
-        }
+        slices_prefix(slices + j, keys, first[j] + before[j]);
     }
     __syncthreads();
-    warp_positions(s0, s1, next, key_of, [&](long long i, int key, int p) {
+    warp_positions(s0, s1, next, [&](long long i) { return i == own0 ? key0 : key_of(i); }, [&](long long i, int key, int p) {
         if (TOKENS) {
             int row = -1;
             if (p >= 0 && !over) {
