@@ -42,6 +42,7 @@ namespace {
 
 struct KParams {
     int64_t lambda_ns, granule;
+    double inv_granule;
     int k_target, n_start, i_aa, k_max;
     int max_tasks, stage_terms, stage_fam, stage_bucket, drem_in_smem;
     int big_stage, big_cross, big_task_warps, big_emit_warp;    // vp_schedule_big_kernel: task tables in shared memory, a task is two warps, task warps, first emitting warp
@@ -1193,7 +1194,7 @@ int resolve_params(const vp_catalog* c, const vp_sched_params* p, KParams* kp) {
     if (!c || !p || c->device < 0) return VP_E_BAD_ARG;         // (a host-only handle launches nothing)
     if (p->k_max <= 0 || p->granule_bytes <= 0 || p->lambda_ns < 0 || p->lambda_ns >= VP_ENTRY_LIMIT) return VP_E_BAD_ARG;
     if (p->k_target < 0 || p->n_start < 0 || p->i_aa < 0 || p->n_start > 64) return VP_E_BAD_ARG;
-    kp->lambda_ns = p->lambda_ns; kp->granule = p->granule_bytes;
+    kp->lambda_ns = p->lambda_ns; kp->granule = p->granule_bytes; kp->inv_granule = 1.0 / (double)p->granule_bytes;
     kp->k_target = p->k_target ? p->k_target : 2 * c->dc.N;
     kp->n_start = p->n_start ? p->n_start : c->dc.g;
     kp->i_aa = p->i_aa ? p->i_aa : 3;

@@ -174,7 +174,23 @@ __device__ __forceinline__ void big_fill_bytes(unsigned char* dst, size_t lo, si
 
 // (out of line: 64-bit division is long, and granules are powers of two in practice)
 __device__ __noinline__ bool big_not_multiple(int64_t x, int64_t granule) { return x % granule != 0; }
-__device__ __noinline__ uint32_t big_div_granule(int64_t x, int64_t granule) { return (uint32_t)(x / granule); }
+__device__ __noinline__ int64_t big_wide_ceil_div(int64_t x, int64_t d) { return x / d + (x % d > 0); }
+// What is wrong with the entries of rows ga * 4 .. ga * 4 + 3 (out of line: looked for only when something is).  Whole warp.
+__device__ __noinline__ int big_wrong_entries(const int64_t* rows, int N, int ga, int64_t granule) {
+    int flags = 0;
+#pragma unroll 1
+    for (int e = threadIdx.x & 31; e < 4 * N; e += 32) {
+        const int64_t x = rows[e];
+        const int i = e / N;
+        if (x < 0) flags |= VP_ST_NEGATIVE;
+        else if (x >= VP_ENTRY_LIMIT) flags |= VP_ST_OVERFLOW_RISK;
+        else {
+            if (e - i * N == ga * 4 + i && x != 0) flags |= VP_ST_DIAG_NONZERO;
+            if (big_not_multiple(x, granule)) flags |= VP_ST_NOT_GRANULE;
+        }
+    }
+    return flags;
+}
 
 // An offset row in rank order, whole lines for PCIe, once all of it is up to date: `threads` threads, numbered from 0, whole warps (out of
 // line: for page-locked plans only, and inlined it costs the other case registers).  The barrier's number counts: an SM has 64, and a
@@ -419,6 +435,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
     const int S = dc.S, P = dc.P;
     const bool by_class = big_by_class(dc);
 
+    const double inv_bw = 1.0 / (double)dc.bw_max;
     // ---- stage the catalog once per CTA: bulk asynchronous copies (TMA) onto one mbarrier; should the bounded wait give
     // up, plain loads fetch the same arrays
     {
@@ -527,53 +544,71 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         int64_t* rowsum = Dhat + G * G;
         int64_t* colsum = rowsum + N;
         int64_t* colmax = colsum + N;
-        for (int i = tid; i < N; i += NT) { colsum[i] = 0; colmax[i] = 0; rowsum[i] = 0; send_acc[i] = 0; recv_acc[i] = 0; colmap[i] = BIG_HOT_MAX; if (EXACT) Hi[BIG_HOT_MAX * N + i] = 0; }
+        uint32_t* const colpart = (uint32_t*)colsum;          // [j] low 24 bits of the column's parts, [N + j] the rest (added up below)
+        uint32_t* const coltop = (uint32_t*)colmax;           // largest entry of the column >> 8
+        for (int i = tid; i < N; i += NT) { colpart[i] = 0; colpart[N + i] = 0; coltop[i] = 0; send_acc[i] = 0; recv_acc[i] = 0; colmap[i] = BIG_HOT_MAX; if (EXACT) Hi[BIG_HOT_MAX * N + i] = 0; }
         if (EXACT) for (int i = tid; i < BIG_HOT_MAX; i += NT) s_beyond[i] = 0;
         if (tid == 0) { s_nhot = 0; s_nbig = 0; if (EXACT) s_hot = 0; }
-        for (int e = tid; e < G * G; e += NT) Dhat[e] = 0;
         __syncthreads();
         int flags = 0;
-        // One warp per source group.  A row is read 32 columns per load instruction, its loads (up to eight) all in
-        // flight at once; row sums need one warp reduction per row, column figures are carried over the group's four rows.
-        const int64_t gmask = (kp.granule & (kp.granule - 1)) == 0 ? kp.granule - 1 : -1;     // power-of-two granule
+        // One warp per source group, 32 columns per load, the loads of two to four rows in flight at once and their sums side by side.
+        // An entry's checks are bits that must not be there: of its value from 2^40 on, of the diagonal, of the difference to the next
+        // multiple of the granule (entries are below 2^40, so a product with the reciprocal rounds to the quotient of a multiple).
+        // Column sums as two 32-bit atomics, as 64-bit ones are loops.  Row by row, with 64-bit remainders, this and the second
+        // pass took 45,000 of 912,000 cycles of a matrix of 64 ranks, 134,000 of 1,600,000 with eight CTAs on the SM.
         constexpr int CW = LANES / SPLIT * 4 / 32;           // 32-column pieces of a row
+        constexpr int RB = CW <= 4 ? 4 : 2;
+        const double inv_granule = kp.inv_granule;
+        const auto col_sum = [&](int j) { return ((int64_t)colpart[N + j] << 24) + colpart[j]; };
         for (int ga = warp; ga < G; ga += n_warps) {
-            int64_t colv[CW], colm[CW];
+            int64_t colv[CW];
+            uint32_t colm[CW];
+            uint64_t wrong = 0;
 #pragma unroll
             for (int m = 0; m < CW; m++) { colv[m] = 0; colm[m] = 0; }
 #pragma unroll 1
-            for (int i4 = 0; i4 < 4; i4++) {
-                const int i = ga * 4 + i4;
-                const int64_t* row = D + (size_t)i * N;
-                int64_t v[CW];
+            for (int i4 = 0; i4 < 4; i4 += RB) {
+                const int64_t* row = D + (size_t)(ga * 4 + i4) * N;
+                int64_t v[RB][CW], rsum[RB];
 #pragma unroll
-                for (int m = 0; m < CW; m++) v[m] = m * 32 + lane < N ? row[m * 32 + lane] : 0;
-                int64_t rsum = 0;
+                for (int r = 0; r < RB; r++)
 #pragma unroll
-                for (int m = 0; m < CW; m++) {
-                    const int64_t x = v[m];
-                    if (x < 0) flags |= VP_ST_NEGATIVE;
-                    else if (x >= VP_ENTRY_LIMIT) flags |= VP_ST_OVERFLOW_RISK;
-                    else {
-                        if (m * 32 + lane == i && x != 0) flags |= VP_ST_DIAG_NONZERO;
-                        if (gmask >= 0 ? (x & gmask) != 0 : big_not_multiple(x, kp.granule)) flags |= VP_ST_NOT_GRANULE;
+                    for (int m = 0; m < CW; m++) v[r][m] = m * 32 + lane < N ? row[r * N + m * 32 + lane] : 0;
+#pragma unroll
+                for (int r = 0; r < RB; r++) {
+                    rsum[r] = 0;
+#pragma unroll
+                    for (int m = 0; m < CW; m++) {
+                        const int64_t x = v[r][m];
+                        wrong |= (uint64_t)x >> 40 | (uint64_t)(__double2ll_rn((double)x * inv_granule) * kp.granule ^ x);
+                        if (m * 32 + lane == ga * 4 + i4 + r) wrong |= (uint64_t)x;
+                        rsum[r] += x;
+                        colv[m] += x;
+                        colm[m] = max_v(colm[m], (uint32_t)(x >> 8));
                     }
-                    rsum += x;
-                    colv[m] += x;
-                    colm[m] = max_v(colm[m], x);
                 }
-                rsum = warp_sum_i64(rsum);
-                if (lane == 0) rowsum[i] = rsum;             // (rows of this group belong to this warp alone)
+#pragma unroll
+                for (int o = 16; o; o >>= 1)
+#pragma unroll
+                    for (int r = 0; r < RB; r++) rsum[r] += __shfl_xor_sync(0xffffffffu, rsum[r], o);
+                if (lane == 0)
+#pragma unroll
+                    for (int r = 0; r < RB; r++) rowsum[ga * 4 + i4 + r] = rsum[r];   // (rows of this group belong to this warp alone)
             }
 #pragma unroll
             for (int m = 0; m < CW; m++) {
                 const int j = m * 32 + lane;
+                int64_t pair = colv[m];                          // sum over a destination group's four columns
+                pair += __shfl_xor_sync(0xffffffffu, pair, 1);
+                pair += __shfl_xor_sync(0xffffffffu, pair, 2);
                 if (j < N) {
-                    atomicAdd((unsigned long long*)&colsum[j], (unsigned long long)colv[m]);
-                    atomicMax((long long*)&colmax[j], (long long)colm[m]);
-                    atomicAdd((unsigned long long*)&Dhat[ga * G + (j >> 2)], (unsigned long long)colv[m]);
+                    atomicAdd(&colpart[j], (uint32_t)colv[m] & 0xffffffu);
+                    atomicAdd(&colpart[N + j], (uint32_t)(colv[m] >> 24));
+                    atomicMax(&coltop[j], colm[m]);
+                    if ((lane & 3) == 0) Dhat[ga * G + (j >> 2)] = pair;
                 }
             }
+            if (__any_sync(0xffffffffu, wrong != 0)) flags |= big_wrong_entries(D + (size_t)ga * 4 * N, N, ga, kp.granule);
         }
         const int64_t tau_given = tau_in ? tau_in[b] : 0;
         if (tid == 0 && (tau_given < 0 || tau_given > VP_ENTRY_LIMIT)) flags |= VP_ST_BAD_TAU;
@@ -589,17 +624,27 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         bool deferred = false;
         if (st == 0) {
             // ---- quantum (Section 5) and capacities
-            int64_t est = 0, tot = 0;
+            const RowDiv by_bw{dc.bw_max, inv_bw};
+            const auto ceil_div = [](int64_t x, const RowDiv& by) {
+                if (rarely(x >= (int64_t)1 << 52)) return big_wide_ceil_div(x, by.d);
+                int64_t rem;
+                const int64_t q = by.div(x, rem);
+                return q + (rem > 0);
+            };
+            int64_t tot = 0, most = 0;
             for (int i = tid; i < N; i += NT) {
                 tot += rowsum[i];
-                est = max_v(est, max_v(ceil_div_i64(rowsum[i], dc.bw_max), ceil_div_i64(colsum[i], dc.bw_max)));
+                most = max_v(most, max_v(rowsum[i], col_sum(i)));
             }
+            int64_t est = ceil_div(most, by_bw);
             for (int l = tid; l < dc.n_res; l += NT) {
                 const uint32_t bwl = dc.forced_bw[l];
                 if (!bwl) continue;
                 int64_t f = 0;
-                for (uint32_t e = dc.forced_ptr[l]; e < dc.forced_ptr[l + 1]; e++) f += Dhat[dc.forced_cell[e]];
-                est = max_v(est, ceil_div_i64(f, (int64_t)bwl));
+                const uint32_t e1 = dc.forced_ptr[l + 1];
+#pragma unroll 4
+                for (uint32_t e = dc.forced_ptr[l]; e < e1; e++) f += Dhat[dc.forced_cell[e]];
+                est = max_v(est, ceil_div(f, bwl == (uint32_t)dc.bw_max ? by_bw : RowDiv{(int64_t)bwl, 1.0 / (double)bwl}));
             }
             est = warp_max_i64(est);
             tot = warp_sum_i64(tot);
@@ -608,26 +653,30 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             if (tid == 0) {
                 int64_t e = 0, t = 0;
                 for (int w = 0; w < n_warps; w++) { e = max_v(e, (int64_t)red[w]); t += (int64_t)red[32 + w]; }
-                const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div_i64(e, (int64_t)kp.k_target));
+                const RowDiv by_granule{kp.granule, inv_granule};
+                int64_t rem;
+                const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div(e, RowDiv{(int64_t)kp.k_target, 1.0 / (double)kp.k_target}));
                 int64_t cap_max = 0;
                 for (int cl = 0; cl < dc.n_classes; cl++) {
-                    int64_t cp = (tq * dc.class_bw[cl]) / kp.granule * kp.granule;
-                    if (cp < kp.granule) cp = kp.granule;
+                    // in granules, at least one (rate x quantum may exceed what the reciprocal divides exactly)
+                    const int64_t x = tq * dc.class_bw[cl];
+                    const int64_t cp = max_v((int64_t)1, x < ((int64_t)1 << 52) ? by_granule.div(x, rem) : x / kp.granule);
                     cap_max = max_v(cap_max, cp);
-                    s_cap[cl] = (uint32_t)min_v(cp / kp.granule, (int64_t)0xffffffffll);
+                    s_cap[cl] = (uint32_t)min_v(cp, (int64_t)0xffffffffll);
                     s_tscale[cl] = dc.class_wdiv[cl] * kp.granule;
                 }
                 // 16-bit credits need capacities below 2^16 granules, hot columns capacities below 2^22 (four credits and
                 // a tag share 32 bits); the 32-bit table needs fewer than 2^32 granules in all
-                const bool fits = kp.granule >= 256 && t / kp.granule < ((int64_t)1 << 32);
-                s_mode = !fits ? 0 : (cap_max / kp.granule < big_floor ? 1 : (cap_max / kp.granule < ((int64_t)1 << 22) ? 2 : 0));
-                s_tau = tq; s_left = t / kp.granule;
+                s_left = t < ((int64_t)1 << 52) ? by_granule.div(t, rem) : t / kp.granule;
+                const bool fits = kp.granule >= 256 && s_left < ((int64_t)1 << 32);
+                s_mode = !fits ? 0 : (cap_max < big_floor ? 1 : (cap_max < ((int64_t)1 << 22) ? 2 : 0));
+                s_tau = tq;
             }
             __syncthreads();
             tau = s_tau;
             if (s_mode == 2) {                               // hot columns: those with a cell of 65,535 granules or more
                 for (int j = tid; j < N; j += NT)
-                    if (colmax[j] / kp.granule >= 65535) {
+                    if (coltop[j] >= (uint32_t)min_v(65535 * kp.granule >> 8, (int64_t)0xffffffffll)) {   // (multiples of a granule of 256 or more)
                         const int at = atomicAdd(&s_nhot, 1);
                         if (at < BIG_HOT_MAX) colmap[j] = (uint8_t)at;
                     }
@@ -671,7 +720,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             for (unsigned e = tid; e < chunk / 16; e += NT) {
                 const int i2 = (int)(e % (unsigned)(N / 2));
                 ((longlong2*)(buf + 2 * chunk))[e] = ((const longlong2*)rowsum)[i2];
-                ((longlong2*)(buf + 3 * chunk))[e] = ((const longlong2*)colsum)[i2];
+                ((longlong2*)(buf + 3 * chunk))[e] = make_longlong2(col_sum(2 * i2), col_sum(2 * i2 + 1));
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
@@ -684,37 +733,57 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                     int n2 = n + delta; if (n2 >= P) n2 -= P;
                     s += Dhat[(size_t)(n * S + q) * G + n2 * S + q2];
                 }
-                tbl[e] = (uint32_t)(s / kp.granule);
+                tbl[e] = (uint32_t)__double2ll_rn((double)s * inv_granule);      // (a multiple)
             }
             __syncthreads();
             // ---- pass 2 over D: the residual in granules as 16-bit cells (big cells through the side list)
             const bool hot_mode = s_mode == 2;
-            const int gshift = gmask >= 0 ? 63 - __clzll(kp.granule) : -1;
             uint16_t* const cells = (uint16_t*)wd;
+            // a warp per pair of rows (a word of the matrix per column), 8 or 16 loads in flight
+            constexpr int PU = CW >= 4 ? 1 : 4 / CW;
 #pragma unroll 1
-            for (int e0 = tid; e0 < N * N; e0 += 4 * NT) {       // four loads in flight per thread
-                int64_t raw[4];
+            for (int p0 = warp; p0 < N / 2; p0 += PU * n_warps) {
+                int64_t raw[PU][2][CW];
 #pragma unroll
-                for (int u = 0; u < 4; u++) raw[u] = e0 + u * NT < N * N ? D[e0 + u * NT] : 0;
-#pragma unroll 1
-                for (int u = 0; u < 4; u++) {
-                    const int e = e0 + u * NT;
-                    if (e >= N * N) break;
-                    const uint32_t v = gshift >= 0 ? (uint32_t)(raw[u] >> gshift) : big_div_granule(raw[u], kp.granule);
-                    const int i = e / N, j = e - i * N;
-                    uint32_t code = v;
-                    if (!hot_mode) {
-                        if (v >= (uint32_t)big_floor) {          // a big cell: exact value in the side list, its index in the matrix
-                            const int at = atomicAdd(&s_nbig, 1);
-                            code = (uint32_t)big_floor + (uint32_t)min_v(at, big_max - 1);
-                            if (at < big_max) side[at] = v;
-                        }
-                    } else if (colmap[j] != BIG_HOT_MAX) {       // exact: 32 bits in a hot column, below 65,535 elsewhere
-                        Hi[(int)colmap[j] * N + i] = (uint16_t)(v >> 16);
-                        if (EXACT && v >> 16) { atomicAdd(&s_beyond[colmap[j]], 1); atomicAdd(&s_hot, 1); }
+                for (int u = 0; u < PU; u++)
+#pragma unroll
+                    for (int m = 0; m < CW; m++) {
+                        const int p = p0 + u * n_warps, j = m * 32 + lane;
+                        const bool in = p < N / 2 && j < N;
+                        raw[u][0][m] = in ? D[2 * p * N + j] : 0;
+                        raw[u][1][m] = in ? D[(2 * p + 1) * N + j] : 0;
                     }
-                    cells[((i >> 1) * ST + j) * 2 + (i & 1)] = (uint16_t)code;
-                }
+#pragma unroll
+                for (int u = 0; u < PU; u++)
+#pragma unroll
+                    for (int m = 0; m < CW; m++) {
+                        const int p = p0 + u * n_warps, j = m * 32 + lane;
+                        if (p >= N / 2 || j >= N) continue;
+                        uint32_t v[2];
+#pragma unroll
+                        for (int r = 0; r < 2; r++) v[r] = (uint32_t)__double2ll_rn((double)raw[u][r][m] * inv_granule);
+                        if (!hot_mode) {
+                            if (rarely(max_v(v[0], v[1]) >= (uint32_t)big_floor)) {
+#pragma unroll 1
+                                for (int r = 0; r < 2; r++) {
+                                    const uint32_t x = r ? v[1] : v[0];
+                                    if (x < (uint32_t)big_floor) continue;   // a big cell: exact value in the side list, its index in the matrix
+                                    const int at = atomicAdd(&s_nbig, 1);
+                                    const uint32_t code = (uint32_t)big_floor + (uint32_t)min_v(at, big_max - 1);
+                                    if (at < big_max) side[at] = x;
+                                    if (r) v[1] = code; else v[0] = code;
+                                }
+                            }
+                        } else if (colmap[j] != BIG_HOT_MAX) {   // exact: 32 bits in a hot column, below 65,535 elsewhere
+#pragma unroll 1
+                            for (int r = 0; r < 2; r++) {
+                                const uint32_t high = (r ? v[1] : v[0]) >> 16;
+                                Hi[(int)colmap[j] * N + 2 * p + r] = (uint16_t)high;
+                                if (EXACT && high) { atomicAdd(&s_beyond[colmap[j]], 1); atomicAdd(&s_hot, 1); }
+                            }
+                        }
+                        wd[p * ST + j] = __byte_perm(v[0], v[1], 0x5410);
+                    }
             }
             __syncthreads();
             if (s_nbig > big_max) {                          // more big cells than the side list holds: the general kernel's
@@ -1196,9 +1265,11 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
             big_fill_bytes((unsigned char*)lane_inst_b, lo * 2, hi * 2, 0xff, tid, NT);
             big_fill_bytes((unsigned char*)lane_bytes_b, lo * 8, hi * 8, 0x00, tid, NT);
             if (off_aligned) {                                   // N is a multiple of four: rows are whole 16-byte pairs
-                const int half = N / 2;
+                const int half = N / 2, step = NT % half;
+                int i2 = (int)((unsigned)(lo / 2 + tid) % (unsigned)half) - step;
                 for (size_t e = lo / 2 + tid; e < hi / 2; e += NT) {
-                    const int i2 = (int)(e % half);
+                    i2 += step;
+                    if (i2 >= half) i2 -= half;
                     ((longlong2*)(send_off_b + N))[e] = ((const longlong2*)send_acc)[i2];
                     if (recv_off_b) ((longlong2*)(recv_off_b + N))[e] = ((const longlong2*)recv_acc)[i2];
                 }
