@@ -28,6 +28,9 @@ __device__ __forceinline__ void bulk_load(unsigned dst_smem, const void* src, un
 __device__ __forceinline__ void bulk_store(void* dst, unsigned src_smem, unsigned bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src_smem), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void bulk_prefetch(const void* src, unsigned bytes) {        // into L2
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N_PENDING>
 __device__ __forceinline__ void bulk_wait_read() {

@@ -175,6 +175,12 @@ __device__ __forceinline__ void big_fill_bytes(unsigned char* dst, size_t lo, si
 // (out of line: 64-bit division is long, and granules are powers of two in practice)
 __device__ __noinline__ bool big_not_multiple(int64_t x, int64_t granule) { return x % granule != 0; }
 __device__ __noinline__ int64_t big_wide_ceil_div(int64_t x, int64_t d) { return x / d + (x % d > 0); }
+// Asks for a whole matrix at once (N * N * 8 is a multiple of 16): with 256 ranks the first pass is then 42,000 cycles, where each of its
+// reads waited for DRAM behind the plans that others write 131,000.  (32 KB matrices gain nothing.  In line it cost the loop 2 %.)
+__device__ __noinline__ void big_prefetch(const int64_t* D, int N) {
+    if (threadIdx.x < 32 && ((uintptr_t)D & 15) == 0)
+        for (int at = threadIdx.x * 4096; at < N * N * 8; at += 32 * 4096) bulk_prefetch((const char*)D + at, (unsigned)min(4096, N * N * 8 - at));
+}
 // What is wrong with the entries of rows ga * 4 .. ga * 4 + 3 (out of line: looked for only when something is).  Whole warp.
 __device__ __noinline__ int big_wrong_entries(const int64_t* rows, int N, int ga, int64_t granule) {
     int flags = 0;
@@ -531,6 +537,7 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         cnt.t_mark = clock64();
 #endif
         const int64_t* D = demand + (size_t)b * N * N;
+        if (RECORD) big_prefetch(D, N);
         const size_t lane_base = (size_t)b * kp.k_max * N, off_base = (size_t)b * (kp.k_max + 1) * N;
         int32_t* chan_id_b = chan_id + (size_t)b * kp.k_max;
         int16_t* lane_dst_b = lane_dst + lane_base;
@@ -551,13 +558,13 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
         if (tid == 0) { s_nhot = 0; s_nbig = 0; if (EXACT) s_hot = 0; }
         __syncthreads();
         int flags = 0;
-        // One warp per source group, 32 columns per load, the loads of two to four rows in flight at once and their sums side by side.
+        // One warp per source group, 32 columns per load, four rows in flight at once (one of eight pieces) and their sums side by side.
         // An entry's checks are bits that must not be there: of its value from 2^40 on, of the diagonal, of the difference to the next
         // multiple of the granule (entries are below 2^40, so a product with the reciprocal rounds to the quotient of a multiple).
         // Column sums as two 32-bit atomics, as 64-bit ones are loops.  Row by row, with 64-bit remainders, this and the second
         // pass took 45,000 of 912,000 cycles of a matrix of 64 ranks, 134,000 of 1,600,000 with eight CTAs on the SM.
         constexpr int CW = LANES / SPLIT * 4 / 32;           // 32-column pieces of a row
-        constexpr int RB = CW <= 4 ? 4 : 2;
+        constexpr int RB = CW <= 4 ? 4 : 1;                  // (256 ranks: with two rows the loop behind lost 1 % to registers)
         const double inv_granule = kp.inv_granule;
         const auto col_sum = [&](int j) { return ((int64_t)colpart[N + j] << 24) + colpart[j]; };
         for (int ga = warp; ga < G; ga += n_warps) {
@@ -939,9 +946,9 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                         if (fill_lo <= k + 1) {                    // the activations have reached filled rows: those copies must be over
                             bulk_wait_all();
                             asm volatile("fence.proxy.async;" ::: "memory");
-                        } else if (fill_lo - 4 * L.fill_rows >= k + 64) {
-                            fill_block(fill_lo - 4 * L.fill_rows, fill_lo);
-                            fill_lo -= 4 * L.fill_rows;
+                        } else if (fill_lo - 2 * L.fill_rows >= k + 64) {       // (8 rows: with 16 the SMs write 5.9 TB/s in bursts, 512 x 256 ranks 10.57 -> 10.71 ms; with 4 10.8)
+                            fill_block(fill_lo - 2 * L.fill_rows, fill_lo);
+                            fill_lo -= 2 * L.fill_rows;
                         }
                     }
 
