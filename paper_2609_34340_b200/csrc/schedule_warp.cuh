@@ -683,6 +683,9 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
             for (uint32_t e = dc.forced_ptr[lane]; e < dc.forced_ptr[lane + 1]; e++) forced |= 1u << dc.forced_cell[e];
     }
     const bool masks = dc.n_res <= 32;                     // (else the lists are read for every matrix)
+    // reciprocals, while the kernel ahead still runs (worked out behind the wait they and the addresses took 1,400 cycles of a call)
+    const RowDiv granule{kp.granule, kp.inv_granule}, bw_max{dc.bw_max, 1.0 / (double)dc.bw_max}, by_target{(int64_t)kp.k_target, 1.0 / (double)kp.k_target};
+    const RowDiv by_forced{(int64_t)max(forced_bw, 1u), 1.0 / (double)max(forced_bw, 1u)};
     __syncthreads();
     grid_wait();
     WCtx c;
@@ -705,7 +708,6 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
     int64_t* const cap64 = ws<int64_t>(c.o_cap64);
     int64_t* const tscale = ws<int64_t>(c.o_tscale);
     uint32_t* const cap32 = ws<uint32_t>(c.o_cap32);
-    const RowDiv granule{kp.granule, 1.0 / (double)kp.granule}, bw_max{dc.bw_max, 1.0 / (double)dc.bw_max};
     auto ceil_div = [](int64_t x, const RowDiv& by) {      // x below 2^52
         int64_t rem;
         const int64_t q = by.div(x, rem);
@@ -816,7 +818,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
                 if (forced) {
                     int64_t f = 0;
                     for (uint32_t m = forced; m; m &= m - 1) f += Dhat[__ffs((int)m) - 1];
-                    est = max_v(est, ceil_div(f * unit, RowDiv{(int64_t)forced_bw, 1.0 / (double)forced_bw}));
+                    est = max_v(est, ceil_div(f * unit, by_forced));
                 }
             } else {
                 for (int l = lane; l < dc.n_res; l += 32) {
@@ -829,7 +831,7 @@ vp_schedule_warp_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ deman
             }
             est = (int64_t)big_warp_max64((uint64_t)est);
             tot = warp_sum_i64(tot);
-            const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div(est, RowDiv{(int64_t)kp.k_target, 1.0 / (double)kp.k_target}));
+            const int64_t tq = tau_given > 0 ? tau_given : max_v((int64_t)1, ceil_div(est, by_target));
             // capacities in granules, at least one (rate x quantum may exceed what the reciprocal divides exactly)
             int64_t cap_gr = 0;
             if (lane < dc.n_classes) {
