@@ -3,6 +3,7 @@ and in bytes, one and two lanes per rank group, tasks of a part of a warp up to 
 other numbers of starts and sweeps than four and three, plans cut short."""
 import numpy as np
 import pytest
+import torch
 
 import tests.test_gpu_schedule as ts
 from tests.test_gpu_schedule import vp  # noqa: F401  (fixture)
@@ -171,3 +172,31 @@ def test_first_maximum_by_class(vp, oracle_lib, nodes, rails):  # noqa: F811
         w = WParams(granule_bytes=256, k_max=12 * N, **extra).resolved(N)
         got, want, *_ = ts._both(vp, oracle_lib, cat, D, w)
         ts._assert_same(got, want)
+
+
+@pytest.mark.parametrize("granule", [256, 7392, 14336, 999983])
+@pytest.mark.parametrize("nodes", [2, 4, 8, 12, 32])
+def test_set_up_of_a_matrix(vp, oracle_lib, nodes, granule):  # noqa: F811
+    """Entries up to the limit of 2^40 (quotients by a reciprocal; capacities in every mode), one wrong entry of each kind at the edges of
+    a matrix, and demand at addresses that are multiples of eight only."""
+    cat, N = node_template_catalog(tree_topology(nodes)), 8 * nodes
+    rng = np.random.default_rng(nodes * 1000003 + granule)
+    most = ((1 << 40) - 1) // granule
+    D = np.zeros((7, N, N), dtype=np.int64)
+    D[0, 0, N - 1] = D[0, N - 1, 0] = D[0, 1, 6] = most * granule
+    for i, j in rng.integers(0, N, size=(9, 2)):
+        if i != j:
+            D[1, i, j] = int(rng.integers(1, 65536 * 3)) * granule
+    D[2:] = D[1]
+    D[2, N - 1, N - 2] = granule * 5 + 1
+    D[3, 0, N - 1] = 1 << 40
+    D[4, N - 1, N - 1] = granule
+    D[5, N - 1, 0] = -granule
+    D[6, N // 2, 0] = (most - 1) * granule + granule // 2
+    w = WParams(granule_bytes=granule, k_max=6 * N).resolved(N)
+    got, want, _, dc = ts._both(vp, oracle_lib, cat, D, w)
+    ts._assert_same(got, want)
+    assert want["n_steps"][:2].min() > 0 and want["status"].tolist()[2:] == [vp.ST_NOT_GRANULE, vp.ST_OVERFLOW_RISK, vp.ST_DIAG_NONZERO, vp.ST_NEGATIVE, vp.ST_NOT_GRANULE]
+    flat = torch.zeros(D.size + 1, dtype=torch.int64, device="cuda")
+    flat[1:] = torch.from_numpy(D).cuda().view(-1)
+    ts._assert_same(vp.schedule_batch(dc, ts._params(vp, w), flat[1:].view(7, N, N)).cpu(), want)
