@@ -1205,7 +1205,7 @@ int resolve_params(const vp_catalog* c, const vp_sched_params* p, KParams* kp) {
 
 // Works out kernel, launch shape and shared-memory layout for a batch of B matrices.  This sets function attributes
 // and asks the runtime for occupancies, so vp_catalog keeps the last few results (see plan_launch).
-int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, Launch* out) {
+int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, bool host_rows, Launch* out) {
     const DevCat& dc = c->dc;
     Launch L;
     memset(&L, 0, sizeof(L));
@@ -1256,13 +1256,17 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
         // Above 32 groups a CTA has its SM to itself, two warps per task, which emit as well: 3, with the tables staged if they fit and
         // the batch is one wave.
         // Measured on both sides of each line, microseconds for a batch of MoE matrices, last batch in the wave and one more:
-        //   0 | 1:  64 ranks 148: 820 | 838, 149: 1,328 | 838.  Staging gives 1 to 2 % at 40 to 64 ranks and nothing at 24 and 32; with one
-        //           lane per group it was never faster (32 ranks, 741 and 1,184: 535 and 628 staged, 525 and 619 not)
-        //   1 | 2:  64 ranks 296: 890 | 1,053, 297: 1,384 | 1,063;  96 ranks 148: 1,460 | 1,436, 149: 2,480 | 1,509 (17 to 32 groups: two
-        //           lanes are two warps per task, 5 % faster on sequence-parallel matrices, 1 to 6 % slower on MoE ones)
-        //   2 | 3:  64 ranks 297: 1,063 | 1,088, 592: 1,243 | 1,239, 593: 1,781 | 1,272;  96 ranks 296: 1,665 | 1,746, 297: 2,652 | 1,829
-        //   1 | 3 up to 8 groups:  32 ranks 740: 468 | 516, 741: 644 | 512;  1,184 by shape 2: 619, by 3: 534
-        for (int shape = dc.G > 32 ? 3 : 0; shape < 4; shape++) {
+        //   0 | 1:  64 ranks 148: 536 | 549, 149: 859 | 554
+        //   1 | 2:  64 ranks 296: 610 | 719, 297: 930 | 724
+        //   2 | 3:  64 ranks 297: 724 | 712, 400: 764 | 797, 592: 834 | 818, 593: 1,134 | 870;  96 ranks 296: 1,293 | 1,322, 297: 1,985 | 1,379
+        //   1 | 3 up to 8 groups:  32 ranks 740: 320 | 357, 741: 442 | 358;  1,184 by shape 2: 461, by 3: 367
+        // With 17 to 32 groups two lanes per group are two warps per task, which only the exact credits of hot columns are worth: 128 ranks,
+        // half sequence parallel and half MoE in granules of 256 B, 148 matrices 2,617 by 1 and 2,856 by 2; without them 2 is faster
+        // at every batch size (MoE, 16 matrices of 72, 96 and 128 ranks 749 | 823, 1,057 | 1,157, 1,501 | 1,650; 148 of 96 1,100 | 1,206).
+        // Capacities of 2^16 granules come with small granules, so granules of 4 KB and more (rows) start at 2,
+        // but not for plans in host memory, whose rows only 0 and 1 write in order (96 ranks, 128 matrices: 3,504 | 3,595).
+        const bool two_warps = L.kp.granule < 4096 || dc.G <= 16 || host_rows;
+        for (int shape = dc.G > 32 ? 3 : (two_warps ? 0 : 2); shape < 4; shape++) {
             if (shape == 2 && dc.G <= 8) continue;
             const int split = shape < 2 ? 2 : 1;
             const bool apart = shape < 3;                        // warps of their own for the emit step
@@ -1297,13 +1301,14 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
     // in 32-bit granule units (granule >= 256 bytes; the choice between units and bytes is made per matrix, so the
     // granule decides here); with smaller granules when the batch exceeds the CTAs of one wave (16 ranks, granule 64, CTA | warp
     // per matrix: 296 matrices 224 | 234 us, 592 275 | 232, 593 362 | 257: between two and four matrices per SM a warp is already
-    // the faster one).  Up to four matrices per SM get a CTA of one warp each (a scheduler to themselves: 64 matrices of 16 ranks
-    // 114.8 us, in pairs 117.6; 592 and 593 the same), larger batches two warps per CTA and beyond eight per SM four, which
-    // measure the same (1,185 matrices 134 and 136 us; CTAs of one warp 189: an SM holds eight of them).
+    // the faster one).  A CTA is one
+    // warp up to four matrices per SM (a scheduler to themselves; 592 matrices of 16 ranks, one warp | two: 82.9 | 83.0), two warps up to six
+    // (600: 87.5 | 84.4, 888: 91.0 | 91.2), one again up to eight, which is what an SM holds of them (pairs share schedulers unevenly then;
+    // 1,036: 91.7 | 102.8, 1,184: 92.6 | 102.7), and four beyond (1,185: one 142.9, two 102.9, four 102.7).
     if (dc.g == 4 && dc.G <= 4 && !dc.sym && (B > cap || p->granule_bytes >= 256)) {
         const bool units = p->granule_bytes >= 256;
         const WarpKernelFn wf = pick_warp_kernel(dc, units);
-        const int warps = B <= 4 * c->sm_count ? 1 : (B <= 8 * c->sm_count ? 2 : 4);
+        const int warps = B > 8 * c->sm_count ? 4 : (B > 4 * c->sm_count && B <= 6 * c->sm_count ? 2 : 1);
         const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
         if (smem <= (size_t)dynamic_smem_limit(c->max_smem_optin)) {
             if (set_dynamic_smem_limit((const void*)wf, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
@@ -1325,22 +1330,22 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, L
 // plan_launch_uncached through the catalog's memo of the last four launches, by batch size and parameters.  A hit saves what the
 // attributes and occupancies cost: 0.5 us of host time, 1.6 at the most.  The memo is not locked: calls that share a catalog
 // handle from several host threads must be serialised by the caller (as must anything else that shares a workspace).
-int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* out) {
+int plan_launch(const vp_catalog* cc, int B, const vp_sched_params* p, Launch* out, bool host_rows = false) {
     vp_catalog* c = const_cast<vp_catalog*>(cc);
     if (!c || !p) return VP_E_BAD_ARG;
     for (vp_launch_memo& m : c->memo) {
-        if (!m.valid || m.B != B || m.k_target != p->k_target || m.n_start != p->n_start || m.i_aa != p->i_aa ||
+        if (!m.valid || m.B != B || m.host_rows != host_rows || m.k_target != p->k_target || m.n_start != p->n_start || m.i_aa != p->i_aa ||
             m.k_max != p->k_max || m.lambda_ns != p->lambda_ns || m.granule != p->granule_bytes)
             continue;
         memcpy(out, m.launch, sizeof(Launch));
         return VP_OK;
     }
     Launch L;
-    const int rc = plan_launch_uncached(c, B, p, &L);
+    const int rc = plan_launch_uncached(c, B, p, host_rows, &L);
     if (rc) return rc;
     vp_launch_memo& m = c->memo[c->memo_next];
     c->memo_next = (c->memo_next + 1) % (int)(sizeof(c->memo) / sizeof(c->memo[0]));
-    m.valid = 1; m.B = B;
+    m.valid = 1; m.B = B; m.host_rows = host_rows;
     m.k_target = p->k_target; m.n_start = p->n_start; m.i_aa = p->i_aa; m.k_max = p->k_max;
     m.lambda_ns = p->lambda_ns; m.granule = p->granule_bytes;
     memcpy(m.launch, &L, sizeof(Launch));
@@ -1392,7 +1397,7 @@ int vp_schedule_launch(const vp_catalog* c, const vp_sched_params* p, const int6
     cudaGetDevice(&prev);
     if (prev != c->device && cudaSetDevice(c->device) != cudaSuccess) return VP_E_CUDA;
     Launch L;
-    int rc = plan_launch(c, B, p, &L);
+    int rc = plan_launch(c, B, p, &L, host_rows);     // (which of the two does not change the workspace)
     L.kp.host_rows = host_rows;
     if (!rc && (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes_given < workspace_bytes(c, L, B))) rc = VP_E_WORKSPACE;
     if (!rc) {

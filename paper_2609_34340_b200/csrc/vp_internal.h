@@ -82,6 +82,7 @@ struct DevCat {
 
 // A launch shape worked out once per (catalog, batch size, parameters) and reused by later calls.
 struct vp_launch_memo {
+    bool host_rows;
     int valid;
     int B;
     int32_t k_target, n_start, i_aa, k_max;
