@@ -424,7 +424,10 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
                 for (int cl = 0; cl < n && by_lane; cl++) {
                     for (size_t place = 0; place < lists[cl].size(); place++) {
                         const size_t at = std::find(second.begin(), second.end(), lists[cl][place]) - second.begin();
-                        lane_rows[4 * (32 + at) + 3] |= 1u << cl | (uint32_t)place << (5 + 5 * cl);
+                        uint32_t& word = lane_rows[4 * (32 + at) + 3];
+                        if (word >> cl & 1u) continue;         // (a shape that the catalog repeats: the first of equal ones is chosen)
+                        by_lane = by_lane && place < 32;       // (a list with repeats may be longer than the rows are many)
+                        word |= 1u << cl | (uint32_t)place << (5 + 5 * cl);
                     }
                 }
                 if (by_lane && !rc) rc = upload(c, lane_rows, &dc.lane_rows);

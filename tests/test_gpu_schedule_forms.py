@@ -8,7 +8,7 @@ import torch
 import tests.test_gpu_schedule as ts
 from tests.test_gpu_schedule import vp  # noqa: F401  (fixture)
 from workloads import SchedParams as WParams, complete_catalog, node_template_catalog, tree_topology
-from workloads.topology import _assemble, ring_topology
+from workloads.topology import Catalog, _assemble, ring_topology
 
 pytestmark = pytest.mark.gpu
 
@@ -172,6 +172,47 @@ def test_first_maximum_by_class(vp, oracle_lib, nodes, rails):  # noqa: F811
         w = WParams(granule_bytes=256, k_max=12 * N, **extra).resolved(N)
         got, want, *_ = ts._both(vp, oracle_lib, cat, D, w)
         ts._assert_same(got, want)
+
+
+def _repeated(cat, shapes):
+    """The catalog with each of `shapes` followed by copies of itself: (shape, copies)."""
+    order = [s for s in range(cat.n_shapes) for _ in range(1 + dict(shapes).get(s, 0))]
+    return Catalog(cat.topology, [cat.shapes[s] for s in order], [cat.buckets[s] for s in order])
+
+
+def _second_rows(cat):
+    """Per run of shapes that share their first row: the shapes."""
+    def first(shape):
+        return tuple((d, c) for a, d, c in shape if a == 0)
+    runs = {}
+    for s, shape in enumerate(cat.shapes):
+        runs.setdefault(first(shape), []).append(s)
+    return list(runs.values())
+
+
+@pytest.mark.parametrize("nodes,rails", [(2, 2), (4, 2), (8, 2), (9, 2), (5, 1)])
+@pytest.mark.parametrize("where", ["one", "every", "ends", "long"])
+def test_repeated_shapes(vp, oracle_lib, nodes, rails, where):  # noqa: F811
+    """A catalog may hold a shape more than once: the first of the equal ones is chosen.  One repeated shape, all of them, the last of
+    every list of second rows, and lists of more than 32 entries by repeats alone."""
+    cat = node_template_catalog(tree_topology(nodes)) if rails == 2 else _one_rail(nodes)
+    runs = _second_rows(cat)
+    again = {"one": {cat.n_shapes // 2: 1}, "every": {s: 1 for s in range(cat.n_shapes)}, "ends": {r[-1]: 2 for r in runs},
+             "long": {s: 35 for r in runs for s in r[:1]}}[where]
+    cat = _repeated(cat, again)
+    N = cat.topology.N
+    rng = np.random.default_rng(100 * nodes + rails)
+    D = (rng.integers(0, 900, size=(5, N, N)) * (rng.random((5, N, N)) < 0.3)).astype(np.int64)
+    D[1] = 1000
+    D[2] = 0
+    D[2][1, N - 2] = 77
+    D[3] = rng.integers(0, 3, size=(N, N))
+    D *= 256
+    for b in range(5):
+        np.fill_diagonal(D[b], 0)
+    got, want, *_ = ts._both(vp, oracle_lib, cat, D, WParams(granule_bytes=256, k_max=12 * N).resolved(N))
+    assert (want["status"] == 0).all()
+    ts._assert_same(got, want)
 
 
 @pytest.mark.parametrize("granule", [256, 7392, 14336, 999983])
