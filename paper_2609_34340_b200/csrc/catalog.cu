@@ -401,7 +401,14 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
                     dc.dec_words = (int)dec.size();
                     dc.dec_chunks = (int)n_chunks;
                     dc.dec_stride = stride;
-                    c->dec_host = dec;
+                    if (S == 2) {                                          // what a caller is shown: two rails, entries without padding terms
+                        c->dec_host.assign(dec.begin(), dec.begin() + kHeader);
+                        c->dec_host[1] = (uint32_t)max_row + 1;
+                        for (size_t at = kHeader; at < dec.size(); at += stride) {
+                            c->dec_host.insert(c->dec_host.end(), dec.begin() + at, dec.begin() + at + max_row);
+                            c->dec_host.push_back(dec[at + stride - 1]);
+                        }
+                    }
                     rc = upload(c, dec, &dc.dec);
                 }
                 // a row per lane (see DevCat::lane_rows)
@@ -499,7 +506,7 @@ extern "C" int vp_load_catalog(const void* topology, size_t topo_bytes, const vo
     I.N = N; I.G = G; I.g = g; I.groups_per_node = S; I.n_resources = n_res; I.n_instances = n_inst;
     I.n_shapes = n_shapes; I.n_families = n_fam; I.max_nnz = max_nnz; I.max_bucket = max_bucket;
     I.covered = covered; I.node_symmetric = sym; I.rate_lcm = W;
-    I.row_patterns = dc.n_patterns; I.argmax_classes = dc.dec_classes;
+    I.row_patterns = dc.n_patterns; I.argmax_classes = S == 2 ? dc.dec_classes : 0;
     if (prev >= 0) cudaSetDevice(prev);
     *out = c;
     return VP_OK;

@@ -121,7 +121,7 @@ struct vp_catalog {
     int max_smem_optin;
     vp_launch_memo memo[4];
     int memo_next;
-    std::vector<uint32_t> dec_host;   // host copy of DevCat::dec (vp_catalog_argmax_classes)
+    std::vector<uint32_t> dec_host;   // DevCat::dec of two rails as vp_catalog_argmax_classes returns it
     // the host-buffer scheduler call's own copy stream and events (created on first use, see host_api.cu)
     cudaStream_t copy_stream;
     cudaEvent_t host_ev[4];

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 from workloads import complete_catalog, crossbar_catalog, crossbar_topology, node_template_catalog, tree_topology
+from workloads.topology import _assemble
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -186,6 +187,25 @@ def test_argmax_classes_reproduce_every_shape(nodes, nic_bw):
                 assert rows_of_shape[run_start + place] == (p0, p1), (cl, run_start, place)
                 seen[run_start + place] += 1
     assert (seen == 1).all()
+
+
+def test_argmax_classes_of_one_rail_and_of_short_rows():
+    """The public figure concerns two rails: a catalog of one rail reports none, whatever the scheduler makes of it.  An entry has as many
+    terms as the longest row, and its tie-break word."""
+    import paper_2609_34340_b200 as vp
+    topo = tree_topology(4, switches_per_node=1)
+    by_key = {(r.src_group, r.dst_group): i for i, r in enumerate(topo.instances)}
+    one = _assemble(topo, [tuple(sorted(x for a in range(4) for x in [by_key[a, a]] * (3 if d else 4) + ([by_key[a, (a + d) % 4]] if d else [])))
+                           for d in range(4)])
+    dc = vp.load_catalog(one.topology.blob(), one.blob(), device=-1)
+    assert dc.node_symmetric == 1 and dc.argmax_classes == 0 and len(vp.catalog_argmax_classes(dc)) == 0
+    full = node_template_catalog(tree_topology(3))
+    keep = [s for s in range(full.n_shapes) if all(sum(a == g for a, _, _ in full.shapes[s]) <= 2 for g in range(full.topology.G))]
+    short = type(full)(full.topology, [full.shapes[s] for s in keep], [full.buckets[s] for s in keep])
+    for cat, terms in ((full, 3), (short, 2)):
+        dc = vp.load_catalog(cat.topology.blob(), cat.blob(), device=-1)
+        d = vp.catalog_argmax_classes(dc)
+        assert dc.argmax_classes > 0 and int(d[1]) == terms + 1 and len(d) == int(d[2]) + 32 * int(d[0]) * (terms + 1)
 
 
 def test_extension_is_built_again_for_another_torch_or_python(monkeypatch, tmp_path):
