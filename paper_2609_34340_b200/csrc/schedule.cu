@@ -1303,14 +1303,17 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, b
     // per matrix: 296 matrices 224 | 234 us, 592 275 | 232, 593 362 | 257: between two and four matrices per SM a warp is already
     // the faster one).  A CTA is one
     // warp up to four matrices per SM (a scheduler to themselves; 592 matrices of 16 ranks, one warp | two: 82.9 | 83.0), two warps up to six
-    // (600: 87.5 | 84.4, 888: 91.0 | 91.2), one again up to eight, which is what an SM holds of them (pairs share schedulers unevenly then;
-    // 1,036: 91.7 | 102.8, 1,184: 92.6 | 102.7), and four beyond (1,185: one 142.9, two 102.9, four 102.7).
+    // (600: 87.5 | 84.4, 888: 91.0 | 91.2), one again up to eight (pairs share schedulers unevenly then; 1,036: 91.7 | 102.8, 1,184:
+    // 92.6 | 102.7), and four beyond (1,185: one 142.9, two 102.9, four 102.7).  CTAs of more warps, which share the catalog's tables, are
+    // taken where one wave of fewer does not hold the batch (a ring of three switches, 468 families, an SM holds four CTAs of one warp and
+    // three of two: 900 matrices by one 135.5, two 120.9, four 93.0; 1,184 145.8, 141.5, 93.1).
     if (dc.g == 4 && dc.G <= 4 && !dc.sym && (B > cap || p->granule_bytes >= 256)) {
         const bool units = p->granule_bytes >= 256;
         const WarpKernelFn wf = pick_warp_kernel(dc, units);
-        const int warps = B > 8 * c->sm_count ? 4 : (B > 4 * c->sm_count && B <= 6 * c->sm_count ? 2 : 1);
-        const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
-        if (smem <= (size_t)dynamic_smem_limit(c->max_smem_optin)) {
+        const int first = B > 8 * c->sm_count ? 4 : (B > 4 * c->sm_count && B <= 6 * c->sm_count ? 2 : 1);
+        for (int warps = first; warps <= 4; warps *= 2) {
+            const size_t smem = (size_t)warp_smem_layout(dc, L.kp, warps, units).total;
+            if (smem > (size_t)dynamic_smem_limit(c->max_smem_optin)) break;
             if (set_dynamic_smem_limit((const void*)wf, c->max_smem_optin) != VP_OK) return VP_E_CUDA;
             int wper_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper_sm, wf, warps * 32, smem) != cudaSuccess || wper_sm < 1)
@@ -1320,6 +1323,7 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, b
             L.kp.drem_in_smem = 1; L.kp.stage_terms = L.kp.stage_fam = L.kp.stage_bucket = 1;
             L.grid = (int)(want < wcap ? want : wcap);
             L.wave = (int)wcap * warps;
+            if (wcap >= want) break;
         }
     }
 #endif

@@ -142,6 +142,21 @@ def test_launch_shapes_of_node_symmetric_catalogs(vp, oracle_lib, name, batches)
     test_work_counters_and_batches(vp, oracle_lib, name, batches)
 
 
+@pytest.mark.parametrize("name,warps", [("two_nodes_64_50", 1), ("ring_of_three", 4)])
+def test_warps_per_cta_by_what_an_sm_holds(vp, oracle_lib, name, warps):  # noqa: F811
+    """Six to eight matrices per SM: a warp per CTA where an SM holds as many of them, else CTAs of more warps, which share the tables (52
+    KB with the 468 families of a ring of three switches); a wave holds the batch either way."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cat = CATALOGS[name]()
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob())
+    p = ts._params(vp, WParams(granule_bytes=4096).resolved(cat.topology.N))
+    for B in (6 * sms + 1, 8 * sms):
+        info = vp.schedule_launch_info(dc, B, p)
+        assert info["threads"] == 32 * warps and info["ctas"] == (B + warps - 1) // warps
+    assert vp.schedule_launch_info(dc, 6 * sms, p)["threads"] == 64
+    test_work_counters_and_batches(vp, oracle_lib, name, (7 * sms,))
+
+
 def _one_rail(nodes):
     """One switch per node: every rank group keeps its four lanes, or sends one to the group `delta` further on."""
     topo = tree_topology(nodes, switches_per_node=1)
