@@ -21,9 +21,11 @@ on the host cores instead (rank 0 only).
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -276,11 +278,21 @@ def time_sched_config(vp, torch, idx, dev, local_rank, flush, peaks_now, counter
     return out
 
 
+def scheduler_code_id() -> str:
+    """What the scheduler's counters were captured of: a hash of its kernels' sources without comments and white space."""
+    h = hashlib.sha256()
+    for name in ("schedule.cu", "schedule_big.cuh", "schedule_warp.cuh"):
+        with open(os.path.join(ROOT, "paper_2609_34340_b200", "csrc", name)) as f:
+            h.update("".join(re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S).split()).encode())
+    return h.hexdigest()[:16]
+
+
 def issue_fraction(counters: dict, key: str, activations: int, ms: float, sm_mhz) -> dict:
     """Issue-slot and shared-memory-pipe use from the warp instructions / wavefronts per activation that an ncu
-    capture of the same kernel and config recorded (profiles/ncu_counters.json), over this run's time and clock."""
+    capture of the same kernel and config recorded (profiles/ncu_counters.json), over this run's time and clock.
+    Null when the capture is of other code than this."""
     c = (counters.get("scheduler") or {}).get(key)
-    if not c or not sm_mhz:
+    if not c or not sm_mhz or c.get("code") != scheduler_code_id():
         return {"issue_slot_frac": None, "shared_wavefront_frac": None}
     cycles = ms * 1e-3 * sm_mhz * 1e6
     inst = c["warp_inst_per_activation"] * activations

@@ -75,3 +75,12 @@ def test_exchange_tables_over_two_gloo_ranks():
     for rc, out, err in res:
         assert rc == 0, err
         assert json.loads(out.strip().splitlines()[-1]) == [[0x1000, 0x2000], [0x2008, 0x4008], [4096 * 3, 4096 * 4]]
+
+
+def test_issue_fraction_is_null_for_counters_of_other_code():
+    import bench
+    one = {"warp_inst_per_activation": 1000.0, "shared_wavefronts_per_activation": 100.0, "commit": "x"}
+    of = lambda code: bench.issue_fraction({"scheduler": {"config3": dict(one, code=code)}}, "config3", 1_000_000, 1.0, 1965)  # noqa: E731
+    assert of(bench.scheduler_code_id())["issue_slot_frac"] == round(1e9 / (1965e3 * bench.SM_COUNT * bench.SCHEDULERS_PER_SM), 4)
+    assert of("0" * 16)["issue_slot_frac"] is None
+    assert bench.issue_fraction({"scheduler": {"config3": one}}, "config3", 1_000_000, 1.0, 1965)["shared_wavefront_frac"] is None
