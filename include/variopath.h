@@ -61,6 +61,8 @@ extern "C" {
  * bounded wait for an asynchronous copy into shared memory gave up (2^22 polls; never seen in practice).  The kernel
  * then issues no further loads, lets the stores it already issued finish and returns; the output buffer is INCOMPLETE
  * and the call must be repeated (vp_exchange_put: what the CTA that gave up has stored is not counted in arrived).
+ * The single launch of small pack, unpack and return calls moves what is left by plain loads instead: its output is
+ * complete, with the bit or without it (which the CTA that writes the status may overwrite there).
  * Nothing faults and the context stays usable. */
 #define VP_ST_INTERNAL_TIMEOUT (1 << 30)
 /* Bits 1..16 reject the matrix before scheduling: n_steps[b] = 0 and an empty plan. */

@@ -20,7 +20,7 @@ ST_NEGATIVE, ST_OVERFLOW_RISK, ST_DIAG_NONZERO, ST_NOT_GRANULE = 1, 2, 4, 8
 ST_BAD_TAU, ST_UNCOVERED, ST_NO_PROGRESS, ST_STEP_LIMIT = 16, 32, 64, 128
 ST_PACK_MISMATCH, ST_PACK_CAPACITY = 256, 512
 ST_EXCHANGE_TIMEOUT = 2048
-ST_INTERNAL_TIMEOUT = 1 << 30    # a row-copy kernel gave up a bounded wait: the output buffer is incomplete
+ST_INTERNAL_TIMEOUT = 1 << 30    # a bounded wait for a row copy gave up: the output may be incomplete
 
 
 class VpError(RuntimeError):

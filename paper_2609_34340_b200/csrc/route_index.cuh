@@ -476,7 +476,8 @@ struct SmallLaunch {
     bool bulk;
 };
 
-struct OwnRing {
+template <unsigned SPINS>
+struct OwnRingOf {
     const char* rows;
     char* out;
     long long row_bytes;
@@ -519,7 +520,7 @@ struct OwnRing {
     __device__ __forceinline__ bool drain() {
         bool ok = true;
         for (int s = 0; s < kOwnStages; s++)
-            if (loaded >> s & 1) ok &= mbar_wait_bounded(bars + 8 * s, phase >> s & 1u, kOwnSpins);
+            if (loaded >> s & 1) ok &= mbar_wait_bounded(bars + 8 * s, phase >> s & 1u, SPINS);
         loaded = 0;
         return ok;
     }
@@ -531,17 +532,36 @@ struct OwnRing {
         const bool mine = lane < min(units, kOwnStages) && issue(lane, src);
         loaded = __ballot_sync(0xffffffffu, mine);
     }
-    // Stores every unit to its destination rows dst[i * fanout + f] (-1: none) and loads the others; false: a wait gave up.
+    // Unit u by plain loads and stores, the whole warp.
+    template <typename Src>
+    __device__ __forceinline__ void move_plain(int u, int fanout, const int* dst, Src src) const {
+        const Unit n = unit(u);
+        const int from = src(n.row), vecs = min(piece, cols - n.at) / 16;
+        if (from < 0) return;
+        const uint4* const x = (const uint4*)(rows + from * row_bytes + col0 + n.at);
+#pragma unroll 1
+        for (int f = 0; f < fanout; f++) {
+            const int d = dst[n.row * fanout + f];
+            if (d < 0) continue;
+            uint4* const to = (uint4*)(out + d * row_bytes + col0 + n.at);
+#pragma unroll 1
+            for (int v = threadIdx.x & 31; v < vecs; v += 32) to[v] = x[v];
+        }
+    }
+    // Stores every unit to its destination rows dst[i * fanout + f] (-1: none) and loads the others; false: a wait gave up.  All units
+    // are stored either way, those that are left then by plain loads: the caller reports it by a bit in the status word, which another CTA
+    // writes by a plain store, so the bit may be lost, and no output may depend on it.
     template <typename Src>
     __device__ __forceinline__ bool finish(int fanout, const int* dst, Src src) {
         constexpr int S = kOwnStages, D = S / 2;    // a stage is loaded again D units after its stores
         const int lane = threadIdx.x & 31;
         bool failed = false;
-        for (int u = 0; u < units; u++) {
+        int u = 0;
+        for (; u < units; u++) {
             const int s = u % S;
             const Unit n = unit(u);
             if (loaded >> s & 1) {
-                failed = __any_sync(0xffffffffu, !mbar_wait_bounded(bars + 8 * s, phase >> s & 1u, kOwnSpins));
+                failed = __any_sync(0xffffffffu, !mbar_wait_bounded(bars + 8 * s, phase >> s & 1u, SPINS));
                 if (failed) break;
                 loaded &= ~(1u << s);
                 phase ^= 1u << s;
@@ -560,11 +580,16 @@ struct OwnRing {
                 if (__any_sync(0xffffffffu, mine)) loaded |= 1u << (u + S - D) % S;
             }
         }
-        drain();                                    // (nothing is in flight unless a wait gave up)
+        if (__builtin_expect(failed, 0)) {          // (no load is in flight otherwise)
+#pragma unroll 1
+            for (; u < units; u++) move_plain(u, fanout, dst, src);
+            drain();
+        }
         bulk_wait_read<0>();                        // the stores have read shared memory
         return !failed;
     }
 };
+using OwnRing = OwnRingOf<kOwnSpins>;
 
 // Copies of `width` bytes; ints(own) words of index in shared memory when a CTA owns up to `own` of the n rows.  With rings one CTA
 // per SM, as a CTA's index costs the same however many rows it owns; by plain loads two, for the loads in flight.  While there are

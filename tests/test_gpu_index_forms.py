@@ -1,6 +1,10 @@
 """GPU parity of the pack and both unpack directions where their index work changes form: one self-contained launch up to
 16,384 items (return: 12,288) and 1,024 plan rows, chunked histograms beyond; the plan's senders read in place or resolved by a kernel of
 their own; fewer rows than SMs (a row split over CTAs) and more; every copy width."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -13,6 +17,7 @@ from workloads.configs import catalog_for
 from workloads.demand import demand_from_routing, moe_routing
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _case(nodes, tokens, topk, row_bytes, k_max=0, seed=0):
@@ -208,3 +213,41 @@ def test_demand_of_more_copies_than_32_bits_count(vp, large):  # noqa: F811
     idx[0, 7, :3], idx[0, -1, 0] = 1, -1                       # three copies to the source itself, one dropped
     got, st = vp.demand_from_routing(idx, 1, 2, 3, src0=1)
     assert int(st.item()) == 0 and got.tolist() == [[3 * (2 ** 32 + 8 - 4), 0]]
+
+
+@pytest.fixture(scope="module")
+def ring(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("ring") / "libring.so")
+    subprocess.check_call(["/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
+                           "-shared", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2609_34340_b200", "csrc"),
+                           os.path.join(ROOT, "tests", "own_ring_wait.cu"), "-o", out], timeout=300)
+    fn = ctypes.CDLL(out).run_ring
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
+                   ctypes.c_int, ctypes.c_void_p]
+    return fn
+
+
+@pytest.mark.parametrize("own,fanout,row_bytes", [(1, 1, 2048), (2, 8, 14336), (9, 3, 7392), (13, 1, 33008), (31, 2, 4096)])
+@pytest.mark.parametrize("at", [0, 1, 4, 6])
+def test_rows_are_complete_when_a_wait_gives_up(vp, ring, own, fanout, row_bytes, at):  # noqa: F811
+    """The status bit of a wait that gave up may be overwritten by the CTA that writes the status, so no output may depend on it: what
+    is left is moved by plain loads.  The wait runs out at the first, the second or the fifth stage of the rings, or (six) not at all."""
+    gen = torch.Generator().manual_seed(own * 100 + at)
+    rows = torch.randint(0, 256, (own + 3, row_bytes), dtype=torch.uint8, generator=gen)
+    src = torch.randperm(own + 3, generator=gen)[:own].to(torch.int32)
+    dst = torch.randperm(own * fanout + 5, generator=gen)[:own * fanout].to(torch.int32)
+    dst[torch.rand(own * fanout, generator=gen) < 0.2] = -1
+    if own > 2:
+        src[own // 2] = -1
+    want = torch.zeros(own * fanout + 5, row_bytes, dtype=torch.uint8)
+    for i in range(own):
+        for d in dst[i * fanout:(i + 1) * fanout].tolist():
+            if src[i] >= 0 and d >= 0:
+                want[d] = rows[src[i]]
+    rows_d, src_d, dst_d, gave_up = rows.cuda(), src.cuda(), dst.cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.zeros_like(want, device="cuda")
+    assert ring(rows_d.data_ptr(), out.data_ptr(), row_bytes, own, fanout, src_d.data_ptr(), dst_d.data_ptr(), at, gave_up.data_ptr()) == 0
+    piece = min(row_bytes if own > 1 else row_bytes // 32 * 16, 16384)
+    units = [i for i in range(own) for _ in range(-(-row_bytes // piece))]             # own row of every unit; two warps take turns
+    assert int(gave_up.item()) == sum(any(src[i] >= 0 for i in units[w::2][at:6]) for w in (0, 1))
+    assert torch.equal(out.cpu(), want)
