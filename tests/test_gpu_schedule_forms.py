@@ -1,6 +1,8 @@
 """GPU parity of the scheduler where its kernels change form: one warp per matrix (up to four groups of four) in 32-bit granules
 and in bytes, one and two lanes per rank group, tasks of a part of a warp up to two warps, scores within and beyond 32 bits,
 other numbers of starts and sweeps than four and three, plans cut short."""
+import itertools
+
 import numpy as np
 import pytest
 import torch
@@ -187,6 +189,74 @@ def test_first_maximum_by_class(vp, oracle_lib, nodes, rails):  # noqa: F811
         w = WParams(granule_bytes=256, k_max=12 * N, **extra).resolved(N)
         got, want, *_ = ts._both(vp, oracle_lib, cat, D, w)
         ts._assert_same(got, want)
+
+
+def _reordered(nodes):
+    """The node template catalog with its shapes in another order: a first row has several runs, so there are no classes."""
+    cat = node_template_catalog(tree_topology(nodes))
+    order = np.random.default_rng(nodes).permutation(cat.n_shapes)
+    return Catalog(cat.topology, [cat.shapes[s] for s in order], [cat.buckets[s] for s in order])
+
+
+def _thinned(nodes):
+    """All but five or six of its shapes: the lists of second rows differ, so the classes are many."""
+    cat = node_template_catalog(tree_topology(nodes))
+    keep = [s for s in range(cat.n_shapes) if s % (cat.n_shapes // 5) != 7]
+    return Catalog(cat.topology, [cat.shapes[s] for s in keep], [cat.buckets[s] for s in keep])
+
+
+def _rails(nodes, S):
+    """Three or four switches per node: every rail sends one lane to its own rail `d` nodes further on (a `d` per rail, none if 0), or
+    all rails to the next rail."""
+    topo = tree_topology(nodes, switches_per_node=S)
+    by_key = {(r.src_group, r.dst_group, r.kind): i for i, r in enumerate(topo.instances)}
+
+    def family(to):                                        # to(node, rail) -> the group it sends a lane to
+        fam = []
+        for n in range(nodes):
+            for q in range(S):
+                a, d = n * S + q, to(n, q)
+                fam += [by_key[a, a, 0]] * (4 if d == a else 3) + ([by_key[a, d, 2]] if d != a else [])
+        return tuple(sorted(fam))
+    several = itertools.product(range(nodes), repeat=S) if nodes ** S < 700 else ((d,) * S for d in range(nodes))
+    fams = [family(lambda n, q: (n + ds[q]) % nodes * S + q) for ds in several]
+    fams += [family(lambda n, q: (n + d) % nodes * S + (q + r) % S) for r in range(1, S) for d in range(nodes)]
+    return _assemble(topo, fams)
+
+
+WITHOUT_CLASSES = {
+    "reordered_4": lambda: _reordered(4), "reordered_8": lambda: _reordered(8), "reordered_12": lambda: _reordered(12), "reordered_17": lambda: _reordered(17),
+    "thinned_4": lambda: _thinned(4), "thinned_8": lambda: _thinned(8),
+    "three_rails": lambda: _rails(4, 3), "four_rails": lambda: _rails(5, 4), "three_rails_of_36_groups": lambda: _rails(12, 3),
+}
+
+
+@pytest.mark.parametrize("name", list(WITHOUT_CLASSES))
+def test_first_maximum_without_classes(vp, oracle_lib, name):  # noqa: F811
+    """Catalogs whose first maximum is not taken class by class: two rails in another order or of more classes than a lane's rows
+    allow, three and four rails.  All launch shapes; scores within 32 bits and beyond."""
+    cat = WITHOUT_CLASSES[name]()
+    N = cat.topology.N
+    dc = vp.load_catalog(cat.topology.blob(), cat.blob(), device=0)
+    assert dc.node_symmetric == 1 and (dc.argmax_classes > 5 if "thinned" in name else dc.argmax_classes == 0)
+    w = WParams(granule_bytes=256, k_max=8 * N).resolved(N)
+    assert vp.schedule_launch_info(dc, 4, ts._params(vp, w))["kernel"] == "CTA per matrix, 16-bit credits"
+    rng = np.random.default_rng(N)
+    D = (rng.integers(0, 900, size=(6, N, N)) * (rng.random((6, N, N)) < 0.3)).astype(np.int64)
+    D[1] = 1000
+    D[2] = 0
+    D[2][1, N - 2] = 77
+    D[3] = rng.integers(0, 3, size=(N, N))
+    D[4] *= 1 << 20                                            # scores beyond 32 bits
+    D *= 256
+    for b in range(6):
+        np.fill_diagonal(D[b], 0)
+    got, want, *_ = ts._both(vp, oracle_lib, cat, D, w)
+    ts._assert_same(got, want)
+    for B in (300, 700) if N <= 64 else (300,):                # the other launch shapes
+        plan = vp.schedule_batch(dc, ts._params(vp, w), torch.from_numpy(np.tile(D, (-(-B // 6), 1, 1))[:B].copy()).cuda()).cpu()
+        for r in range(0, B, 6):
+            ts._assert_same({key: plan[key][r:r + 6] for key in ts.KEYS}, {key: want[key][:min(6, B - r)] for key in ts.KEYS})
 
 
 def _repeated(cat, shapes):
