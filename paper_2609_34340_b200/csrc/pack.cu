@@ -288,7 +288,7 @@ extern "C" int vp_pack(const int32_t* n_steps_b, const int16_t* lane_dst_b, cons
     if (!sms) return VP_E_CUDA;
     if (E <= kSmallItems && k_max <= kSmallSteps && row_bytes <= kSmallRow) {
         const int width = copy_width(rows, staged, row_bytes);
-        const SmallLaunch z = small_launch(T, sms, topk, row_bytes, width, [&](int own) { return pack_small_layout(N, k_max, own * topk).ints; });
+        const SmallLaunch z = small_launch(T, sms, topk, row_bytes, width, kMinOwnBulk, [&](int own) { return pack_small_layout(N, k_max, own * topk).ints; });
         if (z.own <= kSmallOwn) {
             const char* from = (const char*)rows;
             vp_prof_mark(2, 0, stream);

@@ -456,7 +456,7 @@ __device__ __forceinline__ void move_rows(const char* __restrict__ rows, char* _
     }
 }
 
-// The same by bulk asynchronous copies (TMA): rows of at least kMinOwnBulk bytes at 16-byte addresses.  A unit is one piece of one
+// The same by bulk asynchronous copies (TMA): rows of at least kMinOwnBulk (return: kMinReturnBulk) bytes at 16-byte addresses.  A unit is one piece of one
 // own row; warp w < kOwnWarps drives every kOwnWarps-th unit through a ring of its own.  Loads need no index where the source rows
 // are known before it (pack, unpack): they are in flight while it is worked out, and what follows it is the stores alone.  (They start
 // behind the loads that the index waits for: ahead of them they keep those waiting, 4 us with six stages full on every SM.)  Pack of
@@ -466,6 +466,10 @@ constexpr int kOwnWarps = 2;
 constexpr int kOwnStages = 6;
 constexpr int kOwnPiece = 16384;                    // bytes per unit, at most
 constexpr int kMinOwnBulk = 2048;
+// The return knows its source rows behind the index only, and two warps issue a unit per row: rows below 7 KB move faster by plain
+// loads (8,192 copies, by rings | plain, us, 16 ranks: rows of 2,048 B 18.3 | 11.1, 4,096 20.7 | 18.0, 6,144 24.3 | 23.5, 7,392 26.8 | 26.8,
+// 8,192 27.9 | 28.4, 14,336 43.8 | 45.4; 64 ranks 20.2 | 13.3, 22.6 | 20.3, 26.3 | 25.9, 28.8 | 29.3, 30.0 | 31.0, 46.9 | 48.5).
+constexpr int kMinReturnBulk = 7168;
 constexpr unsigned kOwnSpins = 1u << 22;            // bounded mbarrier wait
 
 // How a small problem is dealt, and what a one-launch kernel is told about it.
@@ -591,13 +595,13 @@ struct OwnRingOf {
 };
 using OwnRing = OwnRingOf<kOwnSpins>;
 
-// Copies of `width` bytes; ints(own) words of index in shared memory when a CTA owns up to `own` of the n rows.  With rings one CTA
+// Copies of `width` bytes, by rings from rows of min_bulk bytes on; ints(own) words of index in shared memory when a CTA owns up to `own` of the n rows.  With rings one CTA
 // per SM, as a CTA's index costs the same however many rows it owns; by plain loads two, for the loads in flight.  While there are
 // fewer rows than that, up to eight CTAs take a row's columns.
 template <typename Ints>
-inline SmallLaunch small_launch(int n, int sms, int fanout, long long row_bytes, int width, Ints ints) {
+inline SmallLaunch small_launch(int n, int sms, int fanout, long long row_bytes, int width, int min_bulk, Ints ints) {
     SmallLaunch z{};
-    for (int per_sm = width == 16 && row_bytes >= kMinOwnBulk ? 1 : 2; per_sm <= 2; per_sm++) {
+    for (int per_sm = width == 16 && row_bytes >= min_bulk ? 1 : 2; per_sm <= 2; per_sm++) {
         const int most = per_sm * sms;
         z.pieces = n >= sms ? 1 : (most / n < 8 ? most / n : 8);
         z.grid = n >= sms ? (n < most ? n : most) : n * z.pieces;

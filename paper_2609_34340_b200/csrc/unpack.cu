@@ -577,7 +577,7 @@ int unpack_launch(const UnpackArgs& a, const void* recv, void* out, void* worksp
     cudaError_t e = cudaSuccess;
     if (items <= (TOKENS ? kSmallReturn : kSmallItems) && a.k_max <= kSmallSteps && inline_steps && a.row.d <= kSmallRow) {
         const int width = copy_width(recv, out, a.row.d);
-        const SmallLaunch z = small_launch(a.items, sms, 1, a.row.d, width, [&](int own) { return unpack_small_layout(a.N, a.keys, a.k_max, own, TOKENS).ints; });
+        const SmallLaunch z = small_launch(a.items, sms, 1, a.row.d, width, TOKENS ? kMinReturnBulk : kMinOwnBulk, [&](int own) { return unpack_small_layout(a.N, a.keys, a.k_max, own, TOKENS).ints; });
         if (z.own <= kSmallOwn) {
             const char* from = (const char*)recv;
             vp_prof_mark(3, 0, stream);

@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kOwnWarps * 32) ring_kernel(const char* rows, 
 
 // own rows of row_bytes (a multiple of 16, at least 2 KB); src [own], dst [own * fanout]; gave_up: warps whose wait ran out.
 extern "C" int run_ring(const void* rows, void* out, long long row_bytes, int own, int fanout, const int* src, const int* dst, int at, int* gave_up) {
-    SmallLaunch z = small_launch(own, 1, fanout, row_bytes, 16, [](int) { return 0; });
+    SmallLaunch z = small_launch(own, 1, fanout, row_bytes, 16, kMinOwnBulk, [](int) { return 0; });
     if (!z.bulk || z.grid != 1) return -1;
     if (cudaFuncSetAttribute(ring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)z.smem) != cudaSuccess) return -2;
     ring_kernel<<<1, kOwnWarps * 32, z.smem>>>((const char*)rows, (char*)out, row_bytes, own, fanout, src, dst, at, z, gave_up);

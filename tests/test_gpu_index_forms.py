@@ -40,11 +40,12 @@ def _case(nodes, tokens, topk, row_bytes, k_max=0, seed=0):
 
 # (nodes, tokens, topk, row bytes, k_max): one CTA per token; a token over several CTAs; exactly the limit of the one-launch
 # form and one token more; long plans (k_max above 1,024, above what a count CTA reads itself); 64, 128 and 256 ranks; rows that
-# are multiples of 16, 4 and 1 bytes on both sides of 2 KB, and rows of more than one 16 KB piece
+# are multiples of 16, 4 and 1 bytes on both sides of 2 KB, rows of more than one 16 KB piece, and (return) both sides of 7 KB
 CASES = [(2, 1, 1, 4096, 0), (2, 5, 8, 14336, 0), (1, 149, 3, 4100, 0), (2, 700, 6, 333, 0), (2, 1024, 8, 96, 0), (2, 1025, 8, 96, 0),
          (2, 2400, 8, 2064, 0), (2, 2100, 8, 4100, 0), (2, 300, 8, 2048, 1025), (2, 300, 8, 2048, 40000), (8, 40, 6, 7392, 0),
          (2, 1536, 8, 2064, 0), (2, 1537, 8, 2064, 0), (2, 2048, 8, 96, 0), (2, 2049, 8, 96, 0), (2, 600, 8, 33008, 0), (2, 297, 8, 2048, 0),
-         (2, 74, 1, 2064, 0), (2, 75, 1, 16400, 0), (8, 1200, 8, 4096, 0), (8, 2300, 8, 1536, 0), (16, 30, 4, 4096, 2048), (32, 12, 8, 512, 4096), (2, 2100, 8, 16400, 0)]
+         (2, 74, 1, 2064, 0), (2, 75, 1, 16400, 0), (8, 1200, 8, 4096, 0), (8, 2300, 8, 1536, 0), (16, 30, 4, 4096, 2048), (32, 12, 8, 512, 4096), (2, 2100, 8, 16400, 0),
+         (2, 1000, 8, 7152, 0), (2, 1000, 8, 7168, 0)]
 
 
 @pytest.mark.parametrize("nodes,tokens,topk,row_bytes,k_max", CASES)
