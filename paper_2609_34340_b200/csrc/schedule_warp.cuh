@@ -259,7 +259,7 @@ __device__ __noinline__ uint64_t warp_families(const WarpUnits m, const uint32_t
     unsigned n_sweeps = 0;
 #pragma unroll 1
     for (int task0 = 0; task0 < n_tasks; task0 += 4) {
-        const int task = min(task0 + tsub, n_tasks - 1), h = task / n_start, t = task - h * n_start;
+        const int task = min(task0 + tsub, n_tasks - 1), h = H == 1 ? 0 : task / n_start, t = task - h * n_start;
         const bool mine = task0 + tsub < n_tasks, act = mine && a < G;
         const uint32_t* const fam = fam_task + ((f0 + h) * G + ag) * 8 + part * 2;
         const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
@@ -269,22 +269,24 @@ __device__ __noinline__ uint64_t warp_families(const WarpUnits m, const uint32_t
         const uint32_t bind = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
                               (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
         if (act) *(uint32_t*)(bindings + task * m.N + a * 4 + part * 2) = bind;
-        // Evaluate (Eq. 9, 10), needed only when several families compete: slowest lane under the final bindings
-        int64_t den = 1;
-        if (H > 1) {
-            int64_t tmax = 0;
-            if (act) {
-#pragma unroll
-                for (int i = 0; i < 2; i++) {
-                    const uint32_t bw = bind >> (16 * i), cl = ((i ? uo.y : uo.x) >> 24) & 0xfu;
-                    const uint32_t x = min_v(m.D[(int)(bw & 0xffu) * m.N + (int)((bw >> 8) & 0xffu)], m.cap[cl]);
-                    tmax = max_v(tmax, (int64_t)x * tscale[cl]);
-                }
-            }
-            tmax = team_max(tmax);
-            tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
-            den = F > 0 ? lambda_w + tmax : 1;
+        if (H == 1) {                                        // largest F, lowest start (F is 0 without a task)
+            const uint32_t best = __reduce_max_sync(0xffffffffu, F << 2 | (uint32_t)(3 - tsub));
+            if ((int64_t)(best >> 2) > bf) { bf = best >> 2; bt = task0 + 3 - (int)(best & 3u); }
+            continue;
         }
+        // Evaluate (Eq. 9, 10): slowest lane under the final bindings
+        int64_t tmax = 0;
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                const uint32_t bw = bind >> (16 * i), cl = ((i ? uo.y : uo.x) >> 24) & 0xfu;
+                const uint32_t x = min_v(m.D[(int)(bw & 0xffu) * m.N + (int)((bw >> 8) & 0xffu)], m.cap[cl]);
+                tmax = max_v(tmax, (int64_t)x * tscale[cl]);
+            }
+        }
+        tmax = team_max(tmax);
+        tmax = max_v(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
+        const int64_t den = F > 0 ? lambda_w + tmax : 1;
         // the round's results in task order (every lane follows along)
 #pragma unroll 1
         for (int s = 0; s < 4; s++) {
@@ -337,7 +339,7 @@ __device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams&
     const unsigned gmask = 0xffu << (8 * tsub);
     const uint32_t dst_1 = big_family_and_start(tsub, 4) & 0xffu;
     const uint32_t my_fam = (uint32_t)(ag * 8 + part * 2);
-    const bool act = a < G;
+    const bool mine_1 = tsub < kp.n_start, act = mine_1 && a < G;
     const int my_slot = lane < N ? lane : 0;
     unsigned n_sweeps = 0, n_done = 0;
     RowScores by_rows;
@@ -391,17 +393,19 @@ __device__ __forceinline__ void decompose_units(const DevCat& dc, const KParams&
             // (B) MultiStartAA, (C) best start per family, best family
             uint32_t wF, bind;                                   // F of the best start, source | destination << 8 of slot `lane`
             int wfam = f0;
-            if (usually(H == 1 && kp.n_start == 4)) {            // one family, one round: largest F, lowest start; bindings stay in registers
+            // One family, one round: largest F, lowest start; bindings stay in registers.  (Fewer starts than four leave lanes without a
+            // task, whose F is 0.  By the route out of line 256 matrices of 16 ranks took 128 and 139 us with one start and three, here 74 and 84.)
+            if (usually(H == 1 && kp.n_start <= 4)) {
                 const uint32_t* const fam = fam_task + (uint32_t)(f0 * G) * 8u + my_fam;
                 const uint2 uo = *(const uint2*)fam, ui = *(const uint2*)(fam + 4);
                 if (usually(pend)) write_row(k - 1, inst);
                 uint32_t src;
                 int dt0, dt1;
-                const uint32_t F = warp_tasks<ONE>(units, uo, ui, dst_1, true, act, part, gmask, kp.i_aa, n_sweeps, src, dt0, dt1);
+                const uint32_t F = warp_tasks<ONE>(units, uo, ui, dst_1, mine_1, act, part, gmask, kp.i_aa, n_sweeps, src, dt0, dt1);
                 VP_TICK(2);
                 const uint32_t mine = (uint32_t)(ag * 4 + 3 - (int)((src >> (6 - 4 * part)) & 3u)) | (uint32_t)((int)((uo.x >> 16) & 0xffu) * 4 + 3 - dt0) << 8 |
                                       (uint32_t)(ag * 4 + 3 - (int)((src >> (4 - 4 * part)) & 3u)) << 16 | (uint32_t)((int)((uo.y >> 16) & 0xffu) * 4 + 3 - dt1) << 24;
-                n_done += 4;
+                n_done += (unsigned)kp.n_start;
                 const uint32_t best = __reduce_max_sync(0xffffffffu, F << 2 | (uint32_t)(3 - tsub));     // (F is at most sixteen lanes of 2^22 granules)
                 wF = best >> 2;
                 bind = (__shfl_sync(0xffffffffu, mine, (int)(3u - (best & 3u)) << 3 | ((lane >> 1) & 7)) >> (16 * (lane & 1))) & 0xffffu;

@@ -259,6 +259,24 @@ def test_first_maximum_without_classes(vp, oracle_lib, name):  # noqa: F811
             ts._assert_same({key: plan[key][r:r + 6] for key in ts.KEYS}, {key: want[key][:min(6, B - r)] for key in ts.KEYS})
 
 
+@pytest.mark.parametrize("name", ["one_node", "two_nodes_64_50", "ring_of_three"])
+@pytest.mark.parametrize("n_start,i_aa", [(1, 3), (2, 1), (3, 3), (4, 2), (5, 3), (8, 4)])
+def test_starts_of_the_warp_kernel(vp, oracle_lib, name, n_start, i_aa):  # noqa: F811
+    """Fewer starts than the four that fill a warp, and more: one family of a shape and several; ties between starts."""
+    cat = CATALOGS[name]()
+    N = cat.topology.N
+    rng = np.random.default_rng(n_start)
+    D = (rng.integers(0, 900, size=(6, N, N)) * (rng.random((6, N, N)) < 0.5)).astype(np.int64)
+    D[1] = 1000
+    D[2] = 0
+    D[2][1, N - 2] = 77
+    D *= 256
+    for b in range(6):
+        np.fill_diagonal(D[b], 0)
+    got, want, *_ = ts._both(vp, oracle_lib, cat, D, WParams(granule_bytes=256, n_start=n_start, i_aa=i_aa).resolved(N))
+    ts._assert_same(got, want)
+
+
 def _repeated(cat, shapes):
     """The catalog with each of `shapes` followed by copies of itself: (shape, copies)."""
     order = [s for s in range(cat.n_shapes) for _ in range(1 + dict(shapes).get(s, 0))]
