@@ -243,6 +243,32 @@ __device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t
     __syncthreads();
     return big_warp_max64(lane < NT / 32 ? red[lane] : 0ull);
 }
+// The same class by class in 64 bits, for the chunks of more than sixteen groups (out of line, see there): a matrix of 2^30 granules and
+// more.  All threads of the CTA; the first maximal shape, -1 if all score zero.  (By the scan of all 4,095 shapes above, 16 matrices of
+// 256 ranks and 1.9 x 10^9 granules took 4,630 us, here 3,660.)
+__device__ __noinline__ int big_chunks_maximum(const uint32_t* tbl, uint64_t* red, const uint32_t* dec, int n_chunks, int n_classes) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int c = threadIdx.x >> 5; c < n_chunks; c += blockDim.x >> 5) {
+        const uint4 w = __ldg((const uint4*)(dec + dec[2]) + c * 32 + lane);
+        const uint64_t score = (uint64_t)tbl[w.x & 0xffffu] * (w.x >> 16) + (uint64_t)tbl[w.y & 0xffffu] * (w.y >> 16) + (uint64_t)tbl[w.z & 0xffffu] * (w.z >> 16);
+        const uint64_t key = big_warp_max64(w.w == 0xffffffffu ? 0ull : (score + 1) << 16 | (0xffffu - w.w));   // (equal scores: the lowest word)
+        if (lane == 0) red[c] = key;
+    }
+    __syncthreads();
+    uint64_t sum = 0;
+    if (lane < n_classes) {
+        uint64_t k0 = 0, k1 = 0;
+        const int c0 = (int)dec[3 + 2 * lane], c1 = (int)dec[4 + 2 * lane], c2 = (int)dec[5 + 2 * lane];
+#pragma unroll 1
+        for (int c = c0; c < c1; c++) k0 = max_v(k0, red[c]);
+#pragma unroll 1
+        for (int c = c1; c < c2; c++) k1 = max_v(k1, red[c]);
+        sum = ((k0 >> 16) + (k1 >> 16)) << 16 | ((k0 & 0xffffu) + (k1 & 0xffffu) - 0xffffu);      // 65535 - (run start + place)
+    }
+    sum = big_warp_max64(sum);
+    return (sum >> 16) > 2 ? 65535 - (int)(sum & 0xffffu) : -1;
+}
 // Family (of those that compete) and initial binding of a (family, start) task: h << 8 | binding, as a byte per group (see (B)).  Start t
 // binds in-slot q to row (q + t) mod 4.
 __device__ __noinline__ uint32_t big_family_and_start(int task, int n_start) {
@@ -903,6 +929,8 @@ vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand
                                 if (best > 2u) best_s = (int)s;
                             }
                         }
+                    } else if (!BY_LANE && by_class) {
+                        best_s = big_chunks_maximum(tbl, red, dc.dec, dc.dec_chunks, dc.dec_classes);
                     } else {
                         const uint64_t key = big_first_maximum(tbl, rs, red, pat, spat, dc.n_patterns, dc.max_row_terms, dc.n_shapes, S);
                         if (warp < n_task_warps && (key >> 16) != 0) best_s = 65535 - (int)(key & 0xffffu);

@@ -259,6 +259,24 @@ def test_first_maximum_without_classes(vp, oracle_lib, name):  # noqa: F811
             ts._assert_same({key: plan[key][r:r + 6] for key in ts.KEYS}, {key: want[key][:min(6, B - r)] for key in ts.KEYS})
 
 
+@pytest.mark.parametrize("nodes,k_max", [(17, 120), (24, 150), (32, 300)])
+def test_first_maximum_by_class_beyond_32_bits(vp, oracle_lib, nodes, k_max):  # noqa: F811
+    """Matrices of 2^30 granules and more with capacities of 16 bits, in the chunks of more than sixteen groups: every cell equal (all
+    scores tie; 17 nodes cross 2^30 on the way), random cells, and a cell left alone."""
+    cat = node_template_catalog(tree_topology(nodes))
+    N = cat.topology.N
+    rng = np.random.default_rng(nodes)
+    D = np.full((3, N, N), 58600 if nodes == 17 else 40000, dtype=np.int64)
+    D[1] += rng.integers(0, 2800 if nodes == 17 else 20000, size=(N, N))
+    D[2] = D[1] * (rng.random((N, N)) < 0.99)
+    D *= 256
+    for b in range(3):
+        np.fill_diagonal(D[b], 0)
+    assert D[0].sum() // 256 >= 1 << 30
+    got, want, *_ = ts._both(vp, oracle_lib, cat, D, WParams(granule_bytes=256, k_target=4 * N, k_max=k_max).resolved(N))
+    ts._assert_same(got, want)
+
+
 @pytest.mark.parametrize("name", ["one_node", "two_nodes_64_50", "ring_of_three"])
 @pytest.mark.parametrize("n_start,i_aa", [(1, 3), (2, 1), (3, 3), (4, 2), (5, 3), (8, 4)])
 def test_starts_of_the_warp_kernel(vp, oracle_lib, name, n_start, i_aa):  # noqa: F811
