@@ -27,7 +27,8 @@ constexpr int kMaxKeys = 1024;                      // experts_per_rank x N
 // which the two launches ahead of a copy that they replace (4 to 6 us) pay for up to here.  One launch | chunked, us, 16 ranks, rows of
 // 14,336 B: pack of 8,192 copies 24.1 | 29.8, 12,288 35.6 | 39.4, 16,384 46.9 | 49.0; unpack 19.5 | 25.8, 26.9 | 32.7, 34.5 | 39.7; return
 // 43.3 | 47.5, 63.5 | 64.6, 82.5 | 81.2.  Rows of 4,096 B, 16,384 items: 18.6 | 21.8, 17.3 | 20.5, 35.6 | 34.3; of 1,536 B 11.4 | 13.9,
-// 11.4 | 14.6, 17.1 | 21.3.  (The return counts twice, for both sides of its own range, over more keys: its line lies lower.)
+// 11.4 | 14.6, 17.1 | 21.3; of 96 B with 16 and 64 ranks against the chunked form as it was then, 8,704 items: pack 7.9 | 11.3 and 9.7 | 11.8,
+// return 8.5 | 16.1 and 10.5 | 18.6; 16,384 items: pack 9.5 | 11.9 and 11.3 | 13.4.  (The return counts twice, for both sides of its own range, over more keys: its line lies lower.)
 constexpr int kSmallItems = 16384;
 constexpr int kSmallReturn = 12288;
 constexpr int kSmallSteps = 1024;                   // plan arrays longer than this do not fit its run table
@@ -597,7 +598,8 @@ using OwnRing = OwnRingOf<kOwnSpins>;
 
 // Copies of `width` bytes, by rings from rows of min_bulk bytes on; ints(own) words of index in shared memory when a CTA owns up to `own` of the n rows.  With rings one CTA
 // per SM, as a CTA's index costs the same however many rows it owns; by plain loads two, for the loads in flight.  While there are
-// fewer rows than that, up to eight CTAs take a row's columns.
+// fewer rows than that, up to eight CTAs take a row's columns: with rings 74 rows are 148 CTAs and 75 rows 75 (pack of 74, 75, 96, 128, 147 and
+// 148 tokens x 8 of 14,336 B 5.9, 6.3, 6.5, 6.7, 6.8, 7.0 us; by plain loads and up to 296 CTAs 7.4, 7.4, 7.5, 8.3, 8.4, 8.4 before).
 template <typename Ints>
 inline SmallLaunch small_launch(int n, int sms, int fanout, long long row_bytes, int width, int min_bulk, Ints ints) {
     SmallLaunch z{};

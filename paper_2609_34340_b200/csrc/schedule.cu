@@ -1263,8 +1263,12 @@ int plan_launch_uncached(const vp_catalog* c, int B, const vp_sched_params* p, b
         // With 17 to 32 groups two lanes per group are two warps per task, which only the exact credits of hot columns are worth: 128 ranks,
         // half sequence parallel and half MoE in granules of 256 B, 148 matrices 2,617 by 1 and 2,856 by 2; without them 2 is faster
         // at every batch size (MoE, 16 matrices of 72, 96 and 128 ranks 749 | 823, 1,057 | 1,157, 1,501 | 1,650; 148 of 96 1,100 | 1,206).
-        // Capacities of 2^16 granules come with small granules, so granules of 4 KB and more (rows) start at 2,
-        // but not for plans in host memory, whose rows only 0 and 1 write in order (96 ranks, 128 matrices: 3,504 | 3,595).
+        // What decides is whether capacities reach 2^16 granules, which only the matrices tell; the granule stands for it.  Skewed MoE
+        // batches of 16,384 tokens a rank, rows of 14,336 B, shape 1 | 2, by granule: 148 of 128 ranks 256 B 7,140 | 7,407, 512 B 2,598 | 2,891,
+        // 1 KB 2,470 | 2,783, 2 KB 1,707 | 1,554; 148 of 72 ranks 3,299 | 3,470, 1,255 | 1,425, 1,226 | 1,379, 1,099 | 1,198.  Matrices whose
+        // capacities stay below lose 7 to 10 % by 1 at every granule (148 of 96 ranks, few tokens, 256 B to 8 KB: 1,198 | 1,098; sequence
+        // parallel 590 | 541).  So granules of 4 KB and more (rows, whose counts stay below 2^16) start at 2, but not for plans in host
+        // memory, whose rows only 0 and 1 write in order (96 ranks, 128 matrices: 3,504 | 3,595).
         const bool two_warps = L.kp.granule < 4096 || dc.G <= 16 || host_rows;
         for (int shape = dc.G > 32 ? 3 : (two_warps ? 0 : 2); shape < 4; shape++) {
             if (shape == 2 && dc.G <= 8) continue;

@@ -209,7 +209,9 @@ __device__ __noinline__ void big_write_in_order(int64_t* row, const int64_t* acc
 }
 
 // Eq. (6) by the general route, in 64 bits (out of line, as the loop should stay small for the instruction caches): scores beyond
-// 32 bits, and catalogs that have no class structure (see big_by_class).  All threads of the CTA; every
+// 32 bits (up to sixteen groups), and catalogs that have no class structure (see big_by_class; the template catalogs with their shapes in
+// another order, before the classes were the usual route and now: 16 and 1,024 matrices of 64 ranks 774 -> 668 and 1,567 -> 1,429 us, 148 of
+// 128 ranks 2,266 -> 1,976, 16 of 256 ranks 6,308 -> 6,088).  All threads of the CTA; every
 // warp gets the key of the first maximum, score << 16 | (65535 - shape): a score is at most four times what is left, so below 2^34,
 // and there are fewer than 2^16 shapes.
 __device__ __noinline__ uint64_t big_first_maximum(const uint32_t* tbl, uint64_t* rs, uint64_t* red, const uint32_t* pat, const uint32_t* spat,
@@ -412,9 +414,9 @@ __global__ void __launch_bounds__(256) big_rank_kernel(const int* __restrict__ k
 // a quarter more in all, so it is taken while the batch leaves SMs room.  Up to 32 lanes a task is part of a warp, 64 lanes
 // are two warps that meet at a barrier of their own.  Task warps are the first warps of the CTA (kp.big_task_warps),
 // the threads from warp kp.big_emit_warp on emit, a slot each.
-// ONE: all paths have one rate, so every slot the same capacity.  Selected per slot at run time it costs 5 to 9 %: 16 and 1,024 matrices
-// of 64 ranks 791 -> 830 and 1,589 -> 1,724 us, 512 of 256 ranks 12.6 -> 13.8 ms (two rates, links of 64 and NICs of 50 B/ns: 832 us,
-// 1,718 us, 14.2 ms, the last with 3 % more activations).
+// ONE: all paths have one rate, so every slot the same capacity.  Selected per slot at run time it costs 7 to 13 %: 16 and 1,024 matrices
+// of 64 ranks 519 -> 555 and 1,187 -> 1,300 us, 512 of 256 ranks 9.95 -> 11.25 ms (two rates, links of 64 and NICs of 50 B/ns: 559 us,
+// 1,300 us, 11.65 ms).
 template <int LANES, int SPLIT, bool ONE>
 __global__ void __launch_bounds__(LANES == 64 ? 384 : (SPLIT == 2 ? LANES * 6 : LANES * 8), LANES == 64 ? 1 : 64 / LANES)
 vp_schedule_big_kernel(DevCat dc, KParams kp, const int64_t* __restrict__ demand, const int64_t* __restrict__ tau_in, int B,

@@ -15,7 +15,7 @@
 //    (C) one warp maximum of F and start leaves the best start;
 //    (D) sixteen lanes take the activation off the residual, the credits (row-major and transposed) and D-hat; its plan rows
 //        are written in the shadow of the next activation's tasks.
-//    One matrix of 8 ranks 40.2 -> 30.4 us, 256 of 16 ranks 104.6 -> 81.1, 4,096 of 8 ranks 147.9 -> 111.5 by the code out of
+//    One matrix of 8 ranks 38.1 -> 29.4 us, 256 of 16 ranks 104.6 -> 81.1, 4,096 of 8 ranks 147.9 -> 111.5 by the code out of
 //    line, the credits kept ready and the last sweep's source half left out.
 //  * decompose_bytes: any other matrix, the same algorithm on 64-bit bytes with a lane per rank group.
 //
